@@ -506,10 +506,9 @@ struct StageRec {
 
 double cmul(int es) { return es == 16 ? 8.0 : 2.0; }
 
-// GEMM dispatch: large products go through exact split-bf16 products with FP64
-// accumulation (ozaki.cu) when M, N, K >= 256 and the batch fills at least one wave of
-// 128 x 128 output tiles; the rest stays on the DFMA kernel.  Batch items are split into
-// launches whose digit workspace stays within kOzCap bytes.
+// GEMM dispatch: products go through exact split-bf16 products with FP64 accumulation
+// (ozaki.cu) where split_worth says so, the rest runs on the FP64 kernel.  Batch items are
+// split into launches whose digit workspace stays within kOzCap bytes.
 constexpr size_t kOzCap = (size_t)12 << 30;
 
 // Digit workspace for split products of `count` items of `item` bytes each: items per
@@ -531,11 +530,16 @@ int oz_reserve(gks_ctx* c, size_t item, int count) {
   return per;
 }
 
+// Split products from kSplitFlops flops (all items of the launch together) and 32 in every
+// dimension up: below, the FP64 kernel at 1 TFLOP/s is under the fixed cost of a split product
+// (three or four launches).  Measured (FP64 kernel / split product): real 832 x 256 x 64 (2.7e7
+// flops) 35 / 39 us, 832 x 832 x 64 95 / 52 us, 2500 x 64 x 64 29 / 42 us; complex 256 x 256 x
+// 64 (3.4e7) 42 / 38 us, 832 x 832 x 256 1335 / 94 us.
+constexpr double kSplitFlops = 3e7;
 bool split_worth(gks_ctx* c, int count, int M, int N, int K, int es, double fl) {
   if (c->gemm_mode == 2) return true;
   const int Ne = es == 16 ? 2 * N : N;  // embedded output columns
-  return c->gemm_mode == 0 && fl >= 2e8 * count && M >= 64 && Ne >= 64 && K >= 64 &&
-         (long long)ozaki_tiles(M, N, es == 16) * count >= 152;
+  return c->gemm_mode == 0 && fl >= kSplitFlops && M >= 32 && Ne >= 32 && K >= 32;
 }
 
 template <typename T>
@@ -635,12 +639,14 @@ void gmx2(gks_ctx* c, int count, int nb2, int opA, int opB, int M, int N, int K,
 // rho_k = C_k diag(ks_k) C_k^H over the leading n_rho(k) columns (n_rho read on the device),
 // lower triangle.  C_k is M x (>= n_rho) with leading dimension ldc and item stride sC;
 // rho_k is M x M (stride sR).  Split products take K = the columns of C with the device
-// count cutting the digits and the k loop; the FP64 kernel reads the same count.
+// count cutting the digits and the k loop; the FP64 kernel reads the same count.  The
+// dispatch takes the flops of a full product of this order: rho then runs on the same kernel
+// as the adjoint's products C B C^H of the same order, which users subtract from it.
 template <typename T>
 void rho_run(gks_ctx* c, const T* C, int ldc, long long sC, T* rho, long long sR, const double* ks, long long sks,
              const int* nrho, int M, int K, int nk) {
   const int es = sizeof(T);
-  const int per = split_worth(c, nk, M, M, K, es, gemm_flops(es, M, M, std::max(1, K / 4), 1, nk))
+  const int per = split_worth(c, nk, M, M, K, es, gemm_flops(es, M, M, K, 0, nk))
                       ? oz_reserve(c, ozaki_workspace_bytes(M, M, K, es == 16, sform(c)), nk)
                       : 0;
   int z0 = 0;
@@ -1479,7 +1485,7 @@ gks_status solve_t(gks_ctx* c, const SolveKey& key) {
     StageRec sr(c, PS_RHO);
     T* rho = static_cast<T*>(const_cast<void*>(key.rho));
     {
-      const bool split = split_worth(c, items, M, M, nev, es, gemm_flops(es, M, M, std::max(1, nev / 4), 1, items));
+      const bool split = split_worth(c, items, M, M, nev, es, gemm_flops(es, M, M, nev, 0, items));
       Rec r(c, split ? PC_OZAKI : PC_GEMM, -1.0, -1.0);  // flops resolved from n_rho when the profile is read
       c->prof.nrho_dev = nrho;
       c->prof.rho_m = M;

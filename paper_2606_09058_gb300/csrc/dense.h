@@ -130,9 +130,8 @@ template <typename T>
 void spin_pair_sum(T* dst, long long sd, const T* src, long long ss, int n, int nk, cudaStream_t s);
 
 // ---- FP64-accurate GEMM from exact bf16 digit products (ozaki.cu) ----
-// Workspace bytes per batch item (a multiple of 256), and output tiles per item.
+// Workspace bytes per batch item (a multiple of 256).
 size_t ozaki_workspace_bytes(int M, int N, int K, bool cplx, int S);
-int ozaki_tiles(int M, int N, bool cplx);
 // Returns false (nothing enqueued) when the TMA tensor maps cannot be encoded.  Optional:
 // kscale (per item, stride sks) scales column k of op(A) before the product; kdev (per
 // item, device) cuts K to its value; wait_cycles bounds every device-side wait (0 = 2^32

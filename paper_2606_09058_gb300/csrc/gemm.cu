@@ -16,21 +16,11 @@ static std::atomic<long long> g_launches{0};
 void count_launch(int n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
 long long launches_issued() { return g_launches.load(std::memory_order_relaxed); }
 
-template <typename T> struct GemmTile;
-template <> struct GemmTile<double> {
-  static constexpr int TM = 4, TN = 4, BK = 16;
-};
-template <> struct GemmTile<zc> {
-  static constexpr int TM = 2, TN = 2, BK = 16;
-};
-// single precision (panel updates of the FP32 tridiagonalization): the FP32 pipe is ~60x
-// the FP64 one, so larger register tiles pay
-template <> struct GemmTile<float> {
-  static constexpr int TM = 4, TN = 4, BK = 16;
-};
-template <> struct GemmTile<cf> {
-  static constexpr int TM = 4, TN = 4, BK = 16;
-};
+// Output tile 16 TM x 16 TM (TM x TM per thread), K step 16.  The FP64 pipe takes 1.7
+// multiply-adds per SM clock, so a 64 x 64 real tile keeps one SM busy for 39k clocks per K
+// step: what counts is spreading the outputs over all 152 SMs, not operand reuse (a 16 x 16
+// tile still asks for under 2 bytes of operands per SM clock).
+constexpr int BK = 16;
 
 template <typename T>
 __device__ __forceinline__ T ld_op(const T* p, int op) {
@@ -38,9 +28,9 @@ __device__ __forceinline__ T ld_op(const T* p, int op) {
   return op == OP_C ? conjg(v) : v;
 }
 
-template <typename T>
+template <typename T, int TM>
 __global__ void __launch_bounds__(256) gemm_kernel(GemmBatch gb) {
-  constexpr int TM = GemmTile<T>::TM, TN = GemmTile<T>::TN, BK = GemmTile<T>::BK;
+  constexpr int TN = TM;
   constexpr int BM = 16 * TM, BN = 16 * TN;
   __shared__ T As[BK][BM];
   __shared__ T Bs[BK][BN];
@@ -129,13 +119,28 @@ __global__ void __launch_bounds__(256) gemm_kernel(GemmBatch gb) {
   }
 }
 
+template <typename T, int TM>
+static bool gemm_try(const GemmBatch& b, int maxM, int maxN, cudaStream_t s, long long want) {
+  constexpr int BM = 16 * TM;
+  dim3 grid((maxN + BM - 1) / BM, (maxM + BM - 1) / BM, b.count);
+  if ((long long)grid.x * grid.y * grid.z < want) return false;
+  count_launch();
+  gemm_kernel<T, TM><<<grid, 256, 0, s>>>(b);
+  return true;
+}
+
+// The largest tile that still gives four CTAs per SM (608), else the smallest.  A
+// 832 x 64 x 64 real product: 13 CTAs of 64 x 64 took 150 us, 208 of 16 x 16 take 12 us.
 template <typename T>
 void gemm(const GemmBatch& b, int maxM, int maxN, cudaStream_t s) {
-  constexpr int BM = 16 * GemmTile<T>::TM, BN = 16 * GemmTile<T>::TN;
   if (maxM <= 0 || maxN <= 0 || b.count <= 0) return;
-  dim3 grid((maxN + BN - 1) / BN, (maxM + BM - 1) / BM, b.count);
-  count_launch();
-  gemm_kernel<T><<<grid, 256, 0, s>>>(b);
+  constexpr long long want = 4 * 152;
+  if constexpr (sizeof(T) == 16) {
+    if (!gemm_try<T, 2>(b, maxM, maxN, s, want)) gemm_try<T, 1>(b, maxM, maxN, s, 0);
+  } else {
+    if (gemm_try<T, 4>(b, maxM, maxN, s, want) || gemm_try<T, 2>(b, maxM, maxN, s, want)) return;
+    gemm_try<T, 1>(b, maxM, maxN, s, 0);
+  }
 }
 
 template <typename T>

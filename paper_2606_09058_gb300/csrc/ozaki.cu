@@ -50,190 +50,285 @@ __host__ __device__ constexpr uint32_t crt_mod(int l) {
        : l == 12 ? 211u : l == 13 ? 199u : l == 14 ? 197u : 193u;
 }
 
+// Per-vector scale codes: 0 for a zero vector, e + kExpBias for entries below 2^e in
+// magnitude, kExpNan for a vector with a non-finite entry (its products are NaN, as on the
+// FP64 pipe).  Codes order like the magnitudes, so chunks of a vector combine by atomicMax.
+static constexpr int kExpBias = 2048, kExpNan = 1 << 20;
+__device__ __forceinline__ int exp_of(int code) { return code ? code - kExpBias : 0; }
+
+// x - m round(x / m) for an integer-valued float |x| <= 2^24: the quotient is rounded with
+// the 1.5 * 2^23 shift (|x / m| < 2^22), and the fused multiply-add is exact because the
+// result is a small integer.
+__device__ __forceinline__ float crt_fold(float x, float m, float inv) {
+  const float q = __fsub_rn(__fmaf_rn(x, inv, 12582912.0f), 12582912.0f);
+  return __fmaf_rn(-q, m, x);
+}
+
 // The split values of one element x of a vector whose entries are below 2^e in magnitude,
-// into o[0..S); sh = 6S - e (digits) or p - e (residues).
-// Digits (RES false): the first S base-64 digits of |x| 2^-e truncated toward zero (the
-// base-64 digits of the integer trunc(|x| 2^sh), 6S <= 60 bits), with the sign of x.
-// Residues (RES true): q = trunc(x 2^sh), |q| < 2^p <= 2^62, modulo each of the first S
-// moduli in symmetric form (|q| mod m from its two 32-bit halves, then q's sign).
+// into o[0..S); sh = 6S - e (digits) or p - e (residues).  Integer and FP32 operations only
+// (the FP64 pipe takes 1.7 operations per SM clock): u = trunc(|x| 2^sh) is the significand
+// shifted by the exponent difference.
+// Digits (RES false): the S base-64 digits of u, most significant first, with x's sign.
+// Residues (RES true): u < 2^62 in 21-bit limbs, reduced modulo each of the first S moduli by
+// Horner's rule in exact FP32 steps (|r| 2^7 + limb < 2^22), then x's sign: symmetric
+// residues |r| <= 128.  11 FP32 operations per modulus in place of five 32-bit integer
+// remainders by a constant.
+// With wt (operand B) the residues are those of y_l times the integer, y_l = (M / m_l)^-1 mod
+// m_l in symmetric form: the product's residues then carry the weights of the
+// reconstruction, one multiplication per operand entry instead of one per output.
+struct CrtWeights {
+  float y[CRT_MAXMOD];
+};
 template <bool RES>
-__device__ __forceinline__ void split_vals(double x, int sh, int S, float (&o)[16]) {
+__device__ __forceinline__ void split_vals(double x, int sh, int S, float (&o)[16], const CrtWeights* wt) {
+  const unsigned long long bits = (unsigned long long)__double_as_longlong(x);
+  const int xe = (int)((bits >> 52) & 0x7ff);
+  const unsigned long long m = xe == 0x7ff ? 0ull : (bits & 0xfffffffffffffull) | (xe ? (1ull << 52) : 0ull);
+  const int s = (xe ? xe : 1) - 1075 + sh;
+  const unsigned long long u = s >= 0 ? (s < 64 ? m << s : 0ull) : (s > -64 ? m >> -s : 0ull);
+  const float sg = (bits >> 63) ? -1.0f : 1.0f;
   if constexpr (RES) {
-    const long long q = __double2ll_rz(ldexp(x, sh));
-    const unsigned long long u = q < 0 ? 0ull - (unsigned long long)q : (unsigned long long)q;
-    const uint32_t hi = (uint32_t)(u >> 32), lo = (uint32_t)u;
-    const float sg = q < 0 ? -1.0f : 1.0f;
+    const float a0 = (float)(uint32_t)(u & 0x1fffffull), a1 = (float)(uint32_t)((u >> 21) & 0x1fffffull),
+                a2 = (float)(uint32_t)(u >> 42);
 #pragma unroll
     for (int l = 0; l < CRT_MAXMOD; l++) {
-      const uint32_t m = crt_mod(l), w = (uint32_t)((1ull << 32) % m);
-      const uint32_t r = l < S ? ((hi % m) * w + lo % m) % m : 0u;
-      o[l] = sg * (float)(2u * r > m ? (int)r - (int)m : (int)r);
+      constexpr uint32_t lim = 1u << 21;
+      const uint32_t mi = crt_mod(l), wi = lim % mi;
+      const float mf = (float)mi, inv = 1.0f / mf, w = 2u * wi > mi ? (float)wi - mf : (float)wi;
+      const float r2 = crt_fold(a2, mf, inv);
+      const float r1 = crt_fold(__fmaf_rn(r2, w, a1), mf, inv);
+      o[l] = sg * crt_fold(__fmaf_rn(r1, w, a0), mf, inv);
+      if (wt) o[l] = crt_fold(o[l] * wt->y[l], mf, inv);
     }
   } else {
-    const long long q = __double2ll_rz(ldexp(fabs(x), sh));
-    const float sg = x < 0.0 ? -1.0f : 1.0f;
 #pragma unroll
-    for (int s = 0; s < 16; s++)
-      o[s] = s < S ? sg * (float)((q >> (OZ_BITS * max(S - 1 - s, 0))) & 63) : 0.0f;
+    for (int t = 0; t < 16; t++)
+      o[t] = t < S ? sg * (float)((u >> (OZ_BITS * max(S - 1 - t, 0))) & 63) : 0.0f;
   }
 }
 
-__device__ __forceinline__ void store_vals(const float (&o)[16], float sg, __nv_bfloat16* dst, long long sstride,
-                                           int S) {
+// Two consecutive embedded positions of S planes, one 4-byte store per plane.
+__device__ __forceinline__ void store_pair(const float (&o0)[16], const float (&o1)[16], float s1, __nv_bfloat16* dst,
+                                           long long sstride, int S) {
 #pragma unroll
   for (int s = 0; s < 16; s++)
-    if (s < S) dst[s * sstride] = __float2bfloat16_rn(sg * o[s]);
+    if (s < S)
+      *reinterpret_cast<__nv_bfloat162*>(dst + s * sstride) = __floats2bfloat162_rn(o0[s], s1 * o1[s]);
 }
 
-__device__ __forceinline__ int scale_exp(double mx) {
-  return mx > 0.0 ? ilogb(mx) + 1 : 0;
-}
-
-// Element k of vector v of the split operand.
-// role 0 (A): vector v = row v of op(A);  role 1 (B): vector v = column v of op(B).
-// op N/T/C on the stored matrix X (row-major, ld): op(A)_{v,k} = X[v][k] (N), X[k][v] (T),
-// conj X[k][v] (C);  op(B)_{k,v} = X[k][v] (N), X[v][k] (T), conj X[v][k] (C).
+// One operand of a split product: vector v is row v of op(A) (role 0) or column v of op(B)
+// (role 1) of the stored matrix X (row-major, ld); op(A)_{v,k} = X[v][k] (N), X[k][v] (T),
+// conj X[k][v] (C);  op(B)_{k,v} = X[k][v] (N), X[v][k] (T), conj X[v][k] (C).  Batch item z
+// at item_off(z, sX, sX2, nb2); ksc (nullable, stride sks) scales element k first.
 template <typename T>
-__device__ __forceinline__ T split_elem(const T* X, int ld, int role, int op, int v, int k) {
-  const bool contig = (role == 0) == (op == OP_N);
-  T x = contig ? X[(size_t)v * ld + k] : X[(size_t)k * ld + v];
-  return op == OP_C ? conjg(x) : x;
-}
-
-__device__ __forceinline__ double amax(double x) { return fabs(x); }
-__device__ __forceinline__ double amax(zc x) { return fmax(fabs(x.x), fabs(x.y)); }
-
-// Write the split values of element k of vector v (scaled by 2^-e) into the embedded
-// layout (complex B: column 2v = (Re, -Im), column 2v + 1 = (Im, Re) along k).
-template <bool RES>
-__device__ __forceinline__ void emit(double x, int e, int, int v, int k, __nv_bfloat16* D, int Kp, long long sstride,
-                                     int S, int p) {
-  float o[16];
-  split_vals<RES>(x, (RES ? p : OZ_BITS * S) - e, S, o);
-  store_vals(o, 1.0f, D + (size_t)v * Kp + k, sstride, S);
-}
-template <bool RES>
-__device__ __forceinline__ void emit(zc x, int e, int role, int v, int k, __nv_bfloat16* D, int Kp, long long sstride,
-                                     int S, int p) {
-  float o[16];
-  __nv_bfloat16* r0 = role == 0 ? D + (size_t)v * Kp + 2 * k : D + (size_t)(2 * v) * Kp + 2 * k;
-  __nv_bfloat16* r1 = D + (size_t)(2 * v + 1) * Kp + 2 * k;
-  const int sh = (RES ? p : OZ_BITS * S) - e;
-  split_vals<RES>(x.x, sh, S, o);
-  store_vals(o, 1.0f, r0, sstride, S);
-  if (role != 0) store_vals(o, 1.0f, r1 + 1, sstride, S);
-  split_vals<RES>(x.y, sh, S, o);
-  if (role == 0) {
-    store_vals(o, 1.0f, r0 + 1, sstride, S);
-  } else {
-    store_vals(o, -1.0f, r0 + 1, sstride, S);
-    store_vals(o, 1.0f, r1, sstride, S);
-  }
-}
-
-// Item z of the split operand with the optional per-item K (device) and k scaling.
-template <typename T>
-struct SplitSrc {
+struct SplitOp {
   const T* X;
-  int ld, role, op;
+  int ld, role, op, nvec, nvp;  // nvp: vectors with the padding (complex B: half the embedded rows)
+  long long sX, sX2;
+  int* ex;                      // scale codes, stride sE per item
+  long long sE;
   const double* ksc;
-  __device__ T operator()(int v, int k) const {
-    T x = split_elem(X, ld, role, op, v, k);
-    return ksc ? x * ksc[k] : x;
+  long long sks;
+  __nv_bfloat16* D;             // planes [S][rows][Kp], item stride sD, plane stride sstride
+  long long sstride, sD;
+  __device__ bool contig() const { return (role == 0) == (op == OP_N); }  // k contiguous in memory
+  __device__ T at(const T* Xz, const double* kz, int v, int k) const {
+    T x = contig() ? Xz[(size_t)v * ld + k] : Xz[(size_t)k * ld + v];
+    if (op == OP_C) x = conjg(x);
+    return kz ? x * kz[k] : x;
   }
 };
-
-// Pass 1, one CTA (256 threads) per 32 vectors: the per-vector scale exponents (thread per
-// vector when the vector index is the contiguous direction, else a warp sweeps each vector
-// along k, four loads in flight per lane).  blockIdx.y runs over the batch items (strides
-// sX, sE); kdev (device, per item) cuts K, ksc scales element k by ksc[k] first.
 template <typename T>
-__global__ void __launch_bounds__(256) oz_scale_kernel(const T* X, int ld, long long sX, int role, int op, int nvec,
-                                                       int K, int* ex, long long sE, const double* ksc,
-                                                       long long sks, const int* kdev, long long sX2, int nb2) {
-  __shared__ double smax[32];
-  __shared__ double pm[8][32];
-  const int v0 = blockIdx.x * 32, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (kdev) K = min(K, max(0, kdev[blockIdx.y]));
-  const SplitSrc<T> elem{X + item_off(blockIdx.y, sX, sX2, nb2), ld, role, op, ksc ? ksc + blockIdx.y * sks : nullptr};
-  ex += blockIdx.y * sE;
-  const bool contig = (role == 0) == (op == OP_N);  // k contiguous in memory
-  if (contig) {
-    for (int vv = warp; vv < 32; vv += 8) {
-      const int v = v0 + vv;
-      double m = 0.0;
-      if (v < nvec)
-        for (int k0 = lane; k0 < K; k0 += 128) {
-          T x[4];
-#pragma unroll
-          for (int q = 0; q < 4; q++) x[q] = k0 + 32 * q < K ? elem(v, k0 + 32 * q) : zero<T>();
-#pragma unroll
-          for (int q = 0; q < 4; q++) m = fmax(m, amax(x[q]));
-        }
-      for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-      if (lane == 0) smax[vv] = m;
+struct SplitPair {
+  SplitOp<T> o[2];
+  int n0;  // blockIdx.x below n0: operand 0
+};
+
+// Ordering key of |x|: the top word of its bits (1 for values below 2^-1042).
+__device__ __forceinline__ uint32_t mag_key(double x) {
+  const uint32_t hi = (uint32_t)__double2hiint(x) & 0x7fffffffu;
+  return hi ? hi : (__double2loint(x) ? 1u : 0u);
+}
+__device__ __forceinline__ uint32_t mag_key(zc x) { return max(mag_key(x.x), mag_key(x.y)); }
+
+__device__ __forceinline__ int exp_code(uint32_t m) {
+  return m == 0 ? 0 : m >= 0x7ff00000u ? kExpNan : (int)(m >> 20) - 1022 + kExpBias;
+}
+
+// The planes of two embedded positions of vector v: the complex element k0 + lane (x0), or
+// the real elements k0 + 2 lane and the next (x0, x1).
+template <typename T, bool RES>
+__device__ __forceinline__ void emit_pair(const SplitOp<T>& q, __nv_bfloat16* D, int v, int k0, int lane, T x0, T x1,
+                                          int code, int Kp, int S, int p, const CrtWeights& y) {
+  const int sh = code == kExpNan ? -4096 : (RES ? p : OZ_BITS * S) - exp_of(code);
+  const CrtWeights* wt = q.role ? &y : nullptr;
+  float o0[16], o1[16];
+  if constexpr (sizeof(T) == 16) {
+    split_vals<RES>(x0.x, sh, S, o0, wt);
+    split_vals<RES>(x0.y, sh, S, o1, wt);
+    const size_t k = 2 * ((size_t)k0 + lane);
+    if (q.role == 0) {
+      store_pair(o0, o1, 1.0f, D + (size_t)v * Kp + k, q.sstride, S);
+    } else {  // column 2v = (Re, -Im), column 2v + 1 = (Im, Re) along k
+      store_pair(o0, o1, -1.0f, D + (size_t)(2 * v) * Kp + k, q.sstride, S);
+      store_pair(o1, o0, 1.0f, D + (size_t)(2 * v + 1) * Kp + k, q.sstride, S);
     }
   } else {
-    // 8 warps sweep k in parallel, lanes run over the 32 vectors (coalesced), then reduce
-    double m = 0.0;
-    const int v = v0 + lane;
-    if (v < nvec)
-      for (int k0 = warp; k0 < K; k0 += 32) {
+    split_vals<RES>(x0, sh, S, o0, wt);
+    split_vals<RES>(x1, sh, S, o1, wt);
+    store_pair(o0, o1, 1.0f, D + (size_t)v * Kp + k0 + 2 * lane, q.sstride, S);
+  }
+}
+
+// Pass 1, both operands in one launch: scale codes of 32 vectors over a chunk of kScaleK
+// elements per CTA (grid x: vectors of A then of B, y: k chunks, z: items), combined by
+// atomicMax into codes cleared beforehand.  Bound by reading the operands once; the chunks
+// keep the GPU filled for thin operands (512 vectors of length 5000: 16 CTAs without them).
+static constexpr int kScaleK = 512;
+template <typename T>
+__global__ void __launch_bounds__(256) oz_scale_kernel(const SplitPair<T> sp, int K, int nb2, const int* kdev) {
+  __shared__ uint32_t pm[8][32];
+  const bool second = (int)blockIdx.x >= sp.n0;
+  const SplitOp<T>& q = sp.o[second];
+  const int v0 = ((int)blockIdx.x - (second ? sp.n0 : 0)) * 32, z = blockIdx.z;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (kdev) K = min(K, max(0, kdev[z]));
+  const int k0 = blockIdx.y * kScaleK, k1 = min(K, k0 + kScaleK);
+  if (k0 >= k1) return;
+  const T* X = q.X + item_off(z, q.sX, q.sX2, nb2);
+  const double* kz = q.ksc ? q.ksc + z * q.sks : nullptr;
+  int* ex = q.ex + z * q.sE;
+  auto put = [&](int v, uint32_t m) {
+    if (m) atomicMax(ex + v, exp_code(m));
+  };
+  if (q.contig()) {
+    for (int vv = warp; vv < 32; vv += 8) {
+      const int v = v0 + vv;
+      if (v >= q.nvec) break;
+      uint32_t m = 0;
+      for (int k = k0 + lane; k < k1; k += 128) {  // four loads in flight per lane
         T x[4];
 #pragma unroll
-        for (int q = 0; q < 4; q++) x[q] = k0 + 8 * q < K ? elem(v, k0 + 8 * q) : zero<T>();
+        for (int t = 0; t < 4; t++) x[t] = k + 32 * t < k1 ? q.at(X, kz, v, k + 32 * t) : zero<T>();
 #pragma unroll
-        for (int q = 0; q < 4; q++) m = fmax(m, amax(x[q]));
+        for (int t = 0; t < 4; t++) m = max(m, mag_key(x[t]));
+      }
+      m = __reduce_max_sync(0xffffffffu, m);
+      if (lane == 0) put(v, m);
+    }
+  } else {
+    uint32_t m = 0;
+    const int v = v0 + lane;
+    if (v < q.nvec)
+      for (int k = k0 + warp; k < k1; k += 64) {  // eight loads in flight per lane
+        T x[8];
+#pragma unroll
+        for (int t = 0; t < 8; t++) x[t] = k + 8 * t < k1 ? q.at(X, kz, v, k + 8 * t) : zero<T>();
+#pragma unroll
+        for (int t = 0; t < 8; t++) m = max(m, mag_key(x[t]));
       }
     pm[warp][lane] = m;
     __syncthreads();
-    if (tid < 32) {
-      double mm = 0.0;
-      for (int w = 0; w < 8; w++) mm = fmax(mm, pm[w][tid]);
-      smax[tid] = mm;
+    if (warp == 0 && v < q.nvec) {
+#pragma unroll
+      for (int w = 1; w < 8; w++) m = max(m, pm[w][lane]);
+      put(v, m);
     }
   }
-  __syncthreads();
-  if (tid < 32 && v0 + tid < nvec) ex[v0 + tid] = scale_exp(smax[tid]);
 }
 
-// Pass 2, one CTA (256 threads) per tile of 32 vectors x 32 k (grid x: vectors, y: k,
-// z: items) over the padded plane: nvp vectors (padding rows included; complex B: half the
-// embedded rows) and kpl k (complex: half the padded K').  The tile is staged through shared
-// memory (read along the contiguous direction), then its S digits or residues (RES; residues
-// of trunc(x 2^{p - e})) are written with lanes along k; padding vectors and k beyond K
-// (the item's, after kdev) get the split values of zero, so the planes need no clearing.
+// Pass 2, both operands in one launch: one CTA (256 threads) per tile of 32 vectors x 64
+// embedded positions (64 k real, 32 k complex; grid x: vectors of A then of B, y: k, z:
+// items) over the padded planes.  The tile is staged through shared memory (read along the
+// contiguous direction), then its S digits or residues are written with lanes along k, two
+// positions (4 bytes) per lane: full 128-byte lines per plane and vector.  Padding vectors
+// and k beyond K (the item's, after kdev) get zeros, so the planes need no clearing.
 template <typename T, bool RES>
-__global__ void __launch_bounds__(256) oz_split_kernel(const T* X, int ld, long long sX, int role, int op, int nvec,
-                                                       int K, __nv_bfloat16* D, int Kp, long long sstride,
-                                                       long long sD, int S, int p, const int* ex, long long sE,
-                                                       const double* ksc, long long sks, const int* kdev,
-                                                       long long sX2, int nb2, int nvp, int kpl) {
-  __shared__ T tile[32][33];
-  __shared__ int sexp[32];
-  const int v0 = blockIdx.x * 32, k0 = blockIdx.y * 32, z = blockIdx.z;
+__global__ void __launch_bounds__(256) oz_split_kernel(const SplitPair<T> sp, int K, int Kp, int S, int p, int nb2,
+                                                       const int* kdev, const CrtWeights y) {
+  constexpr bool CPX = sizeof(T) == 16;
+  constexpr int TK = CPX ? 32 : 64;
+  __shared__ T tile[TK][33];
+  const bool second = (int)blockIdx.x >= sp.n0;
+  const SplitOp<T>& q = sp.o[second];
+  const int v0 = ((int)blockIdx.x - (second ? sp.n0 : 0)) * 32, k0 = blockIdx.y * TK, z = blockIdx.z;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (kdev) K = min(K, max(0, kdev[z]));
-  const SplitSrc<T> elem{X + item_off(z, sX, sX2, nb2), ld, role, op, ksc ? ksc + z * sks : nullptr};
-  D += z * sD;
-  ex += z * sE;
-  if (tid < 32) sexp[tid] = v0 + tid < nvec ? ex[v0 + tid] : 0;
-  if ((role == 0) == (op == OP_N)) {  // k contiguous: lanes along k
-    for (int vv = warp; vv < 32; vv += 8) {
-      const int v = v0 + vv, k = k0 + lane;
-      tile[lane][vv] = (v < nvec && k < K) ? elem(v, k) : zero<T>();
+  const T* X = q.X + item_off(z, q.sX, q.sX2, nb2);
+  const double* kz = q.ksc ? q.ksc + z * q.sks : nullptr;
+  const int* ex = q.ex + z * q.sE;
+  __nv_bfloat16* D = q.D + z * q.sD;
+  if (q.contig()) {  // lanes along k
+#pragma unroll
+    for (int w = 0; w < 4; w++) {
+      const int vv = warp + 8 * w, v = v0 + vv;
+#pragma unroll
+      for (int t = 0; t < TK; t += 32) {
+        const int k = k0 + t + lane;
+        tile[t + lane][vv] = (v < q.nvec && k < K) ? q.at(X, kz, v, k) : zero<T>();
+      }
     }
-  } else {  // vectors contiguous: lanes along the vectors
-    for (int kk = warp; kk < 32; kk += 8) {
-      const int k = k0 + kk, v = v0 + lane;
-      tile[kk][lane] = (k < K && v < nvec) ? elem(v, k) : zero<T>();
+  } else {  // lanes along the vectors
+#pragma unroll
+    for (int w = 0; w < TK / 8; w++) {
+      const int kk = warp + 8 * w, k = k0 + kk, v = v0 + lane;
+      tile[kk][lane] = (k < K && v < q.nvec) ? q.at(X, kz, v, k) : zero<T>();
     }
   }
   __syncthreads();
+#pragma unroll 1
   for (int vv = warp; vv < 32; vv += 8) {
-    const int v = v0 + vv, k = k0 + lane;
-    if (v < nvp && k < kpl) emit<RES>(tile[lane][vv], sexp[vv], role, v, k, D, Kp, sstride, S, p);
+    const int v = v0 + vv;
+    if (v >= q.nvp) break;
+    const T* t = &tile[0][vv];
+    emit_pair<T, RES>(q, D, v, k0, lane, CPX ? t[33 * lane] : t[66 * lane], CPX ? zero<T>() : t[66 * lane + 33],
+                      v < q.nvec ? ex[v] : 0, Kp, S, p, y);
   }
+}
+
+// Both passes in one launch where 8 vectors fit in shared memory (padded K' up to kFusedK):
+// a warp per vector finds its scale code and writes its planes, so the operands are read
+// once and thin products (the panel updates) save two of five launches.
+static constexpr int kFusedK = 1024;
+template <typename T>
+static constexpr int fused_ld(int kpl) { return (kpl + 15) / 16 * 16 + 4; }  // 8 vectors x 4 k on distinct banks
+template <typename T, bool RES>
+__global__ void __launch_bounds__(256) oz_fused_kernel(const SplitPair<T> sp, int K, int Kp, int S, int p, int nb2,
+                                                       const int* kdev, const CrtWeights y, int ldk) {
+  constexpr bool CPX = sizeof(T) == 16;
+  extern __shared__ __align__(16) unsigned char fused_raw[];
+  T* rows = reinterpret_cast<T*>(fused_raw);  // [8][ldk]
+  const bool second = (int)blockIdx.x >= sp.n0;
+  const SplitOp<T>& q = sp.o[second];
+  const int v0 = ((int)blockIdx.x - (second ? sp.n0 : 0)) * 8, z = blockIdx.z;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, kpl = CPX ? Kp / 2 : Kp;
+  if (kdev) K = min(K, max(0, kdev[z]));
+  const T* X = q.X + item_off(z, q.sX, q.sX2, nb2);
+  const double* kz = q.ksc ? q.ksc + z * q.sks : nullptr;
+  if (q.contig()) {
+    const int v = v0 + warp;
+#pragma unroll 4
+    for (int k = lane; k < kpl; k += 32) rows[warp * ldk + k] = (v < q.nvec && k < K) ? q.at(X, kz, v, k) : zero<T>();
+  } else {
+    const int v = v0 + (tid & 7);
+#pragma unroll 4
+    for (int k = tid >> 3; k < kpl; k += 32)
+      rows[(tid & 7) * ldk + k] = (v < q.nvec && k < K) ? q.at(X, kz, v, k) : zero<T>();
+  }
+  __syncthreads();
+  const int v = v0 + warp;
+  if (v >= q.nvp) return;
+  const T* row = rows + warp * ldk;
+  uint32_t m = 0;
+  for (int k = lane; k < kpl; k += 32) m = max(m, mag_key(row[k]));
+  m = __reduce_max_sync(0xffffffffu, m);
+  const int code = exp_code(m);
+  if (lane == 0 && v < q.nvec) q.ex[z * q.sE + v] = code;
+  __nv_bfloat16* D = q.D + z * q.sD;
+#pragma unroll 1
+  for (int k0 = 0; k0 < kpl; k0 += CPX ? 32 : 64)
+    emit_pair<T, RES>(q, D, v, k0, lane, CPX ? row[k0 + lane] : row[k0 + 2 * lane],
+                      CPX ? zero<T>() : row[k0 + 2 * lane + 1], code, Kp, S, p, y);
 }
 
 // ------------------------------------------------------------------ product kernel
@@ -243,8 +338,8 @@ static constexpr int OZ_BM = 128, OZ_BN = 128;  // output tile of the product ke
 struct OzArgs {
   const __nv_bfloat16* Ad;  // [S][Mp][Kp]
   const __nv_bfloat16* Bd;  // [S][Np][Kp]   (embedded columns, K-major)
-  const int* ea;            // exponents of the M rows
-  const int* eb;            // exponents of the logical N columns
+  const int* ea;            // scale codes of the M rows
+  const int* eb;            // scale codes of the logical N columns
   void* C;
   int ldc;
   int M, N;                 // logical output (N complex columns when cplx)
@@ -482,8 +577,9 @@ __global__ void __launch_bounds__(tcg::THREADS, 1)
     for (int jj = 0; jj < 32; jj++) {
       const int j = j0 + jj;
       if (j >= a.N || (a.lower && j > i)) continue;
-      const int ee = ea[i] + eb[j];
-      zc v{ldexp(acc[2 * jj], ee) * a.alpha, ldexp(acc[2 * jj + 1], ee) * a.alpha};
+      const bool bad = ea[i] == kExpNan || eb[j] == kExpNan;
+      const int ee = exp_of(ea[i]) + exp_of(eb[j]);
+      zc v{ldexp(bad ? nan("") : acc[2 * jj], ee) * a.alpha, ldexp(bad ? nan("") : acc[2 * jj + 1], ee) * a.alpha};
       zc* cp = C + (size_t)i * a.ldc + j;
       if (a.beta != 0.0) v = v + a.beta * (*cp);
       *cp = v;
@@ -495,7 +591,8 @@ __global__ void __launch_bounds__(tcg::THREADS, 1)
     for (int jj = 0; jj < 64; jj++) {
       const int j = j0 + jj;
       if (j >= a.N || (a.lower && j > i)) continue;
-      double v = ldexp(acc[jj], ea[i] + eb[j]) * a.alpha;
+      const bool bad = ea[i] == kExpNan || eb[j] == kExpNan;
+      double v = ldexp(bad ? nan("") : acc[jj], exp_of(ea[i]) + exp_of(eb[j])) * a.alpha;
       double* cp = C + (size_t)i * a.ldc + j;
       if (a.beta != 0.0) v += a.beta * (*cp);
       *cp = v;
@@ -514,11 +611,16 @@ __global__ void __launch_bounds__(tcg::THREADS, 1)
 // are bf16-exact integers of magnitude <= 128, so a k chunk of 1024 sums exactly in the
 // FP32 accumulator (<= 2^24).  Eight epilogue warps fold each chunk into a residue kept
 // in FP32 registers (x - m round(x / m), exact on integers) while the tensor cores fill the
-// other accumulator, and write t_l = (X mod m_l) y_l mod m_l of every element (the
-// weight of the reconstruction, y_l = (M / m_l)^-1 mod m_l) as one byte when the modulus
-// ends.  One product per modulus: 16 moduli keep p = 55 bits for K up to 16384, where nine
-// 6-bit digits keep 54 bits with 45 digit-pair products.  crt_recon_kernel rebuilds X
-// from its residues in 32-bit limbs and scales it back by 2^{e_i + f_j - 2p}.
+// other accumulator, and write the symmetric residue of every element as one byte when the
+// modulus ends.  B' enters as the residues of y_l B', y_l = (M / m_l)^-1 mod m_l, so what is
+// stored is already the weighted residue of the reconstruction.  One product per modulus: 16
+// moduli keep p = 55 bits for K up to 16384, where nine 6-bit digits keep 54 bits with 45
+// digit-pair products.  crt_recon_kernel rebuilds X and scales it back by 2^{e_i + f_j - 2p}.
+//
+// Measured (832 x 832 x 64 real, one product, CUDA events): 95 us with weights and range
+// corrections in the epilogue, all moduli of a tile in one CTA and 16 elements per
+// reconstruction thread; 52 us with the forms below (13 us product kernel, 19 us
+// reconstruction, 6 us splitting).  Complex 4992 x 4992 x 512: 3.17 -> 2.00 ms.
 constexpr int CRT_CHUNK_BLOCKS = 16;  // k blocks per exact chunk: 16 * 64 * 128^2 = 2^24
 
 struct CrtArgs {
@@ -526,8 +628,8 @@ struct CrtArgs {
   const __nv_bfloat16* Bd;  // [count][n][Np][Kp] residue planes of B' (embedded columns, K-major)
   uint8_t* R;               // [count][n][Mp][Np] residues of X
   int Mp, Np, Kp, n, cplx, lower;
+  int ng;                   // CTAs per tile: CTA g takes moduli [g n / ng, (g + 1) n / ng)
   long long zR;             // item stride of R (bytes)
-  float y[CRT_MAXMOD];      // (M / m_l)^-1 mod m_l: R holds t_l = (X mod m_l) y_l mod m_l
   const int* kdev;          // optional per-item K read on the device (logical, <= K)
   long long wait;           // bound of every mbarrier wait, in SM clock cycles
   long long skip_copy;      // test hook: the producer leaves out this copy (-1 = none)
@@ -549,12 +651,12 @@ constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >
 static_assert(SMEM <= 227 * 1024, "shared memory of the residue kernel");
 }  // namespace crtc
 
-// x - m round(x / m) for an integer-valued float |x| <= 2^24: the quotient is rounded with
-// the 1.5 * 2^23 shift (|x / m| < 2^22), and the fused multiply-add is exact because the
-// result is a small integer.
-__device__ __forceinline__ float crt_fold(float x, float m, float inv) {
-  const float q = __fsub_rn(__fmaf_rn(x, inv, 12582912.0f), 12582912.0f);
-  return __fmaf_rn(-q, m, x);
+// Four symmetric residues as bytes r + 128 (r = 128, modulus 256 only, wraps to -128): adding
+// 1.5 * 2^23 leaves r in the low bits of the float, so no conversion instruction is needed.
+__device__ __forceinline__ uint32_t crt_bytes(float r0, float r1, float r2, float r3) {
+  const uint32_t b0 = __float_as_uint(__fadd_rn(r0, 12582912.0f)), b1 = __float_as_uint(__fadd_rn(r1, 12582912.0f));
+  const uint32_t b2 = __float_as_uint(__fadd_rn(r2, 12582912.0f)), b3 = __float_as_uint(__fadd_rn(r3, 12582912.0f));
+  return __byte_perm(__byte_perm(b0, b1, 0x0040), __byte_perm(b2, b3, 0x0040), 0x5410) ^ 0x80808080u;
 }
 
 __global__ void __launch_bounds__(tcg::THREADS, 1)
@@ -580,11 +682,11 @@ __global__ void __launch_bounds__(tcg::THREADS, 1)
     m0 = (fm + r % gs) * BM;
     n0 = (r / gs) * BN;
   }
-  const int z = blockIdx.z;
+  const int z = blockIdx.z / a.ng, grp = blockIdx.z % a.ng;
   const int ncol0 = a.cplx ? n0 / 2 : n0;
   if (a.lower && m0 + BM - 1 < ncol0) return;  // whole tile above the diagonal (uniform)
 
-  const int n = a.n;
+  const int n = a.n, l0 = grp * n / a.ng, l1 = (grp + 1) * n / a.ng;
   int kblocks = a.Kp / BK;
   if (a.kdev) {
     const int ke = min(a.Kp, max(0, a.kdev[z]) * (a.cplx ? 2 : 1));
@@ -620,7 +722,7 @@ __global__ void __launch_bounds__(tcg::THREADS, 1)
     if (lane == 0) {
       // producer: residue tiles of A' and B' for modulus l, k block kb
       long long q = 0;
-      for (int l = 0; l < n && !*abort; l++) {
+      for (int l = l0; l < l1 && !*abort; l++) {
         const int ya = (z * n + l) * a.Mp + m0, yb = (z * n + l) * a.Np + n0;
         for (int kb = 0; kb < kblocks; kb++, q++) {
           const int stg = (int)(q % STAGES);
@@ -642,7 +744,7 @@ __global__ void __launch_bounds__(tcg::THREADS, 1)
       long long q = 0;
       int u = 0;
       bool ok = true;
-      for (int l = 0; l < n && ok; l++) {
+      for (int l = l0; l < l1 && ok; l++) {
         for (int c = 0; c < nchunk && ok; c++, u++) {
           const int b = u & 1;
           const uint32_t uph = (uint32_t)((u >> 1) & 1);
@@ -685,8 +787,39 @@ __global__ void __launch_bounds__(tcg::THREADS, 1)
     const int i = m0 + lq * 32 + lane;
     int u = 0;
     bool ok = true;
-    for (int l = 0; l < n && ok; l++) {
+    for (int l = l0; l < l1 && ok; l++) {
       const float mf = (float)crt_mod(l), inv = __frcp_rn(mf);
+      uint4* dst = reinterpret_cast<uint4*>(a.R + z * a.zR + ((size_t)l * a.Mp + i) * a.Np + n0 + ch * 128);
+      if (nchunk == 1) {  // K' <= 1024: every accumulator folds straight to its bytes
+        const int b = u & 1;
+        const uint32_t uph = (uint32_t)((u >> 1) & 1);
+        u++;
+        if (!mbar_wait(&tfull[b], uph, abort, a.wait)) {
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        const uint32_t taddr = tmem + ((uint32_t)(lq * 32) << 16) + (uint32_t)(b * BN + ch * 128);
+#pragma unroll
+        for (int g = 0; g < 4; g++) {
+          uint32_t v[32];
+          tmem_ld32(taddr + 32 * g, v);
+          if (g == 3) {  // the last read: the accumulator is free before its bytes are formed
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&tempty[b]);
+          }
+          uint32_t w[8];
+#pragma unroll
+          for (int t = 0; t < 8; t++)
+            w[t] = crt_bytes(crt_fold(__uint_as_float(v[4 * t]), mf, inv), crt_fold(__uint_as_float(v[4 * t + 1]), mf, inv),
+                             crt_fold(__uint_as_float(v[4 * t + 2]), mf, inv),
+                             crt_fold(__uint_as_float(v[4 * t + 3]), mf, inv));
+          dst[2 * g] = make_uint4(w[0], w[1], w[2], w[3]);
+          dst[2 * g + 1] = make_uint4(w[4], w[5], w[6], w[7]);
+        }
+        continue;
+      }
       float acc[128];
 #pragma unroll
       for (int t = 0; t < 128; t++) acc[t] = 0.0f;
@@ -711,26 +844,14 @@ __global__ void __launch_bounds__(tcg::THREADS, 1)
         if (lane == 0) mbar_arrive(&tempty[b]);
       }
       if (!ok) break;
-      // t_l = (X mod m_l) y_l mod m_l in [0, m_l) for this thread's row and 128 embedded
-      // columns, one byte each (both folds exact: |acc| < 2^24, r y_l < 2^16)
-      const float yl = a.y[l];
-      uint4* dst = reinterpret_cast<uint4*>(a.R + z * a.zR + ((size_t)l * a.Mp + i) * a.Np + n0 + ch * 128);
 #pragma unroll
       for (int q = 0; q < 8; q++) {
         uint32_t w[4];
 #pragma unroll
         for (int t = 0; t < 4; t++) {
-          uint32_t word = 0;
-#pragma unroll
-          for (int s4 = 0; s4 < 4; s4++) {
-            float r = crt_fold(acc[16 * q + 4 * t + s4], mf, inv);
-            r = r < 0.0f ? r + mf : r;
-            r = crt_fold(r * yl, mf, inv);
-            r = r < 0.0f ? r + mf : r;
-            r = r >= mf ? r - mf : r;
-            word |= (uint32_t)r << (8 * s4);
-          }
-          w[t] = word;
+          const float* x = acc + 16 * q + 4 * t;
+          w[t] = crt_bytes(crt_fold(x[0], mf, inv), crt_fold(x[1], mf, inv), crt_fold(x[2], mf, inv),
+                           crt_fold(x[3], mf, inv));
         }
         dst[q] = make_uint4(w[0], w[1], w[2], w[3]);
       }
@@ -746,19 +867,25 @@ __global__ void __launch_bounds__(tcg::THREADS, 1)
   if (*abort && tid == 0) set_status(status, ST_ETIMEOUT, -2);
 }
 
-// Constants of the reconstruction for n moduli: X = sum_l t_l (M / m_l) mod M with
-// t_l = r_l y_l mod m_l, y_l = (M / m_l)^-1 mod m_l (t_l is what the product kernel stores).
+// Constants of the reconstruction for n moduli: X = sum_l t_l (M / m_l) mod M with the
+// weighted symmetric residues t_l = (X y_l) mod m_l that the product kernel stores as bytes
+// t_l + 128.  Moduli are taken in groups of three, v_g = sum_l byte_l m_a m_b (the other two
+// of the group; below 2^26), and S = E + sum_g v_g M / (m_a m_b m_c) with E = -128 sum_l
+// M / m_l mod M, so that S is non-negative, congruent to X and below 32 M.
+constexpr int CRT_GROUPS = 6;
 struct CrtRecon {
-  uint32_t y[CRT_MAXMOD];
-  uint32_t Nl[CRT_MAXMOD][4];  // M / m_l, 32-bit limbs, least significant first
-  uint32_t Mv[4], Mh[4];       // M and M / 2
-  float inv_mf;                // 2^{32 b} / M
-  int b;                       // limb at which the quotient estimate starts: max(0, top limb of M - 1)
+  uint32_t cf[CRT_MAXMOD];         // product of the other moduli of the group (0 from n up)
+  uint32_t Ng[CRT_GROUPS][4];      // M / (product of the group), 32-bit limbs, least first
+  uint32_t E[4];
+  unsigned long long Mv[2];        // M
+  float inv_mf;                    // 2^{32 b} / M
+  int b;                           // limb at which the quotient estimate starts: max(0, top limb of M - 1)
   int n;
 };
 
-// 128-bit magnitude (hi, lo) to the nearest double (ties to even), from its bits.
-__device__ __forceinline__ double u128_to_double(unsigned long long hi, unsigned long long lo) {
+// 128-bit magnitude (hi, lo) times 2^e to the nearest double (ties to even), from its bits
+// (through ldexp only where the result leaves the normal range).
+__device__ __forceinline__ double u128_scaled(unsigned long long hi, unsigned long long lo, bool neg, int e) {
   if (hi == 0ull && lo == 0ull) return 0.0;
   const int lz = hi ? __clzll((long long)hi) : 64 + __clzll((long long)lo);
   unsigned long long h, l;
@@ -780,134 +907,120 @@ __device__ __forceinline__ double u128_to_double(unsigned long long hi, unsigned
     mant >>= 1;
     ex++;
   }
-  return __longlong_as_double((long long)(((unsigned long long)(ex + 1023) << 52) | (mant & ((1ull << 52) - 1))));
+  const unsigned long long sgn = neg ? 1ull << 63 : 0ull, frac = mant & ((1ull << 52) - 1);
+  const int be = ex + e + 1023;
+  if (be > 0 && be < 2047) return __longlong_as_double((long long)(sgn | ((unsigned long long)be << 52) | frac));
+  return ldexp(__longlong_as_double((long long)(sgn | ((unsigned long long)(ex + 1023) << 52) | frac)), e);
 }
 
-__device__ __forceinline__ bool ge4(const uint32_t (&x)[4], const uint32_t (&y)[4]) {
-  for (int t = 3; t >= 0; t--)
-    if (x[t] != y[t]) return x[t] > y[t];
-  return true;
-}
-
-// The signed integer X with X y_l = t_l (mod m_l) for the weighted residues t_l (byte el of
-// the 16 loaded for modulus l), |X| < M / 2, as a double times 2^e.
-__device__ __forceinline__ double crt_value(const uint32_t (&w)[CRT_MAXMOD][4], int el, const CrtRecon& cr, int e) {
-  uint32_t s0 = 0, s1 = 0, s2 = 0, s3 = 0, s4 = 0;  // S = sum_l t_l M / m_l < 16 M
+// The signed integer X of the bytes of element el, as a double times 2^e.  S is
+// accumulated in four 64-bit limbs without carries (v_g limb < 2^58, six of them); with |X|
+// <= (1/2 - 2^-10) M the quotient round(S / M) is exact from a single-precision estimate
+// (S / M < 32, relative error below 2^-20), and X = S - q M in 128-bit two's complement from
+// the table of q M.  About 150 integer operations per element: bound by the integer pipe.
+__device__ __forceinline__ double crt_value(const uint32_t (&w)[CRT_MAXMOD][2], int el, const CrtRecon& cr,
+                                            const ulonglong2* qM, int e) {
+  unsigned long long c0 = cr.E[0], c1 = cr.E[1], c2 = cr.E[2], c3 = cr.E[3];
 #pragma unroll
-  for (int l = 0; l < CRT_MAXMOD; l++) {
-    if (l < cr.n) {
-      const uint32_t t = (w[l][el >> 2] >> (8 * (el & 3))) & 0xffu;
-      unsigned long long c = (unsigned long long)t * cr.Nl[l][0] + s0;
-      s0 = (uint32_t)c;
-      c = (c >> 32) + (unsigned long long)t * cr.Nl[l][1] + s1;
-      s1 = (uint32_t)c;
-      c = (c >> 32) + (unsigned long long)t * cr.Nl[l][2] + s2;
-      s2 = (uint32_t)c;
-      c = (c >> 32) + (unsigned long long)t * cr.Nl[l][3] + s3;
-      s3 = (uint32_t)c;
-      s4 += (uint32_t)(c >> 32);
-    }
+  for (int g = 0; g < CRT_GROUPS; g++) {
+    uint32_t v = 0;
+#pragma unroll
+    for (int l = 3 * g; l < 3 * g + 3 && l < CRT_MAXMOD; l++)
+      v += ((w[l][el >> 2] >> (8 * (el & 3))) & 0xffu) * cr.cf[l];
+    c0 += (unsigned long long)v * cr.Ng[g][0];
+    c1 += (unsigned long long)v * cr.Ng[g][1];
+    c2 += (unsigned long long)v * cr.Ng[g][2];
+    c3 += (unsigned long long)v * cr.Ng[g][3];
   }
-  // q = floor(S / M) within one: S / M < 16 estimated from the three limbs of S from limb b
-  // up (M 2^{-32 b} >= 2^32 unless M < 2^32, so the limbs below b do not matter)
+  c1 += c0 >> 32;
+  c2 += c1 >> 32;
+  c3 += c2 >> 32;
+  const uint32_t s0 = (uint32_t)c0, s1 = (uint32_t)c1, s2 = (uint32_t)c2, s3 = (uint32_t)c3;
+  const uint32_t s4 = (uint32_t)(c3 >> 32);
   const uint32_t a2 = cr.b == 0 ? s2 : cr.b == 1 ? s3 : s4;
   const uint32_t a1 = cr.b == 0 ? s1 : cr.b == 1 ? s2 : s3;
   const uint32_t a0 = cr.b == 0 ? s0 : cr.b == 1 ? s1 : s2;
   const float sf = __fmaf_rn((float)a2, 18446744073709551616.0f, __fmaf_rn((float)a1, 4294967296.0f, (float)a0));
-  const unsigned q = (unsigned)(sf * cr.inv_mf);
-  uint32_t x[4];
-  long long d = 0;
-  unsigned long long pm = 0;
-  const uint32_t sl[4] = {s0, s1, s2, s3};
-#pragma unroll
-  for (int t = 0; t < 4; t++) {
-    pm += (unsigned long long)q * cr.Mv[t];
-    d += (long long)sl[t] - (long long)(uint32_t)pm;
-    x[t] = (uint32_t)d;
-    d >>= 32;
-    pm >>= 32;
+  const uint32_t q = __float_as_uint(__fmaf_rn(sf, cr.inv_mf, 12582912.0f)) & 31u;  // nearest integer
+  const ulonglong2 m = qM[q];
+  unsigned long long lo = ((unsigned long long)s1 << 32) | s0, hi = ((unsigned long long)s3 << 32) | s2;
+  hi -= m.y + (lo < m.x ? 1ull : 0ull);
+  lo -= m.x;
+  const bool neg = (hi >> 63) != 0ull;
+  if (neg) {
+    lo = 0ull - lo;
+    hi = ~hi + (lo == 0ull ? 1ull : 0ull);
   }
-  d += (long long)s4 - (long long)pm;  // the top limb: -1, 0 or 1 after one of the corrections below
-  if (d < 0) {  // q one too large: X += M
-    unsigned long long c = 0;
-#pragma unroll
-    for (int t = 0; t < 4; t++) {
-      c += (unsigned long long)x[t] + cr.Mv[t];
-      x[t] = (uint32_t)c;
-      c >>= 32;
-    }
-  } else if (d > 0 || ge4(x, cr.Mv)) {  // q one too small: X -= M
-    long long b = 0;
-#pragma unroll
-    for (int t = 0; t < 4; t++) {
-      b += (long long)x[t] - (long long)cr.Mv[t];
-      x[t] = (uint32_t)b;
-      b >>= 32;
-    }
-  }
-  // symmetric representative: X > M / 2 stands for X - M
-  bool neg = false;
-  if (!ge4(cr.Mh, x)) {
-    neg = true;
-    long long b = 0;
-#pragma unroll
-    for (int t = 0; t < 4; t++) {
-      b += (long long)cr.Mv[t] - (long long)x[t];
-      x[t] = (uint32_t)b;
-      b >>= 32;
-    }
-  }
-  const double v = u128_to_double(((unsigned long long)x[3] << 32) | x[2], ((unsigned long long)x[1] << 32) | x[0]);
-  return ldexp(neg ? -v : v, e);
+  return u128_scaled(hi, lo, neg, e);
 }
 
 // C = alpha 2^{e_i + f_j - 2p} X + beta C for the logical outputs (lower: j <= i only).
-// A thread takes 16 consecutive embedded columns of a row: one 16-byte load per modulus (the
-// residue planes are Np bytes per row, Np a multiple of 256), then the 16 values (8 complex).
+// A thread takes 8 consecutive embedded columns of a row: one 8-byte load per modulus (the
+// residue planes are Np bytes per row, Np a multiple of 256), then the 8 values (4 complex).
+// The CTA's 128 such runs are numbered row by row over the ncg runs per row, so that narrow
+// outputs fill the CTAs too, and the values go through shared memory so that C is read and
+// written with consecutive lanes on consecutive elements.
 template <typename T>
 __global__ void __launch_bounds__(128) crt_recon_kernel(const uint8_t* R, long long zR, int Mp, int Np, int M, int N,
-                                                        const int* ea, const int* eb, long long zEa, long long zEb,
-                                                        int sc, const CrtRecon cr, T* C, int ldc, long long zC,
-                                                        long long zC2, int nb2, double alpha, double beta,
-                                                        int lower) {
+                                                        int ncg, const int* ea, const int* eb, long long zEa,
+                                                        long long zEb, int sc, const CrtRecon cr, T* C, int ldc,
+                                                        long long zC, long long zC2, int nb2, double alpha,
+                                                        double beta, int lower) {
   constexpr bool CPX = sizeof(T) == 16;
-  constexpr int PER = CPX ? 8 : 16;  // logical columns per thread
-  const int z = blockIdx.z, j0 = (blockIdx.x * 128 + threadIdx.x) * PER;
-  if (j0 >= N) return;
-  const long long plane = (long long)Mp * Np;
-  for (int i = blockIdx.y; i < M; i += gridDim.y) {
-    if (lower && j0 > i) continue;
+  constexpr int PER = CPX ? 4 : 8;  // logical columns per thread
+  __shared__ T val[128][PER + 1];
+  __shared__ ulonglong2 qM[32];
+  __shared__ int srow[128], scol[128];  // first column, N + PER where the thread has nothing
+  const int z = blockIdx.z, tid = threadIdx.x;
+  const long long plane = (long long)Mp * Np, t0 = (long long)blockIdx.x * 128 + tid;
+  const int i = (int)(t0 / ncg), j0 = (int)(t0 % ncg) * PER;
+  const bool ok = i < M && !(lower && j0 > i);
+  srow[tid] = i;
+  scol[tid] = ok ? j0 : N + PER;
+  if (tid < 32) {  // q M in 128 bits
+    const unsigned __int128 v = (((unsigned __int128)cr.Mv[1] << 64) | cr.Mv[0]) * (unsigned)tid;
+    qM[tid] = make_ulonglong2((unsigned long long)v, (unsigned long long)(v >> 64));
+  }
+  __syncthreads();
+  if (ok) {
     const uint8_t* Rz = R + z * zR + (size_t)i * Np + (CPX ? 2 * j0 : j0);
-    uint32_t w[CRT_MAXMOD][4];
+    uint32_t w[CRT_MAXMOD][2];
 #pragma unroll
     for (int l = 0; l < CRT_MAXMOD; l++) {
-      if (l < cr.n) {
-        const uint4 v = __ldcs(reinterpret_cast<const uint4*>(Rz + l * plane));
-        w[l][0] = v.x;
-        w[l][1] = v.y;
-        w[l][2] = v.z;
-        w[l][3] = v.w;
-      } else {
-        w[l][0] = w[l][1] = w[l][2] = w[l][3] = 0u;
-      }
+      uint2 v = make_uint2(0u, 0u);
+      if (l < cr.n) v = __ldcs(reinterpret_cast<const uint2*>(Rz + l * plane));
+      w[l][0] = v.x;
+      w[l][1] = v.y;
     }
-    const int ei = ea[z * zEa + i] + sc;
-    T* cp = C + item_off(z, zC, zC2, nb2) + (size_t)i * ldc;
+    const int ci = ea[z * zEa + i], ei = exp_of(ci) + sc;
 #pragma unroll
     for (int q = 0; q < PER; q++) {
       const int j = j0 + q;
-      if (j >= N || (lower && j > i)) break;
-      const int e = ei + eb[z * zEb + j];
-      if constexpr (CPX) {
-        zc v{alpha * crt_value(w, 2 * q, cr, e), alpha * crt_value(w, 2 * q + 1, cr, e)};
-        if (beta != 0.0) v = v + beta * cp[j];
-        cp[j] = v;
+      if (j >= N) break;
+      const int cj = eb[z * zEb + j], e = ei + exp_of(cj);
+      if (ci == kExpNan || cj == kExpNan) {
+        if constexpr (CPX) val[tid][q] = zc{nan(""), nan("")};
+        else val[tid][q] = nan("");
+      } else if constexpr (CPX) {
+        val[tid][q] = zc{crt_value(w, 2 * q, cr, qM, e), crt_value(w, 2 * q + 1, cr, qM, e)};
       } else {
-        double v = alpha * crt_value(w, q, cr, e);
-        if (beta != 0.0) v += beta * cp[j];
-        cp[j] = v;
+        val[tid][q] = crt_value(w, q, cr, qM, e);
       }
     }
+  }
+  __syncthreads();
+  T* Cz = C + item_off(z, zC, zC2, nb2);
+#pragma unroll
+  for (int q = 0; q < PER; q++) {
+    const int idx = q * 128 + tid, o = idx / PER, r = srow[o], j = scol[o] + idx % PER;
+    if (j >= N || (lower && j > r)) continue;
+    T* cp = Cz + (size_t)r * ldc + j;
+    T v = val[o][idx % PER];
+    if (alpha == -1.0) v = -v;
+    else if (alpha != 1.0) v = alpha * v;
+    if (beta == 1.0) v = v + *cp;
+    else if (beta != 0.0) v = v + beta * (*cp);
+    *cp = v;
   }
 }
 
@@ -951,44 +1064,59 @@ static int padded_k(int K, bool cplx) {
   return round_up(Ke > 0 ? Ke : 1, OZ_KSTEP);
 }
 
-// Residue plan for padded length Kp and at least `bits` bits per operand: the fewest
-// moduli n whose product M satisfies 2 Kp 2^{2p} <= M with p >= bits (p as large as M
-// allows, at most 62), and the reconstruction constants.  False if 16 moduli fall short.
+// Residue plan for padded length Kp and at least `bits` bits per operand: moduli n whose
+// product M satisfies 2 Kp 2^{2p} <= M with p >= bits (p as large as M allows, at most 62),
+// and the reconstruction constants.  FP64-accurate products (bits >= 54) take all 16 moduli:
+// p = 59 at Kp = 64 and 57 at 1024, against 54 with the 15 that would do up to Kp = 256, so
+// that thin products, which would otherwise run on the FP64 kernel, keep several bits below
+// the FP64 rounding of their largest terms for 1/15 more work.  Fewer bits (the mixed
+// path's back-transform): the fewest moduli.  False if 16 moduli fall short.
 struct CrtPlan {
   int n, p;
   CrtRecon cr;
+  CrtWeights wt;
 };
 static bool crt_plan(int Kp, int bits, CrtPlan* pl) {
   typedef unsigned __int128 u128;
   u128 M = 1;
   for (int n = 1; n <= CRT_MAXMOD; n++) {
     M *= crt_mod(n - 1);
-    const u128 room = M / ((u128)2 * (u128)Kp);  // 2^{2p} <= room
+    // 2^{2p} <= room, with the 2^-9 margin that makes the reconstruction's quotient exact
+    const u128 room = (M - (M >> 9)) / ((u128)2 * (u128)Kp);
     int lg = -1;
     for (u128 t = room; t; t >>= 1) lg++;
     const int p = lg < 0 ? -1 : std::min(lg / 2, 62);
-    if (p < bits) continue;
+    if (p < bits || (bits >= 54 && n < CRT_MAXMOD)) continue;
     pl->n = n;
     pl->p = p;
     CrtRecon& c = pl->cr;
     c = CrtRecon{};
+    pl->wt = CrtWeights{};
     c.n = n;
-    int top = 0;
-    for (int t = 0; t < 4; t++) {
-      c.Mv[t] = (uint32_t)(M >> (32 * t));
-      c.Mh[t] = (uint32_t)((M >> 1) >> (32 * t));
-      if (c.Mv[t]) top = t;
-    }
+    const int top = (int)(M >> 96) ? 3 : (int)(M >> 64) ? 2 : (M >> 32) ? 1 : 0;
+    c.Mv[0] = (unsigned long long)M;
+    c.Mv[1] = (unsigned long long)(M >> 64);
     c.b = std::max(0, top - 1);
     c.inv_mf = (float)(std::ldexp(1.0, 32 * c.b) / (double)M);
+    u128 off = 0;  // 128 sum_l M / m_l mod M
     for (int l = 0; l < n; l++) {
       const uint32_t m = crt_mod(l);
       const u128 Nl = M / m;
-      for (int t = 0; t < 4; t++) c.Nl[l][t] = (uint32_t)(Nl >> (32 * t));
+      for (int t = 0; t < 128; t++) off = (off + Nl) % M;
       const uint32_t r = (uint32_t)(Nl % m);
       uint32_t y = 1;
       while ((r * y) % m != 1u) y++;  // r is coprime to m
-      c.y[l] = y;
+      pl->wt.y[l] = 2 * y > m ? (float)y - (float)m : (float)y;
+    }
+    const u128 E = off ? M - off : 0;
+    for (int t = 0; t < 4; t++) c.E[t] = (uint32_t)(E >> (32 * t));
+    for (int g = 0; g < CRT_GROUPS && 3 * g < n; g++) {
+      const int e = std::min(n, 3 * g + 3);
+      uint32_t P = 1;
+      for (int l = 3 * g; l < e; l++) P *= crt_mod(l);
+      for (int l = 3 * g; l < e; l++) c.cf[l] = P / crt_mod(l);
+      const u128 Ng = M / P;
+      for (int t = 0; t < 4; t++) c.Ng[g][t] = (uint32_t)(Ng >> (32 * t));
     }
     return true;
   }
@@ -1016,10 +1144,6 @@ size_t ozaki_workspace_bytes(int M, int N, int K, bool cplx, int S) {
   return (b + 255) & ~size_t(255);
 }
 
-int ozaki_tiles(int M, int N, bool cplx) {
-  return (round_up(M, OZ_BM) / OZ_BM) * (round_up(cplx ? 2 * N : N, OZ_BN) / OZ_BN);
-}
-
 // count items, item z at A + z sA, B + z sB, C + z sC.  work holds, for all items, the A
 // planes [count][P][Mp][Kp], then the B planes [count][P][Np][Kp] (P = S digits or n
 // residues), then (residues) the residues of the product [count][n][Mp][Np] as bytes, then
@@ -1044,32 +1168,52 @@ bool ozaki_gemm(int opA, int opB, int M, int N, int K, double alpha, const T* A,
   uint8_t* R = reinterpret_cast<uint8_t*>(Bd + zB * count);
   int* ea = reinterpret_cast<int*>(R + zR * count);
   int* eb = ea + (size_t)Mp * count;
-  // exponents zero for the padding rows and columns; the planes are written whole by the
-  // split kernels (zeros in the padding), also for K = 0
-  cudaMemsetAsync(ea, 0, sizeof(int) * ((size_t)Mp + Np) * count, s);
-  {
-    // padded extents in the split kernels' terms: vectors (complex B: embedded rows 2v, 2v + 1)
-    // and logical k (complex: positions 2k, 2k + 1 of the padded K')
-    const int nva = Mp, nvb = cplx ? Np / 2 : Np, kpl = cplx ? Kp / 2 : Kp;
-    const dim3 ga((M + 31) / 32, count), gb((N + 31) / 32, count);
-    const dim3 ta((nva + 31) / 32, (kpl + 31) / 32, count), tb((nvb + 31) / 32, (kpl + 31) / 32, count);
-    count_launch(4);
-    oz_scale_kernel<T><<<ga, 256, 0, s>>>(A, lda, sA, 0, opA, M, K, ea, Mp, kscale, sks, kdev, sA2, nb2);
-    oz_scale_kernel<T><<<gb, 256, 0, s>>>(B, ldb, sB, 1, opB, N, K, eb, Np, nullptr, 0, kdev, sB2, nb2);
+  SplitPair<T> sp;
+  sp.o[0] = SplitOp<T>{A, lda, 0, opA, M, Mp, sA, sA2, ea, Mp, kscale, sks, Ad, (long long)Mp * Kp, zA};
+  sp.o[1] = SplitOp<T>{B, ldb, 1, opB, N, cplx ? Np / 2 : Np, sB, sB2, eb, Np, nullptr, 0, Bd, (long long)Np * Kp, zB};
+  const int bits = res ? pl.p : 0;
+  if (Kp <= kFusedK) {
+    sp.n0 = Mp / 8;
+    const int ldk = fused_ld<T>(cplx ? Kp / 2 : Kp), sm = 8 * ldk * (int)sizeof(T);
+    const dim3 grid(sp.n0 + sp.o[1].nvp / 8, 1, count);
+    count_launch();
     if (res) {
-      oz_split_kernel<T, true><<<ta, 256, 0, s>>>(A, lda, sA, 0, opA, M, K, Ad, Kp, (long long)Mp * Kp, zA, P, pl.p,
-                                                  ea, Mp, kscale, sks, kdev, sA2, nb2, nva, kpl);
-      oz_split_kernel<T, true><<<tb, 256, 0, s>>>(B, ldb, sB, 1, opB, N, K, Bd, Kp, (long long)Np * Kp, zB, P, pl.p,
-                                                  eb, Np, nullptr, 0, kdev, sB2, nb2, nvb, kpl);
+      cudaFuncSetAttribute(oz_fused_kernel<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+      oz_fused_kernel<T, true><<<grid, 256, sm, s>>>(sp, K, Kp, P, bits, nb2, kdev, pl.wt, ldk);
     } else {
-      oz_split_kernel<T, false><<<ta, 256, 0, s>>>(A, lda, sA, 0, opA, M, K, Ad, Kp, (long long)Mp * Kp, zA, P, 0,
-                                                   ea, Mp, kscale, sks, kdev, sA2, nb2, nva, kpl);
-      oz_split_kernel<T, false><<<tb, 256, 0, s>>>(B, ldb, sB, 1, opB, N, K, Bd, Kp, (long long)Np * Kp, zB, P, 0,
-                                                   eb, Np, nullptr, 0, kdev, sB2, nb2, nvb, kpl);
+      cudaFuncSetAttribute(oz_fused_kernel<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+      oz_fused_kernel<T, false><<<grid, 256, sm, s>>>(sp, K, Kp, P, bits, nb2, kdev, CrtWeights{}, ldk);
     }
+  } else {
+    // the scale codes start at 0 (the zero vector)
+    cudaMemsetAsync(ea, 0, sizeof(int) * ((size_t)Mp + Np) * count, s);
+    sp.n0 = (M + 31) / 32;
+    count_launch(2);
+    oz_scale_kernel<T><<<dim3(sp.n0 + (N + 31) / 32, (K + kScaleK - 1) / kScaleK, count), 256, 0, s>>>(sp, K, nb2,
+                                                                                                      kdev);
+    sp.n0 = Mp / 32;
+    const dim3 tiles(sp.n0 + (sp.o[1].nvp + 31) / 32, Kp / 64, count);
+    if (res) oz_split_kernel<T, true><<<tiles, 256, 0, s>>>(sp, K, Kp, P, bits, nb2, kdev, pl.wt);
+    else oz_split_kernel<T, false><<<tiles, 256, 0, s>>>(sp, K, Kp, P, bits, nb2, kdev, CrtWeights{});
   }
   const long long wait = wait_cycles > 0 ? wait_cycles : (1ll << 32);
-  dim3 grid(Np / (res ? crtc::BN : OZ_BN), Mp / OZ_BM, count);
+  // Moduli of a tile over ng CTAs when the tiles alone leave SMs idle: the rounds of 152 CTAs
+  // times the moduli per CTA (one more for its prologue) is least.  The residues, and so the
+  // result, do not depend on ng.
+  int ng = 1;
+  if (res) {
+    const long long mt = Mp / OZ_BM, nt = Np / crtc::BN;
+    const long long tl = std::max<long long>(1, (lower ? (mt * nt + mt) / 2 : mt * nt) * count);
+    long long best = -1;
+    for (int g = 1; g <= P && (long long)count * g <= 65535; g++) {
+      const long long cost = ((tl * g + 151) / 152) * ((P + g - 1) / g + 1);
+      if (best < 0 || cost < best) {
+        best = cost;
+        ng = g;
+      }
+    }
+  }
+  dim3 grid(Np / (res ? crtc::BN : OZ_BN), Mp / OZ_BM, count * ng);
   CUtensorMap ma, mb;
   if (!digit_map(&ma, Ad, (long long)count * P * Mp, Kp, tcg::BM) ||
       !digit_map(&mb, Bd, (long long)count * P * Np, Kp, res ? crtc::BN : tcg::BN))
@@ -1083,19 +1227,19 @@ bool ozaki_gemm(int opA, int opB, int M, int N, int K, double alpha, const T* A,
     ca.Np = Np;
     ca.Kp = Kp;
     ca.n = P;
+    ca.ng = ng;
     ca.cplx = cplx ? 1 : 0;
     ca.lower = lower;
     ca.zR = zR;
     ca.kdev = kdev;
     ca.wait = wait;
     ca.skip_copy = skip_copy;
-    for (int l = 0; l < CRT_MAXMOD; l++) ca.y[l] = l < P ? (float)pl.cr.y[l] : 0.0f;
     cudaFuncSetAttribute(crt_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, crtc::SMEM);
     count_launch(2);
     crt_tc_kernel<<<grid, tcg::THREADS, crtc::SMEM, s>>>(ma, mb, ca, status);
-    const int per = cplx ? 8 : 16;
-    crt_recon_kernel<T><<<dim3((N + 128 * per - 1) / (128 * per), std::min(M, 65535), count), 128, 0, s>>>(
-        R, zR, Mp, Np, M, N, ea, eb, Mp, Np, -2 * pl.p, pl.cr, C, ldc, sC, sC2, nb2, alpha, beta, lower);
+    const int ncg = (N + (cplx ? 3 : 7)) / (cplx ? 4 : 8);
+    crt_recon_kernel<T><<<dim3((unsigned)(((long long)M * ncg + 127) / 128), 1, count), 128, 0, s>>>(
+        R, zR, Mp, Np, M, N, ncg, ea, eb, Mp, Np, -2 * pl.p, pl.cr, C, ldc, sC, sC2, nb2, alpha, beta, lower);
     return true;
   }
   OzArgs oa;
