@@ -148,7 +148,7 @@ struct gks_ctx {
   int am = -1, ank = -1, aes = -1;
   // offsets (bytes) of per-item arrays; each holds nk items
   size_t oA, oL, oF, oFB, oU, oQ, opart, oy, ouw, oSg, oV, oG, oT, oY, oY2, ou, op, oph, otau, otb, od, oe, oZ, oocc, oks, onrho,
-      oweights, oeb, odc, oticket, oAf, oRY, oRT, oRR, onrm, orstat, operm, oflag, oBd, oV2, otau2, oprog, oerr, oqr, oD, oud, ofu, ormax,
+      oweights, oeb, odc, oticket, oAf, oRY, oRT, oRR, onrm, orstat, operm, oflag, oBd, oV2, otau2, oprog, oerr, oqr, oD, oarow, oppart, opy, opP, opdot, opnrm, opmex, opbar, ormax,
       otau1, oT1, oP1, oP2, oVT, oXb, oGb, oYb, oZb, oXp, oVw, otw, oGw, oTw, oYw, oY2w;
   int ldt2 = 0, nblkmax = 0;
   long long sMM, sF, sFB, sU, spart, sy, sV, sG, sT, sY, sVec;
@@ -293,11 +293,19 @@ gks_status ensure_ws(gks_ctx* c, int m, int n, int nk, int es, int nc) {
   c->ouw = a.take<double>((size_t)3 * m * nk);
   c->oSg = es == 16 && !dig ? a.take<double>(MM * nk) : 0;
   if (dig) {
-    // digit planes of the stale block and of u (14 planes complex, 7 real), scale exponents
+    // digit planes of the stale block (14 planes complex, 7 real), row maxima, and the
+    // panel kernel's rows, shares and barrier counters
     const size_t ldd = ((size_t)m + 15) / 16 * 16, npl = es == 16 ? 14 : 7;
     c->oD = a.take<char>((ldd + 31) / 32 * 32 * ldd * npl * nk);  // rows in tiles of 32
-    c->oud = a.take<char>(ldd * npl * nk);
-    c->ofu = a.take<int>((size_t)nk);
+    const int gs = panel_gs(nk);
+    c->oarow = a.take<char>(elems(2LL * m));
+    c->oppart = a.take<char>(elems(2LL * gs * kPanelMax));
+    c->opy = a.take<char>(elems(2LL * kPanelMax));
+    c->opP = a.take<char>(elems(panel_partials(m, gs)));
+    c->opdot = a.take<char>(elems(gs));
+    c->opnrm = a.take<double>((size_t)gs * nk);
+    c->opmex = a.take<int>((size_t)gs * nk);
+    c->opbar = a.take<unsigned>((size_t)4 * nk);
     c->ormax = a.take<unsigned long long>(ldd * nk);
   }
   c->oV = a.take<char>(elems(c->sV));
@@ -516,16 +524,23 @@ constexpr size_t kOzCap = (size_t)12 << 30;
 int oz_reserve(gks_ctx* c, size_t item, int count) {
   const int maxper = (int)std::max<size_t>(1, std::min<size_t>((size_t)count, kOzCap / item));
   const int nch = (count + maxper - 1) / maxper, per = (count + nch - 1) / nch;
-  const size_t need = item * per;
+  // grown in doublings: each growth waits for the stream
+  const size_t need = item * per, want = std::max(need, std::min(2 * c->oz_bytes, kOzCap));
   if (need > c->oz_bytes) {
     cudaStreamSynchronize(c->stream);
     release_oz(c);
-    if (cudaMalloc(&c->oz, need) != cudaSuccess) {
+    if (cudaMalloc(&c->oz, want) == cudaSuccess) {
+      c->oz_bytes = want;
+    } else {
       cudaGetLastError();
       c->oz = nullptr;
-      return 0;
+      if (want == need || cudaMalloc(&c->oz, need) != cudaSuccess) {
+        cudaGetLastError();
+        c->oz = nullptr;
+        return 0;
+      }
+      c->oz_bytes = need;
     }
-    c->oz_bytes = need;
   }
   return per;
 }
@@ -902,13 +917,108 @@ void hegst_run(gks_ctx* c, T* A, int lda, long long sA, const T* L, int ldl, lon
   }
 }
 
-// One-stage Householder tridiagonalization, steps j = M-1 .. 2, in panels of nbb steps.
+// Deferred update of a panel with kp steps: A[0:n, 0:n] -= U Q^H + Q U^H (lower triangle).
+template <typename T>
+void panel_deferred(gks_ctx* c, T* A, int M, int n, int kp, int nk) {
+  T* U = at<T>(c, c->oU);
+  T* Q = at<T>(c, c->oQ);
+  const int ldu = c->nbb;
+  gmx<T>(c, nk, OP_N, OP_C, n, n, kp, -1.0, U, ldu, c->sU, Q, ldu, c->sU, 1.0, A, M, c->sMM, 1);
+  gmx<T>(c, nk, OP_N, OP_C, n, n, kp, -1.0, Q, ldu, c->sU, U, ldu, c->sU, 1.0, A, M, c->sMM, 1);
+}
+
+// Steps per panel: at most 128 (the per-step corrections grow with the panel length, the
+// deferred update runs fine at K = 128); small orders are latency-bound per step (64).
+int panel_width(const gks_ctx* c, int M) { return M < 2048 ? std::min(NB, c->nbb) : std::min(kPanelMax, c->nbb); }
+
+// One-stage Householder tridiagonalization with the digit form of the matrix-vector step:
+// per panel the digits of the stale block, one persistent launch for its steps, and the
+// deferred update as two lower-triangle products with K = the panel's step count.  False if
+// a cooperative launch was refused.
+template <typename T>
+bool hetrd_digit_run(gks_ctx* c, T* A, int M, int nk) {
+  cudaStream_t s = c->stream;
+  const int es = sizeof(T), pw = panel_width(c, M);
+  const int ldd = (M + 15) / 16 * 16, npl = es == 16 ? 14 : 7;
+  if (M < 3) return true;
+  // items per launch: at least one CTA each, all resident
+  int per = nk;
+  while (per > 1 && hetrd_panel_ctas<T>(M - 1, per) < 1) per = (per + 1) / 2;
+  const int gs = panel_gs(nk);
+  PanelArgs<T> pa{};
+  pa.lda = M;
+  pa.sA = c->sMM;
+  pa.stau = M;
+  pa.ldu = c->nbb;
+  pa.sU = c->sU;
+  pa.sv = M;
+  pa.sP = panel_partials(M, gs);
+  pa.gs = gs;
+  pa.hd.sD = (long long)((ldd + 31) / 32 * 32) * ldd * npl;
+  pa.hd.ldd = ldd;
+  // the grid barriers' CTAs are all resident: a limit chosen for copies does not cut them short
+  pa.wait = std::max(c->wait_cycles, 1ll << 28);
+  cudaMemsetAsync(at<unsigned>(c, c->opbar), 0, sizeof(unsigned) * 4 * nk, s);
+  HemvDigits hd = pa.hd;
+  hd.D = at<signed char>(c, c->oD);
+  hd.rmax = at<unsigned long long>(c, c->ormax);
+  std::vector<unsigned> base((nk + per - 1) / per, 0u), basev(base);
+  for (int jh = M - 1; jh >= 2; jh -= pw) {
+    const int jl = std::max(2, jh - pw + 1), steps = jh - jl + 1;  // steps jh .. jl in this panel
+    {
+      Rec r(c, PC_HETRD_VEC, 0.0, (0.5 * es + npl) * jh * (double)jh * nk);
+      hetrd_digits<T>(A, M, c->sMM, jh, hd, nk, s);
+    }
+    double fl = 0.0, by = 0.0;
+    for (int j = jh; j >= jl; j--) {
+      const double jj = (double)j * j, k = jh - j;
+      fl += cmul(es) * (jj + 4.0 * j * k) * nk;
+      by += (jj * npl + (4.0 * j * k + 8.0 * j) * es) * nk;
+    }
+    {
+      Rec r(c, PC_HETRD_HEMV, fl, by);
+      for (int z0 = 0, q = 0; z0 < nk; z0 += per, q++) {
+        const int cnt = std::min(per, nk - z0), G = std::min(gs, hetrd_panel_ctas<T>(jh, cnt));
+        pa.A = A + z0 * c->sMM;
+        pa.jh = jh;
+        pa.jl = jl;
+        pa.tau = at<double>(c, c->otau) + (size_t)z0 * M;
+        pa.U = at<T>(c, c->oU) + z0 * c->sU;
+        pa.Q = at<T>(c, c->oQ) + z0 * c->sU;
+        pa.arow = at<T>(c, c->oarow) + (size_t)2 * z0 * M;
+        pa.part = at<T>(c, c->oppart) + (size_t)z0 * gs * 2 * kPanelMax;
+        pa.y = at<T>(c, c->opy) + (size_t)z0 * 2 * kPanelMax;
+        pa.P = at<T>(c, c->opP) + z0 * pa.sP;
+        pa.dot = at<T>(c, c->opdot) + (size_t)z0 * gs;
+        pa.nrm = at<double>(c, c->opnrm) + (size_t)z0 * gs;
+        pa.mex = at<int>(c, c->opmex) + (size_t)z0 * gs;
+        pa.bar = at<unsigned>(c, c->opbar) + (size_t)4 * z0;
+        pa.base = base[q];
+        pa.basev = basev[q];
+        pa.hd.D = hd.D + z0 * hd.sD;
+        pa.hd.rmax = hd.rmax + (size_t)z0 * ldd;
+        pa.st = c->st ? c->st + z0 : nullptr;
+        if (!hetrd_panel<T>(pa, G, cnt, s)) {
+          cudaGetLastError();
+          return false;
+        }
+        base[q] += 2u * steps * G;
+        basev[q] += (unsigned)(steps - 1) * G;
+      }
+    }
+    panel_deferred<T>(c, A, M, jl, steps, nk);
+  }
+  return true;
+}
+
+// The same with the matrix-vector step on the FP64 or FP32 pipe (opts.hemv, mixed precision).
 // Each step is two launches (the Hermitian product over the stale trailing block with the
 // panel's corrections, then q, the panel buffers and the next row); each panel ends with
-// the deferred update A[0:j,0:j] -= U Q^H + Q U^H as two lower-triangle GEMMs with K = the
-// panel's step count.
+// the deferred update.
 template <typename T>
-void hetrd_run(gks_ctx* c, T* A, int M, int nk) {
+bool hetrd_run(gks_ctx* c, T* A, int M, int nk) {
+  if constexpr (std::is_same<T, double>::value || std::is_same<T, zc>::value)
+    if (c->wsdig) return hetrd_digit_run<T>(c, A, M, nk);
   cudaStream_t s = c->stream;
   const int es = sizeof(T);
   const int ldu = c->nbb;
@@ -920,62 +1030,39 @@ void hetrd_run(gks_ctx* c, T* A, int M, int nk) {
   T* y = at<T>(c, c->oy);
   double* tau = at<double>(c, c->otau);
   int* tk = at<int>(c, c->oticket);
-  if (M < 3) return;
+  if (M < 3) return true;
   cudaMemsetAsync(tk, 0, sizeof(int) * 2 * nk, s);
-  // panels of at most 128 steps: the per-step corrections grow with the panel length, the
-  // deferred update runs fine at K = 128; small orders are latency-bound per step (64)
-  const int pw = M < 2048 ? std::min(NB, ldu) : std::min(2 * NB, ldu);
-  // digit form of the matrix-vector step (FP64 types): digits of the stale block per panel;
-  // else, complex: three-multiplication products need Re + Im of the stale block (per panel)
-  HemvDigits hdv{};
-  const HemvDigits* hd = nullptr;
-  if constexpr (std::is_same<T, double>::value || std::is_same<T, zc>::value) {
-    if (c->wsdig) {
-      const int ldd = (M + 15) / 16 * 16, npl = es == 16 ? 14 : 7;
-      hdv.D = at<signed char>(c, c->oD);
-      hdv.sD = (long long)((ldd + 31) / 32 * 32) * ldd * npl;
-      hdv.ldd = ldd;
-      hdv.ud = at<signed char>(c, c->oud);
-      hdv.sud = (long long)ldd * npl;
-      hdv.fu = at<int>(c, c->ofu);
-      hdv.rmax = at<unsigned long long>(c, c->ormax);
-      hd = &hdv;
-    }
-  }
-  double* uw = es == 16 && !hd ? at<double>(c, c->ouw) : nullptr;
-  double* Sg = es == 16 && !hd ? at<double>(c, c->oSg) : nullptr;
-  const double npl = es == 16 ? 14.0 : 7.0;
+  const int pw = panel_width(c, M);
+  // complex FP64: three-multiplication products need Re + Im of the stale block (per panel)
+  double* uw = es == 16 ? at<double>(c, c->ouw) : nullptr;
+  double* Sg = es == 16 ? at<double>(c, c->oSg) : nullptr;
   for (int jh = M - 1; jh >= 2; jh -= pw) {
     const int jl = std::max(2, jh - pw + 1);  // steps jh .. jl in this panel
     {
-      Rec r(c, PC_HETRD_VEC, 0.0, (hd ? 0.5 * es + npl : 2.0 * es) * jh * (hd ? jh : 1) * nk);
-      if (hd) hetrd_digits<T>(A, M, c->sMM, jh, hdv, nk, s);
-      else if (Sg) hetrd_sums(reinterpret_cast<const zc*>(A), M, c->sMM, jh, Sg, nk, s);
-      hetrd_reflector<T>(A, M, c->sMM, jh, u, c->sVec, tau, M, nk, s, uw, hd);
+      Rec r(c, PC_HETRD_VEC, 0.0, 2.0 * es * jh * nk);
+      if (Sg) hetrd_sums(reinterpret_cast<const zc*>(A), M, c->sMM, jh, Sg, nk, s);
+      hetrd_reflector<T>(A, M, c->sMM, jh, u, c->sVec, tau, M, nk, s, uw);
     }
     for (int j = jh; j >= jl; j--) {
       const int k = jh - j;  // panel steps already taken
       const double jj = (double)j * j;
       {
-        // algorithmic bytes: the digit planes of the j x j block (full matrix), or the
-        // lower triangle (and Re + Im sums) in FP64
+        // algorithmic bytes: the lower triangle (and Re + Im sums)
         Rec r(c, PC_HETRD_HEMV, cmul(es) * (jj + 2.0 * j * k) * nk,
-              ((hd ? jj * npl : 0.5 * jj * (es == 16 ? 1.5 : 1.0) * es) + (2.0 * j * k + 4.0 * j) * es) * nk);
+              (0.5 * jj * (es == 16 ? 1.5 : 1.0) + 2.0 * j * k + 4.0 * j) * es * nk);
         hetrd_phemv<T>(A, M, c->sMM, j, u, p, c->sVec, tau, M, U, Q, ldu, c->sU, k, part, c->spart, y, c->sy, tk,
-                       nk, s, Sg, uw, hd);
+                       nk, s, Sg, uw);
       }
       const int rowupd = (j > jl) ? 1 : 0;
       {
         Rec r(c, PC_HETRD_RANK2, cmul(es) * 2.0 * j * (k + 1) * (1 + rowupd) * nk, (2.0 * j * (k + 1) + 4.0 * j) * es * nk);
         hetrd_pupdate<T>(A, M, c->sMM, j, u, p, c->sVec, tau, M, U, Q, ldu, c->sU, k, y, c->sy, rowupd, tk + nk, nk,
-                         s, uw, hd);
+                         s, uw);
       }
     }
-    // deferred rank-2k update of the trailing block [0:jl, 0:jl]
-    const int kp = jh - jl + 1;
-    gmx<T>(c, nk, OP_N, OP_C, jl, jl, kp, -1.0, U, ldu, c->sU, Q, ldu, c->sU, 1.0, A, M, c->sMM, 1);
-    gmx<T>(c, nk, OP_N, OP_C, jl, jl, kp, -1.0, Q, ldu, c->sU, U, ldu, c->sU, 1.0, A, M, c->sMM, 1);
+    panel_deferred<T>(c, A, M, jl, jh - jl + 1, nk);
   }
+  return true;
 }
 
 // ---- two-stage tridiagonalization (sbr.cu) ----
@@ -1195,12 +1282,12 @@ void backtransform_run(gks_ctx* c, const TA* A, T* X, int ldx, long long sX, int
 // destroyed): w (M per item, ascending) and X (M x M, ldx M, stride sX) with the FP64 stages
 // of the main path (Householder, divide and conquer, back-transform).
 template <typename T>
-void standard_eig(gks_ctx* c, T* A, T* X, long long sX, double* w, int M, int items) {
+bool standard_eig(gks_ctx* c, T* A, T* X, long long sX, double* w, int M, int items) {
   cudaStream_t s = c->stream;
   double* d = at<double>(c, c->od);
   double* e = at<double>(c, c->oe);
   T* ph = at<T>(c, c->oph);
-  hetrd_run<T>(c, A, M, items);
+  if (!hetrd_run<T>(c, A, M, items)) return false;
   {
     Rec r(c, PC_HETRD_VEC);
     hetrd_finish<T>(A, M, c->sMM, M, d, e, M, ph, M, items, s);
@@ -1220,6 +1307,7 @@ void standard_eig(gks_ctx* c, T* A, T* X, long long sX, double* w, int M, int it
     apply_phase<T>(X, M, sX, Z, M, c->sMM, ph, M, M, M, items, s);
   }
   backtransform_run<T>(c, A, X, M, sX, M, M, items);
+  return true;
 }
 
 // Ogita-Aishima sweeps (refine.cu) on X (C, order M, all columns) for the standard problem
@@ -1290,6 +1378,10 @@ gks_status solve_t(gks_ctx* c, const SolveKey& key) {
   gks_status rc = ensure_ws(c, M, n, items, es, key.spin);
   if (rc) return rc;
   cudaStream_t s = c->stream;
+  // the scratch of the largest split product (the density matrix) at once: growing it product
+  // by product would wait for the stream each time
+  if (split_worth(c, items, M, M, nev, es, gemm_flops(es, M, M, nev, 0, items)))
+    oz_reserve(c, ozaki_workspace_bytes(M, M, nev, es == 16, sform(c)), items);
   double* eps = static_cast<double*>(const_cast<void*>(key.eps));
   T* C = static_cast<T*>(const_cast<void*>(key.C));
   const long long sC = (long long)M * nev;
@@ -1309,6 +1401,9 @@ gks_status solve_t(gks_ctx* c, const SolveKey& key) {
     if (!reuse) copy2d<T>(L, n, sLk, S, n, (long long)n * n, n, n, nk, s);
   }
   const bool lowdin = c->reduction == GKS_REDUCE_LOWDIN;
+  auto refused = [c] {
+    return fail(c, GKS_ECUDA, "tridiagonalization: cooperative launch refused (not enough resident CTAs)");
+  };
   // (a1) Cholesky of S, (a2) reduction to the standard problem
   if (!reuse && lowdin) {
     // Loewdin (paper Sec. 3.1 Parts 2-1, 2-2): S = U diag(s) U^H by the standard eigensolve
@@ -1321,7 +1416,7 @@ gks_status solve_t(gks_ctx* c, const SolveKey& key) {
       copy2d<T>(A, M, sLk, S, n, (long long)n * n, n, n, nk, s);
       if (sp) copy2d<T>(A + c->sMM, M, sLk, A, M, sLk, n, n, nk, s);
     }
-    standard_eig<T>(c, A, C, sC, eps, M, items);
+    if (!standard_eig<T>(c, A, C, sC, eps, M, items)) return refused();
     {
       Rec r(c, PC_MISC);
       lowdin_factor<T>(C, M, sC, eps, M, L, n, c->sMM, M, c->st, items, s);
@@ -1380,7 +1475,7 @@ gks_status solve_t(gks_ctx* c, const SolveKey& key) {
         Rec r(c, PC_MISC);
         narrow_lower<T, TL>(A, M, c->sMM, Af, M, c->sMM, M, items, s);
       }
-      hetrd_run<TL>(c, Af, M, items);
+      if (!hetrd_run<TL>(c, Af, M, items)) return refused();
       Rec r(c, PC_HETRD_VEC);
       TL* phl = at<TL>(c, c->ou);
       hetrd_finish<TL>(Af, M, c->sMM, M, d, e, M, phl, M, items, s);
@@ -1391,7 +1486,7 @@ gks_status solve_t(gks_ctx* c, const SolveKey& key) {
       if (!hb2st_run<T>(c, A, M, items, d, e))
         return fail(c, GKS_ECUDA, "bulge chasing: cooperative launch refused (not enough resident CTAs)");
     } else {
-      hetrd_run<T>(c, A, M, items);
+      if (!hetrd_run<T>(c, A, M, items)) return refused();
       Rec r(c, PC_HETRD_VEC);
       hetrd_finish<T>(A, M, c->sMM, M, d, e, M, ph, M, items, s);
     }

@@ -50,94 +50,77 @@ __global__ void potf2_kernel(T* A, int lda, long long sA, int k0, int nb, DevSta
   }
 }
 
-// Triangular solves against one nb x nb lower-triangular block L (ldl), by substitution
+// Triangular solves against one nb x nb lower-triangular block L (nb <= 64), by substitution
 // (no explicit inverse: the diagonal blocks of the Cholesky factor of an overcomplete
-// basis have condition numbers near 1e5).  Each CTA takes 64 right-hand sides into
-// shared memory, one thread per right-hand side.
-//   TRSM_RIGHT_CONJ : B (nrhs x nb rows)  <- B L^-H
+// basis have condition numbers near 1e5).
+//   TRSM_RIGHT_CONJ : B (nrhs x nb rows)  <- B L^-H   (x L^H = b: conj(L) x = b per row)
 //   TRSM_LEFT       : B (nb x nrhs cols)  <- L^-1 B
-//   TRSM_LEFT_CONJ  : B (nb x nrhs cols)  <- L^-H B
+//   TRSM_LEFT_CONJ  : B (nb x nrhs cols)  <- L^-H B   (backward: the reversed conj(L)^T)
+// Every mode is forward substitution with one lower matrix, kept in shared memory by
+// columns (conjugated or reversed while loading, padded to 64 with the identity).  Eight
+// lanes share a right-hand side, each holding 8 of its 64 entries in registers (entry 8 i +
+// lane): a step broadcasts the solved entry by shuffles and every lane updates its own
+// entries, so nothing but the columns of L is read.  The FP64 pipe bounds it (1.7
+// multiply-adds per SM clock; nb^2 / 2 per right-hand side, four times that complex), so the
+// right-hand sides are spread over all SMs, 4 per warp and as few warps per CTA as give one
+// CTA per SM.  Measured: 64 x 64 against 832 real right-hand sides 184 us with a thread per
+// right-hand side and 64 of them per CTA, 17 us here; 2500 complex 530 us, 62 us here.
+template <typename T>
+__device__ __forceinline__ T shfl8(T v, int src);
+template <>
+__device__ __forceinline__ double shfl8<double>(double v, int src) { return __shfl_sync(0xffffffffu, v, src, 8); }
+template <>
+__device__ __forceinline__ zc shfl8<zc>(zc v, int src) {
+  return zc{__shfl_sync(0xffffffffu, v.x, src, 8), __shfl_sync(0xffffffffu, v.y, src, 8)};
+}
+
 template <typename T, int MODE>
-__global__ void __launch_bounds__(64) trsm_block_kernel(const T* L, int ldl, long long sL, T* B, int ldb, long long sB,
-                                                        int nb, int nrhs) {
+__global__ void __launch_bounds__(256) trsm_block_kernel(const T* L, int ldl, long long sL, T* B, int ldb,
+                                                         long long sB, int nb, int nrhs) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* x = reinterpret_cast<T*>(smem_raw);  // MODE 0: [64][nb+1] (row per rhs); else [nb][65]
-  const int z = blockIdx.y, tid = threadIdx.x, r0 = blockIdx.x * 64;
+  T* lc = reinterpret_cast<T*>(smem_raw);                    // [column][64]
+  double* rd = reinterpret_cast<double*>(lc + 64 * 64);       // 1 / diagonal
+  const int z = blockIdx.y, tid = threadIdx.x, nt = blockDim.x;
   L += z * sL;
   B += z * sB;
-  const int nr = min(64, nrhs - r0);
-  if (MODE == TRSM_RIGHT_CONJ) {
-    const int ld = nb + 1;
-    for (int e = tid; e < nr * nb; e += 64) {
-      int r = e / nb, c = e % nb;
-      x[r * ld + c] = B[(size_t)(r0 + r) * ldb + c];
-    }
-    __syncthreads();
-    if (tid < nr) {
-      T* xr = x + tid * ld;
-      for (int j = 0; j < nb; j++) {  // x L^H = b  <=>  x_j = (b_j - sum_{k<j} x_k conj(L_jk)) / L_jj
-        const T* lj = L + (size_t)j * ldl;
-        T s0 = xr[j], s1 = zero<T>(), s2 = zero<T>(), s3 = zero<T>();  // four chains (latency)
-        int k = 0;
-        for (; k + 3 < j; k += 4) {
-          s0 -= xr[k] * conjg(lj[k]);
-          s1 -= xr[k + 1] * conjg(lj[k + 1]);
-          s2 -= xr[k + 2] * conjg(lj[k + 2]);
-          s3 -= xr[k + 3] * conjg(lj[k + 3]);
-        }
-        for (; k < j; k++) s0 -= xr[k] * conjg(lj[k]);
-        xr[j] = ((s0 + s1) + (s2 + s3)) * (1.0 / re(lj[j]));
-      }
-    }
-    __syncthreads();
-    for (int e = tid; e < nr * nb; e += 64) {
-      int r = e / nb, c = e % nb;
-      B[(size_t)(r0 + r) * ldb + c] = x[r * ld + c];
-    }
-  } else {
-    const int ld = 65;
-    for (int e = tid; e < nb * 64; e += 64) {
-      int i = e / 64, c = e % 64;
-      if (c < nr) x[i * ld + c] = B[(size_t)i * ldb + r0 + c];
-    }
-    __syncthreads();
-    if (tid < nr) {
-      T* xc = x + tid;
-      if (MODE == TRSM_LEFT) {
-        for (int i = 0; i < nb; i++) {  // x_i = (b_i - sum_{k<i} L_ik x_k) / L_ii
-          const T* li = L + (size_t)i * ldl;
-          T s0 = xc[i * ld], s1 = zero<T>(), s2 = zero<T>(), s3 = zero<T>();
-          int k = 0;
-          for (; k + 3 < i; k += 4) {
-            s0 -= li[k] * xc[k * ld];
-            s1 -= li[k + 1] * xc[(k + 1) * ld];
-            s2 -= li[k + 2] * xc[(k + 2) * ld];
-            s3 -= li[k + 3] * xc[(k + 3) * ld];
-          }
-          for (; k < i; k++) s0 -= li[k] * xc[k * ld];
-          xc[i * ld] = ((s0 + s1) + (s2 + s3)) * (1.0 / re(li[i]));
-        }
-      } else {
-        for (int i = nb - 1; i >= 0; i--) {  // x_i = (b_i - sum_{k>i} conj(L_ki) x_k) / L_ii
-          T s0 = xc[i * ld], s1 = zero<T>(), s2 = zero<T>(), s3 = zero<T>();
-          int k = i + 1;
-          for (; k + 3 < nb; k += 4) {
-            s0 -= conjg(L[(size_t)k * ldl + i]) * xc[k * ld];
-            s1 -= conjg(L[(size_t)(k + 1) * ldl + i]) * xc[(k + 1) * ld];
-            s2 -= conjg(L[(size_t)(k + 2) * ldl + i]) * xc[(k + 2) * ld];
-            s3 -= conjg(L[(size_t)(k + 3) * ldl + i]) * xc[(k + 3) * ld];
-          }
-          for (; k < nb; k++) s0 -= conjg(L[(size_t)k * ldl + i]) * xc[k * ld];
-          xc[i * ld] = ((s0 + s1) + (s2 + s3)) * (1.0 / re(L[(size_t)i * ldl + i]));
-        }
-      }
-    }
-    __syncthreads();
-    for (int e = tid; e < nb * 64; e += 64) {
-      int i = e / 64, c = e % 64;
-      if (c < nr) B[(size_t)i * ldb + r0 + c] = x[i * ld + c];
-    }
+#pragma unroll 4
+  for (int e = tid; e < 64 * 64; e += nt) {
+    const int i = e >> 6, j = e & 63;  // stored element (i, j), j <= i
+    T v = (i == j) ? from_real<T>(1.0) : zero<T>();
+    if (i < nb && j <= i) v = L[(size_t)i * ldl + j];
+    if (MODE != TRSM_LEFT) v = conjg(v);
+    if (i == j) rd[MODE == TRSM_LEFT_CONJ && i < nb ? nb - 1 - i : i] = 1.0 / re(v);
+    // lower matrix by columns; backward: (i, j) of L is (nb - 1 - j, nb - 1 - i) of its reverse
+    if (MODE == TRSM_LEFT_CONJ && i < nb && j < nb) lc[(nb - 1 - i) * 64 + nb - 1 - j] = v;
+    else lc[j * 64 + i] = v;
   }
+  __syncthreads();
+  const int g = tid & 7, r = (blockIdx.x * nt + tid) >> 3;
+  const bool ok = r < nrhs;
+  auto at = [&](int i) -> T* {  // entry i of this right-hand side, in solving order
+    const int e = MODE == TRSM_LEFT_CONJ ? nb - 1 - i : i;
+    return MODE == TRSM_RIGHT_CONJ ? B + (size_t)r * ldb + e : B + (size_t)e * ldb + r;
+  };
+  T x[8];
+#pragma unroll
+  for (int i = 0; i < 8; i++) x[i] = (ok && 8 * i + g < nb) ? *at(8 * i + g) : zero<T>();
+#pragma unroll
+  for (int J = 0; J < 8; J++) {
+#pragma unroll
+    for (int jj = 0; jj < 8; jj++) {
+      const int j = 8 * J + jj;
+      const T xj = shfl8<T>(x[J] * rd[j], jj);
+      const T* col = lc + j * 64 + g;
+      if (g > jj) x[J] -= xj * col[8 * J];
+      if (g == jj) x[J] = xj;
+#pragma unroll
+      for (int i = J + 1; i < 8; i++) x[i] -= xj * col[8 * i];
+    }
+    if (8 * J + 8 >= nb) break;
+  }
+#pragma unroll
+  for (int i = 0; i < 8; i++)
+    if (ok && 8 * i + g < nb) *at(8 * i + g) = x[i];
 }
 
 // One CTA per batch item: the diagonal block A11 <- L11^-1 A11 L11^-H (A11 read from its
@@ -337,27 +320,26 @@ void potf2(T* A, int lda, long long sA, int k0, int nb, DevStatus* st, int count
   potf2_kernel<T><<<count, 256, sm, s>>>(A, lda, sA, k0, nb, st);
 }
 
+template <typename T, int MODE>
+static void trsm_launch(const T* L, int ldl, long long sL, T* B, int ldb, long long sB, int nb, int nrhs, int count,
+                        cudaStream_t s) {
+  // warps per CTA: 4 right-hand sides each, at least one CTA per SM where there are enough
+  int w = 8;
+  while (w > 1 && (long long)((nrhs + 4 * w - 1) / (4 * w)) * count < 152) w >>= 1;
+  const int sm = (int)(64 * 64 * sizeof(T) + 64 * sizeof(double));
+  cudaFuncSetAttribute(trsm_block_kernel<T, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+  count_launch();
+  trsm_block_kernel<T, MODE><<<dim3((nrhs + 4 * w - 1) / (4 * w), count), 32 * w, sm, s>>>(L, ldl, sL, B, ldb, sB, nb,
+                                                                                          nrhs);
+}
+
 template <typename T>
 void trsm_block(int mode, const T* L, int ldl, long long sL, T* B, int ldb, long long sB, int nb, int nrhs,
                 int count, cudaStream_t s) {
   if (nrhs <= 0 || nb <= 0 || count <= 0) return;
-  dim3 grid((nrhs + 63) / 64, count);
-  if (mode == TRSM_RIGHT_CONJ) {
-    size_t sm = sizeof(T) * 64 * (nb + 1);
-    cudaFuncSetAttribute(trsm_block_kernel<T, TRSM_RIGHT_CONJ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    count_launch();
-    trsm_block_kernel<T, TRSM_RIGHT_CONJ><<<grid, 64, sm, s>>>(L, ldl, sL, B, ldb, sB, nb, nrhs);
-  } else if (mode == TRSM_LEFT) {
-    size_t sm = sizeof(T) * nb * 65;
-    cudaFuncSetAttribute(trsm_block_kernel<T, TRSM_LEFT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    count_launch();
-    trsm_block_kernel<T, TRSM_LEFT><<<grid, 64, sm, s>>>(L, ldl, sL, B, ldb, sB, nb, nrhs);
-  } else {
-    size_t sm = sizeof(T) * nb * 65;
-    cudaFuncSetAttribute(trsm_block_kernel<T, TRSM_LEFT_CONJ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    count_launch();
-    trsm_block_kernel<T, TRSM_LEFT_CONJ><<<grid, 64, sm, s>>>(L, ldl, sL, B, ldb, sB, nb, nrhs);
-  }
+  if (mode == TRSM_RIGHT_CONJ) trsm_launch<T, TRSM_RIGHT_CONJ>(L, ldl, sL, B, ldb, sB, nb, nrhs, count, s);
+  else if (mode == TRSM_LEFT) trsm_launch<T, TRSM_LEFT>(L, ldl, sL, B, ldb, sB, nb, nrhs, count, s);
+  else trsm_launch<T, TRSM_LEFT_CONJ>(L, ldl, sL, B, ldb, sB, nb, nrhs, count, s);
 }
 
 template <typename T>

@@ -38,35 +38,70 @@ void tune_pencil(T* A, int m, int count, int hermitian, cudaStream_t s);
 // ---- Householder tridiagonalization (hetrd.cu) ----
 // Workspace per batch item: u (m), p (m) vectors, tau (m), two zeroed tickets, and for the
 // panel form U, Q (m x ldu), per-CTA shares (ceil(m/16) x (2 ldu + 2)) and y (2 ldu + 2).
-// hetrd_reflector starts a panel at step j; step j is hetrd_phemv then hetrd_pupdate (which
-// with rowupd also forms the reflector of step j-1).
+// FP64-pipe and single-precision form: hetrd_reflector starts a panel at step j; step j is
+// hetrd_phemv then hetrd_pupdate (which with rowupd also forms the reflector of step j-1).
+// Digit form (hetrd_panel): one persistent launch per panel.
+template <typename T>
+void hetrd_reflector(T* A, int lda, long long sA, int j, T* u, long long sv, double* tau, long long stau, int count,
+                     cudaStream_t s, double* uw = nullptr);
 // Digit form of the panel matrix-vector step.  The stale block A = [0:n, 0:n] is
 // equilibrated symmetrically by powers of two, A = D Ã D with D = diag(2^{d_i}),
 // d_i = ceil(g_i / 2) for row maxima below 2^{g_i} (largest |Re|, |Im| over the full
 // row), so every |Re ã|, |Im ã| < 1; the full Hermitian Ã (upper triangle mirrored,
 // conjugated) is stored as 7 balanced base-256 digits (signed 8-bit) of round(2^54 Re ã)
 // (planes 0..6, most significant first) and of Im ã (planes 7..13, complex only):
-// ã = sum_s d_s 2^{-6 - 8s} up to 2^{-55}.  ũ = D u gets the same digits below its own
-// scale 2^{fu}.  Then (A u)_i = 2^{d_i} sum over digit pairs s + t <= 7 of exact integer
-// dot products (dp4a, int32 sums) weighted by 2^{fu - 12 - 8(s + t)}.
+// ã = sum_s d_s 2^{-6 - 8s} up to 2^{-55}.  The vector ṽ = D v gets the same digits below
+// its own scale 2^{fu}.  Then (A v)_i = 2^{d_i} sum over digit pairs s + t <= 7 of exact
+// integer dot products (dp4a, int32 sums) weighted by 2^{fu - 12 - 8(s + t)}.
 // Layout: tiles of 32 rows x 16 columns, row-tile-major, each tile contiguous (3584 or
-// 7168 bytes: the 32 rows one after the other, a row's 16 columns as the planes' 16 bytes
-// one after the other); ũ per 16 columns the same way.  Rows are padded to a multiple of 32.
+// 7168 bytes) as [plane][row][16 bytes].  Rows are padded to a multiple of 32.
 struct HemvDigits {
-  signed char* D;            // [item][ldd32 / 32][ldd / 16][32][planes][16], ldd32 = ldd rounded up to 32
+  signed char* D;            // [item][ldd32 / 32][ldd / 16][planes][32][16], ldd32 = ldd rounded up to 32
   long long sD;              // item stride (bytes)
   int ldd;                   // columns per row, multiple of 16
-  signed char* ud;           // [item][ldd / 16][planes][16] digits of ũ (zero beyond the step's length)
-  long long sud;             // item stride (bytes)
-  int* fu;                   // [item] scale exponent of ũ
   unsigned long long* rmax;  // [item][ldd] row maxima of the stale block (bits of doubles)
 };
-template <typename T>
-void hetrd_reflector(T* A, int lda, long long sA, int j, T* u, long long sv, double* tau, long long stau, int count,
-                     cudaStream_t s, double* uw = nullptr, const HemvDigits* hd = nullptr);
 // Digits of the stale block [0:n, 0:n] (FP64 forms only).
 template <typename T>
 void hetrd_digits(const T* A, int lda, long long sA, int n, const HemvDigits& hd, int count, cudaStream_t s);
+// One panel of the digit form: steps jh .. jl.  Per item (strides in elements): arow 2 x sv,
+// part gs x 2 kPanelMax, y 2 kPanelMax, P panel_partials(m, gs), dot, nrm and mex gs each (gs:
+// CTAs per item at most), bar 4 counters zeroed once per reduction.  base, basev: arrivals at
+// the two barrier counters so far; a panel of s steps on G CTAs adds 2 s G and (s - 1) G.
+constexpr int kPanelMax = 128;   // steps per panel at most
+constexpr int kPanelCtas = 160;  // CTAs per item at most
+constexpr int panel_gs(int items) { return items >= kPanelCtas ? 1 : kPanelCtas / items; }
+constexpr long long panel_partials(int m, int gs) { return ((long long)(m + 31) / 32 + 2 * gs) * 32; }
+template <typename T>
+struct PanelArgs {
+  T* A;
+  int lda;
+  long long sA;
+  int jh, jl;
+  double* tau;
+  long long stau;
+  T *U, *Q;
+  int ldu;
+  long long sU;
+  T* arow;
+  long long sv;
+  T *part, *y, *P, *dot;
+  long long sP;
+  double* nrm;
+  int* mex;
+  int gs;
+  unsigned* bar;
+  unsigned base, basev;
+  HemvDigits hd;
+  DevStatus* st;
+  long long wait;
+};
+// CTAs per item for a panel of order jh on `items` items (0: not even one per item fits).
+template <typename T>
+int hetrd_panel_ctas(int jh, int items);
+// False if the cooperative launch was refused (then nothing ran).
+template <typename T>
+bool hetrd_panel(const PanelArgs<T>& a, int G, int items, cudaStream_t s);
 // Complex panel form only: Sg = Re + Im of the stale block (lower, leading n x n, stride sA
 // per item, same indexing as A) and uw = (Re u, Im u - Re u, Re u + Im u) per element (3 sv
 // doubles per item); with both, the matrix-vector step uses three real products per
@@ -76,11 +111,11 @@ template <typename T>
 void hetrd_phemv(const T* A, int lda, long long sA, int j, const T* u, T* p, long long sv, const double* tau,
                  long long stau, const T* U, const T* Q, int ldu, long long sU, int k, T* part, long long spart,
                  T* y, long long sy, int* ticket, int count, cudaStream_t s, const double* Sg = nullptr,
-                 const double* uw = nullptr, const HemvDigits* hd = nullptr);
+                 const double* uw = nullptr);
 template <typename T>
 void hetrd_pupdate(T* A, int lda, long long sA, int j, T* u, const T* p, long long sv, double* tau, long long stau,
                    T* U, T* Q, int ldu, long long sU, int k, const T* y, long long sy, int rowupd, int* ticket,
-                   int count, cudaStream_t s, double* uw = nullptr, const HemvDigits* hd = nullptr);
+                   int count, cudaStream_t s, double* uw = nullptr);
 template <typename T>
 void hetrd_finish(const T* A, int lda, long long sA, int m, double* d, double* e, long long sde, T* ph,
                   long long sph, int count, cudaStream_t s);

@@ -15,6 +15,7 @@
 // (16 flops per 16 bytes), above the DFMA pipe's balance point of ~0.15 flop/byte.  The
 // rank-2 updates are therefore deferred over panels of steps and applied as GEMMs (the
 // panel form below), which the product dispatcher can send to the tensor cores.
+#include <algorithm>
 #include <type_traits>
 
 #include "dense.h"
@@ -81,9 +82,9 @@ __device__ __forceinline__ unsigned long long maxbits(T a) {
   else return max(absbits((double)re(a)), absbits((double)im(a)));
 }
 
-// Digits of 16 consecutive entries packed as the layout's block: NPL planes of 16 bytes (the
-// kDig Re planes, then the Im planes for complex), stored with 16-byte writes.  Entry el is
-// cut below 2^{e[el]} (the scale and the equilibration folded into one exponent).
+// Digits of 16 consecutive entries of a row, NPL planes of 16 bytes (the kDig Re planes, then
+// the Im planes for complex) stored 32 rows apart (the tile's plane stride).  Entry el is cut
+// below 2^{e[el]} (the scale and the equilibration folded into one exponent).
 template <typename T, int NPL>
 __device__ __forceinline__ void store_digit_block(const T (&vals)[16], const int (&e)[16], signed char* dst) {
   uint4 o[NPL];
@@ -110,61 +111,11 @@ __device__ __forceinline__ void store_digit_block(const T (&vals)[16], const int
   }
   uint4* out = reinterpret_cast<uint4*>(dst);
 #pragma unroll
-  for (int q = 0; q < NPL; q++) out[q] = o[q];
-}
-
-// Digits of u (length j) into ud (blocks of 16 entries, each the planes' 16 bytes: Re
-// 0..7, Im 8..15; zeros from j up to the next multiple of 16) and its scale exponent fu;
-// every thread of the block takes part.
-template <typename T>
-__device__ void u_digits(const T* u, int j, signed char* ud, int* fu, const unsigned long long* rmax) {
-  constexpr bool CPX = !std::is_same<T, double>::value && !std::is_same<T, float>::value;
-  constexpr int NPL = CPX ? 2 * kDig : kDig;
-  __shared__ int mred[32];
-  const int tid = threadIdx.x, nt = blockDim.x;
-  __syncthreads();
-  // fu: the scale exponent of ũ = D u, the largest bscale(|u_i|) + d_i
-  int m = -100000;
-  for (int i0 = tid; i0 < j; i0 += 8 * nt) {  // eight independent loads in flight per thread
-    unsigned long long mb[8], rb[8];
-#pragma unroll
-    for (int q = 0; q < 8; q++) {
-      const int i = i0 + q * nt;
-      mb[q] = i < j ? maxbits(u[i]) : 0ull;
-      rb[q] = i < j ? rmax[i] : 0ull;
-    }
-#pragma unroll
-    for (int q = 0; q < 8; q++)
-      if (mb[q]) m = max(m, bscale(mb[q]) + deq(rb[q]));
-  }
-  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if ((tid & 31) == 0) mred[tid >> 5] = m;
-  __syncthreads();
-  if (tid < 32) {
-    int v = tid < (nt >> 5) ? mred[tid] : -100000;
-    for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
-    if (tid == 0) mred[0] = v;
-  }
-  __syncthreads();
-  const int e = mred[0] == -100000 ? 0 : mred[0];
-  if (tid == 0) *fu = e;
-  const int nblk = (j + 15) >> 4;
-  for (int b = tid; b < nblk; b += nt) {
-    T vals[16];
-    int ex[16];
-#pragma unroll
-    for (int el = 0; el < 16; el++) {
-      const int i = 16 * b + el;
-      vals[el] = i < j ? u[i] : zero<T>();
-      ex[el] = i < j ? e - deq(rmax[i]) : 0;  // ũ_i 2^{-fu} = u_i 2^{d_i - fu}
-    }
-    store_digit_block<T, NPL>(vals, ex, ud + (size_t)b * (NPL * 16));
-  }
+  for (int q = 0; q < NPL; q++) out[32 * q] = o[q];
 }
 
 template <typename T>
-__device__ void reflector_body(T* A, int lda, int j, T* u, double* tau, double* uw, signed char* ud = nullptr,
-                               int* fu = nullptr, const unsigned long long* rmax = nullptr) {
+__device__ void reflector_body(T* A, int lda, int j, T* u, double* tau, double* uw) {
   __shared__ double redd[32];
   const int tid = threadIdx.x, nt = blockDim.x;
   T* row = A + (size_t)j * lda;
@@ -185,7 +136,6 @@ __device__ void reflector_body(T* A, int lda, int j, T* u, double* tau, double* 
       put_uw(uw, i, i == j - 1 ? 1.0 : 0.0, 0.0);
     }
     if (tid == 0) tau[j] = 0.0;
-    if (ud) u_digits<T>(u, j, ud, fu, rmax);
     return;
   }
   const double xn = sqrt(xnorm2);
@@ -216,16 +166,13 @@ __device__ void reflector_body(T* A, int lda, int j, T* u, double* tau, double* 
     tau[j] = beta * abs2(upiv);
     row[j - 1] = conjg(ph) * (-xn);                     // lower-storage sub-diagonal
   }
-  if (ud) u_digits<T>(u, j, ud, fu, rmax);
 }
 
 template <typename T>
 __global__ void hetrd_reflector_kernel(T* A, int lda, long long sA, int j, T* u, long long sv, double* tau,
-                                       long long stau, double* uw, signed char* ud, long long sud, int* fu,
-                                       const unsigned long long* rmax, int ldr) {
+                                       long long stau, double* uw) {
   const int z = blockIdx.x;
-  reflector_body<T>(A + z * sA, lda, j, u + z * sv, tau + z * stau, uw ? uw + z * 3 * sv : nullptr,
-                    ud ? ud + z * sud : nullptr, fu ? fu + z : nullptr, rmax ? rmax + (size_t)z * ldr : nullptr);
+  reflector_body<T>(A + z * sA, lda, j, u + z * sv, tau + z * stau, uw ? uw + z * 3 * sv : nullptr);
 }
 
 // Sg[r][c] = Re A[r][c] + Im A[r][c] over the lower triangle of the leading n x n block
@@ -505,7 +452,7 @@ __global__ void __launch_bounds__(64) hetrd_digits_kernel(const T* A, int lda, l
       ex[el] = dr + (c < n ? deq(rm[c]) : 0);  // ã = a 2^{-d_r - d_c}, cut below 1
     }
     const size_t tile = (size_t)(r >> 5) * (hd.ldd >> 4) + (C0 >> 4) + cbk;
-    store_digit_block<T, NPL>(vals, ex, hd.D + z * hd.sD + tile * (32 * NPL * 16) + (size_t)(r & 31) * (NPL * 16));
+    store_digit_block<T, NPL>(vals, ex, hd.D + z * hd.sD + tile * (32 * NPL * 16) + (size_t)(r & 31) * 16);
   }
 }
 
@@ -524,139 +471,6 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int N>
 __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
-}
-
-// Shared-memory ring of the digit matrix-vector kernel: per warp STG stages, each the
-// digit planes of 32 rows x 16 columns (row stride RS 16-byte words: an odd count puts a
-// warp's 16-byte reads of 32 rows on distinct bank groups) followed by u's digits of the
-// same 16 columns.
-template <typename T>
-struct DigRing {
-  static constexpr int NPL = sizeof(T) == 16 ? 2 * kDig : kDig;
-  static constexpr int RS = NPL % 2 ? NPL : NPL + 1;
-  static constexpr int STG = 3;
-  static constexpr int SU4 = 32 * RS + NPL;
-  static constexpr int SMEM = 8 * STG * SU4 * 16;
-};
-
-// p_raw = A_stale[0:j, 0:j] u from the digits, 32 rows per CTA (lane = row), the columns in
-// eight ranges (warp w), exact int32 level sums per (row, product, level), summed over the
-// warps in shared memory, then weighted in FP64; then the common tail.  Each warp streams its
-// 16-column blocks through its own ring of STG stages (asynchronous copies, STG - 1 blocks
-// ahead of the one it multiplies; a stage is one contiguous tile, consecutive lanes copying
-// consecutive 16-byte words), and the loads in flight hold no registers.
-// Digit pairs (digits numbered from 0, most significant first) up to level s + t = 7: the
-// dropped pairs lie below 2^-59 of the scales (stopping one level earlier would leave a
-// one-signed error near the FP64 unit per term).
-// Complex: the four real products Re a Re u, Im a Im u, Re a Im u, Im a Re u
-// (Re p = first - second, Im p = third + fourth); real: the first only.
-template <typename T>
-__global__ void __launch_bounds__(256, 1) hetrd_phemv_dig_kernel(int j, const T* u, T* p, long long sv,
-                                                                 const double* tau, long long stau, const T* U,
-                                                                 const T* Q, int ldu, long long sU, int k, T* part,
-                                                                 long long spart, T* y, long long sy, int* ticket,
-                                                                 HemvDigits hd) {
-  constexpr bool CPX = sizeof(T) == 16;
-  constexpr int NP = CPX ? 4 : 1;  // real products
-  constexpr int NPL = DigRing<T>::NPL, RS = DigRing<T>::RS, STG = DigRing<T>::STG, SU4 = DigRing<T>::SU4;
-  constexpr int NL = kMaxLevel + 1;  // levels
-  static_assert(NP * NL * 33 * 8 * 4 <= DigRing<T>::SMEM, "level sums alias the ring");
-  extern __shared__ uint4 ring_all[];
-  __shared__ T prow[32];
-  const int z = blockIdx.y, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int c0 = blockIdx.x * 32, cend = min(c0 + 32, j);
-  const int j16 = (j + 15) & ~15;
-  const int chunk = (((j16 + 7) / 8) + 15) & ~15;
-  const int cb = min(j16, warp * chunk), ce = min(j16, cb + chunk);
-  const int nit = (ce - cb) >> 4;
-  // the CTA's row tile: 16-column tiles of 32 rows, each 32 * NPL 16-byte words
-  const uint4* Dt = reinterpret_cast<const uint4*>(hd.D + z * hd.sD) + (size_t)blockIdx.x * (hd.ldd >> 4) * (32 * NPL);
-  const signed char* ud = hd.ud + z * hd.sud;
-  uint4* ring = ring_all + warp * (STG * SU4);
-  // stage it % STG <- the contiguous tile of the CTA's 32 rows (rows past j - 1 hold stale
-  // digits; their results are unused) and u's digits, columns cb + 16 it .. + 15; an empty
-  // group past the range keeps the group count uniform
-  auto issue = [&](int it) {
-    if (it < nit) {
-      const int cbk = (cb >> 4) + it;
-      const uint4* src = Dt + (size_t)cbk * (32 * NPL);
-      uint4* st = ring + (it % STG) * SU4;
-#pragma unroll
-      for (int w = lane; w < 32 * NPL; w += 32) {
-        const int rr = w / NPL, q = w - rr * NPL;
-        cp_async16(st + rr * RS + q, src + w);
-      }
-      if (lane < NPL)
-        cp_async16(st + 32 * RS + lane, reinterpret_cast<const uint4*>(ud + (size_t)cbk * (NPL * 16)) + lane);
-    }
-    cp_async_commit();
-  };
-  int acc[NP][NL];
-#pragma unroll
-  for (int q = 0; q < NP; q++)
-#pragma unroll
-    for (int L = 0; L < NL; L++) acc[q][L] = 0;
-#pragma unroll
-  for (int it = 0; it < STG - 1; it++) issue(it);
-  for (int it = 0; it < nit; it++) {
-    __syncwarp();  // every lane is done with the stage refilled next
-    issue(it + STG - 1);
-    cp_async_wait<STG - 1>();
-    __syncwarp();  // stage it is complete for every lane (each row comes from several lanes)
-    const uint4* st = ring + (it % STG) * SU4;
-    uint4 av[NPL];
-#pragma unroll
-    for (int q = 0; q < NPL; q++) av[q] = st[lane * RS + q];
-#pragma unroll
-    for (int t = 0; t < kDig; t++) {
-      const uint4 ur = st[32 * RS + t];
-      uint4 ui;
-      if constexpr (CPX) ui = st[32 * RS + kDig + t];
-#pragma unroll
-      for (int s = 0; s < kDig && s + t <= kMaxLevel; s++) {
-        acc[0][s + t] = dp4x4(av[s], ur, acc[0][s + t]);
-        if constexpr (CPX) {
-          acc[1][s + t] = dp4x4(av[kDig + s], ui, acc[1][s + t]);
-          acc[2][s + t] = dp4x4(av[s], ui, acc[2][s + t]);
-          acc[3][s + t] = dp4x4(av[kDig + s], ur, acc[3][s + t]);
-        }
-      }
-    }
-  }
-  cp_async_wait<0>();
-  __syncthreads();  // every ring is idle: the level sums reuse its space
-  auto accs = reinterpret_cast<int(*)[33][8]>(ring_all);
-#pragma unroll
-  for (int q = 0; q < NP; q++)
-#pragma unroll
-    for (int L = 0; L < NL; L++) accs[q * NL + L][lane][warp] = acc[q][L];
-  __syncthreads();
-  if (tid < 32 && c0 + tid < cend) {
-    // exact sums over the warps, then 2^{d_i + fu - 12 - 8L} per level
-    const int E = deq(hd.rmax[(size_t)z * hd.ldd + c0 + tid]) + hd.fu[z] - 12;
-    double pre = 0.0, pim = 0.0;
-#pragma unroll
-    for (int L = NL - 1; L >= 0; L--) {
-      long long s0 = 0, s1 = 0, s2 = 0, s3 = 0;
-#pragma unroll
-      for (int w = 0; w < 8; w++) {
-        s0 += accs[L][tid][w];
-        if constexpr (CPX) {
-          s1 += accs[NL + L][tid][w];
-          s2 += accs[2 * NL + L][tid][w];
-          s3 += accs[3 * NL + L][tid][w];
-        }
-      }
-      pre += ldexp((double)(s0 - s1), E - 8 * L);
-      if constexpr (CPX) pim += ldexp((double)(s2 + s3), E - 8 * L);
-    }
-    if constexpr (CPX) prow[tid] = T{pre, pim};
-    else prow[tid] = pre;
-  }
-  __syncthreads();
-  const double t = tau[z * stau + j];
-  phemv_tail<T>(prow, c0, cend, u + z * sv, p + z * sv, t, U + z * sU, Q + z * sU, ldu, k, part + z * spart,
-                y + z * sy, ticket + z);
 }
 
 // Sum over aligned groups of 8 lanes (every lane of the warp takes part).
@@ -683,9 +497,7 @@ template <typename T>
 __global__ void __launch_bounds__(256) hetrd_pupdate_kernel(T* A, int lda, long long sA, int j, T* u,
                                                             const T* p, long long sv, double* tau, long long stau,
                                                             T* U, T* Q, int ldu, long long sU, int k, const T* y,
-                                                            long long sy, int rowupd, int* ticket, double* uw,
-                                                            signed char* ud, long long sud, int* fu,
-                                                            const unsigned long long* rmax, int ldr) {
+                                                            long long sy, int rowupd, int* ticket, double* uw) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* y1s = reinterpret_cast<T*>(smem_raw);
   T* y2s = y1s + (ldu + 1);
@@ -781,9 +593,542 @@ __global__ void __launch_bounds__(256) hetrd_pupdate_kernel(T* A, int lda, long 
   if (!last) return;
   if (tid == 0) ticket[z] = 0;
   __syncthreads();
-  reflector_body<T>(A, lda, j - 1, u, tau, uw, ud ? ud + z * sud : nullptr, fu ? fu + z : nullptr,
-                    rmax ? rmax + (size_t)z * ldr : nullptr);
+  reflector_body<T>(A, lda, j - 1, u, tau, uw);
 }
+
+// ------------------------------------------------------------------ persistent panel (digit form)
+//
+// All steps of a panel in one cooperative launch, G CTAs per item.  A step is a chain of
+// short dependent parts (norm and reflector, matrix-vector product, the panel's corrections,
+// the next row); as two launches per step with the reductions in a last CTA it took 32 us at
+// order 832 and 127 us at 4992 (one item), against 6 and 25 us of digit traffic and
+// arithmetic.  Here three grid barriers separate the parts and every part is spread over all
+// CTAs:
+//   1. every CTA forms the reflector's scalars from the CTAs' shares of the norm.  Warps 0-7
+//      multiply the CTA's share of the digit tiles (the R x C tiles of the block in row-tile
+//      order, cut into G equal runs, so every CTA streams the same bytes at any order) with
+//      v = conj(a) (the pivot replaced by upiv; u' = v / upiv is applied to the sums), whose
+//      digits each warp makes for the 16 columns it is about to use; warps 8-11 meanwhile
+//      store u' for the CTA's rows, form the rows' shares of Q^H u and U^H u, and after a
+//      barrier of their own add the shares of a few entries each over the CTAs.
+//   2. barrier; p from the runs that touch each row, q, row j-1 with the panel's updates, and
+//      the shares of its norm; barrier.
+// The digit tiles of the next step do not depend on this one: their first copies are issued
+// before the barriers.  Partial sums are added in a fixed order: results do not depend on
+// timing.  Every wait is bounded (a.wait SM cycles): past it the status is set, an abort flag
+// lets every CTA leave.  Bound by HBM and dp4a together at large orders (14 bytes and 34 dp4a
+// per complex entry), by the three barriers (about 1 us each) at small ones.
+// Measured per step (one item, averaged over a reduction): see hetrd_panel_ctas.
+template <typename T>
+struct PanelSmem {
+  static constexpr bool CPX = sizeof(T) == 16;
+  static constexpr int NP = CPX ? 4 : 1, NL = kMaxLevel + 1, NPL = CPX ? 2 * kDig : kDig;
+  static constexpr int STG = 3, TILE4 = 32 * NPL;  // ring stages per warp, 16-byte words per tile
+  static constexpr int RING = 8 * STG * TILE4 * 16;
+  static constexpr int ACC = NP * NL * 33 * 8 * 4;
+  static constexpr int LVL = NL * 33 * (int)sizeof(T);
+  static constexpr int UB = 8 * 2 * NPL * 16;
+  static constexpr int VEC = 4 * (kPanelMax + 1) * (int)sizeof(T);
+  static constexpr int TOTAL = RING + ACC + LVL + UB + VEC;
+  static_assert(TOTAL <= 226 * 1024, "shared memory of the panel kernel");
+};
+constexpr int kPanelThreads = 384;
+
+__device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
+  unsigned v;
+  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];\n" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void red_release(unsigned* p) {
+  asm volatile("red.release.gpu.global.add.u32 [%0], 1;\n" ::"l"(p) : "memory");
+}
+template <int ID, int N>
+__device__ __forceinline__ void bar_named() {
+  asm volatile("bar.sync %0, %1;\n" ::"n"(ID), "n"(N) : "memory");
+}
+// One thread per CTA: arrive on *cnt and wait for target arrivals; false on abort or timeout.
+__device__ __forceinline__ bool grid_arrive_wait(unsigned* cnt, unsigned target, unsigned* abortf, long long limit) {
+  __threadfence();
+  red_release(cnt);
+  const long long t0 = clock64();
+  while ((int)(ld_acquire(cnt) - target) < 0) {
+    if (*(volatile unsigned*)abortf) return false;
+    if (clock64() - t0 > limit) {
+      atomicExch(abortf, 1u);
+      return false;
+    }
+  }
+  __threadfence();
+  return true;
+}
+
+// Runs of digit tiles: T = R C tiles of order j, CTA b of G has [run0(b), run0(b + 1)).
+struct PanelRuns {
+  int C, R;
+  long long T;
+  int G;
+  __device__ PanelRuns(int j, int G_) : C((j + 15) >> 4), R((j + 31) >> 5), T((long long)R * C), G(G_) {}
+  __device__ int run0(int b) const { return (int)((long long)b * T / G); }
+  __device__ int owner(int t) const { return (int)((((long long)t + 1) * G - 1) / T); }  // run holding tile t
+};
+
+template <typename T>
+__global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const PanelArgs<T> a, int maxseg) {
+  using SM = PanelSmem<T>;
+  constexpr bool CPX = SM::CPX;
+  constexpr int NP = SM::NP, NL = SM::NL, NPL = SM::NPL, STG = SM::STG, TILE4 = SM::TILE4;
+  extern __shared__ __align__(128) unsigned char psm[];
+  uint4* ring_all = reinterpret_cast<uint4*>(psm);
+  auto accs = reinterpret_cast<int(*)[33][8]>(psm + SM::RING);
+  T* lvl = reinterpret_cast<T*>(psm + SM::RING + SM::ACC);  // [NL][33]
+  unsigned char* ubuf = psm + SM::RING + SM::ACC + SM::LVL;
+  T* y1s = reinterpret_cast<T*>(psm + SM::RING + SM::ACC + SM::LVL + SM::UB);
+  T* y2s = y1s + (kPanelMax + 1);
+  T* ujs = y2s + (kPanelMax + 1);
+  T* qjs = ujs + (kPanelMax + 1);
+  __shared__ T s_inv, s_upiv, s_sub, s_kq, s_pj, s_us[64];
+  __shared__ double s_tau, s_red[12];
+  __shared__ int s_fu, s_ok, s_abort, s_rede[12];
+
+  const int z = blockIdx.y, b = blockIdx.x, G = gridDim.x;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int lda = a.lda, ldu = a.ldu;
+  T* A = a.A + z * a.sA;
+  T* U = a.U + z * a.sU;
+  T* Q = a.Q + z * a.sU;
+  T* arow2 = a.arow + z * 2 * a.sv;
+  T* part = a.part + (long long)z * a.gs * (2 * kPanelMax);
+  T* y = a.y + (long long)z * (2 * kPanelMax);
+  T* P = a.P + z * a.sP;
+  T* dot = a.dot + (long long)z * a.gs;
+  double* nrm = a.nrm + (long long)z * a.gs;
+  int* mex = a.mex + (long long)z * a.gs;
+  double* tau = a.tau + z * a.stau;
+  unsigned* bar = a.bar + 4 * z;
+  const unsigned long long* rmax = a.hd.rmax + (size_t)z * a.hd.ldd;
+  const uint4* D = reinterpret_cast<const uint4*>(a.hd.D + z * a.hd.sD);
+  const int ldc = a.hd.ldd >> 4;  // tiles per row tile
+  const int cs = (a.jh + G - 1) / G, c0 = b * cs, c1 = min(c0 + cs, a.jh);  // this CTA's rows
+  unsigned arrived = a.base, arrivedv = a.basev;  // targets of the two counters
+  constexpr int NOEXP = -100000;
+
+  // shares of the next reflector's norm (over the entries before the pivot) and scale
+  auto put_norm = [&](double n2, int e) {
+    n2 = warp_sum(n2);
+    e = __reduce_max_sync(0xffffffffu, e);
+    if (lane == 0) {
+      s_red[warp] = n2;
+      s_rede[warp] = e;
+    }
+    __syncthreads();
+    if (tid == 0) {
+      double t = 0.0;
+      int m = NOEXP;
+      for (int w = 0; w < 12; w++) {
+        t += s_red[w];
+        m = max(m, s_rede[w]);
+      }
+      nrm[b] = t;
+      mex[b] = m;
+    }
+  };
+  auto scale_of = [&](T v, int i) -> int {
+    const unsigned long long mb = maxbits(v);
+    return mb ? bscale(mb) + deq(rmax[i]) : NOEXP;
+  };
+  // full barrier over the item's CTAs; false once any wait expired (uniform over the CTA)
+  auto barrier = [&]() -> bool {
+    __syncthreads();
+    arrived += (unsigned)G;
+    if (tid == 0 && !grid_arrive_wait(bar, arrived, bar + 2, a.wait)) s_abort = 1;
+    __syncthreads();
+    return s_abort == 0;
+  };
+  uint4* ring = ring_all + warp * (STG * TILE4);
+  // stage i % STG <- the warp's i-th tile of the run of step j
+  auto issue = [&](const PanelRuns& pr, int i) {
+    const int t = pr.run0(b) + warp + 8 * i;
+    if (t < pr.run0(b + 1)) {
+      const int r = t / pr.C, cb = t - r * pr.C;
+      const uint4* src = D + ((size_t)r * ldc + cb) * TILE4 + lane;
+      uint4* st = ring + (i % STG) * TILE4 + lane;
+#pragma unroll
+      for (int q = 0; q < NPL; q++) cp_async16(st + 32 * q, src + 32 * q);
+    }
+    cp_async_commit();
+  };
+
+  if (tid == 0) s_abort = 0;
+  {
+    const int j = a.jh;
+    T* ar = arow2 + (j & 1) * a.sv;
+    double n2 = 0.0;
+    int e = NOEXP;
+    for (int c = c0 + tid; c < c1; c += kPanelThreads) {
+      const T v = A[(size_t)j * lda + c];
+      ar[c] = v;
+      if (c < j - 1) {
+        n2 += abs2(v);
+        e = max(e, scale_of(v, c));
+      }
+    }
+    __syncthreads();
+    put_norm(n2, e);
+    if (warp < 8) {
+      const PanelRuns pr(j, G);
+#pragma unroll
+      for (int i = 0; i < STG - 1; i++) issue(pr, i);
+    }
+  }
+  bool live = barrier();
+
+  for (int j = a.jh; j >= a.jl && live; j--) {
+    const int k = a.jh - j;
+    const T* ar = arow2 + (j & 1) * a.sv;
+    if (warp == 0) {
+      double tail = 0.0;
+      int e = NOEXP;
+      for (int g = lane; g < G; g += 32) {
+        tail += __ldcg(nrm + g);
+        e = max(e, __ldcg(mex + g));
+      }
+      tail = warp_sum(tail);
+      e = __reduce_max_sync(0xffffffffu, e);
+      if (lane == 0) {
+        const T alpha = conjg(ldcg(ar + j - 1));
+        if (!(tail > 0.0)) {  // nothing to annihilate: P_j = I
+          s_ok = 0;
+          s_inv = s_upiv = from_real<T>(1.0);
+          s_sub = conjg(alpha);
+          s_tau = 0.0;
+          e = scale_of(from_real<T>(1.0), j - 1);
+        } else {
+          const double a2 = abs2(alpha), xn = sqrt(tail + a2), aa = sqrt(a2);
+          const T ph = aa > 0.0 ? alpha * (1.0 / aa) : from_real<T>(1.0);
+          const T upiv = ph * (aa + xn);  // alpha + ph xn
+          const double up2 = abs2(upiv);
+          s_ok = 1;
+          s_upiv = upiv;
+          s_inv = conjg(upiv) * (1.0 / up2);
+          s_sub = conjg(ph) * (-xn);  // lower-storage sub-diagonal
+          s_tau = 2.0 / (tail + up2) * up2;
+          e = max(e, scale_of(upiv, j - 1));
+        }
+        s_fu = e;
+        if (b == 0) tau[j] = s_tau;
+      }
+    }
+    __syncthreads();
+    const T inv = s_inv;
+    const bool refl = s_ok != 0;
+
+    if (warp < 8) {
+      // ---- matrix-vector product over the CTA's run of tiles
+      const PanelRuns pr(j, G);
+      const int t0 = pr.run0(b), t1 = pr.run0(b + 1), fu = s_fu;
+      int acc[NP][NL];
+#pragma unroll
+      for (int q = 0; q < NP; q++)
+#pragma unroll
+        for (int L = 0; L < NL; L++) acc[q][L] = 0;
+      // entry of v this lane makes digits of, for the warp's i-th tile: lane & 15, Re (lanes
+      // 0-15) or Im (lanes 16-31)
+      auto vload = [&](int i, double& x, int& ex) {
+        x = 0.0;
+        ex = 0;
+        const int t = t0 + warp + 8 * i;
+        if (t >= t1) return;
+        const int c = 16 * (t % pr.C) + (lane & 15);
+        if (c >= j) return;
+        ex = fu - deq(rmax[c]);
+        T v = c == j - 1 ? s_upiv : (refl ? conjg(ldcg(ar + c)) : zero<T>());
+        x = lane < 16 ? re(v) : im(v);
+      };
+      double xv;
+      int xe;
+      vload(0, xv, xe);
+      T d0 = zero<T>();
+      int i = 0;
+      for (int seg = 0, r = t0 / pr.C; t0 < t1 && r * pr.C < t1; r++, seg++) {
+        const int te = min(t1, (r + 1) * pr.C);
+        for (; t0 + warp + 8 * i < te; i++) {
+          int d[kDig];
+          digits8(xv, xe, d);
+          unsigned char* ub = ubuf + (warp * 2 + (i & 1)) * (NPL * 16);
+          if (CPX || lane < 16) {
+#pragma unroll
+            for (int q = 0; q < kDig; q++)
+              ub[((lane >> 4) * kDig + q) * 16 + (lane & 15)] = (unsigned char)(d[q] & 0xff);
+          }
+          vload(i + 1, xv, xe);
+          __syncwarp();  // the digits are written, and every lane is done with the stage refilled next
+          issue(pr, i + STG - 1);
+          cp_async_wait<STG - 1>();
+          __syncwarp();
+          const uint4* st = ring + (i % STG) * TILE4 + lane;
+          const uint4* uq = reinterpret_cast<const uint4*>(ub);
+          uint4 av[NPL];
+#pragma unroll
+          for (int q = 0; q < NPL; q++) av[q] = st[32 * q];
+#pragma unroll
+          for (int t = 0; t < kDig; t++) {
+            const uint4 ur = uq[t];
+            uint4 ui;
+            if constexpr (CPX) ui = uq[kDig + t];
+#pragma unroll
+            for (int q = 0; q < kDig && q + t <= kMaxLevel; q++) {
+              acc[0][q + t] = dp4x4(av[q], ur, acc[0][q + t]);
+              if constexpr (CPX) {
+                acc[1][q + t] = dp4x4(av[kDig + q], ui, acc[1][q + t]);
+                acc[2][q + t] = dp4x4(av[q], ui, acc[2][q + t]);
+                acc[3][q + t] = dp4x4(av[kDig + q], ur, acc[3][q + t]);
+              }
+            }
+          }
+        }
+        // the row tile's sums: over the warps exactly, one level per warp, then in FP64
+#pragma unroll
+        for (int q = 0; q < NP; q++)
+#pragma unroll
+          for (int L = 0; L < NL; L++) {
+            accs[q * NL + L][lane][warp] = acc[q][L];
+            acc[q][L] = 0;
+          }
+        bar_named<1, 256>();
+        {
+          long long s0 = 0, s1 = 0, s2 = 0, s3 = 0;
+#pragma unroll
+          for (int w = 0; w < 8; w++) {
+            s0 += accs[warp][lane][w];
+            if constexpr (CPX) {
+              s1 += accs[NL + warp][lane][w];
+              s2 += accs[2 * NL + warp][lane][w];
+              s3 += accs[3 * NL + warp][lane][w];
+            }
+          }
+          const double wl = __longlong_as_double((long long)(1023 - 8 * warp) << 52);  // 2^{-8 L}
+          if constexpr (CPX) lvl[warp * 33 + lane] = T{(double)(s0 - s1) * wl, (double)(s2 + s3) * wl};
+          else lvl[warp * 33 + lane] = (double)s0 * wl;
+        }
+        bar_named<1, 256>();
+        if (warp == 0) {
+          T pv = zero<T>();
+#pragma unroll
+          for (int L = NL - 1; L >= 0; L--) pv += lvl[L * 33 + lane];
+          const int row = 32 * r + lane;
+          if (row < j) {
+            const int E = deq(rmax[row]) + fu - 12;
+            if constexpr (CPX) pv = inv * T{ldexp(pv.x, E), ldexp(pv.y, E)};
+            else pv = inv * ldexp(pv, E);
+            P[((size_t)b * maxseg + seg) * 32 + lane] = pv;
+            const T ur = row == j - 1 ? from_real<T>(1.0) : (refl ? conjg(ldcg(ar + row)) * inv : zero<T>());
+            macc(d0, ur, pv);
+          }
+        }
+      }
+      if (warp == 0) {
+        d0 = warp_sum(d0);
+        if (lane == 0) dot[b] = d0;
+      }
+      if (j > a.jl) {  // the next step's first tiles
+        const PanelRuns pn(j - 1, G);
+        __syncwarp();
+#pragma unroll
+        for (int q = 0; q < STG - 1; q++) issue(pn, q);
+      }
+    } else {
+      // ---- u' for this CTA's rows, and their shares of Q^H u (entries 0..k-1) and U^H u
+      const int vt = tid - 256, ce = min(c1, j);
+      T ya[2] = {zero<T>(), zero<T>()};
+      for (int r0 = c0; r0 < ce; r0 += 64) {
+        const int nr = min(64, ce - r0);
+        bar_named<2, 128>();
+        if (vt < nr) {
+          const int c = r0 + vt;
+          const T av = ldcg(ar + c);
+          const T uv = c == j - 1 ? from_real<T>(1.0) : (refl ? conjg(av) * inv : zero<T>());
+          s_us[vt] = uv;
+          U[(size_t)c * ldu + k] = uv;
+          A[(size_t)j * lda + c] = c == j - 1 ? s_sub : (refl ? uv : av);
+        }
+        bar_named<2, 128>();
+#pragma unroll
+        for (int h = 0; h < 2; h++) {
+          const int en = vt + 128 * h;
+          if (en >= 2 * k) break;
+          const T* src = (en < k ? Q + en : U + (en - k)) + (size_t)r0 * ldu;
+          for (int r = 0; r < nr; r += 8) {  // eight rows' loads in flight
+            T v[8];
+#pragma unroll
+            for (int q = 0; q < 8; q++) v[q] = r + q < nr ? src[(size_t)(r + q) * ldu] : zero<T>();
+#pragma unroll
+            for (int q = 0; q < 8; q++)
+              if (r + q < nr) macc(ya[h], v[q], s_us[r + q]);
+          }
+        }
+      }
+      if (k > 0) {
+#pragma unroll
+        for (int h = 0; h < 2; h++)
+          if (vt + 128 * h < 2 * k) part[(size_t)b * (2 * kPanelMax) + vt + 128 * h] = ya[h];
+        bar_named<2, 128>();
+        arrivedv += (unsigned)G;
+        if (vt == 0 && !grid_arrive_wait(bar + 1, arrivedv, bar + 2, a.wait)) s_abort = 1;
+        bar_named<2, 128>();
+        for (int en = b + G * (warp - 8); en < 2 * k; en += 4 * G) {
+          T v = zero<T>();
+          for (int g = lane; g < G; g += 32) v += ldcg(part + (size_t)g * (2 * kPanelMax) + en);
+          v = warp_sum(v);
+          if (lane == 0) y[en] = v;
+        }
+      }
+    }
+    if (!barrier()) break;
+
+    // ---- p, q, and row j-1 with the panel's updates
+    const bool rowupd = j > a.jl;
+    const double t = s_tau;
+    for (int s = tid; s < k; s += kPanelThreads) {
+      y1s[s] = ldcg(y + s);
+      y2s[s] = ldcg(y + k + s);
+      ujs[s] = ldcg(U + (size_t)(j - 1) * ldu + s);
+      qjs[s] = ldcg(Q + (size_t)(j - 1) * ldu + s);
+    }
+    __syncthreads();
+    const PanelRuns pr(j, G);
+    auto p_of = [&](int row, int l, int nl) -> T {  // lanes l of nl: their share of p_raw[row]
+      const int r = row >> 5;
+      const int b0 = pr.owner(r * pr.C), b1 = pr.owner((r + 1) * pr.C - 1);
+      T v = zero<T>();
+      for (int g = b0 + l; g <= b1; g += nl) {
+        const int g0 = pr.run0(g);
+        if (g0 < pr.run0(g + 1)) v += ldcg(P + ((size_t)g * maxseg + (r - g0 / pr.C)) * 32 + (row & 31));
+      }
+      return v;
+    };
+    if (warp == 0) {
+      T tot = zero<T>(), w = zero<T>();
+      for (int g = lane; g < G; g += 32) tot += ldcg(dot + g);
+      for (int s = lane; s < k; s += 32) {
+        macc(w, y2s[s], y1s[s]);
+        macc(w, y1s[s], y2s[s]);
+      }
+      tot = warp_sum(tot);
+      w = warp_sum(w);
+      if (lane == 0) s_kq = (0.5 * t) * (t * (tot - w));
+    } else if (warp == 1 && rowupd) {  // p[j-1] - U y1 - Q y2 of row j-1
+      T v = p_of(j - 1, lane, 32), corr = zero<T>();
+      for (int s = lane; s < k; s += 32) {
+        mac(corr, ujs[s], y1s[s]);
+        mac(corr, qjs[s], y2s[s]);
+      }
+      v = warp_sum(v - corr);
+      if (lane == 0) s_pj = v;
+    }
+    // groups of 8 lanes, one row each (48 rows at a time)
+    const int grp = tid >> 3, gl = tid & 7, ce = min(c1, j);
+    double n2 = 0.0;
+    int ex = NOEXP;
+    bool synced = false;
+    T* an = arow2 + ((j - 1) & 1) * a.sv;
+    for (int base = c0; base < ce || !synced; base += 48) {
+      const int c = base + grp;
+      const bool ok = c < ce;
+      T pv = zero<T>(), rs = zero<T>(), uc = zero<T>(), aold = zero<T>();
+      if (ok) {
+        pv = p_of(c, gl, 8);
+        const T* Uc = U + (size_t)c * ldu;
+        const T* Qc = Q + (size_t)c * ldu;
+        if (gl == 0) {
+          uc = ldcg(Uc + k);
+          if (rowupd) aold = A[(size_t)(j - 1) * lda + c];
+        }
+        for (int s0 = gl; s0 < k; s0 += 32) {  // four steps' loads in flight
+          T ucv[4], qcv[4];
+#pragma unroll
+          for (int q = 0; q < 4; q++) {
+            const int sq = min(s0 + 8 * q, k - 1);
+            ucv[q] = Uc[sq];
+            qcv[q] = Qc[sq];
+          }
+#pragma unroll
+          for (int q = 0; q < 4; q++) {
+            const int sq = s0 + 8 * q;
+            if (sq < k) {
+              mac(pv, -ucv[q], y1s[sq]);
+              mac(pv, -qcv[q], y2s[sq]);
+              if (rowupd) {
+                mac(rs, ujs[sq], conjg(qcv[q]));
+                mac(rs, qjs[sq], conjg(ucv[q]));
+              }
+            }
+          }
+        }
+      }
+      pv = group8_sum(pv);
+      rs = group8_sum(rs);
+      if (!synced) {  // kq and row j-1's share
+        __syncthreads();
+        synced = true;
+      }
+      if (ok && gl == 0) {
+        const T kq = s_kq, qc = t * pv - kq * uc;
+        Q[(size_t)c * ldu + k] = qc;
+        if (rowupd) {
+          const T qj = t * s_pj - kq;  // u'[j-1] = 1
+          rs += conjg(qc);
+          mac(rs, qj, conjg(uc));
+          const T an_c = aold - rs;
+          if (c == j - 1) {
+            A[(size_t)(j - 1) * lda + c] = an_c;
+          } else {
+            an[c] = an_c;
+            if (c < j - 2) {
+              n2 += abs2(an_c);
+              ex = max(ex, scale_of(an_c, c));
+            }
+          }
+        }
+      }
+    }
+    if (!rowupd) break;
+    put_norm(n2, ex);
+    live = barrier();
+  }
+  cp_async_wait<0>();
+  if (s_abort && tid == 0 && b == 0) set_status(a.st ? a.st + z : nullptr, ST_ETIMEOUT, -3);
+}
+
+// CTAs per item: as many as give each about kPanelTiles digit tiles (fewer CTAs make the
+// barriers cheaper and leave SMs to other streams), at most one per SM over all items.
+constexpr int kPanelTiles = 12;
+template <typename T>
+int hetrd_panel_ctas(int jh, int items) {
+  static const int cap = [] {
+    int dev = 0, sms = 0, per = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    cudaFuncSetAttribute(hetrd_panel_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, PanelSmem<T>::TOTAL);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, hetrd_panel_kernel<T>, kPanelThreads, PanelSmem<T>::TOTAL);
+    cudaGetLastError();
+    return sms * (per > 0 ? 1 : 0);
+  }();
+  const int top = std::min(cap / items, kPanelCtas);
+  const long long tiles = (long long)((jh + 31) / 32) * ((jh + 15) / 16);
+  return (int)std::min<long long>(top, (tiles + kPanelTiles - 1) / kPanelTiles);
+}
+
+template <typename T>
+bool hetrd_panel(const PanelArgs<T>& a, int G, int items, cudaStream_t s) {
+  cudaFuncSetAttribute(hetrd_panel_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, PanelSmem<T>::TOTAL);
+  int maxseg = (a.jh + 31) / 32 / G + 2;
+  PanelArgs<T> arg = a;
+  void* args[] = {&arg, &maxseg};
+  count_launch();
+  return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(hetrd_panel_kernel<T>), dim3(G, items),
+                                     dim3(kPanelThreads), args, PanelSmem<T>::TOTAL, s) == cudaSuccess;
+}
+
 
 // d_i = Re A_ii, e_i = |A_{i+1,i}|, ph_0 = 1, ph_{i+1} = ph_i A_{i+1,i}/|A_{i+1,i}|.
 template <typename T>
@@ -839,11 +1184,9 @@ __global__ void gather_reflectors_kernel(const T* A, int lda, long long sA, cons
 
 template <typename T>
 void hetrd_reflector(T* A, int lda, long long sA, int j, T* u, long long sv, double* tau, long long stau, int count,
-                     cudaStream_t s, double* uw, const HemvDigits* hd) {
+                     cudaStream_t s, double* uw) {
   count_launch();
-  hetrd_reflector_kernel<T><<<count, 256, 0, s>>>(A, lda, sA, j, u, sv, tau, stau, uw, hd ? hd->ud : nullptr,
-                                                  hd ? hd->sud : 0, hd ? hd->fu : nullptr, hd ? hd->rmax : nullptr,
-                                                  hd ? hd->ldd : 0);
+  hetrd_reflector_kernel<T><<<count, 256, 0, s>>>(A, lda, sA, j, u, sv, tau, stau, uw);
 }
 
 template <typename T>
@@ -866,18 +1209,8 @@ void hetrd_sums(const zc* A, int lda, long long sA, int n, double* Sg, int count
 template <typename T>
 void hetrd_phemv(const T* A, int lda, long long sA, int j, const T* u, T* p, long long sv, const double* tau,
                  long long stau, const T* U, const T* Q, int ldu, long long sU, int k, T* part, long long spart,
-                 T* y, long long sy, int* ticket, int count, cudaStream_t s, const double* Sg, const double* uw,
-                 const HemvDigits* hd) {
+                 T* y, long long sy, int* ticket, int count, cudaStream_t s, const double* Sg, const double* uw) {
   count_launch();
-  if constexpr (std::is_same<T, double>::value || std::is_same<T, zc>::value) {
-    if (hd) {
-      constexpr int sm = DigRing<T>::SMEM;
-      cudaFuncSetAttribute(hetrd_phemv_dig_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-      hetrd_phemv_dig_kernel<T><<<dim3((j + 31) / 32, count), 256, sm, s>>>(j, u, p, sv, tau, stau, U, Q, ldu, sU,
-                                                                            k, part, spart, y, sy, ticket, *hd);
-      return;
-    }
-  }
   if ((long long)((j + 63) / 64) * count >= 4 * 152)
     hetrd_phemv_kernel<T, 64><<<dim3((j + 63) / 64, count), 256, 0, s>>>(A, lda, sA, j, u, p, sv, tau, stau, U, Q,
                                                                          ldu, sU, k, part, spart, y, sy, ticket, Sg,
@@ -891,15 +1224,12 @@ void hetrd_phemv(const T* A, int lda, long long sA, int j, const T* u, T* p, lon
 template <typename T>
 void hetrd_pupdate(T* A, int lda, long long sA, int j, T* u, const T* p, long long sv, double* tau, long long stau,
                    T* U, T* Q, int ldu, long long sU, int k, const T* y, long long sy, int rowupd, int* ticket,
-                   int count, cudaStream_t s, double* uw, const HemvDigits* hd) {
+                   int count, cudaStream_t s, double* uw) {
   const int sm = (int)(4 * sizeof(T) * (ldu + 1));
   if (sm > 48 * 1024) cudaFuncSetAttribute(hetrd_pupdate_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
   count_launch();
   hetrd_pupdate_kernel<T><<<dim3((j + 63) / 64, count), 256, sm, s>>>(A, lda, sA, j, u, p, sv, tau, stau, U, Q, ldu,
-                                                                      sU, k, y, sy, rowupd, ticket, uw,
-                                                                      hd ? hd->ud : nullptr, hd ? hd->sud : 0,
-                                                                      hd ? hd->fu : nullptr, hd ? hd->rmax : nullptr,
-                                                                      hd ? hd->ldd : 0);
+                                                                      sU, k, y, sy, rowupd, ticket, uw);
 }
 
 template <typename T>
@@ -958,30 +1288,32 @@ void narrow_lower(const T* A, int lda, long long sA, TL* B, int ldb, long long s
 
 #define INST(T)                                                                                            \
   template void hetrd_reflector<T>(T*, int, long long, int, T*, long long, double*, long long, int,         \
-                                   cudaStream_t, double*, const HemvDigits*);                              \
+                                   cudaStream_t, double*);                                                 \
   template void hetrd_phemv<T>(const T*, int, long long, int, const T*, T*, long long, const double*,        \
                                long long, const T*, const T*, int, long long, int, T*, long long, T*, long long, \
-                               int*, int, cudaStream_t, const double*, const double*, const HemvDigits*);  \
+                               int*, int, cudaStream_t, const double*, const double*);                     \
   template void hetrd_pupdate<T>(T*, int, long long, int, T*, const T*, long long, double*, long long, T*,  \
                                  T*, int, long long, int, const T*, long long, int, int*, int, cudaStream_t, \
-                                 double*, const HemvDigits*);                                              \
+                                 double*);                                                                \
   template void hetrd_finish<T>(const T*, int, long long, int, double*, double*, long long, T*, long long,   \
                                 int, cudaStream_t);                                                        \
   template void gather_reflectors<T, T>(const T*, int, long long, const double*, long long, int, int, T*,    \
                                         int, long long, double*, long long, int, cudaStream_t);               \
-  template void hetrd_digits<T>(const T*, int, long long, int, const HemvDigits&, int, cudaStream_t);
+  template void hetrd_digits<T>(const T*, int, long long, int, const HemvDigits&, int, cudaStream_t);           \
+  template int hetrd_panel_ctas<T>(int, int);                                                              \
+  template bool hetrd_panel<T>(const PanelArgs<T>&, int, int, cudaStream_t);
 INST(double)
 INST(zc)
 #undef INST
 #define INST(T)                                                                                            \
   template void hetrd_reflector<T>(T*, int, long long, int, T*, long long, double*, long long, int,         \
-                                   cudaStream_t, double*, const HemvDigits*);                              \
+                                   cudaStream_t, double*);                                                 \
   template void hetrd_phemv<T>(const T*, int, long long, int, const T*, T*, long long, const double*,        \
                                long long, const T*, const T*, int, long long, int, T*, long long, T*, long long, \
-                               int*, int, cudaStream_t, const double*, const double*, const HemvDigits*);  \
+                               int*, int, cudaStream_t, const double*, const double*);                     \
   template void hetrd_pupdate<T>(T*, int, long long, int, T*, const T*, long long, double*, long long, T*,  \
                                  T*, int, long long, int, const T*, long long, int, int*, int, cudaStream_t, \
-                                 double*, const HemvDigits*);                                              \
+                                 double*);                                                                \
   template void hetrd_finish<T>(const T*, int, long long, int, double*, double*, long long, T*, long long,   \
                                 int, cudaStream_t);
 INST(float)
