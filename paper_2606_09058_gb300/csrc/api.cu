@@ -302,7 +302,7 @@ gks_status ensure_ws(gks_ctx* c, int m, int n, int nk, int es, int nc) {
     c->oppart = a.take<char>(elems(2LL * gs * kPanelMax));
     c->opy = a.take<char>(elems(2LL * kPanelMax));
     c->opP = a.take<char>(elems(panel_partials(m, gs)));
-    c->opdot = a.take<char>(elems(gs));
+    c->opdot = a.take<double>((size_t)gs * nk);
     c->opnrm = a.take<double>((size_t)gs * nk);
     c->opmex = a.take<int>((size_t)gs * nk);
     c->opbar = a.take<unsigned>((size_t)4 * nk);
@@ -978,7 +978,7 @@ bool hetrd_digit_run(gks_ctx* c, T* A, int M, int nk) {
     {
       Rec r(c, PC_HETRD_HEMV, fl, by);
       for (int z0 = 0, q = 0; z0 < nk; z0 += per, q++) {
-        const int cnt = std::min(per, nk - z0), G = std::min(gs, hetrd_panel_ctas<T>(jh, cnt));
+        const int cnt = std::min(per, nk - z0);
         pa.A = A + z0 * c->sMM;
         pa.jh = jh;
         pa.jl = jl;
@@ -989,21 +989,17 @@ bool hetrd_digit_run(gks_ctx* c, T* A, int M, int nk) {
         pa.part = at<T>(c, c->oppart) + (size_t)z0 * gs * 2 * kPanelMax;
         pa.y = at<T>(c, c->opy) + (size_t)z0 * 2 * kPanelMax;
         pa.P = at<T>(c, c->opP) + z0 * pa.sP;
-        pa.dot = at<T>(c, c->opdot) + (size_t)z0 * gs;
+        pa.dot = at<double>(c, c->opdot) + (size_t)z0 * gs;
         pa.nrm = at<double>(c, c->opnrm) + (size_t)z0 * gs;
         pa.mex = at<int>(c, c->opmex) + (size_t)z0 * gs;
         pa.bar = at<unsigned>(c, c->opbar) + (size_t)4 * z0;
-        pa.base = base[q];
-        pa.basev = basev[q];
         pa.hd.D = hd.D + z0 * hd.sD;
         pa.hd.rmax = hd.rmax + (size_t)z0 * ldd;
         pa.st = c->st ? c->st + z0 : nullptr;
-        if (!hetrd_panel<T>(pa, G, cnt, s)) {
+        if (!hetrd_panel<T>(pa, cnt, &base[q], &basev[q], s)) {
           cudaGetLastError();
           return false;
         }
-        base[q] += 2u * steps * G;
-        basev[q] += (unsigned)(steps - 1) * G;
       }
     }
     panel_deferred<T>(c, A, M, jl, steps, nk);

@@ -67,10 +67,11 @@ void hetrd_digits(const T* A, int lda, long long sA, int n, const HemvDigits& hd
 // One panel of the digit form: steps jh .. jl.  Per item (strides in elements): arow 2 x sv,
 // part gs x 2 kPanelMax, y 2 kPanelMax, P panel_partials(m, gs), dot, nrm and mex gs each (gs:
 // CTAs per item at most), bar 4 counters zeroed once per reduction.  base, basev: arrivals at
-// the two barrier counters so far; a panel of s steps on G CTAs adds 2 s G and (s - 1) G.
+// the two barrier counters so far; a panel of s steps on G CTAs adds 2 s G and (s - 1) G
+// (none in the cluster form).
 constexpr int kPanelMax = 128;   // steps per panel at most
 constexpr int kPanelCtas = 160;  // CTAs per item at most
-constexpr int panel_gs(int items) { return items >= kPanelCtas ? 1 : kPanelCtas / items; }
+constexpr int panel_gs(int items) { return items >= kPanelCtas / 16 ? 16 : kPanelCtas / items; }
 constexpr long long panel_partials(int m, int gs) { return ((long long)(m + 31) / 32 + 2 * gs) * 32; }
 template <typename T>
 struct PanelArgs {
@@ -85,7 +86,8 @@ struct PanelArgs {
   long long sU;
   T* arow;
   long long sv;
-  T *part, *y, *P, *dot;
+  T *part, *y, *P;
+  double* dot;
   long long sP;
   double* nrm;
   int* mex;
@@ -96,12 +98,14 @@ struct PanelArgs {
   DevStatus* st;
   long long wait;
 };
-// CTAs per item for a panel of order jh on `items` items (0: not even one per item fits).
+// CTAs per item of the grid form for a panel of order jh on `items` items (0: not even one
+// per item fits).
 template <typename T>
 int hetrd_panel_ctas(int jh, int items);
-// False if the cooperative launch was refused (then nothing ran).
+// base and basev advance by the launch's arrivals.  False if the launch was refused (then
+// nothing ran).
 template <typename T>
-bool hetrd_panel(const PanelArgs<T>& a, int G, int items, cudaStream_t s);
+bool hetrd_panel(PanelArgs<T> a, int items, unsigned* base, unsigned* basev, cudaStream_t s);
 // Complex panel form only: Sg = Re + Im of the stale block (lower, leading n x n, stride sA
 // per item, same indexing as A) and uw = (Re u, Im u - Re u, Re u + Im u) per element (3 sv
 // doubles per item); with both, the matrix-vector step uses three real products per

@@ -486,6 +486,8 @@ __device__ __forceinline__ float group8_sum(float v) {
   return v;
 }
 __device__ __forceinline__ cf group8_sum(cf v) { return cf{group8_sum(v.x), group8_sum(v.y)}; }
+__device__ __forceinline__ double shfl_xor(double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
+__device__ __forceinline__ zc shfl_xor(zc v, int o) { return zc{shfl_xor(v.x, o), shfl_xor(v.y, o)}; }
 
 // Step j, second half: q = tau (p_raw - U y1 - Q y2) - kq u for the rows of this CTA (64
 // per CTA), stored with u as column k of Q and U.  With rowupd, row j-1 of A (columns
@@ -625,8 +627,8 @@ struct PanelSmem {
   static constexpr int NP = CPX ? 4 : 1, NL = kMaxLevel + 1, NPL = CPX ? 2 * kDig : kDig;
   static constexpr int STG = 3, TILE4 = 32 * NPL;  // ring stages per warp, 16-byte words per tile
   static constexpr int RING = 8 * STG * TILE4 * 16;
-  static constexpr int ACC = NP * NL * 33 * 8 * 4;
-  static constexpr int LVL = NL * 33 * (int)sizeof(T);
+  static constexpr int ACC = NP * NL * 8 * 32 * 4;   // [product, level][warp][row]
+  static constexpr int LVL = NL * 32 * (int)sizeof(T);  // [level][row] 64-bit sums, Re then Im
   static constexpr int UB = 8 * 2 * NPL * 16;
   static constexpr int VEC = 4 * (kPanelMax + 1) * (int)sizeof(T);
   static constexpr int TOTAL = RING + ACC + LVL + UB + VEC;
@@ -648,46 +650,73 @@ __device__ __forceinline__ void bar_named() {
 }
 // One thread per CTA: arrive on *cnt and wait for target arrivals; false on abort or timeout.
 __device__ __forceinline__ bool grid_arrive_wait(unsigned* cnt, unsigned target, unsigned* abortf, long long limit) {
-  __threadfence();
   red_release(cnt);
   const long long t0 = clock64();
-  while ((int)(ld_acquire(cnt) - target) < 0) {
+  for (unsigned n = 1; (int)(ld_acquire(cnt) - target) < 0; n++) {
+    if (n & 63u) continue;
     if (*(volatile unsigned*)abortf) return false;
     if (clock64() - t0 > limit) {
       atomicExch(abortf, 1u);
       return false;
     }
   }
-  __threadfence();
   return true;
 }
 
-// Runs of digit tiles: T = R C tiles of order j, CTA b of G has [run0(b), run0(b + 1)).
+// The same over the CTAs of a cluster: an mbarrier of G arrivals in every CTA.  Lanes below G
+// arrive on the barrier of CTA `lane`; a thread waits for its own CTA's phase.
+__device__ __forceinline__ void cluster_arrive(uint64_t* bar, int cta) {
+  asm volatile(
+      "{\n .reg .b32 ra;\n mapa.shared::cluster.u32 ra, %0, %1;\n"
+      " mbarrier.arrive.release.cluster.shared::cluster.b64 _, [ra];\n}\n" ::"r"(
+          (unsigned)__cvta_generic_to_shared(bar)),
+      "r"(cta)
+      : "memory");
+}
+__device__ __forceinline__ bool cluster_wait(uint64_t* bar, unsigned parity, long long limit) {
+  const long long t0 = clock64();
+  unsigned ok = 0;
+  while (true) {
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
+        " selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(ok)
+        : "r"((unsigned)__cvta_generic_to_shared(bar)), "r"(parity)
+        : "memory");
+    if (ok) return true;
+    if (clock64() - t0 > limit) return false;
+  }
+}
+__device__ __forceinline__ void cluster_sync_all() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+}
+
+// Runs of digit tiles: T = R C tiles of order j (T G < 2^31 at every supported order), CTA b
+// of G has [run0(b), run0(b + 1)).
 struct PanelRuns {
-  int C, R;
-  long long T;
-  int G;
-  __device__ PanelRuns(int j, int G_) : C((j + 15) >> 4), R((j + 31) >> 5), T((long long)R * C), G(G_) {}
-  __device__ int run0(int b) const { return (int)((long long)b * T / G); }
-  __device__ int owner(int t) const { return (int)((((long long)t + 1) * G - 1) / T); }  // run holding tile t
+  unsigned C, R, T, G;
+  __device__ PanelRuns(int j, int G_) : C((j + 15) >> 4), R((j + 31) >> 5), T(R * C), G(G_) {}
+  __device__ int run0(int b) const { return (int)((unsigned)b * T / G); }
+  __device__ int owner(int t) const { return (int)((((unsigned)t + 1u) * G - 1u) / T); }  // run holding tile t
 };
 
-template <typename T>
+template <typename T, bool CL>
 __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const PanelArgs<T> a, int maxseg) {
   using SM = PanelSmem<T>;
   constexpr bool CPX = SM::CPX;
   constexpr int NP = SM::NP, NL = SM::NL, NPL = SM::NPL, STG = SM::STG, TILE4 = SM::TILE4;
   extern __shared__ __align__(128) unsigned char psm[];
   uint4* ring_all = reinterpret_cast<uint4*>(psm);
-  auto accs = reinterpret_cast<int(*)[33][8]>(psm + SM::RING);
-  T* lvl = reinterpret_cast<T*>(psm + SM::RING + SM::ACC);  // [NL][33]
+  auto accs = reinterpret_cast<int(*)[8][32]>(psm + SM::RING);
+  long long* lvl = reinterpret_cast<long long*>(psm + SM::RING + SM::ACC);
   unsigned char* ubuf = psm + SM::RING + SM::ACC + SM::LVL;
   T* y1s = reinterpret_cast<T*>(psm + SM::RING + SM::ACC + SM::LVL + SM::UB);
   T* y2s = y1s + (kPanelMax + 1);
   T* ujs = y2s + (kPanelMax + 1);
   T* qjs = ujs + (kPanelMax + 1);
-  __shared__ T s_inv, s_upiv, s_sub, s_kq, s_pj, s_us[64];
-  __shared__ double s_tau, s_red[12];
+  __shared__ T s_inv, s_upiv, s_sub, s_pj, s_us[64];
+  __shared__ double s_tau, s_kq, s_red[12];
+  __shared__ __align__(8) uint64_t s_bar[2];  // cluster form: all threads', the vector warps'
   __shared__ int s_fu, s_ok, s_abort, s_rede[12];
 
   const int z = blockIdx.y, b = blockIdx.x, G = gridDim.x;
@@ -700,7 +729,7 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
   T* part = a.part + (long long)z * a.gs * (2 * kPanelMax);
   T* y = a.y + (long long)z * (2 * kPanelMax);
   T* P = a.P + z * a.sP;
-  T* dot = a.dot + (long long)z * a.gs;
+  double* dot = a.dot + (long long)z * a.gs;
   double* nrm = a.nrm + (long long)z * a.gs;
   int* mex = a.mex + (long long)z * a.gs;
   double* tau = a.tau + z * a.stau;
@@ -709,27 +738,31 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
   const uint4* D = reinterpret_cast<const uint4*>(a.hd.D + z * a.hd.sD);
   const int ldc = a.hd.ldd >> 4;  // tiles per row tile
   const int cs = (a.jh + G - 1) / G, c0 = b * cs, c1 = min(c0 + cs, a.jh);  // this CTA's rows
-  unsigned arrived = a.base, arrivedv = a.basev;  // targets of the two counters
+  // targets of the two counters (cluster form: phases passed)
+  unsigned arrived = CL ? 0u : a.base, arrivedv = CL ? 0u : a.basev;
   constexpr int NOEXP = -100000;
 
   // shares of the next reflector's norm (over the entries before the pivot) and scale
-  auto put_norm = [&](double n2, int e) {
-    n2 = warp_sum(n2);
+  auto put_norm = [&](double n2, int e, bool groups) {
+    if (groups) {  // one value per 8 lanes
+      n2 += __shfl_xor_sync(0xffffffffu, n2, 8);
+      n2 += __shfl_xor_sync(0xffffffffu, n2, 16);
+    } else {
+      n2 = warp_sum(n2);
+    }
     e = __reduce_max_sync(0xffffffffu, e);
     if (lane == 0) {
       s_red[warp] = n2;
       s_rede[warp] = e;
     }
     __syncthreads();
-    if (tid == 0) {
-      double t = 0.0;
-      int m = NOEXP;
-      for (int w = 0; w < 12; w++) {
-        t += s_red[w];
-        m = max(m, s_rede[w]);
+    if (warp == 0) {
+      const double t = warp_sum(lane < 12 ? s_red[lane] : 0.0);
+      const int m = __reduce_max_sync(0xffffffffu, lane < 12 ? s_rede[lane] : NOEXP);
+      if (lane == 0) {
+        nrm[b] = t;
+        mex[b] = m;
       }
-      nrm[b] = t;
-      mex[b] = m;
     }
   };
   auto scale_of = [&](T v, int i) -> int {
@@ -739,17 +772,23 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
   // full barrier over the item's CTAs; false once any wait expired (uniform over the CTA)
   auto barrier = [&]() -> bool {
     __syncthreads();
-    arrived += (unsigned)G;
-    if (tid == 0 && !grid_arrive_wait(bar, arrived, bar + 2, a.wait)) s_abort = 1;
+    arrived += CL ? 1u : (unsigned)G;
+    if (CL) {
+      if (warp == 0) {
+        if (lane < G) cluster_arrive(&s_bar[0], lane);
+        if (lane == 0 && !cluster_wait(&s_bar[0], (arrived - 1) & 1u, a.wait)) s_abort = 1;
+      }
+    } else if (tid == 0 && !grid_arrive_wait(bar, arrived, bar + 2, a.wait)) {
+      s_abort = 1;
+    }
     __syncthreads();
     return s_abort == 0;
   };
   uint4* ring = ring_all + warp * (STG * TILE4);
   // stage i % STG <- the warp's i-th tile of the run of step j
-  auto issue = [&](const PanelRuns& pr, int i) {
-    const int t = pr.run0(b) + warp + 8 * i;
-    if (t < pr.run0(b + 1)) {
-      const int r = t / pr.C, cb = t - r * pr.C;
+  auto issue = [&](int C, int t, int t1, int i) {  // t: the tile, of the run that ends at t1
+    if (t < t1) {
+      const int r = t / C, cb = t - r * C;
       const uint4* src = D + ((size_t)r * ldc + cb) * TILE4 + lane;
       uint4* st = ring + (i % STG) * TILE4 + lane;
 #pragma unroll
@@ -759,6 +798,15 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
   };
 
   if (tid == 0) s_abort = 0;
+  if (CL) {
+    if (tid == 0) {
+      for (int q = 0; q < 2; q++)
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"((unsigned)__cvta_generic_to_shared(&s_bar[q])),
+                     "r"(G));
+      asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    }
+    cluster_sync_all();
+  }
   {
     const int j = a.jh;
     T* ar = arow2 + (j & 1) * a.sv;
@@ -773,11 +821,12 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
       }
     }
     __syncthreads();
-    put_norm(n2, e);
+    put_norm(n2, e, false);
     if (warp < 8) {
       const PanelRuns pr(j, G);
+      const int t0 = pr.run0(b), t1 = pr.run0(b + 1);
 #pragma unroll
-      for (int i = 0; i < STG - 1; i++) issue(pr, i);
+      for (int i = 0; i < STG - 1; i++) issue(pr.C, t0 + warp + 8 * i, t1, i);
     }
   }
   bool live = barrier();
@@ -785,17 +834,38 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
   for (int j = a.jh; j >= a.jl && live; j--) {
     const int k = a.jh - j;
     const T* ar = arow2 + (j & 1) * a.sv;
+    // the entry of a whose digits this lane makes for the warp's next tile: column lane & 15, Re
+    // (lanes 0-15) or Im (lanes 16-31), loaded a tile ahead (the first one before the scalars)
+    const PanelRuns pr(j, G);
+    const int t0 = pr.run0(b), t1 = pr.run0(b + 1);
+    T araw = zero<T>();
+    unsigned long long rraw = 0ull;
+    auto vfetch = [&](int t) {
+      const int c = 16 * (t % (int)pr.C) + (lane & 15);
+      if (t < t1 && c < j) {
+        araw = ldcg(ar + c);
+        rraw = rmax[c];
+      }
+    };
+    if (warp < 8) vfetch(t0 + warp);
     if (warp == 0) {
       double tail = 0.0;
       int e = NOEXP;
+      const T alpha = conjg(ldcg(ar + j - 1));
       for (int g = lane; g < G; g += 32) {
         tail += __ldcg(nrm + g);
         e = max(e, __ldcg(mex + g));
       }
       tail = warp_sum(tail);
       e = __reduce_max_sync(0xffffffffu, e);
+      // |a| and |alpha| in two lanes, then the three reciprocals in three lanes: one square
+      // root and one division deep.  u = alpha + ph |a| at the pivot, tau = 1 + |alpha| / |a|.
+      const double a2 = abs2(alpha), sq = sqrt(lane & 1 ? a2 : tail + a2);
+      const double xn = __shfl_sync(0xffffffffu, sq, 0), aa = __shfl_sync(0xffffffffu, sq, 1);
+      const double rc = 1.0 / (lane == 0 ? aa : lane == 1 ? aa + xn : xn);
+      const double raa = __shfl_sync(0xffffffffu, rc, 0), rsum = __shfl_sync(0xffffffffu, rc, 1);
+      const double rxn = __shfl_sync(0xffffffffu, rc, 2);
       if (lane == 0) {
-        const T alpha = conjg(ldcg(ar + j - 1));
         if (!(tail > 0.0)) {  // nothing to annihilate: P_j = I
           s_ok = 0;
           s_inv = s_upiv = from_real<T>(1.0);
@@ -803,15 +873,13 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
           s_tau = 0.0;
           e = scale_of(from_real<T>(1.0), j - 1);
         } else {
-          const double a2 = abs2(alpha), xn = sqrt(tail + a2), aa = sqrt(a2);
-          const T ph = aa > 0.0 ? alpha * (1.0 / aa) : from_real<T>(1.0);
-          const T upiv = ph * (aa + xn);  // alpha + ph xn
-          const double up2 = abs2(upiv);
+          const T ph = aa > 0.0 ? alpha * raa : from_real<T>(1.0);
+          const T upiv = ph * (aa + xn);
           s_ok = 1;
           s_upiv = upiv;
-          s_inv = conjg(upiv) * (1.0 / up2);
+          s_inv = conjg(ph) * rsum;
           s_sub = conjg(ph) * (-xn);  // lower-storage sub-diagonal
-          s_tau = 2.0 / (tail + up2) * up2;
+          s_tau = (aa + xn) * rxn;
           e = max(e, scale_of(upiv, j - 1));
         }
         s_fu = e;
@@ -824,34 +892,35 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
 
     if (warp < 8) {
       // ---- matrix-vector product over the CTA's run of tiles
-      const PanelRuns pr(j, G);
-      const int t0 = pr.run0(b), t1 = pr.run0(b + 1), fu = s_fu;
+      const int fu = s_fu;
       int acc[NP][NL];
 #pragma unroll
       for (int q = 0; q < NP; q++)
 #pragma unroll
         for (int L = 0; L < NL; L++) acc[q][L] = 0;
-      // entry of v this lane makes digits of, for the warp's i-th tile: lane & 15, Re (lanes
-      // 0-15) or Im (lanes 16-31)
-      auto vload = [&](int i, double& x, int& ex) {
-        x = 0.0;
-        ex = 0;
-        const int t = t0 + warp + 8 * i;
-        if (t >= t1) return;
-        const int c = 16 * (t % pr.C) + (lane & 15);
-        if (c >= j) return;
-        ex = fu - deq(rmax[c]);
-        T v = c == j - 1 ? s_upiv : (refl ? conjg(ldcg(ar + c)) : zero<T>());
-        x = lane < 16 ? re(v) : im(v);
-      };
-      double xv;
-      int xe;
-      vload(0, xv, xe);
-      T d0 = zero<T>();
+      double d0 = 0.0;  // u^H p_raw (real: the block is Hermitian)
       int i = 0;
-      for (int seg = 0, r = t0 / pr.C; t0 < t1 && r * pr.C < t1; r++, seg++) {
-        const int te = min(t1, (r + 1) * pr.C);
-        for (; t0 + warp + 8 * i < te; i++) {
+      const int C = pr.C;
+      for (int seg = 0, r = t0 / C; t0 < t1 && r * C < t1; r++, seg++) {
+        const int te = min(t1, (r + 1) * C), row = 32 * r + lane;
+        T arow = zero<T>();
+        int drow = 0;
+        if (warp == 0 && row < j) {
+          arow = ldcg(ar + row);
+          drow = deq(rmax[row]);
+        }
+        for (int t = t0 + warp + 8 * i; t < te; t += 8, i++) {
+          double xv = 0.0;
+          int xe = 0;
+          {
+            const int c = 16 * (t - r * C) + (lane & 15);
+            if (c < j) {
+              const T v = c == j - 1 ? s_upiv : (refl ? conjg(araw) : zero<T>());
+              xv = lane < 16 ? re(v) : im(v);
+              xe = fu - deq(rraw);
+            }
+          }
+          vfetch(t + 8);
           int d[kDig];
           digits8(xv, xe, d);
           unsigned char* ub = ubuf + (warp * 2 + (i & 1)) * (NPL * 16);
@@ -860,9 +929,8 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
             for (int q = 0; q < kDig; q++)
               ub[((lane >> 4) * kDig + q) * 16 + (lane & 15)] = (unsigned char)(d[q] & 0xff);
           }
-          vload(i + 1, xv, xe);
           __syncwarp();  // the digits are written, and every lane is done with the stage refilled next
-          issue(pr, i + STG - 1);
+          issue(C, t + 8 * (STG - 1), t1, i + STG - 1);
           cp_async_wait<STG - 1>();
           __syncwarp();
           const uint4* st = ring + (i % STG) * TILE4 + lane;
@@ -871,27 +939,28 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
 #pragma unroll
           for (int q = 0; q < NPL; q++) av[q] = st[32 * q];
 #pragma unroll
-          for (int t = 0; t < kDig; t++) {
-            const uint4 ur = uq[t];
+          for (int w = 0; w < kDig; w++) {
+            const uint4 ur = uq[w];
             uint4 ui;
-            if constexpr (CPX) ui = uq[kDig + t];
+            if constexpr (CPX) ui = uq[kDig + w];
 #pragma unroll
-            for (int q = 0; q < kDig && q + t <= kMaxLevel; q++) {
-              acc[0][q + t] = dp4x4(av[q], ur, acc[0][q + t]);
+            for (int q = 0; q < kDig && q + w <= kMaxLevel; q++) {
+              acc[0][q + w] = dp4x4(av[q], ur, acc[0][q + w]);
               if constexpr (CPX) {
-                acc[1][q + t] = dp4x4(av[kDig + q], ui, acc[1][q + t]);
-                acc[2][q + t] = dp4x4(av[q], ui, acc[2][q + t]);
-                acc[3][q + t] = dp4x4(av[kDig + q], ur, acc[3][q + t]);
+                acc[1][q + w] = dp4x4(av[kDig + q], ui, acc[1][q + w]);
+                acc[2][q + w] = dp4x4(av[q], ui, acc[2][q + w]);
+                acc[3][q + w] = dp4x4(av[kDig + q], ur, acc[3][q + w]);
               }
             }
           }
         }
-        // the row tile's sums: over the warps exactly, one level per warp, then in FP64
+        // the row tile's sums: over the warps exactly, one level per warp; then the eight levels
+        // as two 64-bit integers (|sums| < 2^37), weighted in FP64
 #pragma unroll
         for (int q = 0; q < NP; q++)
 #pragma unroll
           for (int L = 0; L < NL; L++) {
-            accs[q * NL + L][lane][warp] = acc[q][L];
+            accs[q * NL + L][warp][lane] = acc[q][L];
             acc[q][L] = 0;
           }
         bar_named<1, 256>();
@@ -899,31 +968,38 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
           long long s0 = 0, s1 = 0, s2 = 0, s3 = 0;
 #pragma unroll
           for (int w = 0; w < 8; w++) {
-            s0 += accs[warp][lane][w];
+            s0 += accs[warp][w][lane];
             if constexpr (CPX) {
-              s1 += accs[NL + warp][lane][w];
-              s2 += accs[2 * NL + warp][lane][w];
-              s3 += accs[3 * NL + warp][lane][w];
+              s1 += accs[NL + warp][w][lane];
+              s2 += accs[2 * NL + warp][w][lane];
+              s3 += accs[3 * NL + warp][w][lane];
             }
           }
-          const double wl = __longlong_as_double((long long)(1023 - 8 * warp) << 52);  // 2^{-8 L}
-          if constexpr (CPX) lvl[warp * 33 + lane] = T{(double)(s0 - s1) * wl, (double)(s2 + s3) * wl};
-          else lvl[warp * 33 + lane] = (double)s0 * wl;
+          lvl[warp * 32 + lane] = s0 - s1;
+          if constexpr (CPX) lvl[(NL + warp) * 32 + lane] = s2 + s3;
         }
         bar_named<1, 256>();
-        if (warp == 0) {
-          T pv = zero<T>();
+        if (warp == 0 && row < j) {
+          const int E = drow + fu - 12;
+          // 2^{E - 24} (sum_L S_L 2^{24 - 8L}, levels 0-3) + 2^{E - 56} (levels 4-7)
+          auto levels = [&](const long long* sl) -> double {
+            long long h = 0, l = 0;
 #pragma unroll
-          for (int L = NL - 1; L >= 0; L--) pv += lvl[L * 33 + lane];
-          const int row = 32 * r + lane;
-          if (row < j) {
-            const int E = deq(rmax[row]) + fu - 12;
-            if constexpr (CPX) pv = inv * T{ldexp(pv.x, E), ldexp(pv.y, E)};
-            else pv = inv * ldexp(pv, E);
-            P[((size_t)b * maxseg + seg) * 32 + lane] = pv;
-            const T ur = row == j - 1 ? from_real<T>(1.0) : (refl ? conjg(ldcg(ar + row)) * inv : zero<T>());
-            macc(d0, ur, pv);
-          }
+            for (int L = 0; L < 4; L++) {
+              h = (h << 8) + sl[L * 32 + lane];
+              l = (l << 8) + sl[(4 + L) * 32 + lane];
+            }
+            const double v = fma((double)l, 0x1p-32, (double)h);
+            const int be = E - 24 + 1023;
+            return be > 0 && be < 2047 ? v * __longlong_as_double((long long)be << 52) : ldexp(v, E - 24);
+          };
+          T pv;
+          if constexpr (CPX) pv = inv * T{levels(lvl), levels(lvl + NL * 32)};
+          else pv = inv * levels(lvl);
+          P[((size_t)b * maxseg + seg) * 32 + lane] = pv;
+          const T ur = row == j - 1 ? from_real<T>(1.0) : (refl ? conjg(arow) * inv : zero<T>());
+          d0 = fma(re(ur), re(pv), d0);
+          if constexpr (CPX) d0 = fma(im(ur), im(pv), d0);
         }
       }
       if (warp == 0) {
@@ -932,9 +1008,10 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
       }
       if (j > a.jl) {  // the next step's first tiles
         const PanelRuns pn(j - 1, G);
+        const int n0 = pn.run0(b), n1 = pn.run0(b + 1);
         __syncwarp();
 #pragma unroll
-        for (int q = 0; q < STG - 1; q++) issue(pn, q);
+        for (int q = 0; q < STG - 1; q++) issue(pn.C, n0 + warp + 8 * q, n1, q);
       }
     } else {
       // ---- u' for this CTA's rows, and their shares of Q^H u (entries 0..k-1) and U^H u
@@ -972,14 +1049,25 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
         for (int h = 0; h < 2; h++)
           if (vt + 128 * h < 2 * k) part[(size_t)b * (2 * kPanelMax) + vt + 128 * h] = ya[h];
         bar_named<2, 128>();
-        arrivedv += (unsigned)G;
-        if (vt == 0 && !grid_arrive_wait(bar + 1, arrivedv, bar + 2, a.wait)) s_abort = 1;
+        arrivedv += CL ? 1u : (unsigned)G;
+        if (CL) {
+          if (warp == 8) {
+            if (lane < G) cluster_arrive(&s_bar[1], lane);
+            if (lane == 0 && !cluster_wait(&s_bar[1], (arrivedv - 1) & 1u, a.wait)) s_abort = 1;
+          }
+        } else if (vt == 0 && !grid_arrive_wait(bar + 1, arrivedv, bar + 2, a.wait)) {
+          s_abort = 1;
+        }
         bar_named<2, 128>();
-        for (int en = b + G * (warp - 8); en < 2 * k; en += 4 * G) {
+        // LG lanes per entry, 32 / LG entries per warp at a time
+        const int LG = G > 16 ? 32 : G > 8 ? 16 : 8, per = 32 / LG, sub = lane / LG, sl = lane % LG;
+        for (int e0 = (warp - 8) * per; b + G * e0 < 2 * k; e0 += 4 * per) {
+          const int en = b + G * (e0 + sub);
           T v = zero<T>();
-          for (int g = lane; g < G; g += 32) v += ldcg(part + (size_t)g * (2 * kPanelMax) + en);
-          v = warp_sum(v);
-          if (lane == 0) y[en] = v;
+          if (en < 2 * k)
+            for (int g = sl; g < G; g += LG) v += ldcg(part + (size_t)g * (2 * kPanelMax) + en);
+          for (int o = LG >> 1; o > 0; o >>= 1) v += shfl_xor(v, o);
+          if (sl == 0 && en < 2 * k) y[en] = v;
         }
       }
     }
@@ -988,6 +1076,42 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
     // ---- p, q, and row j-1 with the panel's updates
     const bool rowupd = j > a.jl;
     const double t = s_tau;
+    auto p_of = [&](int row, int l, int nl) -> T {  // lanes l of nl: their share of p_raw[row]
+      const int r = row >> 5;
+      const int b0 = pr.owner(r * pr.C), b1 = pr.owner((r + 1) * pr.C - 1);
+      T v = zero<T>();
+      for (int g = b0 + l; g <= b1; g += nl) {
+        const int g0 = pr.run0(g);
+        if (g0 < pr.run0(g + 1)) v += ldcg(P + ((size_t)g * maxseg + (r - g0 / (int)pr.C)) * 32 + (row & 31));
+      }
+      return v;
+    };
+    // groups of 8 lanes of warps 0-9, one row each (40 rows at a time); the first rows' loads go
+    // out before y arrives
+    const int grp = tid >> 3, gl = tid & 7, ce = min(c1, j);
+    T pv0 = zero<T>(), uc0 = zero<T>(), aold0 = zero<T>(), u0[4], q0[4];
+    double dsum = 0.0;
+    if (grp < 40) {
+      if (c0 + grp < ce) {
+        const T* Uc = U + (size_t)(c0 + grp) * ldu;
+        const T* Qc = Q + (size_t)(c0 + grp) * ldu;
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+          const int sq = min(gl + 8 * q, k > 0 ? k - 1 : 0);
+          u0[q] = k > 0 ? Uc[sq] : zero<T>();
+          q0[q] = k > 0 ? Qc[sq] : zero<T>();
+        }
+        if (gl == 0) {
+          uc0 = ldcg(Uc + k);
+          if (rowupd) aold0 = A[(size_t)(j - 1) * lda + c0 + grp];
+        }
+        pv0 = p_of(c0 + grp, gl, 8);
+      }
+    } else if (warp == 10) {
+      for (int g = lane; g < G; g += 32) dsum += __ldcg(dot + g);
+    } else if (rowupd) {
+      pv0 = p_of(j - 1, lane, 32);
+    }
     for (int s = tid; s < k; s += kPanelThreads) {
       y1s[s] = ldcg(y + s);
       y2s[s] = ldcg(y + k + s);
@@ -995,29 +1119,16 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
       qjs[s] = ldcg(Q + (size_t)(j - 1) * ldu + s);
     }
     __syncthreads();
-    const PanelRuns pr(j, G);
-    auto p_of = [&](int row, int l, int nl) -> T {  // lanes l of nl: their share of p_raw[row]
-      const int r = row >> 5;
-      const int b0 = pr.owner(r * pr.C), b1 = pr.owner((r + 1) * pr.C - 1);
-      T v = zero<T>();
-      for (int g = b0 + l; g <= b1; g += nl) {
-        const int g0 = pr.run0(g);
-        if (g0 < pr.run0(g + 1)) v += ldcg(P + ((size_t)g * maxseg + (r - g0 / pr.C)) * 32 + (row & 31));
-      }
-      return v;
-    };
-    if (warp == 0) {
-      T tot = zero<T>(), w = zero<T>();
-      for (int g = lane; g < G; g += 32) tot += ldcg(dot + g);
+    if (warp == 10) {  // kq = (tau / 2) u^H p = (tau^2 / 2) (u^H p_raw - 2 Re y2^H y1)
+      double tot = dsum;
       for (int s = lane; s < k; s += 32) {
-        macc(w, y2s[s], y1s[s]);
-        macc(w, y1s[s], y2s[s]);
+        tot = fma(-2.0 * re(y2s[s]), re(y1s[s]), tot);
+        if constexpr (CPX) tot = fma(-2.0 * im(y2s[s]), im(y1s[s]), tot);
       }
       tot = warp_sum(tot);
-      w = warp_sum(w);
-      if (lane == 0) s_kq = (0.5 * t) * (t * (tot - w));
-    } else if (warp == 1 && rowupd) {  // p[j-1] - U y1 - Q y2 of row j-1
-      T v = p_of(j - 1, lane, 32), corr = zero<T>();
+      if (lane == 0) s_kq = (0.5 * t) * (t * tot);
+    } else if (warp == 11 && rowupd) {  // p[j-1] - U y1 - Q y2 of row j-1
+      T v = pv0, corr = zero<T>();
       for (int s = lane; s < k; s += 32) {
         mac(corr, ujs[s], y1s[s]);
         mac(corr, qjs[s], y2s[s]);
@@ -1025,57 +1136,61 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
       v = warp_sum(v - corr);
       if (lane == 0) s_pj = v;
     }
-    // groups of 8 lanes, one row each (48 rows at a time)
-    const int grp = tid >> 3, gl = tid & 7, ce = min(c1, j);
     double n2 = 0.0;
     int ex = NOEXP;
     bool synced = false;
     T* an = arow2 + ((j - 1) & 1) * a.sv;
-    for (int base = c0; base < ce || !synced; base += 48) {
+    for (int base = c0; base < ce || !synced; base += 40) {
       const int c = base + grp;
-      const bool ok = c < ce;
-      T pv = zero<T>(), rs = zero<T>(), uc = zero<T>(), aold = zero<T>();
+      const bool ok = c < ce && grp < 40;
+      T pv = pv0, rs = zero<T>(), uc = uc0, aold = aold0;
       if (ok) {
-        pv = p_of(c, gl, 8);
         const T* Uc = U + (size_t)c * ldu;
         const T* Qc = Q + (size_t)c * ldu;
-        if (gl == 0) {
-          uc = ldcg(Uc + k);
-          if (rowupd) aold = A[(size_t)(j - 1) * lda + c];
+        if (synced) {
+          pv = p_of(c, gl, 8);
+          if (gl == 0) {
+            uc = ldcg(Uc + k);
+            if (rowupd) aold = A[(size_t)(j - 1) * lda + c];
+          }
         }
         for (int s0 = gl; s0 < k; s0 += 32) {  // four steps' loads in flight
-          T ucv[4], qcv[4];
+          if (synced || s0 > gl) {
 #pragma unroll
-          for (int q = 0; q < 4; q++) {
-            const int sq = min(s0 + 8 * q, k - 1);
-            ucv[q] = Uc[sq];
-            qcv[q] = Qc[sq];
+            for (int q = 0; q < 4; q++) {
+              const int sq = min(s0 + 8 * q, k - 1);
+              u0[q] = Uc[sq];
+              q0[q] = Qc[sq];
+            }
           }
 #pragma unroll
           for (int q = 0; q < 4; q++) {
             const int sq = s0 + 8 * q;
             if (sq < k) {
-              mac(pv, -ucv[q], y1s[sq]);
-              mac(pv, -qcv[q], y2s[sq]);
+              mac(pv, -u0[q], y1s[sq]);
+              mac(pv, -q0[q], y2s[sq]);
               if (rowupd) {
-                mac(rs, ujs[sq], conjg(qcv[q]));
-                mac(rs, qjs[sq], conjg(ucv[q]));
+                mac(rs, ujs[sq], conjg(q0[q]));
+                mac(rs, qjs[sq], conjg(u0[q]));
               }
             }
           }
         }
       }
-      pv = group8_sum(pv);
-      rs = group8_sum(rs);
+      if (grp < 40) {
+        pv = group8_sum(pv);
+        if (rowupd) rs = group8_sum(rs);
+      }
       if (!synced) {  // kq and row j-1's share
         __syncthreads();
         synced = true;
       }
       if (ok && gl == 0) {
-        const T kq = s_kq, qc = t * pv - kq * uc;
+        const double kq = s_kq;
+        const T qc = t * pv - kq * uc;
         Q[(size_t)c * ldu + k] = qc;
         if (rowupd) {
-          const T qj = t * s_pj - kq;  // u'[j-1] = 1
+          const T qj = t * s_pj - from_real<T>(kq);  // u'[j-1] = 1
           rs += conjg(qc);
           mac(rs, qj, conjg(uc));
           const T an_c = aold - rs;
@@ -1092,43 +1207,111 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
       }
     }
     if (!rowupd) break;
-    put_norm(n2, ex);
+    put_norm(n2, ex, true);
     live = barrier();
   }
   cp_async_wait<0>();
-  if (s_abort && tid == 0 && b == 0) set_status(a.st ? a.st + z : nullptr, ST_ETIMEOUT, -3);
+  if (CL) cluster_sync_all();  // no CTA leaves while another may still arrive on its barriers
+  if (s_abort && tid == 0) set_status(a.st ? a.st + z : nullptr, ST_ETIMEOUT, -3);
 }
 
-// CTAs per item: as many as give each about kPanelTiles digit tiles (fewer CTAs make the
-// barriers cheaper and leave SMs to other streams), at most one per SM over all items.
+// CTAs per item: as many as give each about kPanelTiles digit tiles, at most one per SM over
+// all items.
 constexpr int kPanelTiles = 12;
 template <typename T>
-int hetrd_panel_ctas(int jh, int items) {
+static int panel_capacity() {
   static const int cap = [] {
     int dev = 0, sms = 0, per = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaFuncSetAttribute(hetrd_panel_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, PanelSmem<T>::TOTAL);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, hetrd_panel_kernel<T>, kPanelThreads, PanelSmem<T>::TOTAL);
+    cudaFuncSetAttribute(hetrd_panel_kernel<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         PanelSmem<T>::TOTAL);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, hetrd_panel_kernel<T, false>, kPanelThreads,
+                                                  PanelSmem<T>::TOTAL);
     cudaGetLastError();
     return sms * (per > 0 ? 1 : 0);
   }();
-  const int top = std::min(cap / items, kPanelCtas);
+  return cap;
+}
+// Largest cluster of panel CTAs that can be resident (16, 8 or 0), attributes set.
+template <typename T>
+static int panel_cluster() {
+  static const int best = [] {
+    auto k = hetrd_panel_kernel<T, true>;
+    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, PanelSmem<T>::TOTAL);
+    cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    for (int c = 16; c >= 8; c /= 2) {
+      cudaLaunchConfig_t cfg{};
+      cudaLaunchAttribute at{};
+      at.id = cudaLaunchAttributeClusterDimension;
+      at.val.clusterDim.x = c;
+      at.val.clusterDim.y = at.val.clusterDim.z = 1;
+      cfg.gridDim = dim3(c);
+      cfg.blockDim = dim3(kPanelThreads);
+      cfg.dynamicSmemBytes = PanelSmem<T>::TOTAL;
+      cfg.attrs = &at;
+      cfg.numAttrs = 1;
+      int n = 0;
+      if (cudaOccupancyMaxActiveClusters(&n, k, &cfg) == cudaSuccess && n > 0) return c;
+      cudaGetLastError();
+    }
+    return 0;
+  }();
+  return best;
+}
+
+template <typename T>
+int hetrd_panel_ctas(int jh, int items) {
+  const int top = std::min(panel_capacity<T>() / items, kPanelCtas);
   const long long tiles = (long long)((jh + 31) / 32) * ((jh + 15) / 16);
   return (int)std::min<long long>(top, (tiles + kPanelTiles - 1) / kPanelTiles);
 }
 
+// The cluster form (one cluster of up to 16 CTAs per item, barriers through shared-memory
+// mbarriers, no co-residency of the whole grid needed, so that several streams' reductions
+// run side by side) up to kClusterTiles digit tiles per item, or where the grid form cannot
+// give every item a CTA.
 template <typename T>
-bool hetrd_panel(const PanelArgs<T>& a, int G, int items, cudaStream_t s) {
-  cudaFuncSetAttribute(hetrd_panel_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, PanelSmem<T>::TOTAL);
-  int maxseg = (a.jh + 31) / 32 / G + 2;
-  PanelArgs<T> arg = a;
-  void* args[] = {&arg, &maxseg};
-  count_launch();
-  return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(hetrd_panel_kernel<T>), dim3(G, items),
-                                     dim3(kPanelThreads), args, PanelSmem<T>::TOTAL, s) == cudaSuccess;
+static int panel_cluster_ctas(int jh, int items) {
+  constexpr long long kClusterTiles = sizeof(T) == 16 ? 400 : 1000;
+  const int c = panel_cluster<T>();
+  const long long tiles = (long long)((jh + 31) / 32) * ((jh + 15) / 16);
+  if (c == 0 || (tiles > kClusterTiles && hetrd_panel_ctas<T>(jh, items) >= 1)) return 0;
+  int g = c;
+  while (g > 2 && tiles <= 4 * g) g >>= 1;
+  return g;
 }
 
+template <typename T>
+bool hetrd_panel(PanelArgs<T> a, int items, unsigned* base, unsigned* basev, cudaStream_t s) {
+  const int cl = std::min(panel_cluster_ctas<T>(a.jh, items), a.gs >= 16 ? 16 : a.gs >= 8 ? 8 : 0);
+  const int G = cl > 0 ? cl : std::min(a.gs, hetrd_panel_ctas<T>(a.jh, items));
+  int maxseg = (a.jh + 31) / 32 / G + 2;
+  const int steps = a.jh - a.jl + 1;
+  a.base = *base;
+  a.basev = *basev;
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute at{};
+  cfg.gridDim = dim3(G, items);
+  cfg.blockDim = dim3(kPanelThreads);
+  cfg.dynamicSmemBytes = PanelSmem<T>::TOTAL;
+  cfg.stream = s;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  count_launch();
+  if (cl > 0) {
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = G;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    return cudaLaunchKernelEx(&cfg, hetrd_panel_kernel<T, true>, a, maxseg) == cudaSuccess;
+  }
+  *base += 2u * steps * G;
+  *basev += (unsigned)(steps - 1) * G;
+  cudaFuncSetAttribute(hetrd_panel_kernel<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, PanelSmem<T>::TOTAL);
+  at.id = cudaLaunchAttributeCooperative;
+  at.val.cooperative = 1;
+  return cudaLaunchKernelEx(&cfg, hetrd_panel_kernel<T, false>, a, maxseg) == cudaSuccess;
+}
 
 // d_i = Re A_ii, e_i = |A_{i+1,i}|, ph_0 = 1, ph_{i+1} = ph_i A_{i+1,i}/|A_{i+1,i}|.
 template <typename T>
@@ -1301,7 +1484,7 @@ void narrow_lower(const T* A, int lda, long long sA, TL* B, int ldb, long long s
                                         int, long long, double*, long long, int, cudaStream_t);               \
   template void hetrd_digits<T>(const T*, int, long long, int, const HemvDigits&, int, cudaStream_t);           \
   template int hetrd_panel_ctas<T>(int, int);                                                              \
-  template bool hetrd_panel<T>(const PanelArgs<T>&, int, int, cudaStream_t);
+  template bool hetrd_panel<T>(PanelArgs<T>, int, unsigned*, unsigned*, cudaStream_t);
 INST(double)
 INST(zc)
 #undef INST
