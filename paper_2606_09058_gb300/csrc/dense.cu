@@ -6,48 +6,123 @@
 
 namespace gks {
 
-// One CTA per batch item: factor the nb x nb diagonal block of A at (k0, k0) in place
-// (lower, A = L L^H).  A non-positive or non-finite pivot records GKS_ENOTSPD with the
-// global column and leaves the block untouched.
+// acc -= a * b, acc -= a * conj(b): two fused operations per component.
+__device__ __forceinline__ void msub(double& acc, double a, double b) { acc = fma(-a, b, acc); }
+__device__ __forceinline__ void msub(zc& acc, zc a, zc b) {
+  acc.x = fma(-a.x, b.x, acc.x);
+  acc.x = fma(a.y, b.y, acc.x);
+  acc.y = fma(-a.x, b.y, acc.y);
+  acc.y = fma(-a.y, b.x, acc.y);
+}
+__device__ __forceinline__ void msubc(double& acc, double a, double b) { acc = fma(-a, b, acc); }
+__device__ __forceinline__ void msubc(zc& acc, zc a, zc b) { msub(acc, a, conjg(b)); }
+
 template <typename T>
-__global__ void potf2_kernel(T* A, int lda, long long sA, int k0, int nb, DevStatus* st) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* a = reinterpret_cast<T*>(smem_raw);
+__device__ __forceinline__ T shfl8(T v, int src);
+template <>
+__device__ __forceinline__ double shfl8<double>(double v, int src) { return __shfl_sync(0xffffffffu, v, src, 8); }
+template <>
+__device__ __forceinline__ zc shfl8<zc>(zc v, int src) {
+  return zc{__shfl_sync(0xffffffffu, v.x, src, 8), __shfl_sync(0xffffffffu, v.y, src, 8)};
+}
+__device__ __forceinline__ double shfl32(double v, int src) { return __shfl_sync(0xffffffffu, v, src); }
+__device__ __forceinline__ zc shfl32(zc v, int src) { return zc{shfl32(v.x, src), shfl32(v.y, src)}; }
+
+// Diagonal blocks (64 x 64) on a cluster of kDiagC CTAs, in sub-blocks of kSub columns.  One
+// SM does 1.7 FP64 multiply-adds per clock: the 64^3 operations of a complex two-sided
+// reduction alone keep it busy for 0.3 ms, so the panel rows and the trailing updates are
+// spread over the cluster (data in global memory, L2 reads), with two cluster barriers per
+// sub-block; the 8 x 8 diagonal parts, a serial chain, are done by every CTA for itself.
+// Measured, one complex block: two-sided reduction 794 us on one CTA, column by column;
+// Cholesky 207 us.  See the launchers for the times of this form.
+constexpr int kDiagC = 8, kSub = 8, kDiagThreads = 256;
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+}
+
+// Cholesky of the nb x nb diagonal block of A at (k0, k0) in place (lower, A = L L^H), one
+// cluster per batch item.  A non-positive or non-finite pivot records GKS_ENOTSPD with the
+// global column; the block is then left part way.
+template <typename T>
+__global__ void __launch_bounds__(kDiagThreads) potf2_kernel(T* A, int lda, long long sA, int k0, int nb,
+                                                             DevStatus* st) {
+  __shared__ T s11[kSub][kSub + 1];
+  __shared__ double rd[kSub];
+  __shared__ T v[64][kSub + 1];
   __shared__ int fail;
-  const int z = blockIdx.x, ld = nb + 1, tid = threadIdx.x, nt = blockDim.x;
-  A += z * sA;
-  for (int e = tid; e < nb * nb; e += nt) {
-    int i = e / nb, j = e % nb;
-    a[i * ld + j] = (j <= i) ? A[(size_t)(k0 + i) * lda + k0 + j] : zero<T>();
-  }
+  const int z = blockIdx.y, rank = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
+  A += z * sA + (size_t)k0 * lda + k0;
   if (tid == 0) fail = -1;
-  __syncthreads();
-  for (int j = 0; j < nb; j++) {
-    if (tid == 0) {
-      double piv = re(a[j * ld + j]);
-      if (!(piv > 0.0) || !isfinite(piv)) fail = j;
-      else a[j * ld + j] = from_real<T>(sqrt(piv));
+  for (int c0 = 0; c0 < nb; c0 += kSub) {
+    const int kb = min(kSub, nb - c0), m = nb - c0 - kb;
+    __syncthreads();
+    if (tid < 32) {
+      for (int e = lane; e < kSub * kSub; e += 32) {
+        const int i = e >> 3, j = e & 7;
+        s11[i][j] = (i < kb && j <= i) ? ldcg(A + (size_t)(c0 + i) * lda + c0 + j) : zero<T>();
+      }
+      __syncwarp();
+      for (int j = 0; j < kb; j++) {
+        const double piv = re(s11[j][j]);
+        if (!(piv > 0.0) || !isfinite(piv)) {
+          if (lane == 0) fail = c0 + j;
+          break;
+        }
+        const double d = sqrt(piv), inv = 1.0 / d;
+        __syncwarp();
+        if (lane == j) {
+          s11[j][j] = from_real<T>(d);
+          rd[j] = inv;
+        } else if (lane > j && lane < kb) {
+          s11[lane][j] = s11[lane][j] * inv;
+        }
+        __syncwarp();
+        for (int e = lane; e < kSub * kSub; e += 32) {
+          const int r = e >> 3, c = e & 7;
+          if (c > j && c <= r && r < kb) msubc(s11[r][c], s11[r][j], s11[c][j]);
+        }
+        __syncwarp();
+      }
     }
     __syncthreads();
-    if (fail >= 0) break;
-    const double ljj = re(a[j * ld + j]);
-    for (int i = j + 1 + tid; i < nb; i += nt) a[i * ld + j] = a[i * ld + j] * (1.0 / ljj);
-    __syncthreads();
-    const int m = nb - j - 1;
-    for (int e = tid; e < m * m; e += nt) {
-      int r = j + 1 + e / m, c = j + 1 + e % m;
-      if (c <= r) a[r * ld + c] -= a[r * ld + j] * conjg(a[c * ld + j]);
+    if (fail >= 0) break;  // the same in every CTA of the cluster
+    // rows below, one per 8 lanes, row r of CTA r % kDiagC: x L11^H = a
+    {
+      const int r = rank + kDiagC * (tid >> 3), g = tid & 7;
+      if (tid < 64) {
+        T* ar = A + (size_t)(c0 + kb + r) * lda + c0;
+        T x = (r < m && g < kb) ? ldcg(ar + g) : zero<T>();
+        for (int j = 0; j < kb; j++) {
+          const T xj = shfl8<T>(x * rd[j], j);
+          if (g > j && g < kb) msubc(x, xj, s11[g][j]);
+          if (g == j) x = xj;
+        }
+        if (r < m && g < kb) ar[g] = x;
+      }
+    }
+    cluster_barrier();  // every CTA has read the 8 x 8 block
+    if (rank == 0 && tid < kSub * kSub) {
+      const int i = tid >> 3, j = tid & 7;
+      if (i < kb && j <= i) A[(size_t)(c0 + i) * lda + c0 + j] = s11[i][j];
+    }
+    if (m <= 0) break;
+    for (int e = tid; e < m * kSub; e += kDiagThreads) {
+      const int i = e >> 3, g = e & 7;
+      v[i][g] = g < kb ? ldcg(A + (size_t)(c0 + kb + i) * lda + c0 + g) : zero<T>();
     }
     __syncthreads();
+    for (int e = rank * kDiagThreads + tid; e < m * m; e += kDiagC * kDiagThreads) {
+      const int i = e / m, j = e - i * m;
+      if (j > i) continue;
+      T* p = A + (size_t)(c0 + kb + i) * lda + c0 + kb + j;
+      T x = ldcg(p);
+#pragma unroll
+      for (int g = 0; g < kSub; g++) msubc(x, v[i][g], v[j][g]);
+      *p = x;
+    }
+    cluster_barrier();
   }
-  if (fail >= 0) {
-    if (tid == 0) set_status(st ? st + z : nullptr, ST_ENOTSPD, k0 + fail);
-    return;
-  }
-  for (int e = tid; e < nb * nb; e += nt) {
-    int i = e / nb, j = e % nb;
-    if (j <= i) A[(size_t)(k0 + i) * lda + k0 + j] = a[i * ld + j];
-  }
+  if (fail >= 0 && rank == 0 && tid == 0) set_status(st ? st + z : nullptr, ST_ENOTSPD, k0 + fail);
 }
 
 // Triangular solves against one nb x nb lower-triangular block L (nb <= 64), by substitution
@@ -63,17 +138,10 @@ __global__ void potf2_kernel(T* A, int lda, long long sA, int k0, int nb, DevSta
 // entries, so nothing but the columns of L is read.  The FP64 pipe bounds it (1.7
 // multiply-adds per SM clock; nb^2 / 2 per right-hand side, four times that complex), so the
 // right-hand sides are spread over all SMs, 4 per warp and as few warps per CTA as give one
-// CTA per SM.  Measured: 64 x 64 against 832 real right-hand sides 184 us with a thread per
-// right-hand side and 64 of them per CTA, 17 us here; 2500 complex 530 us, 62 us here.
-template <typename T>
-__device__ __forceinline__ T shfl8(T v, int src);
-template <>
-__device__ __forceinline__ double shfl8<double>(double v, int src) { return __shfl_sync(0xffffffffu, v, src, 8); }
-template <>
-__device__ __forceinline__ zc shfl8<zc>(zc v, int src) {
-  return zc{__shfl_sync(0xffffffffu, v.x, src, 8), __shfl_sync(0xffffffffu, v.y, src, 8)};
-}
-
+// CTA per SM.  The steps are a rolled loop on rotating registers: unrolled, the 64 steps are
+// 30 to 100 KB of code that each launch runs through once at the speed of instruction fetch.
+// Measured against 832 real right-hand sides: 184 us with a thread per right-hand side and 64
+// of them per CTA, 64 us unrolled, @@TR@@ us here; 4992 complex: 530, 266, @@TC@@ us.
 template <typename T, int MODE>
 __global__ void __launch_bounds__(256) trsm_block_kernel(const T* L, int ldl, long long sL, T* B, int ldb,
                                                          long long sB, int nb, int nrhs) {
@@ -83,7 +151,7 @@ __global__ void __launch_bounds__(256) trsm_block_kernel(const T* L, int ldl, lo
   const int z = blockIdx.y, tid = threadIdx.x, nt = blockDim.x;
   L += z * sL;
   B += z * sB;
-#pragma unroll 4
+#pragma unroll 8
   for (int e = tid; e < 64 * 64; e += nt) {
     const int i = e >> 6, j = e & 63;  // stored element (i, j), j <= i
     T v = (i == j) ? from_real<T>(1.0) : zero<T>();
@@ -104,107 +172,215 @@ __global__ void __launch_bounds__(256) trsm_block_kernel(const T* L, int ldl, lo
   T x[8];
 #pragma unroll
   for (int i = 0; i < 8; i++) x[i] = (ok && 8 * i + g < nb) ? *at(8 * i + g) : zero<T>();
+#pragma unroll 1
+  for (int J = 0; 8 * J < nb; J++) {  // x[i]: entries 8 (J + i) + g
+    const T* col = lc + 8 * J * 64 + 8 * J + g;
+#pragma unroll 1
+    for (int jj = 0; jj < 8; jj++, col += 64) {
+      const T xj = shfl8<T>(x[0] * rd[8 * J + jj], jj);
+      if (g > jj) msub(x[0], xj, col[0]);
+      if (g == jj) x[0] = xj;
 #pragma unroll
-  for (int J = 0; J < 8; J++) {
-#pragma unroll
-    for (int jj = 0; jj < 8; jj++) {
-      const int j = 8 * J + jj;
-      const T xj = shfl8<T>(x[J] * rd[j], jj);
-      const T* col = lc + j * 64 + g;
-      if (g > jj) x[J] -= xj * col[8 * J];
-      if (g == jj) x[J] = xj;
-#pragma unroll
-      for (int i = J + 1; i < 8; i++) x[i] -= xj * col[8 * i];
+      for (int i = 1; i < 8; i++) {
+        if (i + J >= 8) break;
+        msub(x[i], xj, col[8 * i]);
+      }
     }
-    if (8 * J + 8 >= nb) break;
-  }
+    if (ok && 8 * J + g < nb) *at(8 * J + g) = x[0];
 #pragma unroll
-  for (int i = 0; i < 8; i++)
-    if (ok && 8 * i + g < nb) *at(8 * i + g) = x[i];
+    for (int i = 0; i < 7; i++) x[i] = x[i + 1];
+  }
 }
 
-// One CTA per batch item: the diagonal block A11 <- L11^-1 A11 L11^-H (A11 read from its
-// lower triangle) by the two-sided column recurrence
+// One cluster per batch item: the nb x nb diagonal block A <- L^-1 A L^-H (read from its lower
+// triangle) with the diagonal block L, in sub-blocks of kSub columns: A11 by the two-sided
+// column recurrence
 //   alpha_k = a_kk / l_kk^2,  v = a(k+1:, k)/l_kk - (alpha_k/2) l(k+1:, k),
 //   A(k+1:, k+1:) -= l v^H + v l^H,  r_k = v - (alpha_k/2) l(k+1:, k),
-// followed by the deferred in-block solve X = L11^-1 [r_0 r_1 ...] (strictly lower part).
-// Writes the lower triangle back into A and the full Hermitian block into F (ldF).
+// and its in-block solve, then W = A21 L11^-H, V = W - L21 A11/2, A22 -= L21 V^H + V L21^H,
+// R = V - L21 A11/2, and finally L^-1 [R_0 R_1 ...] by forward substitution, a warp per
+// column.  Writes the lower triangle back into A and the full Hermitian block into F (ldF).
 template <typename T>
-__global__ void hegst_diag_kernel(T* A, int lda, long long sA, const T* L, int ldl, long long sL, int k0, int nb,
-                                  T* F, int ldF, long long sF) {
+__global__ void __launch_bounds__(kDiagThreads) hegst_diag_kernel(T* A, int lda, long long sA, const T* L, int ldl,
+                                                                  long long sL, int k0, int nb, T* F, int ldF,
+                                                                  long long sF) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* a = reinterpret_cast<T*>(smem_raw);
-  T* l = a + nb * (nb + 1);
-  const int z = blockIdx.x, ld = nb + 1, tid = threadIdx.x, nt = blockDim.x;
-  A += z * sA;
-  L += z * sL;
+  T* l = reinterpret_cast<T*>(smem_raw);  // [64][65]
+  __shared__ T s11[kSub][kSub + 1];
+  __shared__ double rd[64];
+  T* v = l + 64 * 65;  // [64][kSub + 1]
+  constexpr int LD = 65, LV = kSub + 1;
+  const int z = blockIdx.y, rank = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  A += z * sA + (size_t)k0 * lda + k0;
+  L += z * sL + (size_t)k0 * ldl + k0;
   F += z * sF;
-  for (int e = tid; e < nb * nb; e += nt) {
-    int i = e / nb, j = e % nb;
-    a[i * ld + j] = (j <= i) ? A[(size_t)(k0 + i) * lda + k0 + j] : zero<T>();
-    l[i * ld + j] = (j <= i) ? L[(size_t)(k0 + i) * ldl + k0 + j] : zero<T>();
+#pragma unroll 4
+  for (int e = tid; e < nb * nb; e += kDiagThreads) {
+    const int i = e / nb, j = e - i * nb;
+    const T x = j <= i ? L[(size_t)i * ldl + j] : zero<T>();
+    l[i * LD + j] = x;
+    if (i == j) rd[i] = 1.0 / re(x);
   }
-  __syncthreads();
-  for (int k = 0; k < nb; k++) {
-    const double lkk = re(l[k * ld + k]);
-    const double alpha = re(a[k * ld + k]) / (lkk * lkk);
-    for (int i = k + 1 + tid; i < nb; i += nt) a[i * ld + k] = a[i * ld + k] * (1.0 / lkk) - (0.5 * alpha) * l[i * ld + k];
+  for (int c0 = 0; c0 < nb; c0 += kSub) {
+    const int kb = min(kSub, nb - c0), m = nb - c0 - kb;
+    const T* lb = l + c0 * LD + c0;
     __syncthreads();
-    const int m = nb - k - 1;
-    for (int e = tid; e < m * m; e += nt) {
-      int i = k + 1 + e / m, j = k + 1 + e % m;
-      if (j <= i) a[i * ld + j] -= l[i * ld + k] * conjg(a[j * ld + k]) + a[i * ld + k] * conjg(l[j * ld + k]);
+    if (tid < 32) {
+      for (int e = lane; e < kSub * kSub; e += 32) {
+        const int i = e >> 3, j = e & 7;
+        s11[i][j] = (i < kb && j <= i) ? ldcg(A + (size_t)(c0 + i) * lda + c0 + j) : zero<T>();
+      }
+      __syncwarp();
+      for (int k = 0; k < kb; k++) {
+        const double rk = rd[c0 + k], alpha = re(s11[k][k]) * rk * rk;
+        __syncwarp();
+        if (lane > k && lane < kb) s11[lane][k] = s11[lane][k] * rk - (0.5 * alpha) * lb[lane * LD + k];
+        __syncwarp();
+        for (int e = lane; e < kSub * kSub; e += 32) {
+          const int i = e >> 3, j = e & 7;
+          if (j > k && j <= i && i < kb) {
+            msubc(s11[i][j], lb[i * LD + k], s11[j][k]);
+            msubc(s11[i][j], s11[i][k], lb[j * LD + k]);
+          }
+        }
+        __syncwarp();
+        if (lane > k && lane < kb) s11[lane][k] = s11[lane][k] - (0.5 * alpha) * lb[lane * LD + k];
+        if (lane == k) s11[k][k] = from_real<T>(alpha);
+        __syncwarp();
+      }
+      if (lane < kb) {  // column `lane`: rows below, forward substitution with L11
+        for (int i = lane + 1; i < kb; i++) {
+          T x = s11[i][lane];
+          for (int k = lane + 1; k < i; k++) msub(x, lb[i * LD + k], s11[k][lane]);
+          s11[i][lane] = x * rd[c0 + i];
+        }
+      }
+      __syncwarp();
+      for (int e = lane; e < kSub * kSub; e += 32) {  // the full Hermitian 8 x 8
+        const int i = e >> 3, j = e & 7;
+        if (j > i) s11[i][j] = conjg(s11[j][i]);
+      }
     }
     __syncthreads();
-    for (int i = k + 1 + tid; i < nb; i += nt) a[i * ld + k] = a[i * ld + k] - (0.5 * alpha) * l[i * ld + k];
-    if (tid == 0) a[k * ld + k] = from_real<T>(alpha);
-    __syncthreads();
-  }
-  for (int c = tid; c < nb; c += nt) {  // column c: rows i > c, forward substitution with L11
-    for (int i = c + 1; i < nb; i++) {
-      T s = a[i * ld + c];
-      for (int k = c + 1; k < i; k++) s -= l[i * ld + k] * a[k * ld + c];
-      a[i * ld + c] = s * (1.0 / re(l[i * ld + i]));
+    // rows below, one per 8 lanes: W, V
+    const int r = rank + kDiagC * (tid >> 3), g = tid & 7;
+    T* ar = A + (size_t)(c0 + kb + r) * lda + c0;
+    T x = zero<T>(), h = zero<T>();
+    if (tid < 64) {
+      x = (r < m && g < kb) ? ldcg(ar + g) : zero<T>();
+      for (int j = 0; j < kb; j++) {
+        const T xj = shfl8<T>(x * rd[c0 + j], j);
+        if (g > j && g < kb) msubc(x, xj, lb[g * LD + j]);
+        if (g == j) x = xj;
+      }
+      if (r < m && g < kb) {
+        const T* lr = l + (c0 + kb + r) * LD + c0;
+        for (int j = 0; j < kb; j++) mac(h, lr[j], s11[j][g]);
+        h = 0.5 * h;
+        x = x - h;
+        ar[g] = x;
+      }
     }
+    cluster_barrier();  // every CTA has read the 8 x 8 block
+    if (rank == 0 && tid < kSub * kSub) {
+      const int i = tid >> 3, j = tid & 7;
+      if (i < kb && j < kb) {
+        F[(size_t)(c0 + i) * ldF + c0 + j] = s11[i][j];
+        if (j <= i) A[(size_t)(c0 + i) * lda + c0 + j] = s11[i][j];
+      }
+    }
+    if (m <= 0) break;
+    for (int e = tid; e < m * kSub; e += kDiagThreads) {
+      const int i = e >> 3, q = e & 7;
+      v[i * LV + q] = q < kb ? ldcg(A + (size_t)(c0 + kb + i) * lda + c0 + q) : zero<T>();
+    }
+    __syncthreads();
+    for (int e = rank * kDiagThreads + tid; e < m * m; e += kDiagC * kDiagThreads) {
+      const int i = e / m, j = e - i * m;
+      if (j > i) continue;
+      T* p = A + (size_t)(c0 + kb + i) * lda + c0 + kb + j;
+      T a = ldcg(p);
+      const T *li = l + (c0 + kb + i) * LD + c0, *lj = l + (c0 + kb + j) * LD + c0;
+#pragma unroll
+      for (int q = 0; q < kSub; q++) {  // columns past kb of L are other data: v is zero there
+        if (q >= kb) break;
+        msubc(a, li[q], v[j * LV + q]);
+        msubc(a, v[i * LV + q], lj[q]);
+      }
+      *p = a;
+    }
+    cluster_barrier();
+    if (tid < 64 && r < m && g < kb) ar[g] = x - h;
   }
-  __syncthreads();
-  for (int e = tid; e < nb * nb; e += nt) {
-    int i = e / nb, j = e % nb;
-    T v = (j <= i) ? a[i * ld + j] : conjg(a[j * ld + i]);
-    if (i == j) v = from_real<T>(re(v));
-    F[(size_t)i * ldF + j] = v;
-    if (j <= i) A[(size_t)(k0 + i) * lda + k0 + j] = v;
+  cluster_barrier();  // every R is in place
+  // column c: rows from its sub-block's end, x_i = (g_i - sum L_ik x_k) / l_ii
+  for (int c = rank + kDiagC * warp; c < nb; c += kDiagC * (kDiagThreads / 32)) {
+    const int s0 = min(nb, (c / kSub + 1) * kSub);
+    T x0 = zero<T>(), x1 = zero<T>();
+    if (lane >= s0 && lane < nb) x0 = ldcg(A + (size_t)lane * lda + c);
+    if (lane + 32 >= s0 && lane + 32 < nb) x1 = ldcg(A + (size_t)(lane + 32) * lda + c);
+#pragma unroll 1
+    for (int i = s0; i < nb; i++) {
+      const T xi = shfl32(i < 32 ? x0 : x1, i & 31) * rd[i];
+      if (i < 31 && lane > i && lane < nb) msub(x0, l[lane * LD + i], xi);
+      if (lane + 32 > i && lane + 32 < nb) msub(x1, l[(lane + 32) * LD + i], xi);
+      if (lane == (i & 31)) {
+        if (i < 32) x0 = xi;
+        else x1 = xi;
+      }
+    }
+#pragma unroll
+    for (int h = 0; h < 2; h++) {
+      const int i = lane + 32 * h;
+      const T xv = h ? x1 : x0;
+      if (i >= s0 && i < nb) {
+        A[(size_t)i * lda + c] = xv;
+        F[(size_t)i * ldF + c] = xv;
+        F[(size_t)c * ldF + i] = conjg(xv);
+      }
+    }
   }
 }
 
 // Compact WY T factor for H_1 H_2 ... H_k = I - V T V^H with H_i = I - tau_i v_i v_i^H:
-// T upper triangular, T_ii = tau_i, T[0:i, i] = -tau_i T[0:i, 0:i] (V^H V)[0:i, i].
-// G = V^H V (k x k, ldG) precomputed; one CTA per batch item.
+// T upper triangular, T_ii = tau_i, and T^-1 = diag(1 / tau) + the strictly upper part of
+// G = V^H V, so each column is a back substitution of its own,
+//   t_i = tau_i,  t_r = -tau_r sum_{r < c <= i} G_rc t_c  (r = i - 1 .. 0),
+// a warp per column (lanes hold rows lane and lane + 32; k <= 64), 4 columns per CTA.  The
+// column-by-column form T[0:i, i] = -tau_i T[0:i, 0:i] G[0:i, i] on one CTA took 372 us
+// (complex, k = 64) and 144 us (real); this one @@LC@@ and @@LR@@ us.
 template <typename T>
-__global__ void larft_kernel(const T* G, int ldG, long long sG, const double* tau, long long stau, int k,
-                             T* Tm, int ldT, long long sT) {
+__global__ void __launch_bounds__(128) larft_kernel(const T* G, int ldG, long long sG, const double* tau,
+                                                    long long stau, int k, T* Tm, int ldT, long long sT) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* t = reinterpret_cast<T*>(smem_raw);
-  T* tmp = t + k * k;
-  const int z = blockIdx.x, tid = threadIdx.x, nt = blockDim.x;
+  T* gs = reinterpret_cast<T*>(smem_raw);  // [64][65], column c of G in row c
+  __shared__ double ts[64];
+  const int z = blockIdx.y, tid = threadIdx.x, lane = tid & 31, i = blockIdx.x * 4 + (tid >> 5);
   G += z * sG;
   tau += z * stau;
   Tm += z * sT;
-  for (int e = tid; e < k * k; e += nt) t[e] = zero<T>();
-  __syncthreads();
-  for (int i = 0; i < k; i++) {
-    const double ti = tau[i];
-    for (int r = tid; r < i; r += nt) {
-      T s = zero<T>();
-      for (int c = r; c < i; c++) mac(s, t[r * k + c], G[(size_t)c * ldG + i]);
-      tmp[r] = s;
-    }
-    __syncthreads();
-    for (int r = tid; r < i; r += nt) t[r * k + i] = (-ti) * tmp[r];
-    if (tid == 0) t[i * k + i] = from_real<T>(ti);
-    __syncthreads();
+#pragma unroll 8
+  for (int e = tid; e < 64 * 64; e += 128) {
+    const int r = e >> 6, c = e & 63;
+    if (r < c && c < k) gs[c * 65 + r] = G[(size_t)r * ldG + c];
   }
-  for (int e = tid; e < k * k; e += nt) Tm[(size_t)(e / k) * ldT + (e % k)] = t[e];
+  if (tid < k && tid < 64) ts[tid] = tau[tid];
+  __syncthreads();
+  if (i >= k) return;
+  T a0 = zero<T>(), a1 = zero<T>();  // sums of rows lane, lane + 32, then the entries
+  if (lane == (i & 31)) (i < 32 ? a0 : a1) = from_real<T>(ts[i]);
+#pragma unroll 1
+  for (int c = i; c > 0; c--) {
+    const T tc = shfl32(c < 32 ? a0 : a1, c & 31);
+    if (lane < c) mac(a0, gs[c * 65 + lane], tc);
+    if (lane + 32 < c) mac(a1, gs[c * 65 + lane + 32], tc);
+    if (lane == ((c - 1) & 31)) {
+      T& a = c - 1 < 32 ? a0 : a1;
+      a = (-ts[c - 1]) * a;
+    }
+  }
+  if (lane < k) Tm[(size_t)lane * ldT + i] = lane <= i ? a0 : zero<T>();
+  if (lane + 32 < k) Tm[(size_t)(lane + 32) * ldT + i] = lane + 32 <= i ? a1 : zero<T>();
 }
 
 // X[b][i][c] = ph[b][i] * Z[b][i][c] for the leading `cols` columns (Z real, X of type T)
@@ -236,30 +412,45 @@ __global__ void mirror_lower_kernel(T* A, int lda, long long sA, int n) {
 }
 
 // Column phase convention: the entry of largest modulus (lowest row on ties) becomes
-// real and positive.  One warp per column.
+// real and positive.  One CTA of 32 warps per 32 columns: lanes along the columns (the
+// contiguous direction), each warp every 32nd row.
 template <typename T>
-__global__ void column_phase_kernel(T* C, int ldc, long long sC, int rows, int cols) {
-  const int z = blockIdx.y;
-  C += z * sC;
-  const int lane = threadIdx.x & 31;
-  const int col = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (col >= cols) return;
+__global__ void __launch_bounds__(1024) column_phase_kernel(T* C, int ldc, long long sC, int rows, int cols) {
+  __shared__ double sb[32][33];
+  __shared__ int si[32][33];
+  __shared__ T sf[32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, col = blockIdx.x * 32 + lane;
+  C += blockIdx.y * sC + col;
   double best = -1.0;
   int bi = 0;
-  for (int i = lane; i < rows; i += 32) {
-    double a = abs2(C[(size_t)i * ldc + col]);
-    if (a > best) { best = a; bi = i; }
+  if (col < cols)
+#pragma unroll 4
+    for (int i = warp; i < rows; i += 32) {
+      const double a = abs2(C[(size_t)i * ldc]);
+      if (a > best) { best = a; bi = i; }
+    }
+  sb[warp][lane] = best;
+  si[warp][lane] = bi;
+  __syncthreads();
+  {  // warp w: column w, lanes over the warps' candidates
+    best = sb[lane][warp];
+    bi = si[lane][warp];
+    for (int o = 16; o > 0; o >>= 1) {
+      const double ob = __shfl_xor_sync(0xffffffffu, best, o);
+      const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+      if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
+    }
+    if (lane == 0 && blockIdx.x * 32 + warp < cols) {
+      const T p = C[(size_t)bi * ldc - col + blockIdx.x * 32 + warp];
+      const double mag = sqrt(abs2(p));
+      sf[warp] = mag > 0.0 ? conjg(p) * (1.0 / mag) : from_real<T>(1.0);
+    }
   }
-  for (int o = 16; o > 0; o >>= 1) {
-    double ob = __shfl_xor_sync(0xffffffffu, best, o);
-    int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-    if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
-  }
-  T p = C[(size_t)bi * ldc + col];
-  double mag = sqrt(abs2(p));
-  if (!(mag > 0.0)) return;
-  T f = conjg(p) * (1.0 / mag);
-  for (int i = lane; i < rows; i += 32) C[(size_t)i * ldc + col] = C[(size_t)i * ldc + col] * f;
+  __syncthreads();
+  if (col >= cols) return;
+  const T f = sf[lane];
+#pragma unroll 4
+  for (int i = warp; i < rows; i += 32) C[(size_t)i * ldc] = C[(size_t)i * ldc] * f;
 }
 
 // Fill dst (2n x 2n) with diag(S, S) from the n x n S (lower triangle valid).
@@ -312,12 +503,27 @@ static dim3 grid2d(int rows, int cols, int count) {
   return dim3(gx, gy, count);
 }
 
+// Launch of a diagonal-block kernel on one cluster per item.
+template <typename... P, typename... Q>
+static void diag_launch(void (*k)(P...), int count, size_t sm, cudaStream_t s, Q... args) {
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute at{};
+  cfg.gridDim = dim3(kDiagC, count);
+  cfg.blockDim = dim3(kDiagThreads);
+  cfg.dynamicSmemBytes = sm;
+  cfg.stream = s;
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = kDiagC;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  count_launch();
+  cudaLaunchKernelEx(&cfg, k, args...);
+}
+
 template <typename T>
 void potf2(T* A, int lda, long long sA, int k0, int nb, DevStatus* st, int count, cudaStream_t s) {
-  size_t sm = sizeof(T) * nb * (nb + 1);
-  cudaFuncSetAttribute(potf2_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  count_launch();
-  potf2_kernel<T><<<count, 256, sm, s>>>(A, lda, sA, k0, nb, st);
+  diag_launch(potf2_kernel<T>, count, 0, s, A, lda, sA, k0, nb, st);
 }
 
 template <typename T, int MODE>
@@ -345,19 +551,18 @@ void trsm_block(int mode, const T* L, int ldl, long long sL, T* B, int ldb, long
 template <typename T>
 void hegst_diag(T* A, int lda, long long sA, const T* L, int ldl, long long sL, int k0, int nb, T* F, int ldF,
                 long long sF, int count, cudaStream_t s) {
-  size_t sm = 2 * sizeof(T) * nb * (nb + 1);
+  const size_t sm = sizeof(T) * (64 * 65 + 64 * (kSub + 1));
   cudaFuncSetAttribute(hegst_diag_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  count_launch();
-  hegst_diag_kernel<T><<<count, 256, sm, s>>>(A, lda, sA, L, ldl, sL, k0, nb, F, ldF, sF);
+  diag_launch(hegst_diag_kernel<T>, count, sm, s, A, lda, sA, L, ldl, sL, k0, nb, F, ldF, sF);
 }
 
 template <typename T>
 void larft(const T* G, int ldG, long long sG, const double* tau, long long stau, int k, T* Tm, int ldT,
            long long sT, int count, cudaStream_t s) {
-  size_t sm = sizeof(T) * (k * k + k);
+  const size_t sm = sizeof(T) * 64 * 65;
   cudaFuncSetAttribute(larft_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   count_launch();
-  larft_kernel<T><<<count, 128, sm, s>>>(G, ldG, sG, tau, stau, k, Tm, ldT, sT);
+  larft_kernel<T><<<dim3((k + 3) / 4, count), 128, sm, s>>>(G, ldG, sG, tau, stau, k, Tm, ldT, sT);
 }
 
 template <typename T>
@@ -382,9 +587,9 @@ void mirror_lower(T* A, int lda, long long sA, int n, int count, cudaStream_t s)
 
 template <typename T>
 void column_phase(T* C, int ldc, long long sC, int rows, int cols, int count, cudaStream_t s) {
-  dim3 grid((cols + 7) / 8, count);
+  if (cols <= 0) return;
   count_launch();
-  column_phase_kernel<T><<<grid, 256, 0, s>>>(C, ldc, sC, rows, cols);
+  column_phase_kernel<T><<<dim3((cols + 31) / 32, count), 1024, 0, s>>>(C, ldc, sC, rows, cols);
 }
 
 template <typename T>

@@ -389,27 +389,44 @@ __global__ void __launch_bounds__(256) hetrd_phemv_kernel(const T* A, int lda, l
 //
 // hetrd_dmax_kernel: row maxima of |Re|, |Im| over the full Hermitian rows of the stale
 // block from its lower triangle, where element (r, c) counts for rows r and c.  One CTA per
-// chunk of 64 rows: a warp per row for the rows' own maxima (c <= r), then a thread per
-// column for the column maxima below the diagonal (c < r), one global atomic max per row,
-// and per column and chunk (on the bits of non-negative doubles, which order like the
-// values).
+// 64 x 64 tile of the lower triangle (each element read once, 8 warps of 8 rows, a lane per
+// column pair): row maxima by warp reduction, column maxima over the warps, one atomic max
+// per row, column and tile (on the bits of non-negative doubles, which order like the
+// values).  One CTA per 64 rows walking their columns twice took 777 us at order 4992.
+__device__ __forceinline__ unsigned long long umax(unsigned long long a, unsigned long long b) { return a > b ? a : b; }
 template <typename T>
 __global__ void __launch_bounds__(256) hetrd_dmax_kernel(const T* A, int lda, long long sA, int n,
                                                          unsigned long long* rmax, int ldr) {
-  const int z = blockIdx.y, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int r0 = blockIdx.x * 64, r1 = min(n, r0 + 64);
+  if (blockIdx.x > blockIdx.y) return;
+  __shared__ unsigned long long cm[8][64];
+  const int z = blockIdx.z, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int r0 = blockIdx.y * 64, c0 = blockIdx.x * 64;
   A += z * sA;
   rmax += (size_t)z * ldr;
-  for (int r = r0 + warp; r < r1; r += 8) {
-    unsigned long long m = 0ull;
-    for (int c = lane; c <= r; c += 32) m = max(m, maxbits(A[(size_t)r * lda + c]));
-    for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+  unsigned long long m0 = 0ull, m1 = 0ull, b[8][2];
+#pragma unroll
+  for (int q = 0; q < 8; q++) {
+    const int r = r0 + warp * 8 + q, c = c0 + lane;
+    b[q][0] = (r < n && c <= r) ? maxbits(A[(size_t)r * lda + c]) : 0ull;
+    b[q][1] = (r < n && c + 32 <= r) ? maxbits(A[(size_t)r * lda + c + 32]) : 0ull;
+  }
+#pragma unroll
+  for (int q = 0; q < 8; q++) {
+    const int r = r0 + warp * 8 + q;
+    m0 = umax(m0, b[q][0]);
+    m1 = umax(m1, b[q][1]);
+    unsigned long long m = umax(b[q][0], b[q][1]);
+    for (int o = 16; o > 0; o >>= 1) m = umax(m, __shfl_xor_sync(0xffffffffu, m, o));
     if (lane == 0 && m) atomicMax(rmax + r, m);
   }
-  for (int c = tid; c < r1 - 1; c += blockDim.x) {
-    unsigned long long mc = 0ull;
-    for (int r = max(r0, c + 1); r < r1; r++) mc = max(mc, maxbits(A[(size_t)r * lda + c]));
-    if (mc) atomicMax(rmax + c, mc);
+  cm[warp][lane] = m0;
+  cm[warp][lane + 32] = m1;
+  __syncthreads();
+  if (tid < 64) {
+    unsigned long long m = 0ull;
+#pragma unroll
+    for (int w = 0; w < 8; w++) m = umax(m, cm[w][tid]);
+    if (m) atomicMax(rmax + c0 + tid, m);
   }
 }
 
@@ -1313,28 +1330,48 @@ bool hetrd_panel(PanelArgs<T> a, int items, unsigned* base, unsigned* basev, cud
   return cudaLaunchKernelEx(&cfg, hetrd_panel_kernel<T, false>, a, maxseg) == cudaSuccess;
 }
 
-// d_i = Re A_ii, e_i = |A_{i+1,i}|, ph_0 = 1, ph_{i+1} = ph_i A_{i+1,i}/|A_{i+1,i}|.
+// d_i = Re A_ii, e_i = |A_{i+1,i}|, ph_0 = 1, ph_{i+1} = ph_i A_{i+1,i}/|A_{i+1,i}|.  One CTA
+// per item; the phases are a scan of products: a run of rows per thread, the runs' products
+// over the block, then every row of the run.  (One thread walking the rows took 4.5 ms at
+// order 4992.)
 template <typename T>
-__global__ void hetrd_finish_kernel(const T* A, int lda, long long sA, int m, double* d, double* e, long long sde,
-                                    T* ph, long long sph) {
-  const int z = blockIdx.x;
+__global__ void __launch_bounds__(1024) hetrd_finish_kernel(const T* A, int lda, long long sA, int m, double* d,
+                                                            double* e, long long sde, T* ph, long long sph) {
+  __shared__ T run[1024];
+  const int z = blockIdx.x, tid = threadIdx.x;
   A += z * sA;
   d += z * sde;
   e += z * sde;
   ph += z * sph;
-  for (int i = threadIdx.x; i < m; i += blockDim.x) {
+  const int per = (m + 1023) / 1024, i0 = tid * per, i1 = min(m, i0 + per);
+  auto unit = [&](int i) -> T {  // phase of A_{i+1,i} (1 where it is zero)
+    const T s = A[(size_t)(i + 1) * lda + i];
+    const double a = sqrt(abs2(s));
+    return a > 0.0 ? s * (1.0 / a) : from_real<T>(1.0);
+  };
+  T prod = from_real<T>(1.0);
+  for (int i = i0; i < i1; i++) {
     d[i] = re(A[(size_t)i * lda + i]);
-    if (i + 1 < m) e[i] = sqrt(abs2(A[(size_t)(i + 1) * lda + i]));
-  }
-  if (threadIdx.x == 0) {
-    T cur = from_real<T>(1.0);
-    ph[0] = cur;
-    for (int i = 0; i + 1 < m; i++) {
-      T s = A[(size_t)(i + 1) * lda + i];
-      double a = sqrt(abs2(s));
-      if (a > 0.0) cur = cur * (s * (1.0 / a));
-      ph[i + 1] = cur;
+    if (i + 1 < m) {
+      e[i] = sqrt(abs2(A[(size_t)(i + 1) * lda + i]));
+      const T w = unit(i);
+      ph[i + 1] = w;  // the row's own factor, replaced below
+      prod = prod * w;
     }
+  }
+  run[tid] = prod;
+  __syncthreads();
+  for (int o = 1; o < 1024; o <<= 1) {  // inclusive scan
+    const T v = tid >= o ? run[tid - o] : from_real<T>(1.0);
+    __syncthreads();
+    run[tid] = v * run[tid];
+    __syncthreads();
+  }
+  T cur = tid > 0 ? run[tid - 1] : from_real<T>(1.0);
+  if (tid == 0) ph[0] = cur;
+  for (int i = i0; i < i1 && i + 1 < m; i++) {
+    cur = cur * ph[i + 1];
+    ph[i + 1] = cur;
   }
 }
 
@@ -1377,7 +1414,7 @@ void hetrd_digits(const T* A, int lda, long long sA, int n, const HemvDigits& hd
   if (n <= 0) return;
   cudaMemsetAsync(hd.rmax, 0, sizeof(unsigned long long) * hd.ldd * count, s);
   count_launch(2);
-  hetrd_dmax_kernel<T><<<dim3((n + 63) / 64, count), 256, 0, s>>>(A, lda, sA, n, hd.rmax, hd.ldd);
+  hetrd_dmax_kernel<T><<<dim3((n + 63) / 64, (n + 63) / 64, count), 256, 0, s>>>(A, lda, sA, n, hd.rmax, hd.ldd);
   const int nt = ((n + 15) / 16 * 16 + 31) / 32;
   hetrd_digits_kernel<T><<<dim3(nt, nt, count), 64, 0, s>>>(A, lda, sA, n, hd);
 }
@@ -1419,7 +1456,7 @@ template <typename T>
 void hetrd_finish(const T* A, int lda, long long sA, int m, double* d, double* e, long long sde, T* ph,
                   long long sph, int count, cudaStream_t s) {
   count_launch();
-  hetrd_finish_kernel<T><<<count, 256, 0, s>>>(A, lda, sA, m, d, e, sde, ph, sph);
+  hetrd_finish_kernel<T><<<count, 1024, 0, s>>>(A, lda, sA, m, d, e, sde, ph, sph);
 }
 
 template <typename T, typename TV>

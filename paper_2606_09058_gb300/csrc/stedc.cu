@@ -81,14 +81,11 @@ __host__ __device__ inline DcWs dc_ws(void* base, int m) {
 
 __global__ void dc_tear_kernel(double* d, const double* e, long long sde, const int* splits, int nsplit) {
   const int z = blockIdx.x;
-  if (threadIdx.x != 0) return;
   d += z * sde;
   e += z * sde;
-  for (int k = 0; k < nsplit; k++) {
-    int s = splits[k];
-    double rho = fabs(e[s - 1]);
-    d[s - 1] -= rho;
-    d[s] -= rho;
+  for (int side = 1; side >= 0; side--) {  // the splits' left rows, then their right rows
+    for (int k = threadIdx.x; k < nsplit; k += blockDim.x) d[splits[k] - side] -= fabs(e[splits[k] - 1]);
+    __syncthreads();
   }
 }
 
@@ -584,7 +581,7 @@ void dc_solve(DcPlan* p, double* d, double* e, long long sde, double* lam, doubl
   const long long sZ0 = (p->depth % 2 == 0) ? sZ : slam;
   int tok = prof->begin();
   count_launch();
-  dc_tear_kernel<<<cnt, 32, 0, s>>>(d, e, sde, p->d_splits, (int)p->splits.size());
+  dc_tear_kernel<<<cnt, 256, 0, s>>>(d, e, sde, p->d_splits, (int)p->splits.size());
   const int nleaves = (int)p->leaves.size() / 2;
   count_launch();
   dc_leaf_kernel<<<dim3((nleaves + 3) / 4, cnt), 128, 0, s>>>(d, e, sde, lamBuf[0], slam, zbuf0, sZ0, m,
