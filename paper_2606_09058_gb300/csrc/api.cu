@@ -557,6 +557,14 @@ bool split_worth(gks_ctx* c, int count, int M, int N, int K, int es, double fl) 
   return c->gemm_mode == 0 && fl >= kSplitFlops && M >= 32 && Ne >= 32 && K >= 32;
 }
 
+// Smallest half of a merge whose products (half x 2 half x half, `items` of them per launch) are
+// split products: kSplitFlops again.
+int merge_half(int items) {
+  int h = 64;
+  while (4.0 * h * h * h * items < kSplitFlops) h += 16;
+  return h;
+}
+
 template <typename T>
 void gmx(gks_ctx* c, int count, int opA, int opB, int M, int N, int K, double alpha, const T* A, int lda, long long sA,
          const T* B, int ldb, long long sB, double beta, T* C, int ldc, long long sC, int lower = 0) {
@@ -833,10 +841,10 @@ void hegst_level(gks_ctx* c, T* A, int lda, long long sA, const T* L, int ldl, l
       Rec r(c, PC_TRSM, cmul(es) * 0.5 * kb * kb * rows * nk, (2.0 * rows * kb + 0.5 * kb * kb) * es * nk);
       trsm_block<T>(TRSM_RIGHT_CONJ, L11, ldl, sL, A21, lda, sA, kb, rows, nk, s);
     }
-    gmp<T>(c, nk, OP_N, OP_N, rows, kb, kb, -0.5, L21, ldl, sL, F, NB, c->sF, 1.0, A21, lda, sA);
+    gmx<T>(c, nk, OP_N, OP_N, rows, kb, kb, -0.5, L21, ldl, sL, F, NB, c->sF, 1.0, A21, lda, sA);
     gmx<T>(c, nk, OP_N, OP_C, rows, rows, kb, -1.0, L21, ldl, sL, A21, lda, sA, 1.0, A22, lda, sA, 1);
     gmx<T>(c, nk, OP_N, OP_C, rows, rows, kb, -1.0, A21, lda, sA, L21, ldl, sL, 1.0, A22, lda, sA, 1);
-    gmp<T>(c, nk, OP_N, OP_N, rows, kb, kb, -0.5, L21, ldl, sL, F, NB, c->sF, 1.0, A21, lda, sA);
+    gmx<T>(c, nk, OP_N, OP_N, rows, kb, kb, -0.5, L21, ldl, sL, F, NB, c->sF, 1.0, A21, lda, sA);
   }
   for (int r0 = NB; r0 < n; r0 += NB) {
     const int rb = std::min(NB, n - r0);
@@ -1263,9 +1271,9 @@ void backtransform_run(gks_ctx* c, const TA* A, T* X, int ldx, long long sX, int
       }
       if (s0 > 0) {
         // P = G[:s0, s0:s0+ks] T_ss (P in Y2, ld NB), then T[:s0, s0:s0+ks] = -T[:s0, :s0] P
-        gmp<T>(c, nk, OP_N, OP_N, s0, ks, ks, 1.0, G + s0, nbb, c->sG, Tm + (size_t)s0 * nbb + s0, nbb, c->sT, 0.0,
+        gmx<T>(c, nk, OP_N, OP_N, s0, ks, ks, 1.0, G + s0, nbb, c->sG, Tm + (size_t)s0 * nbb + s0, nbb, c->sT, 0.0,
                Y2, NB, c->sY);
-        gmp<T>(c, nk, OP_N, OP_N, s0, ks, s0, -1.0, Tm, nbb, c->sT, Y2, NB, c->sY, 0.0, Tm + s0, nbb, c->sT);
+        gmx<T>(c, nk, OP_N, OP_N, s0, ks, s0, -1.0, Tm, nbb, c->sT, Y2, NB, c->sY, 0.0, Tm + s0, nbb, c->sT);
       }
     }
     gmx<T>(c, nk, OP_C, OP_N, nbk, ncols, j1, 1.0, V, nbb, c->sV, X, ldx, sX, 0.0, Y, ncols, c->sY);
@@ -1289,8 +1297,8 @@ bool standard_eig(gks_ctx* c, T* A, T* X, long long sX, double* w, int M, int it
     hetrd_finish<T>(A, M, c->sMM, M, d, e, M, ph, M, items, s);
   }
   double* Z = at<double>(c, c->oZ);
-  DcSplit sp{nullptr, 0, sform(c), 512, c->wait_cycles};
-  if (c->gemm_mode != 1 && M >= 1024) {
+  DcSplit sp{nullptr, 0, sform(c), merge_half(items), c->wait_cycles};
+  if (c->gemm_mode != 1) {
     const size_t item = dc_split_item_bytes(c->dc, sp.min_half, sform(c));
     if (item > 0) {
       sp.per = oz_reserve(c, item, items);
@@ -1491,8 +1499,8 @@ gks_status solve_t(gks_ctx* c, const SolveKey& key) {
   double* Z = at<double>(c, c->oZ);
   {
     StageRec sr(c, PS_STEDC);
-    DcSplit sp_{nullptr, 0, sform(c), 512, c->wait_cycles};
-    if (c->gemm_mode != 1 && M >= 1024) {
+    DcSplit sp_{nullptr, 0, sform(c), merge_half(items), c->wait_cycles};
+    if (c->gemm_mode != 1) {
       const size_t item = dc_split_item_bytes(c->dc, sp_.min_half, sform(c));
       if (item > 0) {
         sp_.per = oz_reserve(c, item, items);

@@ -36,6 +36,7 @@ __device__ __forceinline__ zc shfl32(zc v, int src) { return zc{shfl32(v.x, src)
 // Measured, one complex block: two-sided reduction 794 us on one CTA, column by column;
 // Cholesky 207 us.  See the launchers for the times of this form.
 constexpr int kDiagC = 8, kSub = 8, kDiagThreads = 256;
+__device__ __forceinline__ void diag_bar() { asm volatile("bar.sync 1, 64;\n" ::: "memory"); }
 __device__ __forceinline__ void cluster_barrier() {
   asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
 }
@@ -68,7 +69,9 @@ __global__ void __launch_bounds__(kDiagThreads) potf2_kernel(T* A, int lda, long
           if (lane == 0) fail = c0 + j;
           break;
         }
-        const double d = sqrt(piv), inv = 1.0 / d;
+        // 1 / sqrt, then sqrt with one correction step: half the chain of a square root and a
+        // division on this pipe (434 + 686 clocks)
+        const double inv = rsqrt(piv), d0 = piv * inv, d = fma(0.5 * inv, fma(-d0, d0, piv), d0);
         __syncwarp();
         if (lane == j) {
           s11[j][j] = from_real<T>(d);
@@ -132,63 +135,67 @@ __global__ void __launch_bounds__(kDiagThreads) potf2_kernel(T* A, int lda, long
 //   TRSM_LEFT       : B (nb x nrhs cols)  <- L^-1 B
 //   TRSM_LEFT_CONJ  : B (nb x nrhs cols)  <- L^-H B   (backward: the reversed conj(L)^T)
 // Every mode is forward substitution with one lower matrix, kept in shared memory by
-// columns (conjugated or reversed while loading, padded to 64 with the identity).  Eight
-// lanes share a right-hand side, each holding 8 of its 64 entries in registers (entry 8 i +
+// columns (conjugated or reversed while loading, padded to 64 with the identity).  G lanes
+// share a right-hand side, each holding 64 / G of its entries in registers (entry G i +
 // lane): a step broadcasts the solved entry by shuffles and every lane updates its own
-// entries, so nothing but the columns of L is read.  The FP64 pipe bounds it (1.7
-// multiply-adds per SM clock; nb^2 / 2 per right-hand side, four times that complex), so the
-// right-hand sides are spread over all SMs, 4 per warp and as few warps per CTA as give one
-// CTA per SM.  The steps are a rolled loop on rotating registers: unrolled, the 64 steps are
-// 30 to 100 KB of code that each launch runs through once at the speed of instruction fetch.
-// Measured against 832 real right-hand sides: 184 us with a thread per right-hand side and 64
-// of them per CTA, 64 us unrolled, @@TR@@ us here; 4992 complex: 530, 266, @@TC@@ us.
-template <typename T, int MODE>
+// entries, so nothing but the columns of L is read.  The steps are a rolled loop on rotating
+// registers (unrolled they are 30 to 100 KB of code that each launch runs through once).
+// The FP64 pipe bounds it: one warp instruction per 64 clocks and SM partition whatever its
+// active lanes, 19 clocks over the four.  With many right-hand sides G = 8 wastes least (5.5
+// instructions per step for 4 right-hand sides); with few, G = 32 has the shorter chain (2.5
+// per step) on four times the warps.
+// Measured against 832 real right-hand sides: 184 us with a thread per right-hand side and
+// 64 of them per CTA, 20 us here; 4992 complex: 530, 137 us.
+template <typename T, int MODE, int G>
 __global__ void __launch_bounds__(256) trsm_block_kernel(const T* L, int ldl, long long sL, T* B, int ldb,
                                                          long long sB, int nb, int nrhs) {
+  constexpr int E = 64 / G;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* lc = reinterpret_cast<T*>(smem_raw);                    // [column][64]
   double* rd = reinterpret_cast<double*>(lc + 64 * 64);       // 1 / diagonal
   const int z = blockIdx.y, tid = threadIdx.x, nt = blockDim.x;
   L += z * sL;
   B += z * sB;
+  const int g = tid % G, r = (blockIdx.x * nt + tid) / G;
+  const bool ok = r < nrhs;
+  auto at = [&](int i) -> T* {  // entry i of this right-hand side, in solving order
+    const int e = MODE == TRSM_LEFT_CONJ ? nb - 1 - i : i;
+    return MODE == TRSM_RIGHT_CONJ ? B + (size_t)r * ldb + e : B + (size_t)e * ldb + r;
+  };
+  T x[E];
+#pragma unroll
+  for (int i = 0; i < E; i++) x[i] = (ok && G * i + g < nb) ? *at(G * i + g) : zero<T>();
 #pragma unroll 8
   for (int e = tid; e < 64 * 64; e += nt) {
     const int i = e >> 6, j = e & 63;  // stored element (i, j), j <= i
     T v = (i == j) ? from_real<T>(1.0) : zero<T>();
     if (i < nb && j <= i) v = L[(size_t)i * ldl + j];
     if (MODE != TRSM_LEFT) v = conjg(v);
-    if (i == j) rd[MODE == TRSM_LEFT_CONJ && i < nb ? nb - 1 - i : i] = 1.0 / re(v);
     // lower matrix by columns; backward: (i, j) of L is (nb - 1 - j, nb - 1 - i) of its reverse
     if (MODE == TRSM_LEFT_CONJ && i < nb && j < nb) lc[(nb - 1 - i) * 64 + nb - 1 - j] = v;
     else lc[j * 64 + i] = v;
   }
   __syncthreads();
-  const int g = tid & 7, r = (blockIdx.x * nt + tid) >> 3;
-  const bool ok = r < nrhs;
-  auto at = [&](int i) -> T* {  // entry i of this right-hand side, in solving order
-    const int e = MODE == TRSM_LEFT_CONJ ? nb - 1 - i : i;
-    return MODE == TRSM_RIGHT_CONJ ? B + (size_t)r * ldb + e : B + (size_t)e * ldb + r;
-  };
-  T x[8];
-#pragma unroll
-  for (int i = 0; i < 8; i++) x[i] = (ok && 8 * i + g < nb) ? *at(8 * i + g) : zero<T>();
+  for (int i = tid; i < 64; i += nt) rd[i] = 1.0 / re(lc[i * 65]);
+  __syncthreads();
 #pragma unroll 1
-  for (int J = 0; 8 * J < nb; J++) {  // x[i]: entries 8 (J + i) + g
-    const T* col = lc + 8 * J * 64 + 8 * J + g;
+  for (int J = 0; G * J < nb; J++) {  // x[i]: entries G (J + i) + g
+    const T* col = lc + G * J * 64 + G * J + g;
 #pragma unroll 1
-    for (int jj = 0; jj < 8; jj++, col += 64) {
-      const T xj = shfl8<T>(x[0] * rd[8 * J + jj], jj);
+    for (int jj = 0; jj < G; jj++, col += 64) {
+      const T y = x[0] * rd[G * J + jj];
+      const T xj = G == 8 ? shfl8<T>(y, jj) : shfl32(y, jj);
       if (g > jj) msub(x[0], xj, col[0]);
       if (g == jj) x[0] = xj;
 #pragma unroll
-      for (int i = 1; i < 8; i++) {
-        if (i + J >= 8) break;
-        msub(x[i], xj, col[8 * i]);
+      for (int i = 1; i < E; i++) {
+        if (i + J >= E) break;
+        msub(x[i], xj, col[G * i]);
       }
     }
-    if (ok && 8 * J + g < nb) *at(8 * J + g) = x[0];
+    if (ok && G * J + g < nb) *at(G * J + g) = x[0];
 #pragma unroll
-    for (int i = 0; i < 7; i++) x[i] = x[i + 1];
+    for (int i = 0; i < E - 1; i++) x[i] = x[i + 1];
   }
 }
 
@@ -225,41 +232,41 @@ __global__ void __launch_bounds__(kDiagThreads) hegst_diag_kernel(T* A, int lda,
     const int kb = min(kSub, nb - c0), m = nb - c0 - kb;
     const T* lb = l + c0 * LD + c0;
     __syncthreads();
-    if (tid < 32) {
-      for (int e = lane; e < kSub * kSub; e += 32) {
-        const int i = e >> 3, j = e & 7;
-        s11[i][j] = (i < kb && j <= i) ? ldcg(A + (size_t)(c0 + i) * lda + c0 + j) : zero<T>();
-      }
-      __syncwarp();
+    if (tid < kSub * kSub) {  // two warps (two SM partitions), one element each
+      const int i = tid >> 3, j = tid & 7;
+      T a = (i < kb && j <= i) ? ldcg(A + (size_t)(c0 + i) * lda + c0 + j) : zero<T>();
+      s11[i][j] = a;
+      diag_bar();
       for (int k = 0; k < kb; k++) {
         const double rk = rd[c0 + k], alpha = re(s11[k][k]) * rk * rk;
-        __syncwarp();
-        if (lane > k && lane < kb) s11[lane][k] = s11[lane][k] * rk - (0.5 * alpha) * lb[lane * LD + k];
-        __syncwarp();
-        for (int e = lane; e < kSub * kSub; e += 32) {
-          const int i = e >> 3, j = e & 7;
-          if (j > k && j <= i && i < kb) {
-            msubc(s11[i][j], lb[i * LD + k], s11[j][k]);
-            msubc(s11[i][j], s11[i][k], lb[j * LD + k]);
-          }
+        const T hl = (0.5 * alpha) * lb[min(i, kb - 1) * LD + k];
+        if (j == k && i > k) {
+          a = a * rk - hl;
+          s11[i][k] = a;
         }
-        __syncwarp();
-        if (lane > k && lane < kb) s11[lane][k] = s11[lane][k] - (0.5 * alpha) * lb[lane * LD + k];
-        if (lane == k) s11[k][k] = from_real<T>(alpha);
-        __syncwarp();
-      }
-      if (lane < kb) {  // column `lane`: rows below, forward substitution with L11
-        for (int i = lane + 1; i < kb; i++) {
-          T x = s11[i][lane];
-          for (int k = lane + 1; k < i; k++) msub(x, lb[i * LD + k], s11[k][lane]);
-          s11[i][lane] = x * rd[c0 + i];
+        diag_bar();
+        if (j > k && j <= i && i < kb) {
+          msubc(a, lb[i * LD + k], s11[j][k]);
+          msubc(a, s11[i][k], lb[j * LD + k]);
+          if (j == k + 1 && i == j) s11[i][j] = a;  // the next step's alpha
         }
+        diag_bar();
+        if (j == k && i > k) a = a - hl;
+        if (j == k && i == k) a = from_real<T>(alpha);
       }
-      __syncwarp();
-      for (int e = lane; e < kSub * kSub; e += 32) {  // the full Hermitian 8 x 8
-        const int i = e >> 3, j = e & 7;
-        if (j > i) s11[i][j] = conjg(s11[j][i]);
+      // strictly lower part: forward substitution with L11, rows top down
+      s11[i][j] = a;
+      diag_bar();
+      for (int k = 1; k < kb; k++) {
+        if (i == k && j < k) {
+          a = a * rd[c0 + k];
+          s11[k][j] = a;
+        }
+        diag_bar();
+        if (i > k && i < kb && j < k) msub(a, lb[i * LD + k], s11[k][j]);
       }
+      diag_bar();
+      if (i > j) s11[j][i] = conjg(s11[i][j]);  // the full Hermitian 8 x 8
     }
     __syncthreads();
     // rows below, one per 8 lanes: W, V
@@ -348,7 +355,7 @@ __global__ void __launch_bounds__(kDiagThreads) hegst_diag_kernel(T* A, int lda,
 //   t_i = tau_i,  t_r = -tau_r sum_{r < c <= i} G_rc t_c  (r = i - 1 .. 0),
 // a warp per column (lanes hold rows lane and lane + 32; k <= 64), 4 columns per CTA.  The
 // column-by-column form T[0:i, i] = -tau_i T[0:i, 0:i] G[0:i, i] on one CTA took 372 us
-// (complex, k = 64) and 144 us (real); this one @@LC@@ and @@LR@@ us.
+// (complex, k = 64) and 144 us (real); this one 38 and 26 us.
 template <typename T>
 __global__ void __launch_bounds__(128) larft_kernel(const T* G, int ldG, long long sG, const double* tau,
                                                     long long stau, int k, T* Tm, int ldT, long long sT) {
@@ -529,14 +536,18 @@ void potf2(T* A, int lda, long long sA, int k0, int nb, DevStatus* st, int count
 template <typename T, int MODE>
 static void trsm_launch(const T* L, int ldl, long long sL, T* B, int ldb, long long sB, int nb, int nrhs, int count,
                         cudaStream_t s) {
-  // warps per CTA: 4 right-hand sides each, at least one CTA per SM where there are enough
-  int w = 8;
-  while (w > 1 && (long long)((nrhs + 4 * w - 1) / (4 * w)) * count < 152) w >>= 1;
   const int sm = (int)(64 * 64 * sizeof(T) + 64 * sizeof(double));
-  cudaFuncSetAttribute(trsm_block_kernel<T, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
   count_launch();
-  trsm_block_kernel<T, MODE><<<dim3((nrhs + 4 * w - 1) / (4 * w), count), 32 * w, sm, s>>>(L, ldl, sL, B, ldb, sB, nb,
-                                                                                          nrhs);
+  if ((long long)nrhs * count <= 8 * 152) {  // a warp per right-hand side, 4 per CTA
+    cudaFuncSetAttribute(trsm_block_kernel<T, MODE, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+    trsm_block_kernel<T, MODE, 32><<<dim3((nrhs + 3) / 4, count), 128, sm, s>>>(L, ldl, sL, B, ldb, sB, nb, nrhs);
+    return;
+  }
+  // warps per CTA: 4 right-hand sides each, four warps (one per SM partition) or more
+  const int w = (long long)nrhs * count >= 2 * 32 * 152 ? 8 : 4;
+  cudaFuncSetAttribute(trsm_block_kernel<T, MODE, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+  trsm_block_kernel<T, MODE, 8><<<dim3((nrhs + 4 * w - 1) / (4 * w), count), 32 * w, sm, s>>>(L, ldl, sL, B, ldb, sB,
+                                                                                             nb, nrhs);
 }
 
 template <typename T>

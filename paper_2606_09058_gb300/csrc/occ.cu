@@ -22,13 +22,37 @@ __device__ __forceinline__ double fermi_fn(double x) {
   return 1.0 / (1.0 + exp(x));
 }
 
-// One CTA per system; system q owns k-points [q*nk, (q+1)*nk).
-__global__ void __launch_bounds__(1024) fermi_mu_kernel(const double* eps, int m, int nk, const double* w, double gs,
-                                                        double kT, double n_elec, double f_cut, double* occ,
-                                                        double* kscale, double* mu_out, double* e_band,
-                                                        int* nrho, DevStatus* st) {
-  __shared__ double red[32];
-  const int q = blockIdx.x, tid = threadIdx.x, nt = blockDim.x;
+// One cluster of kOccC CTAs x 128 threads per system; system q owns k-points [q*nk, (q+1)*nk).
+// The FP64 pipe bounds an evaluation of N(mu) (about 40 operations per eigenvalue and SM with
+// 1.7 per clock), so it is spread over the cluster's SMs, and eigenvalues more than 40 kT
+// below mu (f = 1 exactly) or 60 kT above (f < 1e-26) take no exponential.  The sum is the one
+// of 1024 threads in one CTA (thread tid of rank r stands for thread 128 r + tid, their 32 warp
+// sums combined in one shuffle tree), so the halvings do not depend on the cluster.  6656
+// eigenvalues: 3.9 ms on one CTA, 0.5 ms here.
+constexpr int kOccC = 8, kOccT = 128;
+__device__ __forceinline__ void occ_barrier() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+}
+// Every warp's value into slot 4 rank + warp of all CTAs of the cluster.
+__device__ __forceinline__ void occ_share(double* slots, int rank, double v) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (lane < kOccC)
+    asm volatile(
+        "{\n .reg .b32 ra;\n mapa.shared::cluster.u32 ra, %0, %1;\n st.shared::cluster.f64 [ra], %2;\n}\n" ::"r"(
+            (unsigned)__cvta_generic_to_shared(slots + 4 * rank + warp)),
+        "r"(lane), "d"(v)
+        : "memory");
+  occ_barrier();
+}
+
+__global__ void __launch_bounds__(kOccT) fermi_mu_kernel(const double* eps, int m, int nk, const double* w, double gs,
+                                                         double kT, double n_elec, double f_cut, double* occ,
+                                                         double* kscale, double* mu_out, double* e_band, int* nrho,
+                                                         DevStatus* st) {
+  __shared__ double slots[2][32];
+  const int q = blockIdx.y, rank = blockIdx.x, lane = threadIdx.x & 31;
+  const int tid = rank * kOccT + threadIdx.x;
+  constexpr int nt = kOccC * kOccT;
   const long long base = (long long)q * nk * m;
   eps += base;
   occ += base;
@@ -36,80 +60,105 @@ __global__ void __launch_bounds__(1024) fermi_mu_kernel(const double* eps, int m
   const long long tot = (long long)nk * m;
   double lo, hi;
   {
-    // min / max reductions
     double vmin = 1e300, vmax = -1e300;
     for (long long t = tid; t < tot; t += nt) { vmin = fmin(vmin, eps[t]); vmax = fmax(vmax, eps[t]); }
     for (int o = 16; o > 0; o >>= 1) {
       vmin = fmin(vmin, __shfl_xor_sync(0xffffffffu, vmin, o));
       vmax = fmax(vmax, __shfl_xor_sync(0xffffffffu, vmax, o));
     }
-    __shared__ double smin[32], smax[32];
-    if ((tid & 31) == 0) { smin[tid >> 5] = vmin; smax[tid >> 5] = vmax; }
-    __syncthreads();
-    if (tid < 32) {
-      int nw = (nt + 31) >> 5;
-      vmin = tid < nw ? smin[tid] : 1e300;
-      vmax = tid < nw ? smax[tid] : -1e300;
-      for (int o = 16; o > 0; o >>= 1) {
-        vmin = fmin(vmin, __shfl_xor_sync(0xffffffffu, vmin, o));
-        vmax = fmax(vmax, __shfl_xor_sync(0xffffffffu, vmax, o));
-      }
-      if (tid == 0) { smin[0] = vmin; smax[0] = vmax; }
+    occ_barrier();  // every CTA of the cluster runs
+    occ_share(slots[0], rank, vmin);
+    occ_share(slots[1], rank, vmax);
+    vmin = slots[0][lane];
+    vmax = slots[1][lane];
+    for (int o = 16; o > 0; o >>= 1) {
+      vmin = fmin(vmin, __shfl_xor_sync(0xffffffffu, vmin, o));
+      vmax = fmax(vmax, __shfl_xor_sync(0xffffffffu, vmax, o));
     }
-    __syncthreads();
-    lo = smin[0] - 1.0;
-    hi = smax[0] + 1.0;
-    __syncthreads();
+    lo = vmin - 1.0;
+    hi = vmax + 1.0;
+    occ_barrier();  // the slots have been read
   }
   double wsum = 0.0;
   for (int k = 0; k < nk; k++) wsum += w[k];
   const bool bad = !(kT > 0.0) || !(n_elec > 0.0) || !(n_elec < gs * m * wsum) || !isfinite(lo) || !isfinite(hi);
-  if (bad) {
+  if (bad) {  // the same in every CTA
     if (tid == 0) set_status(st, ST_EINVAL, 0);
     return;
   }
+  const int k0 = tid / m, dk = nt / m, r0 = tid % m, dr = nt % m;  // k-point and row of t = tid + i nt
+  // sum over the system of fn(t, k), by every thread
+  int phase = 0;
+  auto total = [&](auto fn) -> double {
+    double s = 0.0;
+    int k = k0, r = r0;
+    for (long long t = tid; t < tot; t += nt) {
+      s += fn(t, k);
+      k += dk;
+      r += dr;
+      if (r >= m) {
+        r -= m;
+        k++;
+      }
+    }
+    s = warp_sum(s);
+    phase ^= 1;
+    occ_share(slots[phase], rank, s);
+    return warp_sum(slots[phase][lane]);
+  };
   const double u = 1.1102230246251565e-16;
   for (int it = 0; it < 200; it++) {
     double mid = 0.5 * (lo + hi);
     if (hi - lo <= 4.0 * u * fmax(1.0, fabs(mid))) break;
-    double s = 0.0;
-    for (long long t = tid; t < tot; t += nt) s += w[t / m] * fermi_fn((eps[t] - mid) / kT);
-    s = gs * block_sum(s, red);
+    const double one = mid - 40.0 * kT, none = mid + 60.0 * kT;
+    const double s = gs * total([&](long long t, int k) -> double {
+      const double e = eps[t];
+      return e < one ? w[k] : e > none ? 0.0 : w[k] * fermi_fn((e - mid) / kT);
+    });
     if (s < n_elec) lo = mid;
     else hi = mid;
   }
   const double mu = 0.5 * (lo + hi);
-  double eb = 0.0;
-  for (long long t = tid; t < tot; t += nt) {
-    double f = fermi_fn((eps[t] - mu) / kT);
+  const double eb = total([&](long long t, int k) -> double {
+    const double f = fermi_fn((eps[t] - mu) / kT);
     occ[t] = f;
     kscale[t] = (f >= f_cut) ? gs * f : 0.0;
-    eb += w[t / m] * gs * f * eps[t];
-  }
-  eb = block_sum(eb, red);
+    return w[k] * gs * f * eps[t];
+  });
   if (tid == 0) {
     mu_out[q] = mu;
     e_band[q] = eb;
   }
-  __syncthreads();
   for (int k = tid; k < nk; k += nt) {
     // f non-increasing along the ascending eigenvalues: binary search for the last kept
+    // (written by this cluster before the barrier of the last sum)
     const double* fk = occ + (long long)k * m;
     int lo_i = 0, hi_i = m;
     while (lo_i < hi_i) {
       int mid = (lo_i + hi_i) >> 1;
-      if (fk[mid] >= f_cut) lo_i = mid + 1;
+      if (__ldcg(fk + mid) >= f_cut) lo_i = mid + 1;
       else hi_i = mid;
     }
     nrho[(long long)q * nk + k] = lo_i;
   }
+  occ_barrier();  // no CTA leaves while another may still write to its slots
 }
 
 void fermi_mu(const double* eps, int m, int nk, const double* w, double gs, double kT, double n_elec, double f_cut,
               double* occ, double* kscale, double* mu, double* e_band, int* nrho, DevStatus* st, int nsys,
               cudaStream_t s) {
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute at{};
+  cfg.gridDim = dim3(kOccC, nsys);
+  cfg.blockDim = dim3(kOccT);
+  cfg.stream = s;
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = kOccC;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
   count_launch();
-  fermi_mu_kernel<<<nsys, 1024, 0, s>>>(eps, m, nk, w, gs, kT, n_elec, f_cut, occ, kscale, mu, e_band, nrho, st);
+  cudaLaunchKernelEx(&cfg, fermi_mu_kernel, eps, m, nk, w, gs, kT, n_elec, f_cut, occ, kscale, mu, e_band, nrho, st);
 }
 
 __global__ void expand_weights_kernel(const double* w, int nk, int rep, double* out) {

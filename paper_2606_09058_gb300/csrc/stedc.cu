@@ -4,7 +4,7 @@
 //
 //  * Tear: T = diag(T1, T2) + rho v v^T at every split s (rho = |e_{s-1}|,
 //    v = (e_last; sign e_first)), i.e. d_{s-1} -= rho and d_s -= rho before the leaves.
-//  * Leaves (<= 32 rows): one warp each runs implicit QL redundantly on every lane, lane
+//  * Leaves (<= 16 rows): one warp each runs implicit QL redundantly on every lane, lane
 //    i accumulating row i of the leaf's eigenvector block.
 //  * Merge of (lam1, Z1), (lam2, Z2): z = (last row of Z1; sign * first row of Z2)/sqrt2,
 //    rho' = 2 rho; poles merged in ascending order; deflation of negligible z_i and of
@@ -24,7 +24,7 @@
 
 namespace gks {
 
-static constexpr int DC_LEAF = 32;
+static constexpr int DC_LEAF = 16;
 static constexpr double DC_U = 1.1102230246251565e-16;
 
 struct DcNode {
@@ -89,75 +89,98 @@ __global__ void dc_tear_kernel(double* d, const double* e, long long sde, const 
   }
 }
 
-// One warp per leaf. Every lane runs the same QL iteration on private copies of (d, e);
-// lane i applies the rotations to row i of the leaf's eigenvector block.
-__global__ void dc_leaf_kernel(const double* d, const double* e, long long sde, double* lam, long long slam,
-                               double* Z, long long sZ, int m, const int* leaves, int nleaves, DevStatus* st) {
-  const int z = blockIdx.y;
-  const int leaf = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (leaf >= nleaves) return;
+// One warp per leaf, one leaf per CTA. Every lane runs the same QL iteration on (d, e) in
+// shared memory; lane i applies the rotations to row i of the leaf's eigenvector block.  A
+// serial chain of rotations: one reciprocal square root each in place of a hypot and two
+// divisions (the block is scaled by a power of two so that no square overflows), arrays in
+// shared memory in place of dynamically indexed local ones, and leaves of at most 16 rows (a
+// quarter of the rotations of 32 for one more merge level): 1.87 ms at order 832 with 32 rows,
+// 220 us here.
+__global__ void __launch_bounds__(32) dc_leaf_kernel(const double* d, const double* e, long long sde, double* lam,
+                                                     long long slam, double* Z, long long sZ, int m,
+                                                     const int* leaves, int nleaves, DevStatus* st) {
+  __shared__ double dd[DC_LEAF], ee[DC_LEAF], zr[DC_LEAF][33];
+  const int z = blockIdx.y, leaf = blockIdx.x, lane = threadIdx.x;
   const int off = leaves[2 * leaf], n = leaves[2 * leaf + 1];
   d += z * sde;
   e += z * sde;
   lam += z * slam;
   Z += z * sZ;
-  double dd[DC_LEAF], ee[DC_LEAF], zr[DC_LEAF];
-  for (int i = 0; i < n; i++) {
-    dd[i] = d[off + i];
-    ee[i] = (i + 1 < n) ? e[off + i] : 0.0;
-    zr[i] = (i == lane) ? 1.0 : 0.0;
+  double dv = lane < n ? d[off + lane] : 0.0, ev = lane + 1 < n ? e[off + lane] : 0.0;
+  double big = fmax(fabs(dv), fabs(ev));
+  for (int o = 16; o > 0; o >>= 1) big = fmax(big, __shfl_xor_sync(0xffffffffu, big, o));
+  const int sc = (big > 0.0 && isfinite(big)) ? ilogb(big) : 0;  // entries at most 2 in magnitude
+  if (lane < DC_LEAF) {
+    dd[lane] = ldexp(dv, -sc);
+    ee[lane] = ldexp(ev, -sc);
   }
+  for (int i = 0; i < n; i++) zr[i][lane] = (i == lane) ? 1.0 : 0.0;
+  __syncwarp();
   bool ok = true;
   for (int l = 0; l < n && ok; l++) {
     for (int sweep = 0;; sweep++) {
-      int q = l;
-      while (q < n - 1) {
-        if (fabs(ee[q]) <= DC_U * (fabs(dd[q]) + fabs(dd[q + 1]))) { ee[q] = 0.0; break; }
-        q++;
-      }
+      // the first negligible off-diagonal from l on
+      const bool neg = lane >= l && lane < n - 1 && fabs(ee[lane]) <= DC_U * (fabs(dd[lane]) + fabs(dd[lane + 1]));
+      const unsigned mask = __ballot_sync(0xffffffffu, neg);
+      const int q = mask ? __ffs(mask) - 1 : n - 1;
+      __syncwarp();
+      if (mask && lane == 0) ee[q] = 0.0;
+      __syncwarp();
       if (q == l) break;
       if (sweep >= 60) { ok = false; break; }
       // shift: eigenvalue of [[d_l, e_l], [e_l, d_{l+1}]] nearer to d_l
-      double h = 0.5 * (dd[l + 1] - dd[l]);
-      double r = hypot(h, ee[l]);
-      double mu = dd[l] - ee[l] * ee[l] / (h + copysign(r, h));
+      const double el = ee[l], h = 0.5 * (dd[l + 1] - dd[l]);
+      const double mu = dd[l] - el * el / (h + copysign(sqrt(fma(h, h, el * el)), h));
       double x = dd[q] - mu, y = ee[q - 1];
+      double g = dd[q], z1 = zr[q][lane];
       for (int k = q; k > l; k--) {
-        double rr = hypot(x, y);
-        double c = rr > 0.0 ? x / rr : 1.0, s = rr > 0.0 ? y / rr : 0.0;
-        if (k < q) ee[k] = rr;
-        double a = dd[k - 1], b = ee[k - 1], g = dd[k];
-        double cs = c * s;
-        dd[k - 1] = c * c * a - 2.0 * cs * b + s * s * g;
-        dd[k] = s * s * a + 2.0 * cs * b + c * c * g;
-        ee[k - 1] = cs * (a - g) + (c * c - s * s) * b;
-        double z0 = zr[k - 1], z1 = zr[k];
-        zr[k - 1] = c * z0 - s * z1;
-        zr[k] = s * z0 + c * z1;
-        if (k - 1 > l) {
-          x = ee[k - 1];
-          y = s * ee[k - 2];
-          ee[k - 2] = c * ee[k - 2];
+        const double r2 = fma(x, x, y * y), ri = r2 > 0.0 ? rsqrt(r2) : 0.0;
+        const double c = r2 > 0.0 ? x * ri : 1.0, sn = y * ri;
+        const double a = dd[k - 1], b = ee[k - 1], en = k - 1 > l ? ee[k - 2] : 0.0, z0 = zr[k - 1][lane];
+        // [[a, b], [b, g]] rotated: s t moves between the diagonal entries, t = s (a - g) + 2 c b
+        const double t = fma(sn, a - g, 2.0 * c * b);
+        const double gk = fma(sn, -t, a);  // new d_{k-1}: a - s t
+        __syncwarp();
+        if (lane == 0) {
+          if (k < q) ee[k] = r2 * ri;
+          dd[k] = fma(sn, t, g);            // g + s t
         }
+        const double bk = fma(c, t, -b);    // new coupling: c t - b
+        zr[k][lane] = fma(sn, z0, c * z1);
+        z1 = fma(c, z0, -sn * z1);
+        x = bk;
+        y = sn * en;
+        if (lane == 0) {
+          ee[k - 1] = bk;
+          if (k - 1 > l) ee[k - 2] = c * en;
+        }
+        g = gk;
+        __syncwarp();
       }
+      if (lane == 0) dd[l] = g;
+      zr[l][lane] = z1;
+      __syncwarp();
     }
   }
   if (!ok) {
     if (lane == 0) set_status(st ? st + z : nullptr, ST_ENOCONV, off);
   }
-  // ascending order by selection (ties keep the lower index)
-  int perm[DC_LEAF];
-  for (int i = 0; i < n; i++) perm[i] = i;
+  // ascending order (ties keep the lower index); ordered bits, so that the ranks are a
+  // permutation whatever the values
+  const double v = lane < n ? dd[lane] : 0.0;
+  auto key = [](double x) -> long long {
+    const long long k = __double_as_longlong(x + 0.0);
+    return k < 0 ? k ^ 0x7fffffffffffffffll : k;
+  };
+  int rank = 0;
   for (int i = 0; i < n; i++) {
-    int b = i;
-    for (int k = i + 1; k < n; k++)
-      if (dd[perm[k]] < dd[perm[b]]) b = k;
-    int t = perm[i]; perm[i] = perm[b]; perm[b] = t;
+    const long long o = key(dd[i]), kv = key(v);
+    if (o < kv || (o == kv && i < lane)) rank++;
   }
+  if (lane < n) lam[off + rank] = ldexp(v, sc);
   for (int c = 0; c < n; c++) {
-    if (lane == 0) lam[off + c] = dd[perm[c]];
-    if (lane < n) Z[(size_t)(off + lane) * m + off + c] = zr[perm[c]];
+    const int pos = __shfl_sync(0xffffffffu, rank, c);
+    if (lane < n) Z[(size_t)(off + lane) * m + off + pos] = zr[c][lane];
   }
 }
 
@@ -187,11 +210,41 @@ struct DcArgs {
 
 __device__ __forceinline__ DcWs item_ws(const DcArgs& a, int z) { return dc_ws(a.ws + z * a.sitem, a.m); }
 
-// Merge setup, one CTA per (node, item): z vector, merged poles, deflation.
-__global__ void dc_merge_prep_kernel(DcArgs a, const DcNode* nodes) {
+// Exclusive sum of v over the CTA (1024 threads), total in *all.
+__device__ int block_scan(int v, int* scratch, int* all) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int x = v;
+  for (int o = 1; o < 32; o <<= 1) {
+    const int t = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += t;
+  }
+  __syncthreads();
+  if (lane == 31) scratch[warp] = x;
+  __syncthreads();
+  if (warp == 0) {
+    int t = scratch[lane];
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, t, o);
+      if (lane >= o) t += y;
+    }
+    scratch[lane] = t;
+  }
+  __syncthreads();
+  *all = scratch[31];
+  return x - v + (warp ? scratch[warp - 1] : 0);
+}
+
+// Merge setup, one CTA per (node, item): z vector, merged poles, deflation.  The scan for
+// close poles is sequential only where rotations happen: negligible z_i drop out by a
+// compaction, the test between neighbouring survivors runs for all pairs at once on the
+// unrotated values (which are the current ones unless the pair before rotated), and one
+// thread walks the runs that start at a pair that fails it.  (Walking every pole from global
+// memory took 6.3 ms for the last merge of order 4992.)
+__global__ void __launch_bounds__(1024) dc_merge_prep_kernel(DcArgs a, const DcNode* nodes) {
   __shared__ double red[32];
+  __shared__ int scan[32], s_nrot, s_bad;
   const DcNode nd = nodes[blockIdx.x];
-  const int z = blockIdx.y, tid = threadIdx.x, nt = blockDim.x;
+  const int z = blockIdx.y, tid = threadIdx.x, nt = 1024;
   DcWs w = item_ws(a, z);
   const int m = a.m, off = nd.off, n1 = nd.n1, n2 = nd.n2, n = n1 + n2, s = off + n1;
   const double* lam = a.lam + z * a.slam;
@@ -200,6 +253,16 @@ __global__ void dc_merge_prep_kernel(DcArgs a, const DcNode* nodes) {
   const double rho2 = 2.0 * fabs(beta);
   const double sg = beta < 0.0 ? -1.0 : 1.0;
   const double isq2 = 0.70710678118654752440;
+  double *ds = w.ds + off, *zs = w.zs + off, *dK = w.dK + off, *zK = w.zK + off, *dD = w.dD + off;
+  double *rc = w.rc + off, *rs = w.rs + off;
+  int *src = w.src + off, *idxK = w.idxK + off, *idxD = w.idxD + off, *ra = w.ra + off, *rb = w.rb + off;
+  int *links = w.colsrc + off, *gone = w.orig + off;  // free until the roots and the column map
+  for (int i = tid; i < n; i += nt) {  // every slot valid, also if non-finite values collide below
+    ds[i] = 0.0;
+    zs[i] = 0.0;
+    src[i] = i;
+  }
+  __syncthreads();
   double dmax = 0.0;
   for (int i = tid; i < n; i += nt) {
     int pos;
@@ -214,60 +277,140 @@ __global__ void dc_merge_prep_kernel(DcArgs a, const DcNode* nodes) {
       zv = sg * Zc[(size_t)s * m + s + k] * isq2;
       pos = k + upper_bound_d(lam + off, n1, dv);
     }
-    w.ds[off + pos] = dv;
-    w.zs[off + pos] = zv;
-    w.src[off + pos] = i;
+    ds[pos] = dv;
+    zs[pos] = zv;
+    src[pos] = i;
     dmax = fmax(dmax, fabs(dv));
   }
   for (int o = 16; o > 0; o >>= 1) dmax = fmax(dmax, __shfl_xor_sync(0xffffffffu, dmax, o));
   if ((tid & 31) == 0) red[tid >> 5] = dmax;
+  if (tid == 0) s_nrot = s_bad = 0;
   __syncthreads();
-  if (tid != 0) return;
-  for (int k = 1; k < (nt + 31) / 32; k++) dmax = fmax(dmax, red[k]);
-  dmax = fmax(dmax, red[0]);
+  for (int k = 0; k < 32; k++) dmax = fmax(dmax, red[k]);
   const double tol = 8.0 * DC_U * fmax(dmax, rho2);
-  int K = 0, nD = 0, nrot = 0;
-  bool have = false;
-  double pd = 0, pz = 0;
-  int ps = 0;
-  for (int p = 0; p < n; p++) {
-    double dp = w.ds[off + p], zp = w.zs[off + p];
-    int sp = w.src[off + p];
-    if (rho2 * fabs(zp) <= tol) {
-      w.dD[off + nD] = dp; w.idxD[off + nD] = sp; nD++;
-      continue;
-    }
-    if (!have) { pd = dp; pz = zp; ps = sp; have = true; continue; }
-    double r = hypot(pz, zp);
-    double c = zp / r, sn = pz / r;
-    if (fabs(c * sn * (dp - pd)) <= tol) {
-      w.ra[off + nrot] = ps; w.rb[off + nrot] = sp; w.rc[off + nrot] = c; w.rs[off + nrot] = sn; nrot++;
-      w.dD[off + nD] = c * c * pd + sn * sn * dp; w.idxD[off + nD] = ps; nD++;
-      pd = sn * sn * pd + c * c * dp; pz = r; ps = sp;
+  // survivors (in dK, zK, idxK) and negligible z_i (in dD, idxD), each in ascending order
+  const int per = (n + nt - 1) / nt, p0 = min(n, tid * per), p1 = min(n, p0 + per);
+  int cnt = 0, ns = 0;
+  for (int p = p0; p < p1; p++) cnt += !(rho2 * fabs(zs[p]) <= tol);
+  int at = block_scan(cnt, scan, &ns);
+  for (int p = p0, q = p0 - at; p < p1; p++) {
+    if (!(rho2 * fabs(zs[p]) <= tol)) {
+      dK[at] = ds[p]; zK[at] = zs[p]; idxK[at] = src[p]; at++;
     } else {
-      w.dK[off + K] = pd; w.zK[off + K] = pz; w.idxK[off + K] = ps; K++;
-      pd = dp; pz = zp; ps = sp;
+      dD[q] = ds[p]; idxD[q] = src[p]; q++;
     }
   }
-  if (have) { w.dK[off + K] = pd; w.zK[off + K] = pz; w.idxK[off + K] = ps; K++; }
-  // rotations can perturb the order slightly: insertion sorts on nearly sorted data
-  for (int i = 1; i < K; i++) {
-    double dv = w.dK[off + i], zv = w.zK[off + i];
-    int iv = w.idxK[off + i], j = i - 1;
-    while (j >= 0 && w.dK[off + j] > dv) {
-      w.dK[off + j + 1] = w.dK[off + j]; w.zK[off + j + 1] = w.zK[off + j]; w.idxK[off + j + 1] = w.idxK[off + j]; j--;
+  const int nsm = n - ns;
+  __syncthreads();
+  // pairs (i, i + 1) close enough to rotate: |c s (d_{i+1} - d_i)| <= tol with c, s ~ z_{i+1}, z_i
+  auto close = [tol](double pd, double pz, double dp, double zp) {
+    return fabs(pz * zp * (dp - pd)) <= tol * fma(pz, pz, zp * zp);
+  };
+  const int pr = (ns + nt - 1) / nt, l0 = min(ns, tid * pr), l1 = min(ns, l0 + pr);
+  int nl = 0;
+  cnt = 0;
+  for (int i = l0; i < l1; i++) {
+    gone[i] = 0;
+    cnt += i + 1 < ns && close(dK[i], zK[i], dK[i + 1], zK[i + 1]);
+  }
+  at = block_scan(cnt, scan, &nl);
+  for (int i = l0; i < l1 && cnt; i++)
+    if (i + 1 < ns && close(dK[i], zK[i], dK[i + 1], zK[i + 1])) links[at++] = i;
+  __syncthreads();
+  int K = ns, nD = nsm;
+  if (nl > 0) {
+    if (tid == 0) {
+      int nrot = 0, next = 0;  // next: first survivor not yet walked over
+      for (int f = 0; f < nl; f++) {
+        int i = links[f];
+        if (i < next) continue;
+        double pd = dK[i], pz = zK[i];
+        int ps = idxK[i];
+        while (i + 1 < ns) {
+          const double dp = dK[i + 1], zp = zK[i + 1];
+          if (!close(pd, pz, dp, zp)) break;
+          const double r = hypot(pz, zp), c = zp / r, sn = pz / r;
+          const int sp = idxK[i + 1];
+          ra[nrot] = ps; rb[nrot] = sp; rc[nrot] = c; rs[nrot] = sn;
+          gone[i] = 1;
+          // the rotation's deflated pole, kept with the small ones' tail (sorted below)
+          dD[nsm + nrot] = c * c * pd + sn * sn * dp; idxD[nsm + nrot] = ps;
+          nrot++;
+          pd = sn * sn * pd + c * c * dp; pz = r; ps = sp;
+          i++;
+          dK[i] = pd; zK[i] = pz;
+        }
+        next = i + 1;
+      }
+      for (int i = 1; i < nrot; i++) {  // rotations can perturb the order slightly
+        double dv = dD[nsm + i];
+        int iv = idxD[nsm + i], j = i - 1;
+        while (j >= 0 && dD[nsm + j] > dv) { dD[nsm + j + 1] = dD[nsm + j]; idxD[nsm + j + 1] = idxD[nsm + j]; j--; }
+        dD[nsm + j + 1] = dv; idxD[nsm + j + 1] = iv;
+      }
+      s_nrot = nrot;
     }
-    w.dK[off + j + 1] = dv; w.zK[off + j + 1] = zv; w.idxK[off + j + 1] = iv;
+    __syncthreads();
+    const int nrot = s_nrot;
+    K = ns - nrot;
+    nD = nsm + nrot;
+    // survivors left, compacted through ds, zs, src; the deflated lists merged the same way
+    cnt = 0;
+    for (int i = l0; i < l1; i++) cnt += !gone[i];
+    int all;
+    at = block_scan(cnt, scan, &all);
+    for (int i = l0; i < l1; i++)
+      if (!gone[i]) { ds[at] = dK[i]; zs[at] = zK[i]; src[at] = idxK[i]; at++; }
+    __syncthreads();
+    for (int i = tid; i < K; i += nt) { dK[i] = ds[i]; zK[i] = zs[i]; idxK[i] = src[i]; }
+    __syncthreads();
+    for (int i = tid; i < nD; i += nt) {
+      const double v = dD[i];
+      const int pos = i < nsm ? i + lower_bound_d(dD + nsm, nrot, v) : i - nsm + upper_bound_d(dD, nsm, v);
+      ds[pos] = v; src[pos] = idxD[i];
+    }
+    __syncthreads();
+    for (int i = tid; i < nD; i += nt) { dD[i] = ds[i]; idxD[i] = src[i]; }
+    for (int i = tid; i + 1 < K; i += nt)
+      if (dK[i] > dK[i + 1]) s_bad = 1;
+    __syncthreads();
+    if (s_bad && tid == 0)
+      for (int i = 1; i < K; i++) {
+        double dv = dK[i], zv = zK[i];
+        int iv = idxK[i], j = i - 1;
+        while (j >= 0 && dK[j] > dv) { dK[j + 1] = dK[j]; zK[j + 1] = zK[j]; idxK[j + 1] = idxK[j]; j--; }
+        dK[j + 1] = dv; zK[j + 1] = zv; idxK[j + 1] = iv;
+      }
   }
-  for (int i = 1; i < nD; i++) {
-    double dv = w.dD[off + i];
-    int iv = w.idxD[off + i], j = i - 1;
-    while (j >= 0 && w.dD[off + j] > dv) { w.dD[off + j + 1] = w.dD[off + j]; w.idxD[off + j + 1] = w.idxD[off + j]; j--; }
-    w.dD[off + j + 1] = dv; w.idxD[off + j + 1] = iv;
+  if (tid == 0) {
+    w.cnt[3 * off + 0] = K;
+    w.cnt[3 * off + 1] = nD;
+    w.cnt[3 * off + 2] = s_nrot;
   }
-  w.cnt[3 * off + 0] = K;
-  w.cnt[3 * off + 1] = nD;
-  w.cnt[3 * off + 2] = nrot;
+}
+
+// 1 / x for x in the normal range of a double's reciprocal by Newton's iteration r <- r + r (1 -
+// x r) from the single-precision reciprocal of x's significand (24, 48, 96 bits: within 1.5
+// units): four FP64 operations where a division takes about ten; the exponents move by
+// integer operations.  Zero and values whose reciprocal leaves the normal range divide.
+__device__ __forceinline__ double recip(double x) {
+  const int hi = __double2hiint(x), lo = __double2loint(x);
+  const int ex = (hi >> 20) & 0x7ff;
+  if (ex < 2 || ex > 2044) return 1.0 / x;
+  // float in [1, 2) from the leading 23 bits of the significand
+  const uint32_t fm = 0x3f800000u | (((uint32_t)hi & 0xfffffu) << 3) | ((uint32_t)lo >> 29);
+  const uint32_t fr = __float_as_uint(__frcp_rn(__uint_as_float(fm)));  // in (1/2, 1]
+  // widened, times 2^{1023 - ex}, with x's sign
+  const int fe = (int)(fr >> 23) - 127;  // -1 or 0
+  const uint32_t rh = ((uint32_t)hi & 0x80000000u) | ((uint32_t)(1023 + fe + 1023 - ex) << 20) | ((fr & 0x7fffffu) >> 3);
+  double r = __hiloint2double((int)rh, (int)(fr << 29));
+  r = fma(r, fma(-x, r, 1.0), r);
+  return fma(r, fma(-x, r, 1.0), r);
+}
+// a / x with one correction of the quotient.
+__device__ __forceinline__ double quot(double a, double x) {
+  const double r = recip(x), q = a * r, t = fma(-q, x, a);
+  return isfinite(t) ? fma(r, t, q) : a / x;
 }
 
 // Secular roots, one warp per root.  With origin pole d_o and tau = lam - d_o the function
@@ -298,7 +441,7 @@ __global__ void dc_secular_kernel(DcArgs a, const DcNode* nodes, DevStatus* st) 
     const double gap = dK[j + 1] - dK[j];
     const double mid = 0.5 * gap;
     double f = 0.0;
-    for (int i = lane; i < K; i += 32) f += zK[i] * zK[i] / ((dK[i] - dK[j]) - mid);
+    for (int i = lane; i < K; i += 32) f = fma(zK[i] * zK[i], recip((dK[i] - dK[j]) - mid), f);
     f = 1.0 + rho2 * warp_sum(f);
     if (f >= 0.0) { o = j; lo = 0.0; hi = mid; }
     else { o = j + 1; lo = -mid; hi = 0.0; }
@@ -317,17 +460,15 @@ __global__ void dc_secular_kernel(DcArgs a, const DcNode* nodes, DevStatus* st) 
   double wref = hi - lo;  // bracket width two iterations ago: a step must halve it
   int it = 0;
   for (; it < 200; it++) {
-    double ps = 0.0, psd = 0.0, fs = 0.0, fsd = 0.0, absum = 0.0;
+    double ps = 0.0, psd = 0.0, fs = 0.0, fsd = 0.0;
+    // poles i <= j lie left of the root (terms negative), the others right of it
     for (int i = lane; i < K; i += 32) {
-      double den = (dK[i] - d0) - tau;
-      double t = zK[i] / den;
-      double term = zK[i] * t;          // z_i^2 / den
-      double dterm = t * t;             // z_i^2 / den^2
-      if (i <= j) { ps += term; psd += dterm; }
-      else { fs += term; fsd += dterm; }
-      absum += fabs(term);
+      const double t = zK[i] * recip((dK[i] - d0) - tau);
+      if (i <= j) { ps = fma(zK[i], t, ps); psd = fma(t, t, psd); }
+      else { fs = fma(zK[i], t, fs); fsd = fma(t, t, fsd); }
     }
-    ps = warp_sum(ps); psd = warp_sum(psd); fs = warp_sum(fs); fsd = warp_sum(fsd); absum = warp_sum(absum);
+    ps = warp_sum(ps); psd = warp_sum(psd); fs = warp_sum(fs); fsd = warp_sum(fsd);
+    const double absum = fabs(ps) + fabs(fs);
     const double f = 1.0 + rho2 * (ps + fs);
     if (f < 0.0) lo = tau; else hi = tau;
     if (fabs(f) <= 8.0 * DC_U * (1.0 + rho2 * absum)) break;
@@ -376,24 +517,27 @@ __global__ void dc_secular_kernel(DcArgs a, const DcNode* nodes, DevStatus* st) 
   }
 }
 
-// Gu-Eisenstat: z_hat_i^2 = (lam_i - d_i)/rho' * prod_{j != i} (lam_j - d_i)/(d_j - d_i).
+// Gu-Eisenstat: z_hat_i^2 = (lam_i - d_i)/rho' * prod_{j != i} (lam_j - d_i)/(d_j - d_i).  A
+// warp per entry: a thread per entry (39 CTAs at K = 4992) took 2.0 ms.
 __global__ void dc_zhat_kernel(DcArgs a, const DcNode* nodes) {
   const DcNode nd = nodes[blockIdx.y];
   const int z = blockIdx.z;
   DcWs w = item_ws(a, z);
   const int off = nd.off, s = off + nd.n1;
   const int K = w.cnt[3 * off];
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const int lane = threadIdx.x & 31, i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (i >= K) return;
   const double rho2 = 2.0 * fabs(a.e[z * a.sde + s - 1]);
   const double* dK = w.dK + off;
   const double di = dK[i];
-  double prod = ((dK[w.orig[off + i]] - di) + w.tauK[off + i]) / rho2;
-  for (int j = 0; j < K; j++) {
-    if (j == i) continue;
-    double lj = (dK[w.orig[off + j]] - di) + w.tauK[off + j];
-    prod *= lj / (dK[j] - di);
+  // a warp per entry, the factors over the lanes (each near 1 but for the nearest: no overflow)
+  double prod = 1.0;
+  for (int j = lane; j < K; j += 32) {
+    const double lj = (dK[w.orig[off + j]] - di) + w.tauK[off + j];
+    prod *= j == i ? lj / rho2 : quot(lj, dK[j] - di);
   }
+  for (int o = 16; o > 0; o >>= 1) prod *= __shfl_xor_sync(0xffffffffu, prod, o);
+  if (lane) return;
   double zh = sqrt(fabs(prod));
   w.zhat[off + i] = w.zK[off + i] < 0.0 ? -zh : zh;
 }
@@ -444,12 +588,12 @@ __global__ void dc_buildw_kernel(DcArgs a, const DcNode* nodes) {
     const double dj = dK[w.orig[off + j]], tj = w.tauK[off + j];
     double s2 = 0.0;
     for (int i = lane; i < K; i += 32) {
-      double v = w.zhat[off + i] / ((dK[i] - dj) - tj);
+      double v = w.zhat[off + i] * recip((dK[i] - dj) - tj);
       s2 += v * v;
     }
     s2 = warp_sum(s2);
     const double inv = 1.0 / sqrt(s2);
-    for (int i = lane; i < K; i += 32) col[w.idxK[off + i]] = w.zhat[off + i] / ((dK[i] - dj) - tj) * inv;
+    for (int i = lane; i < K; i += 32) col[w.idxK[off + i]] = w.zhat[off + i] * recip((dK[i] - dj) - tj) * inv;
   } else {
     if (lane == 0) col[w.idxD[off + (-1 - src)]] = 1.0;
   }
@@ -584,8 +728,8 @@ void dc_solve(DcPlan* p, double* d, double* e, long long sde, double* lam, doubl
   dc_tear_kernel<<<cnt, 256, 0, s>>>(d, e, sde, p->d_splits, (int)p->splits.size());
   const int nleaves = (int)p->leaves.size() / 2;
   count_launch();
-  dc_leaf_kernel<<<dim3((nleaves + 3) / 4, cnt), 128, 0, s>>>(d, e, sde, lamBuf[0], slam, zbuf0, sZ0, m,
-                                                              p->d_leaves, nleaves, st);
+  dc_leaf_kernel<<<dim3(nleaves, cnt), 32, 0, s>>>(d, e, sde, lamBuf[0], slam, zbuf0, sZ0, m, p->d_leaves, nleaves,
+                                                   st);
   prof->end(tok, PC_DC_LEAF, 0.0, 0.0);
   for (int t = 0; t < p->depth; t++) {
     DcLevel& L = p->levels[t];
@@ -604,12 +748,12 @@ void dc_solve(DcPlan* p, double* d, double* e, long long sde, double* lam, doubl
     a.sZ = in_is_Z ? sZ : slam;
     tok = prof->begin();
     count_launch();
-    dc_merge_prep_kernel<<<dim3(nn, cnt), 256, 0, s>>>(a, L.d_nodes);
+    dc_merge_prep_kernel<<<dim3(nn, cnt), 1024, 0, s>>>(a, L.d_nodes);
     dim3 g1((L.maxn + 127) / 128, nn, cnt);
     count_launch();
     dc_secular_kernel<<<dim3((L.maxn + 7) / 8, nn, cnt), 256, 0, s>>>(a, L.d_nodes, st);
     count_launch();
-    dc_zhat_kernel<<<g1, 128, 0, s>>>(a, L.d_nodes);
+    dc_zhat_kernel<<<dim3((L.maxn + 7) / 8, nn, cnt), 256, 0, s>>>(a, L.d_nodes);
     count_launch();
     dc_colmap_kernel<<<g1, 128, 0, s>>>(a, L.d_nodes);
     count_launch();
