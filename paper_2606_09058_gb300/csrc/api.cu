@@ -256,12 +256,23 @@ int pick_width(const gks_ctx* c, int m, int es, int nc) {
 // collinear class (same order and element type).
 int shape_spin(int spin) { return spin == GKS_NONCOLLINEAR ? 1 : 0; }
 
+// Reduction of the mixed path: single precision with two launches per step (1), or the
+// persistent digit form on an FP64 copy of H' (2), which is more accurate and, its steps being
+// shorter, faster until its traffic (14 bytes per complex entry against 4) outweighs them.
+// Measured per step (single precision / digits): real order 1404 35 / 15 us, 6000 55 / 32 us;
+// complex 1404 41 / 22 us, 4000 59 / 39 us, eight items of 1404 47 / 50 us.
+constexpr double kMixedDigitBytes = 2.4e8;
+int mixed_form(const gks_ctx* c, int m, int nk, int es) {
+  if (c->precision == GKS_FP64) return 0;
+  return (double)m * m * nk * es <= kMixedDigitBytes ? 2 : 1;
+}
+
 // Workspace for nk items of order m (element size es, n = basis per spin, nc = spin mode).
 gks_status ensure_ws(gks_ctx* c, int m, int n, int nk, int es, int nc) {
   const int want = pick_width(c, m, es, shape_spin(nc));
-  const int mixed = c->precision != GKS_FP64 ? 1 : 0;
+  const int mixed = mixed_form(c, m, nk, es);
   const int two = c->tridiag == GKS_TRIDIAG_TWO_STAGE ? c->band : 0;
-  const int dig = c->hemv == 0 && !mixed ? 1 : 0;
+  const int dig = (c->hemv == 0 && !mixed) || mixed == 2 ? 1 : 0;
   if (c->ws && c->m == m && c->n == n && c->nk == nk && c->es == es && c->nc == nc && c->nbb == want &&
       c->wsmixed == mixed && c->wstwo == two && c->wsdig == dig)
     return GKS_OK;
@@ -359,9 +370,9 @@ gks_status ensure_ws(gks_ctx* c, int m, int n, int nk, int es, int nc) {
     c->oY2w = a.take<char>(elems((long long)c->nblkmax * m * bb));
   }
   if (mixed) {
-    // single-precision copy of H' for the tridiagonalization, refinement products Y, T, R,
-    // the per-item norms, and the reordering buffers
-    c->oAf = a.take<char>(elems(c->sMM) / 2);
+    // copy of H' for the tridiagonalization (single precision, or FP64 for the digit form),
+    // refinement products Y, T, R, the per-item norms, and the reordering buffers
+    c->oAf = a.take<char>(elems(c->sMM) / (mixed == 2 ? 1 : 2));
     c->oRY = a.take<char>(elems(c->sMM));
     c->oRT = a.take<char>(elems(c->sMM));
     c->oRR = a.take<char>(elems(c->sMM));
@@ -1469,10 +1480,21 @@ gks_status solve_t(gks_ctx* c, const SolveKey& key) {
   const bool mixed = c->precision == GKS_MIXED_SPLITBF16;
   const bool two = !mixed && c->tridiag == GKS_TRIDIAG_TWO_STAGE;
   using TL = typename Low<T>::type;
+  const bool mixdig = mixed && c->wsmixed == 2;
   TL* Af = mixed ? at<TL>(c, c->oAf) : nullptr;
   {
     StageRec sr(c, PS_HETRD);
-    if (mixed) {
+    if (mixdig) {
+      // mixed precision, small orders: an FP64 copy of H' (H' stays in A for the refinement)
+      T* Ad = at<T>(c, c->oAf);
+      {
+        Rec r(c, PC_MISC);
+        copy2d<T>(Ad, M, c->sMM, A, M, c->sMM, M, M, items, s);
+      }
+      if (!hetrd_run<T>(c, Ad, M, items)) return refused();
+      Rec r(c, PC_HETRD_VEC);
+      hetrd_finish<T>(Ad, M, c->sMM, M, d, e, M, ph, M, items, s);
+    } else if (mixed) {
       // mixed precision: H' rounded to single precision and tridiagonalized on the FP32
       // pipe (FP64 H' stays in A for the refinement)
       {
@@ -1532,9 +1554,15 @@ gks_status solve_t(gks_ctx* c, const SolveKey& key) {
       q1_apply_run<T>(c, A, C, nev, sC, M, nev, items);
     } else if (mixed) {
       // single-precision reflectors, products on fewer digits (about FP32 accuracy)
-      const int sv = c->slices;
+      const int sv = c->slices, gm = c->gemm_mode;
       c->slices = std::min(sv, kLowSlices);
-      backtransform_run<T, TL>(c, Af, C, nev, sC, M, nev, items);
+      if (mixdig) {
+        if (gm == 0) c->gemm_mode = 2;  // about single precision at every order
+        backtransform_run<T>(c, at<T>(c, c->oAf), C, nev, sC, M, nev, items);
+      } else {
+        backtransform_run<T, TL>(c, Af, C, nev, sC, M, nev, items);
+      }
+      c->gemm_mode = gm;
       c->slices = sv;
     } else {
       backtransform_run<T>(c, A, C, nev, sC, M, nev, items);

@@ -67,7 +67,8 @@ void hetrd_digits(const T* A, int lda, long long sA, int n, const HemvDigits& hd
 // One panel of the digit form: steps jh .. jl.  Per item (strides in elements): arow 2 x sv,
 // part gs x 2 kPanelMax, y 2 kPanelMax, P panel_partials(m, gs), dot, nrm and mex gs each (gs:
 // CTAs per item at most), bar 4 counters zeroed once per reduction.  base, basev: arrivals at
-// the two barrier counters so far; a panel of s steps on G CTAs adds 2 s G and (s - 1) G
+// the two barrier counters so far; a panel of s steps on G CTAs adds 2 s G and (s - 1) G, or
+// twice the latter with early set
 // (none in the cluster form).
 constexpr int kPanelMax = 128;   // steps per panel at most
 constexpr int kPanelCtas = 160;  // CTAs per item at most
@@ -94,6 +95,7 @@ struct PanelArgs {
   int gs;
   unsigned* bar;
   unsigned base, basev;
+  int early;
   HemvDigits hd;
   DevStatus* st;
   long long wait;

@@ -627,11 +627,15 @@ __global__ void __launch_bounds__(256) hetrd_pupdate_kernel(T* A, int lda, long 
 //      multiply the CTA's share of the digit tiles (the R x C tiles of the block in row-tile
 //      order, cut into G equal runs, so every CTA streams the same bytes at any order) with
 //      v = conj(a) (the pivot replaced by upiv; u' = v / upiv is applied to the sums), whose
-//      digits each warp makes for the 16 columns it is about to use; warps 8-11 meanwhile
-//      store u' for the CTA's rows, form the rows' shares of Q^H u and U^H u, and after a
-//      barrier of their own add the shares of a few entries each over the CTAs.
-//   2. barrier; p from the runs that touch each row, q, row j-1 with the panel's updates, and
-//      the shares of its norm; barrier.
+//      digits each warp makes for the 16 columns it is about to use.  Warps 8-11 meanwhile
+//      store u' for the CTA's rows, form the rows' shares of y1 = Q^H u and y2 = U^H u and,
+//      after a barrier of their own, add the shares of a few entries each over the CTAs.
+//      Where the product is long enough to hide it (a.early) they also wait for y and form
+//      U y1 + Q y2 and row j-1 with the panel's earlier updates, which takes the panel's FP64
+//      work off the chain (order 4992: 44 -> 40 us per step; order 832: 13 -> 16 us, the
+//      product being shorter than that work).
+//   2. barrier; p from the runs that touch each row, those corrections unless done, q, row j-1
+//      with this step's update, and the shares of its norm; barrier.
 // The digit tiles of the next step do not depend on this one: their first copies are issued
 // before the barriers.  Partial sums are added in a fixed order: results do not depend on
 // timing.  Every wait is bounded (a.wait SM cycles): past it the status is set, an abort flag
@@ -665,9 +669,9 @@ template <int ID, int N>
 __device__ __forceinline__ void bar_named() {
   asm volatile("bar.sync %0, %1;\n" ::"n"(ID), "n"(N) : "memory");
 }
-// One thread per CTA: arrive on *cnt and wait for target arrivals; false on abort or timeout.
-__device__ __forceinline__ bool grid_arrive_wait(unsigned* cnt, unsigned target, unsigned* abortf, long long limit) {
-  red_release(cnt);
+// One thread per CTA (which has arrived on *cnt): wait for target arrivals; false on abort or
+// timeout.
+__device__ __forceinline__ bool grid_wait(unsigned* cnt, unsigned target, unsigned* abortf, long long limit) {
   const long long t0 = clock64();
   for (unsigned n = 1; (int)(ld_acquire(cnt) - target) < 0; n++) {
     if (n & 63u) continue;
@@ -795,8 +799,9 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
         if (lane < G) cluster_arrive(&s_bar[0], lane);
         if (lane == 0 && !cluster_wait(&s_bar[0], (arrived - 1) & 1u, a.wait)) s_abort = 1;
       }
-    } else if (tid == 0 && !grid_arrive_wait(bar, arrived, bar + 2, a.wait)) {
-      s_abort = 1;
+    } else if (tid == 0) {
+      red_release(bar);
+      if (!grid_wait(bar, arrived, bar + 2, a.wait)) s_abort = 1;
     }
     __syncthreads();
     return s_abort == 0;
@@ -814,6 +819,24 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
     cp_async_commit();
   };
 
+  // y and row j-1 of U and Q (their earlier steps) into shared memory, threads t of nt
+  int j = a.jh, k = 0;
+  auto load_panel_vectors = [&](int t, int nt) {
+    for (int s = t; s < k; s += nt) {
+      y1s[s] = ldcg(y + s);
+      y2s[s] = ldcg(y + k + s);
+      ujs[s] = ldcg(U + (size_t)(j - 1) * ldu + s);
+      qjs[s] = ldcg(Q + (size_t)(j - 1) * ldu + s);
+    }
+  };
+  // one earlier step's share of U y1 + Q y2 and of row j-1's updates
+  auto correct = [&](T& corr, T& rs, T u, T q, int s) {
+    mac(corr, u, y1s[s]);
+    mac(corr, q, y2s[s]);
+    mac(rs, ujs[s], conjg(q));
+    mac(rs, qjs[s], conjg(u));
+  };
+
   if (tid == 0) s_abort = 0;
   if (CL) {
     if (tid == 0) {
@@ -825,7 +848,6 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
     cluster_sync_all();
   }
   {
-    const int j = a.jh;
     T* ar = arow2 + (j & 1) * a.sv;
     double n2 = 0.0;
     int e = NOEXP;
@@ -848,8 +870,8 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
   }
   bool live = barrier();
 
-  for (int j = a.jh; j >= a.jl && live; j--) {
-    const int k = a.jh - j;
+  for (; j >= a.jl && live; j--) {
+    k = a.jh - j;
     const T* ar = arow2 + (j & 1) * a.sv;
     // the entry of a whose digits this lane makes for the warp's next tile: column lane & 15, Re
     // (lanes 0-15) or Im (lanes 16-31), loaded a tile ahead (the first one before the scalars)
@@ -1061,21 +1083,24 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
           }
         }
       }
+      // barrier of the vector warps over the item's CTAs
+      auto vbarrier = [&]() {
+        bar_named<2, 128>();
+        arrivedv += CL ? 1u : (unsigned)G;
+        if (CL) {
+          if (warp == 8 && lane < G) cluster_arrive(&s_bar[1], lane);
+          if (vt == 0 && !cluster_wait(&s_bar[1], (arrivedv - 1) & 1u, a.wait)) s_abort = 1;
+        } else if (vt == 0) {
+          red_release(bar + 1);
+          if (!grid_wait(bar + 1, arrivedv, bar + 2, a.wait)) s_abort = 1;
+        }
+        bar_named<2, 128>();
+      };
       if (k > 0) {
 #pragma unroll
         for (int h = 0; h < 2; h++)
           if (vt + 128 * h < 2 * k) part[(size_t)b * (2 * kPanelMax) + vt + 128 * h] = ya[h];
-        bar_named<2, 128>();
-        arrivedv += CL ? 1u : (unsigned)G;
-        if (CL) {
-          if (warp == 8) {
-            if (lane < G) cluster_arrive(&s_bar[1], lane);
-            if (lane == 0 && !cluster_wait(&s_bar[1], (arrivedv - 1) & 1u, a.wait)) s_abort = 1;
-          }
-        } else if (vt == 0 && !grid_arrive_wait(bar + 1, arrivedv, bar + 2, a.wait)) {
-          s_abort = 1;
-        }
-        bar_named<2, 128>();
+        vbarrier();
         // LG lanes per entry, 32 / LG entries per warp at a time
         const int LG = G > 16 ? 32 : G > 8 ? 16 : 8, per = 32 / LG, sub = lane / LG, sl = lane % LG;
         for (int e0 = (warp - 8) * per; b + G * e0 < 2 * k; e0 += 4 * per) {
@@ -1085,6 +1110,43 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
             for (int g = sl; g < G; g += LG) v += ldcg(part + (size_t)g * (2 * kPanelMax) + en);
           for (int o = LG >> 1; o > 0; o >>= 1) v += shfl_xor(v, o);
           if (sl == 0 && en < 2 * k) y[en] = v;
+        }
+      }
+      if (a.early) {
+        if (k > 0) {
+          vbarrier();
+          load_panel_vectors(vt, 128);
+          bar_named<2, 128>();
+        }
+        // groups of 8 lanes, one row each (16 rows at a time): U y1 + Q y2 into Q's new column
+        // (replaced by q below), row j-1 with the earlier updates into the next row's buffer
+        const int grp = vt >> 3, gl = vt & 7;
+        T* an = arow2 + ((j - 1) & 1) * a.sv;
+        for (int base = c0; base < ce; base += 16) {
+          const int c = base + grp;
+          T corr = zero<T>(), rs = zero<T>();
+          if (c < ce) {
+            const T* Uc = U + (size_t)c * ldu;
+            const T* Qc = Q + (size_t)c * ldu;
+            for (int s0 = gl; s0 < k; s0 += 32) {  // four steps' loads in flight
+              T u0[4], q0[4];
+#pragma unroll
+              for (int q = 0; q < 4; q++) {
+                const int sq = min(s0 + 8 * q, k - 1);
+                u0[q] = Uc[sq];
+                q0[q] = Qc[sq];
+              }
+#pragma unroll
+              for (int q = 0; q < 4; q++)
+                if (s0 + 8 * q < k) correct(corr, rs, u0[q], q0[q], s0 + 8 * q);
+            }
+          }
+          corr = group8_sum(corr);
+          rs = group8_sum(rs);
+          if (c < ce && gl == 0) {
+            Q[(size_t)c * ldu + k] = corr;
+            if (j > a.jl) an[c] = A[(size_t)(j - 1) * lda + c] - rs;
+          }
         }
       }
     }
@@ -1103,10 +1165,12 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
       }
       return v;
     };
-    // groups of 8 lanes of warps 0-9, one row each (40 rows at a time); the first rows' loads go
-    // out before y arrives
+    // groups of 8 lanes of warps 0-9, one row each (40 rows at a time); kq and row j-1's p on
+    // the other two warps; the first rows' loads go out before y arrives
     const int grp = tid >> 3, gl = tid & 7, ce = min(c1, j);
-    T pv0 = zero<T>(), uc0 = zero<T>(), aold0 = zero<T>(), u0[4], q0[4];
+    T* an = arow2 + ((j - 1) & 1) * a.sv;
+    const int ke = a.early ? 0 : k;  // steps of the corrections still to do
+    T pv0 = zero<T>(), u0[4], q0[4];
     double dsum = 0.0;
     if (grp < 40) {
       if (c0 + grp < ce) {
@@ -1114,13 +1178,9 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
         const T* Qc = Q + (size_t)(c0 + grp) * ldu;
 #pragma unroll
         for (int q = 0; q < 4; q++) {
-          const int sq = min(gl + 8 * q, k > 0 ? k - 1 : 0);
-          u0[q] = k > 0 ? Uc[sq] : zero<T>();
-          q0[q] = k > 0 ? Qc[sq] : zero<T>();
-        }
-        if (gl == 0) {
-          uc0 = ldcg(Uc + k);
-          if (rowupd) aold0 = A[(size_t)(j - 1) * lda + c0 + grp];
+          const int sq = max(min(gl + 8 * q, ke - 1), 0);
+          u0[q] = ke > 0 ? Uc[sq] : zero<T>();
+          q0[q] = ke > 0 ? Qc[sq] : zero<T>();
         }
         pv0 = p_of(c0 + grp, gl, 8);
       }
@@ -1129,53 +1189,44 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
     } else if (rowupd) {
       pv0 = p_of(j - 1, lane, 32);
     }
-    for (int s = tid; s < k; s += kPanelThreads) {
-      y1s[s] = ldcg(y + s);
-      y2s[s] = ldcg(y + k + s);
-      ujs[s] = ldcg(U + (size_t)(j - 1) * ldu + s);
-      qjs[s] = ldcg(Q + (size_t)(j - 1) * ldu + s);
-    }
+    if (!a.early) load_panel_vectors(tid, kPanelThreads);
     __syncthreads();
     if (warp == 10) {  // kq = (tau / 2) u^H p = (tau^2 / 2) (u^H p_raw - 2 Re y2^H y1)
-      double tot = dsum;
       for (int s = lane; s < k; s += 32) {
-        tot = fma(-2.0 * re(y2s[s]), re(y1s[s]), tot);
-        if constexpr (CPX) tot = fma(-2.0 * im(y2s[s]), im(y1s[s]), tot);
+        dsum = fma(-2.0 * re(y2s[s]), re(y1s[s]), dsum);
+        if constexpr (CPX) dsum = fma(-2.0 * im(y2s[s]), im(y1s[s]), dsum);
       }
-      tot = warp_sum(tot);
-      if (lane == 0) s_kq = (0.5 * t) * (t * tot);
+      dsum = warp_sum(dsum);
+      if (lane == 0) s_kq = (0.5 * t) * (t * dsum);
     } else if (warp == 11 && rowupd) {  // p[j-1] - U y1 - Q y2 of row j-1
-      T v = pv0, corr = zero<T>();
       for (int s = lane; s < k; s += 32) {
-        mac(corr, ujs[s], y1s[s]);
-        mac(corr, qjs[s], y2s[s]);
+        mac(pv0, -ujs[s], y1s[s]);
+        mac(pv0, -qjs[s], y2s[s]);
       }
-      v = warp_sum(v - corr);
-      if (lane == 0) s_pj = v;
+      pv0 = warp_sum(pv0);
+      if (lane == 0) s_pj = pv0;
     }
     double n2 = 0.0;
     int ex = NOEXP;
     bool synced = false;
-    T* an = arow2 + ((j - 1) & 1) * a.sv;
     for (int base = c0; base < ce || !synced; base += 40) {
       const int c = base + grp;
       const bool ok = c < ce && grp < 40;
-      T pv = pv0, rs = zero<T>(), uc = uc0, aold = aold0;
+      T pv = pv0, corr = zero<T>(), rs = zero<T>(), uc = zero<T>(), aold = zero<T>();
       if (ok) {
         const T* Uc = U + (size_t)c * ldu;
         const T* Qc = Q + (size_t)c * ldu;
-        if (synced) {
-          pv = p_of(c, gl, 8);
-          if (gl == 0) {
-            uc = ldcg(Uc + k);
-            if (rowupd) aold = A[(size_t)(j - 1) * lda + c];
-          }
+        if (synced) pv = p_of(c, gl, 8);
+        if (gl == 0) {
+          uc = ldcg(Uc + k);
+          if (a.early) corr = ldcg(Qc + k);
+          if (rowupd) aold = a.early ? ldcg(an + c) : A[(size_t)(j - 1) * lda + c];
         }
-        for (int s0 = gl; s0 < k; s0 += 32) {  // four steps' loads in flight
+        for (int s0 = gl; s0 < ke; s0 += 32) {  // four steps' loads in flight
           if (synced || s0 > gl) {
 #pragma unroll
             for (int q = 0; q < 4; q++) {
-              const int sq = min(s0 + 8 * q, k - 1);
+              const int sq = min(s0 + 8 * q, ke - 1);
               u0[q] = Uc[sq];
               q0[q] = Qc[sq];
             }
@@ -1183,20 +1234,13 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
 #pragma unroll
           for (int q = 0; q < 4; q++) {
             const int sq = s0 + 8 * q;
-            if (sq < k) {
-              mac(pv, -u0[q], y1s[sq]);
-              mac(pv, -q0[q], y2s[sq]);
-              if (rowupd) {
-                mac(rs, ujs[sq], conjg(q0[q]));
-                mac(rs, qjs[sq], conjg(u0[q]));
-              }
-            }
+            if (sq < ke) correct(corr, rs, u0[q], q0[q], sq);
           }
         }
       }
       if (grp < 40) {
-        pv = group8_sum(pv);
-        if (rowupd) rs = group8_sum(rs);
+        pv = group8_sum(pv - corr);
+        if (ke > 0 && rowupd) rs = group8_sum(rs);
       }
       if (!synced) {  // kq and row j-1's share
         __syncthreads();
@@ -1300,11 +1344,15 @@ static int panel_cluster_ctas(int jh, int items) {
 }
 
 template <typename T>
+constexpr int kEarlyTiles = sizeof(T) == 16 ? 30 : 150;
+template <typename T>
 bool hetrd_panel(PanelArgs<T> a, int items, unsigned* base, unsigned* basev, cudaStream_t s) {
   const int cl = std::min(panel_cluster_ctas<T>(a.jh, items), a.gs >= 16 ? 16 : a.gs >= 8 ? 8 : 0);
   const int G = cl > 0 ? cl : std::min(a.gs, hetrd_panel_ctas<T>(a.jh, items));
   int maxseg = (a.jh + 31) / 32 / G + 2;
   const int steps = a.jh - a.jl + 1;
+  // U y1 + Q y2 behind the product from kEarlyTiles tiles per CTA up
+  a.early = (long long)((a.jh + 31) / 32) * ((a.jh + 15) / 16) >= (long long)kEarlyTiles<T> * G;
   a.base = *base;
   a.basev = *basev;
   cudaLaunchConfig_t cfg{};
@@ -1323,7 +1371,7 @@ bool hetrd_panel(PanelArgs<T> a, int items, unsigned* base, unsigned* basev, cud
     return cudaLaunchKernelEx(&cfg, hetrd_panel_kernel<T, true>, a, maxseg) == cudaSuccess;
   }
   *base += 2u * steps * G;
-  *basev += (unsigned)(steps - 1) * G;
+  *basev += (a.early ? 2u : 1u) * (unsigned)(steps - 1) * G;
   cudaFuncSetAttribute(hetrd_panel_kernel<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, PanelSmem<T>::TOTAL);
   at.id = cudaLaunchAttributeCooperative;
   at.val.cooperative = 1;

@@ -242,7 +242,8 @@ __global__ void __launch_bounds__(256) oz_scale_kernel(const SplitPair<T> sp, in
 // items) over the padded planes.  The tile is staged through shared memory (read along the
 // contiguous direction), then its S digits or residues are written with lanes along k, two
 // positions (4 bytes) per lane: full 128-byte lines per plane and vector.  Padding vectors
-// and k beyond K (the item's, after kdev) get zeros, so the planes need no clearing.
+// and k beyond K (the item's, after kdev) up to the last k block read get zeros, so the
+// planes need no clearing.
 template <typename T, bool RES>
 __global__ void __launch_bounds__(256) oz_split_kernel(const SplitPair<T> sp, int K, int Kp, int S, int p, int nb2,
                                                        const int* kdev, const CrtWeights y) {
@@ -253,7 +254,10 @@ __global__ void __launch_bounds__(256) oz_split_kernel(const SplitPair<T> sp, in
   const SplitOp<T>& q = sp.o[second];
   const int v0 = ((int)blockIdx.x - (second ? sp.n0 : 0)) * 32, k0 = blockIdx.y * TK, z = blockIdx.z;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (kdev) K = min(K, max(0, kdev[z]));
+  if (kdev) {
+    K = min(K, max(0, kdev[z]));
+    if (k0 >= (K + TK - 1) / TK * TK) return;  // k blocks the product kernel does not read
+  }
   const T* X = q.X + item_off(z, q.sX, q.sX2, nb2);
   const double* kz = q.ksc ? q.ksc + z * q.sks : nullptr;
   const int* ex = q.ex + z * q.sE;
