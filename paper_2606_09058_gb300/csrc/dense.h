@@ -96,6 +96,7 @@ struct PanelArgs {
   unsigned* bar;
   unsigned base, basev;
   int early;
+  bool shared;  // other problems' reductions run beside this one
   HemvDigits hd;
   DevStatus* st;
   long long wait;
@@ -103,7 +104,7 @@ struct PanelArgs {
 // CTAs per item of the grid form for a panel of order jh on `items` items (0: not even one
 // per item fits).
 template <typename T>
-int hetrd_panel_ctas(int jh, int items);
+int hetrd_panel_ctas(int jh, int items, bool shared);
 // base and basev advance by the launch's arrivals.  False if the launch was refused (then
 // nothing ran).
 template <typename T>

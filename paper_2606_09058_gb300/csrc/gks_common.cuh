@@ -121,6 +121,25 @@ template <typename T> struct Low;
 template <> struct Low<double> { using type = float; };
 template <> struct Low<zc> { using type = cf; };
 
+// 1 / x for x in the normal range of a double's reciprocal by Newton's iteration r <- r + r (1 -
+// x r) from the single-precision reciprocal of x's significand (24, 48, 96 bits: within 1.5
+// units): four FP64 operations where a division takes about ten; the exponents move by
+// integer operations.  Zero and values whose reciprocal leaves the normal range divide.
+__device__ __forceinline__ double recip(double x) {
+  const int hi = __double2hiint(x), lo = __double2loint(x);
+  const int ex = (hi >> 20) & 0x7ff;
+  if (ex < 2 || ex > 2044) return 1.0 / x;
+  // float in [1, 2) from the leading 23 bits of the significand
+  const uint32_t fm = 0x3f800000u | (((uint32_t)hi & 0xfffffu) << 3) | ((uint32_t)lo >> 29);
+  const uint32_t fr = __float_as_uint(__frcp_rn(__uint_as_float(fm)));  // in (1/2, 1]
+  // widened, times 2^{1023 - ex}, with x's sign
+  const int fe = (int)(fr >> 23) - 127;  // -1 or 0
+  const uint32_t rh = ((uint32_t)hi & 0x80000000u) | ((uint32_t)(1023 + fe + 1023 - ex) << 20) | ((fr & 0x7fffffu) >> 3);
+  double r = __hiloint2double((int)rh, (int)(fr << 29));
+  r = fma(r, fma(-x, r, 1.0), r);
+  return fma(r, fma(-x, r, 1.0), r);
+}
+
 // ---- warp / block reductions ----
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll

@@ -886,7 +886,10 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
         rraw = rmax[c];
       }
     };
+    const int vt = tid - 256, ce = min(c1, j);
+    T apre = zero<T>();  // the vector warps' rows of a
     if (warp < 8) vfetch(t0 + warp);
+    else if (vt < 64 && c0 + vt < ce) apre = ldcg(ar + c0 + vt);
     if (warp == 0) {
       double tail = 0.0;
       int e = NOEXP;
@@ -901,7 +904,7 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
       // root and one division deep.  u = alpha + ph |a| at the pivot, tau = 1 + |alpha| / |a|.
       const double a2 = abs2(alpha), sq = sqrt(lane & 1 ? a2 : tail + a2);
       const double xn = __shfl_sync(0xffffffffu, sq, 0), aa = __shfl_sync(0xffffffffu, sq, 1);
-      const double rc = 1.0 / (lane == 0 ? aa : lane == 1 ? aa + xn : xn);
+      const double rc = recip(lane == 0 ? aa : lane == 1 ? aa + xn : xn);
       const double raa = __shfl_sync(0xffffffffu, rc, 0), rsum = __shfl_sync(0xffffffffu, rc, 1);
       const double rxn = __shfl_sync(0xffffffffu, rc, 2);
       if (lane == 0) {
@@ -1054,14 +1057,13 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
       }
     } else {
       // ---- u' for this CTA's rows, and their shares of Q^H u (entries 0..k-1) and U^H u
-      const int vt = tid - 256, ce = min(c1, j);
       T ya[2] = {zero<T>(), zero<T>()};
       for (int r0 = c0; r0 < ce; r0 += 64) {
         const int nr = min(64, ce - r0);
         bar_named<2, 128>();
         if (vt < nr) {
           const int c = r0 + vt;
-          const T av = ldcg(ar + c);
+          const T av = r0 == c0 ? apre : ldcg(ar + c);
           const T uv = c == j - 1 ? from_real<T>(1.0) : (refl ? conjg(av) * inv : zero<T>());
           s_us[vt] = uv;
           U[(size_t)c * ldu + k] = uv;
@@ -1076,7 +1078,8 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
           for (int r = 0; r < nr; r += 8) {  // eight rows' loads in flight
             T v[8];
 #pragma unroll
-            for (int q = 0; q < 8; q++) v[q] = r + q < nr ? src[(size_t)(r + q) * ldu] : zero<T>();
+            for (int q = 0; q < 8; q++)
+              v[q] = r + q < nr ? src[(size_t)(r + q) * ldu] : zero<T>();
 #pragma unroll
             for (int q = 0; q < 8; q++)
               if (r + q < nr) macc(ya[h], v[q], s_us[r + q]);
@@ -1167,7 +1170,7 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
     };
     // groups of 8 lanes of warps 0-9, one row each (40 rows at a time); kq and row j-1's p on
     // the other two warps; the first rows' loads go out before y arrives
-    const int grp = tid >> 3, gl = tid & 7, ce = min(c1, j);
+    const int grp = tid >> 3, gl = tid & 7;
     T* an = arow2 + ((j - 1) & 1) * a.sv;
     const int ke = a.early ? 0 : k;  // steps of the corrections still to do
     T pv0 = zero<T>(), u0[4], q0[4];
@@ -1276,9 +1279,14 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
   if (s_abort && tid == 0) set_status(a.st ? a.st + z : nullptr, ST_ETIMEOUT, -3);
 }
 
-// CTAs per item: as many as give each about kPanelTiles digit tiles, at most one per SM over
-// all items.
+// CTAs per item: as many as leave each at most kPanelTiles digit tiles and kPanelRows<T> rows
+// (the FP64 corrections of its rows cost an SM 1.2 us per 4 rows and 32 earlier steps, complex),
+// at most one per SM over all items.
 constexpr int kPanelTiles = 12;
+// With other problems' reductions on other streams (a batch): half the SMs at most.
+constexpr int kPanelShare = 76;
+template <typename T>
+constexpr int kPanelRows = sizeof(T) == 16 ? 4 : 8;
 template <typename T>
 static int panel_capacity() {
   static const int cap = [] {
@@ -1322,33 +1330,35 @@ static int panel_cluster() {
 }
 
 template <typename T>
-int hetrd_panel_ctas(int jh, int items) {
-  const int top = std::min(panel_capacity<T>() / items, kPanelCtas);
+int hetrd_panel_ctas(int jh, int items, bool shared) {
+  const int cap = shared ? std::min(panel_capacity<T>(), kPanelShare) : panel_capacity<T>();
+  const int top = std::min(cap / items, kPanelCtas);
   const long long tiles = (long long)((jh + 31) / 32) * ((jh + 15) / 16);
-  return (int)std::min<long long>(top, (tiles + kPanelTiles - 1) / kPanelTiles);
+  return (int)std::min<long long>(
+      top, std::max<long long>((tiles + kPanelTiles - 1) / kPanelTiles, (jh + kPanelRows<T> - 1) / kPanelRows<T>));
 }
 
-// The cluster form (one cluster of up to 16 CTAs per item, barriers through shared-memory
-// mbarriers, no co-residency of the whole grid needed, so that several streams' reductions
-// run side by side) up to kClusterTiles digit tiles per item, or where the grid form cannot
-// give every item a CTA.
+// The cluster form: one cluster of up to 16 CTAs per item, barriers through shared-memory
+// mbarriers, no co-residency of the whole grid needed.  For a problem of its own it pays at
+// the smallest orders only (16 SMs do the FP64 corrections: order 640 real 20 us per step
+// against 12.7 us on 80 CTAs), beside other streams' reductions up to 1000 digit tiles (eight
+// uneven systems of order 208 to 1144: 61 ms with whole-GPU grids, 52 ms on half the SMs, 37
+// ms with clusters below 1000 tiles), and where the grid form cannot give every item a CTA.
 template <typename T>
-static int panel_cluster_ctas(int jh, int items) {
-  constexpr long long kClusterTiles = sizeof(T) == 16 ? 400 : 1000;
+static int panel_cluster_ctas(int jh, int items, bool shared) {
+  const long long kClusterTiles = shared ? 1000 : 64;
   const int c = panel_cluster<T>();
   const long long tiles = (long long)((jh + 31) / 32) * ((jh + 15) / 16);
-  if (c == 0 || (tiles > kClusterTiles && hetrd_panel_ctas<T>(jh, items) >= 1)) return 0;
-  int g = c;
-  while (g > 2 && tiles <= 4 * g) g >>= 1;
-  return g;
+  if (c == 0 || (tiles > kClusterTiles && hetrd_panel_ctas<T>(jh, items, shared) >= 1)) return 0;
+  return c;
 }
 
 template <typename T>
 constexpr int kEarlyTiles = sizeof(T) == 16 ? 30 : 150;
 template <typename T>
 bool hetrd_panel(PanelArgs<T> a, int items, unsigned* base, unsigned* basev, cudaStream_t s) {
-  const int cl = std::min(panel_cluster_ctas<T>(a.jh, items), a.gs >= 16 ? 16 : a.gs >= 8 ? 8 : 0);
-  const int G = cl > 0 ? cl : std::min(a.gs, hetrd_panel_ctas<T>(a.jh, items));
+  const int cl = std::min(panel_cluster_ctas<T>(a.jh, items, a.shared), a.gs >= 16 ? 16 : a.gs >= 8 ? 8 : 0);
+  const int G = cl > 0 ? cl : std::min(a.gs, hetrd_panel_ctas<T>(a.jh, items, a.shared));
   int maxseg = (a.jh + 31) / 32 / G + 2;
   const int steps = a.jh - a.jl + 1;
   // U y1 + Q y2 behind the product from kEarlyTiles tiles per CTA up
@@ -1568,7 +1578,7 @@ void narrow_lower(const T* A, int lda, long long sA, TL* B, int ldb, long long s
   template void gather_reflectors<T, T>(const T*, int, long long, const double*, long long, int, int, T*,    \
                                         int, long long, double*, long long, int, cudaStream_t);               \
   template void hetrd_digits<T>(const T*, int, long long, int, const HemvDigits&, int, cudaStream_t);           \
-  template int hetrd_panel_ctas<T>(int, int);                                                              \
+  template int hetrd_panel_ctas<T>(int, int, bool);                                                              \
   template bool hetrd_panel<T>(PanelArgs<T>, int, unsigned*, unsigned*, cudaStream_t);
 INST(double)
 INST(zc)
