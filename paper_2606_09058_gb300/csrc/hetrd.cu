@@ -778,7 +778,9 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
     }
     __syncthreads();
     if (warp == 0) {
-      const double t = warp_sum(lane < 12 ? s_red[lane] : 0.0);
+      double t = lane < 12 ? s_red[lane] : 0.0;
+#pragma unroll
+      for (int o = 8; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
       const int m = __reduce_max_sync(0xffffffffu, lane < 12 ? s_rede[lane] : NOEXP);
       if (lane == 0) {
         nrm[b] = t;
@@ -786,9 +788,9 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
       }
     }
   };
-  auto scale_of = [&](T v, int i) -> int {
+  auto scale_of = [&](T v, int d) -> int {  // d: the entry's equilibration exponent
     const unsigned long long mb = maxbits(v);
-    return mb ? bscale(mb) + deq(rmax[i]) : NOEXP;
+    return mb ? bscale(mb) + d : NOEXP;
   };
   // full barrier over the item's CTAs; false once any wait expired (uniform over the CTA)
   auto barrier = [&]() -> bool {
@@ -856,7 +858,7 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
       ar[c] = v;
       if (c < j - 1) {
         n2 += abs2(v);
-        e = max(e, scale_of(v, c));
+        e = max(e, scale_of(v, deq(rmax[c])));
       }
     }
     __syncthreads();
@@ -894,6 +896,7 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
       double tail = 0.0;
       int e = NOEXP;
       const T alpha = conjg(ldcg(ar + j - 1));
+      const int dpiv = deq(rmax[j - 1]);
       for (int g = lane; g < G; g += 32) {
         tail += __ldcg(nrm + g);
         e = max(e, __ldcg(mex + g));
@@ -913,7 +916,7 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
           s_inv = s_upiv = from_real<T>(1.0);
           s_sub = conjg(alpha);
           s_tau = 0.0;
-          e = scale_of(from_real<T>(1.0), j - 1);
+          e = scale_of(from_real<T>(1.0), dpiv);
         } else {
           const T ph = aa > 0.0 ? alpha * raa : from_real<T>(1.0);
           const T upiv = ph * (aa + xn);
@@ -922,7 +925,7 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
           s_inv = conjg(ph) * rsum;
           s_sub = conjg(ph) * (-xn);  // lower-storage sub-diagonal
           s_tau = (aa + xn) * rxn;
-          e = max(e, scale_of(upiv, j - 1));
+          e = max(e, scale_of(upiv, dpiv));
         }
         s_fu = e;
         if (b == 0) tau[j] = s_tau;
@@ -1057,7 +1060,7 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
       }
     } else {
       // ---- u' for this CTA's rows, and their shares of Q^H u (entries 0..k-1) and U^H u
-      T ya[2] = {zero<T>(), zero<T>()};
+      T ya[2] = {zero<T>(), zero<T>()}, yb[2] = {zero<T>(), zero<T>()};  // even and odd rows
       for (int r0 = c0; r0 < ce; r0 += 64) {
         const int nr = min(64, ce - r0);
         bar_named<2, 128>();
@@ -1082,7 +1085,7 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
               v[q] = r + q < nr ? src[(size_t)(r + q) * ldu] : zero<T>();
 #pragma unroll
             for (int q = 0; q < 8; q++)
-              if (r + q < nr) macc(ya[h], v[q], s_us[r + q]);
+              if (r + q < nr) macc(q & 1 ? yb[h] : ya[h], v[q], s_us[r + q]);
           }
         }
       }
@@ -1102,7 +1105,7 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
       if (k > 0) {
 #pragma unroll
         for (int h = 0; h < 2; h++)
-          if (vt + 128 * h < 2 * k) part[(size_t)b * (2 * kPanelMax) + vt + 128 * h] = ya[h];
+          if (vt + 128 * h < 2 * k) part[(size_t)b * (2 * kPanelMax) + vt + 128 * h] = ya[h] + yb[h];
         vbarrier();
         // LG lanes per entry, 32 / LG entries per warp at a time
         const int LG = G > 16 ? 32 : G > 8 ? 16 : 8, per = 32 / LG, sub = lane / LG, sl = lane % LG;
@@ -1153,16 +1156,29 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
         }
       }
     }
+    // where the partial products of this lane's first row of the next part lie (the integer
+    // divisions before the barrier)
+    const int grp = tid >> 3, gl = tid & 7;
+    const int prow = grp < 40 ? c0 + grp : j - 1, pl = grp < 40 ? gl : lane, pn = grp < 40 ? 8 : 32;
+    int pb0 = 0, pb1 = -1, pg0 = 0, pg1 = 0;
+    if (grp < 40 ? prow < ce : warp == 11) {
+      pb0 = pr.owner((prow >> 5) * pr.C) + pl;
+      pb1 = pr.owner(((prow >> 5) + 1) * pr.C - 1);
+      if (pb0 <= pb1) {
+        pg0 = pr.run0(pb0);
+        pg1 = pr.run0(pb0 + 1);
+        pg0 = pg0 < pg1 ? (prow >> 5) - pg0 / (int)pr.C : -1;  // the run's segment, -1: empty run
+      }
+    }
     if (!barrier()) break;
 
     // ---- p, q, and row j-1 with the panel's updates
     const bool rowupd = j > a.jl;
     const double t = s_tau;
-    auto p_of = [&](int row, int l, int nl) -> T {  // lanes l of nl: their share of p_raw[row]
+    auto p_from = [&](int row, int g, int b1, int nl) -> T {  // runs g, g + nl .. b1 of the row
       const int r = row >> 5;
-      const int b0 = pr.owner(r * pr.C), b1 = pr.owner((r + 1) * pr.C - 1);
       T v = zero<T>();
-      for (int g = b0 + l; g <= b1; g += nl) {
+      for (; g <= b1; g += nl) {
         const int g0 = pr.run0(g);
         if (g0 < pr.run0(g + 1)) v += ldcg(P + ((size_t)g * maxseg + (r - g0 / (int)pr.C)) * 32 + (row & 31));
       }
@@ -1170,7 +1186,6 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
     };
     // groups of 8 lanes of warps 0-9, one row each (40 rows at a time); kq and row j-1's p on
     // the other two warps; the first rows' loads go out before y arrives
-    const int grp = tid >> 3, gl = tid & 7;
     T* an = arow2 + ((j - 1) & 1) * a.sv;
     const int ke = a.early ? 0 : k;  // steps of the corrections still to do
     T pv0 = zero<T>(), u0[4], q0[4];
@@ -1185,12 +1200,13 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
           u0[q] = ke > 0 ? Uc[sq] : zero<T>();
           q0[q] = ke > 0 ? Qc[sq] : zero<T>();
         }
-        pv0 = p_of(c0 + grp, gl, 8);
       }
     } else if (warp == 10) {
       for (int g = lane; g < G; g += 32) dsum += __ldcg(dot + g);
-    } else if (rowupd) {
-      pv0 = p_of(j - 1, lane, 32);
+    }
+    if (pb0 <= pb1) {
+      if (pg0 >= 0) pv0 = ldcg(P + ((size_t)pb0 * maxseg + pg0) * 32 + (prow & 31));
+      if (pb0 + pn <= pb1) pv0 += p_from(prow, pb0 + pn, pb1, pn);
     }
     if (!a.early) load_panel_vectors(tid, kPanelThreads);
     __syncthreads();
@@ -1216,14 +1232,18 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
       const int c = base + grp;
       const bool ok = c < ce && grp < 40;
       T pv = pv0, corr = zero<T>(), rs = zero<T>(), uc = zero<T>(), aold = zero<T>();
+      int dc = 0;
       if (ok) {
         const T* Uc = U + (size_t)c * ldu;
         const T* Qc = Q + (size_t)c * ldu;
-        if (synced) pv = p_of(c, gl, 8);
+        if (synced) pv = p_from(c, pr.owner((c >> 5) * pr.C) + gl, pr.owner(((c >> 5) + 1) * pr.C - 1), 8);
         if (gl == 0) {
           uc = ldcg(Uc + k);
           if (a.early) corr = ldcg(Qc + k);
-          if (rowupd) aold = a.early ? ldcg(an + c) : A[(size_t)(j - 1) * lda + c];
+          if (rowupd) {
+            aold = a.early ? ldcg(an + c) : A[(size_t)(j - 1) * lda + c];
+            dc = deq(rmax[c]);
+          }
         }
         for (int s0 = gl; s0 < ke; s0 += 32) {  // four steps' loads in flight
           if (synced || s0 > gl) {
@@ -1264,7 +1284,7 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
             an[c] = an_c;
             if (c < j - 2) {
               n2 += abs2(an_c);
-              ex = max(ex, scale_of(an_c, c));
+              ex = max(ex, scale_of(an_c, dc));
             }
           }
         }

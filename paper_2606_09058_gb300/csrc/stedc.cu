@@ -402,9 +402,10 @@ __device__ __forceinline__ double quot(double a, double x) {
 // part by one pole plus a constant matched in value and slope,
 //   psi ~ p + q/(delta_j - tau),  phi ~ s + t/(delta_{j+1} - tau),
 // and takes the root of the model (a quadratic in u = delta_j - tau) when it falls inside
-// the current sign bracket; otherwise it bisects, and it also bisects whenever two steps
-// failed to halve the bracket.  Stops when f is below its rounding level or the bracket
-// is at the working precision of tau.
+// the current sign bracket and the step is at most half the one before last; otherwise it
+// bisects.  (Asking two steps to halve the bracket instead sends a one-sided convergence back
+// to the middle every second time: half the roots took 20 iterations.)  Stops when f is below
+// its rounding level or the bracket is at the working precision of tau.
 __global__ void dc_secular_kernel(DcArgs a, const DcNode* nodes, DevStatus* st) {
   const DcNode nd = nodes[blockIdx.y];
   const int z = blockIdx.z;
@@ -439,7 +440,7 @@ __global__ void dc_secular_kernel(DcArgs a, const DcNode* nodes, DevStatus* st) 
   const bool last = (j == K - 1);
   const double dr = last ? 0.0 : dK[j + 1] - d0;
   double tau = 0.5 * (lo + hi);
-  double wref = hi - lo;  // bracket width two iterations ago: a step must halve it
+  double s1 = hi - lo, s2 = hi - lo;  // the last step and the one before: a step must halve the latter
   int it = 0;
   for (; it < 200; it++) {
     double ps = 0.0, psd = 0.0, fs = 0.0, fsd = 0.0;
@@ -483,12 +484,10 @@ __global__ void dc_secular_kernel(DcArgs a, const DcNode* nodes, DevStatus* st) 
       }
       cand = dl - u;
     }
-    if ((it & 1) == 1) {
-      if (hi - lo > 0.5 * wref) cand = 0.5 * (lo + hi);  // slow one-sided progress: bisect
-      wref = hi - lo;
-    }
-    if (!(cand > lo && cand < hi)) cand = 0.5 * (lo + hi);
+    if (!(cand > lo && cand < hi) || fabs(cand - tau) > 0.5 * s2) cand = 0.5 * (lo + hi);
     if (cand == tau) break;
+    s2 = s1;
+    s1 = fabs(cand - tau);
     tau = cand;
   }
   if (it >= 200 && lane == 0) set_status(st ? st + z : nullptr, ST_ENOCONV, off + j);
