@@ -947,9 +947,13 @@ void panel_deferred(gks_ctx* c, T* A, int M, int n, int kp, int nk) {
   gmx<T>(c, nk, OP_N, OP_C, n, n, kp, -1.0, Q, ldu, c->sU, U, ldu, c->sU, 1.0, A, M, c->sMM, 1);
 }
 
-// Steps per panel: at most 128 (the per-step corrections grow with the panel length, the
-// deferred update runs fine at K = 128); small orders are latency-bound per step (64).
-int panel_width(const gks_ctx* c, int M) { return M < 2048 ? std::min(NB, c->nbb) : std::min(kPanelMax, c->nbb); }
+// Steps per panel.  The per-step FP64 corrections grow with the panel length, the digits and
+// the deferred update come once per panel.  Reductions in ms at 64 / 96 / 128 steps: complex
+// 1625 (four items) 55.3 / 60.3 / 64.4, 2496 63.2 / 65.3 / 68.3, 4992 242.8 / 237.2 / 238.9; real
+// 832 10.8 / 11.1 / 11.7, 2808 49.9 / 49.6 / 50.2.
+int panel_width(const gks_ctx* c, int M) {
+  return std::min(M < 3072 ? 64 : M < 6144 ? 96 : kPanelMax, c->nbb);
+}
 
 // One-stage Householder tridiagonalization with the digit form of the matrix-vector step:
 // per panel the digits of the stale block, one persistent launch for its steps, and the

@@ -1374,7 +1374,7 @@ static int panel_cluster_ctas(int jh, int items, bool shared) {
 }
 
 template <typename T>
-constexpr int kEarlyTiles = sizeof(T) == 16 ? 30 : 150;
+constexpr int kEarlyTiles = sizeof(T) == 16 ? 60 : 150;
 template <typename T>
 bool hetrd_panel(PanelArgs<T> a, int items, unsigned* base, unsigned* basev, cudaStream_t s) {
   const int cl = std::min(panel_cluster_ctas<T>(a.jh, items, a.shared), a.gs >= 16 ? 16 : a.gs >= 8 ? 8 : 0);
