@@ -557,23 +557,24 @@ int oz_reserve(gks_ctx* c, size_t item, int count) {
   return per;
 }
 
-// Split products from kSplitFlops flops (all items of the launch together) and 32 in every
-// dimension up: below, the FP64 kernel at 1 TFLOP/s is under the fixed cost of a split product
-// (three or four launches).  Measured (FP64 kernel / split product): real 832 x 256 x 64 (2.7e7
-// flops) 35 / 39 us, 832 x 832 x 64 95 / 52 us, 2500 x 64 x 64 29 / 42 us; complex 256 x 256 x
-// 64 (3.4e7) 42 / 38 us, 832 x 832 x 256 1335 / 94 us.
-constexpr double kSplitFlops = 3e7;
-bool split_worth(gks_ctx* c, int count, int M, int N, int K, int es, double fl) {
+// Split products where the FP64 kernel would take longer than their fixed cost (three or four
+// launches, about 30 us) and every dimension is at least 32.  The FP64 kernel's 16 x 16 tiles
+// take 0.073 us (complex 0.294) per inner index on their SM, whatever shares the other SMs.
+// Measured (FP64 kernel / split product): real 832 x 256 x 64 35 / 39 us, 832 x 832 x 64 95 / 52
+// us, 2500 x 64 x 64 29 / 42 us; complex 256 x 256 x 64 42 / 38 us, 192 x 64 x 192 64 / 38 us.
+constexpr double kSplitUs = 32.0;
+bool split_worth(gks_ctx* c, int count, int M, int N, int K, int es, int lower) {
   if (c->gemm_mode == 2) return true;
-  const int Ne = es == 16 ? 2 * N : N;  // embedded output columns
-  return c->gemm_mode == 0 && fl >= kSplitFlops && M >= 32 && Ne >= 32 && K >= 32;
+  if (c->gemm_mode != 0 || M < 32 || (es == 16 ? 2 * N : N) < 32 || K < 32) return false;
+  const long long tiles = (long long)((M + 15) / 16) * ((N + 15) / 16) * count / (lower ? 2 : 1);
+  return (double)((tiles + 151) / 152) * K * (es == 16 ? 0.294 : 0.073) >= kSplitUs;
 }
 
 // Smallest half of a merge whose products (half x 2 half x half, `items` of them per launch) are
-// split products: kSplitFlops again.
+// split products: 3e7 flops (a level's other merges fill the GPU on the FP64 kernel).
 int merge_half(int items) {
   int h = 64;
-  while (4.0 * h * h * h * items < kSplitFlops) h += 16;
+  while (4.0 * h * h * h * items < 3e7) h += 16;
   return h;
 }
 
@@ -588,7 +589,7 @@ void gmx(gks_ctx* c, int count, int opA, int opB, int M, int N, int K, double al
   } else {
   const int es = sizeof(T);
   const double fl = gemm_flops(es, M, N, K, lower, count);
-  const int per = split_worth(c, count, M, N, K, es, fl)
+  const int per = split_worth(c, count, M, N, K, es, lower)
                       ? oz_reserve(c, ozaki_workspace_bytes(M, N, K, es == 16, sform(c)), count)
                       : 0;
   if (per == 0) {
@@ -641,7 +642,7 @@ void gmx2(gks_ctx* c, int count, int nb2, int opA, int opB, int M, int N, int K,
     gemm<T>(g, M, N, c->stream);
     c->prof.end(tok, PC_GEMM, gemm_flops(es, M, N, K, 0, cnt), gemm_bytes(es, M, N, K, 0, cnt, beta != 0.0));
   };
-  const int per = (count % nb2 == 0 && split_worth(c, count, M, N, K, es, fl))
+  const int per = (count % nb2 == 0 && split_worth(c, count, M, N, K, es, 0))
                       ? oz_reserve(c, ozaki_workspace_bytes(M, N, K, es == 16, sform(c)), count)
                       : 0;
   if (per == 0) {
@@ -675,13 +676,13 @@ void gmx2(gks_ctx* c, int count, int nb2, int opA, int opB, int M, int N, int K,
 // lower triangle.  C_k is M x (>= n_rho) with leading dimension ldc and item stride sC;
 // rho_k is M x M (stride sR).  Split products take K = the columns of C with the device
 // count cutting the digits and the k loop; the FP64 kernel reads the same count.  The
-// dispatch takes the flops of a full product of this order: rho then runs on the same kernel
+// dispatch asks for a full product of this order: rho then runs on the same kernel
 // as the adjoint's products C B C^H of the same order, which users subtract from it.
 template <typename T>
 void rho_run(gks_ctx* c, const T* C, int ldc, long long sC, T* rho, long long sR, const double* ks, long long sks,
              const int* nrho, int M, int K, int nk) {
   const int es = sizeof(T);
-  const int per = split_worth(c, nk, M, M, K, es, gemm_flops(es, M, M, K, 0, nk))
+  const int per = split_worth(c, nk, M, M, K, es, 0)
                       ? oz_reserve(c, ozaki_workspace_bytes(M, M, K, es == 16, sform(c)), nk)
                       : 0;
   int z0 = 0;
@@ -1401,7 +1402,7 @@ gks_status solve_t(gks_ctx* c, const SolveKey& key) {
   cudaStream_t s = c->stream;
   // the scratch of the largest split product (the density matrix) at once: growing it product
   // by product would wait for the stream each time
-  if (split_worth(c, items, M, M, nev, es, gemm_flops(es, M, M, nev, 0, items)))
+  if (split_worth(c, items, M, M, nev, es, 0))
     oz_reserve(c, ozaki_workspace_bytes(M, M, nev, es == 16, sform(c)), items);
   double* eps = static_cast<double*>(const_cast<void*>(key.eps));
   T* C = static_cast<T*>(const_cast<void*>(key.C));
@@ -1618,7 +1619,7 @@ gks_status solve_t(gks_ctx* c, const SolveKey& key) {
     StageRec sr(c, PS_RHO);
     T* rho = static_cast<T*>(const_cast<void*>(key.rho));
     {
-      const bool split = split_worth(c, items, M, M, nev, es, gemm_flops(es, M, M, nev, 0, items));
+      const bool split = split_worth(c, items, M, M, nev, es, 0);
       Rec r(c, split ? PC_OZAKI : PC_GEMM, -1.0, -1.0);  // flops resolved from n_rho when the profile is read
       c->prof.nrho_dev = nrho;
       c->prof.rho_m = M;

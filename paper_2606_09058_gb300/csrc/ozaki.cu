@@ -649,7 +649,8 @@ constexpr int STAGES = 4;
 constexpr int B_BYTES = BN * tcg::BK * 2;
 constexpr int STAGE_BYTES = tcg::TILE_BYTES + B_BYTES;
 constexpr int TMEM_COLS = 2 * BN;
-constexpr int SMEM = STAGES * STAGE_BYTES + 1024;
+constexpr int OUT_BYTES = 32 * 128;  // an epilogue warp's 32 rows x 128 residues
+constexpr int SMEM = STAGES * STAGE_BYTES + tcg::EPI_WARPS * OUT_BYTES + 1024;
 constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) |
                            ((uint32_t)(tcg::BM >> 4) << 24);
 static_assert(SMEM <= 227 * 1024, "shared memory of the residue kernel");
@@ -788,12 +789,26 @@ __global__ void __launch_bounds__(tcg::THREADS, 1)
     // epilogue: warp w owns TMEM lanes 32 (w % 4) .. +31 (tile rows) and column half
     // (w - 2) / 4 (128 columns)
     const int lq = warp & 3, ch = (warp - 2) >> 2;
-    const int i = m0 + lq * 32 + lane;
+    uint4* out = reinterpret_cast<uint4*>(ring + (size_t)STAGES * STAGE_BYTES + (warp - 2) * crtc::OUT_BYTES);
+    auto flush = [&](int l) {
+      __syncwarp();
+      uint8_t* dst = a.R + z * a.zR + ((size_t)l * a.Mp + m0 + lq * 32) * a.Np + n0 + ch * 128;
+#pragma unroll
+      for (int q = 0; q < 8; q++) {
+        const int r = 4 * q + (lane >> 3), w = lane & 7;
+        __stcs(reinterpret_cast<uint4*>(dst + (size_t)r * a.Np + 16 * w), out[r * 8 + (w ^ (r & 7))]);
+      }
+      __syncwarp();
+    };
     int u = 0;
     bool ok = true;
     for (int l = l0; l < l1 && ok; l++) {
       const float mf = (float)crt_mod(l), inv = __frcp_rn(mf);
-      uint4* dst = reinterpret_cast<uint4*>(a.R + z * a.zR + ((size_t)l * a.Mp + i) * a.Np + n0 + ch * 128);
+      // the thread's row of residues goes to shared memory in 16-byte words (word w of row r at
+      // w ^ (r & 7): distinct banks), and from there in full 128-byte lines, 4 rows per warp store
+      auto put = [&](int word, uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3) {
+        out[lane * 8 + (word ^ (lane & 7))] = make_uint4(w0, w1, w2, w3);
+      };
       if (nchunk == 1) {  // K' <= 1024: every accumulator folds straight to its bytes
         const int b = u & 1;
         const uint32_t uph = (uint32_t)((u >> 1) & 1);
@@ -819,9 +834,10 @@ __global__ void __launch_bounds__(tcg::THREADS, 1)
             w[t] = crt_bytes(crt_fold(__uint_as_float(v[4 * t]), mf, inv), crt_fold(__uint_as_float(v[4 * t + 1]), mf, inv),
                              crt_fold(__uint_as_float(v[4 * t + 2]), mf, inv),
                              crt_fold(__uint_as_float(v[4 * t + 3]), mf, inv));
-          dst[2 * g] = make_uint4(w[0], w[1], w[2], w[3]);
-          dst[2 * g + 1] = make_uint4(w[4], w[5], w[6], w[7]);
+          put(2 * g, w[0], w[1], w[2], w[3]);
+          put(2 * g + 1, w[4], w[5], w[6], w[7]);
         }
+        flush(l);
         continue;
       }
       float acc[128];
@@ -857,8 +873,9 @@ __global__ void __launch_bounds__(tcg::THREADS, 1)
           w[t] = crt_bytes(crt_fold(x[0], mf, inv), crt_fold(x[1], mf, inv), crt_fold(x[2], mf, inv),
                            crt_fold(x[3], mf, inv));
         }
-        dst[q] = make_uint4(w[0], w[1], w[2], w[3]);
+        put(q, w[0], w[1], w[2], w[3]);
       }
+      flush(l);
     }
   }
   tc_fence_before();
