@@ -28,15 +28,16 @@ __device__ __forceinline__ zc shfl8<zc>(zc v, int src) {
 __device__ __forceinline__ double shfl32(double v, int src) { return __shfl_sync(0xffffffffu, v, src); }
 __device__ __forceinline__ zc shfl32(zc v, int src) { return zc{shfl32(v.x, src), shfl32(v.y, src)}; }
 
-// Diagonal blocks (64 x 64) on a cluster of kDiagC CTAs, in sub-blocks of kSub columns.  One
-// SM does 1.7 FP64 multiply-adds per clock: the 64^3 operations of a complex two-sided
-// reduction alone keep it busy for 0.3 ms, so the panel rows and the trailing updates are
-// spread over the cluster (data in global memory, L2 reads), with two cluster barriers per
-// sub-block; the 8 x 8 diagonal parts, a serial chain, are done by every CTA for itself.
-// Measured, one complex block: two-sided reduction 794 us on one CTA, column by column;
-// Cholesky 207 us.  See the launchers for the times of this form.
-constexpr int kDiagC = 8, kSub = 8, kDiagThreads = 256;
-__device__ __forceinline__ void diag_bar() { asm volatile("bar.sync 1, 64;\n" ::: "memory"); }
+// Diagonal blocks (64 x 64) on a cluster of kDiagC CTAs, in sub-blocks (32 columns of the
+// Cholesky factorization, 8 of the two-sided reduction).  One SM does 1.7 FP64 multiply-adds
+// per clock: the 64^3 operations of a complex two-sided reduction alone keep it busy for 0.3
+// ms, so the panel rows and the trailing updates are spread over the cluster (data in global
+// memory, L2 reads), with two cluster barriers per sub-block; the diagonal parts, a serial
+// chain of 67-clock operations, are done by every CTA for itself.
+// Measured, one block (complex / real): two-sided reduction 794 / 265 us on one CTA column by
+// column, 175 / 91 us here (190 / 90 with sub-blocks of 16); Cholesky 207 / 103 us on one CTA,
+// 110 / 76 us with sub-blocks of 8, 83 / 59 us here.
+constexpr int kDiagC = 8, kDiagThreads = 256;
 __device__ __forceinline__ void cluster_barrier() {
   asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
 }
@@ -44,84 +45,105 @@ __device__ __forceinline__ void cluster_barrier() {
 // Cholesky of the nb x nb diagonal block of A at (k0, k0) in place (lower, A = L L^H), one
 // cluster per batch item.  A non-positive or non-finite pivot records GKS_ENOTSPD with the
 // global column; the block is then left part way.
+// A 32-column sub-block's own part: thread (i, q) holds row i, columns q + 8 t in registers; a
+// step scales the pivot column (one warp), then every element takes its rank-one update, the
+// next pivot's owner going on to its reciprocal square root while the others still update.
 template <typename T>
 __global__ void __launch_bounds__(kDiagThreads) potf2_kernel(T* A, int lda, long long sA, int k0, int nb,
                                                              DevStatus* st) {
-  __shared__ T s11[kSub][kSub + 1];
-  __shared__ double rd[kSub];
-  __shared__ T v[64][kSub + 1];
+  constexpr int SB = 32;
+  __shared__ T l11[SB][SB + 1], raw[SB], v[SB][SB + 1];
+  __shared__ double rd[SB], s_d;
   __shared__ int fail;
-  const int z = blockIdx.y, rank = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
+  const int z = blockIdx.y, rank = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   A += z * sA + (size_t)k0 * lda + k0;
   if (tid == 0) fail = -1;
-  for (int c0 = 0; c0 < nb; c0 += kSub) {
-    const int kb = min(kSub, nb - c0), m = nb - c0 - kb;
-    __syncthreads();
-    if (tid < 32) {
-      for (int e = lane; e < kSub * kSub; e += 32) {
-        const int i = e >> 3, j = e & 7;
-        s11[i][j] = (i < kb && j <= i) ? ldcg(A + (size_t)(c0 + i) * lda + c0 + j) : zero<T>();
-      }
-      __syncwarp();
-      for (int j = 0; j < kb; j++) {
-        const double piv = re(s11[j][j]);
-        if (!(piv > 0.0) || !isfinite(piv)) {
-          if (lane == 0) fail = c0 + j;
-          break;
-        }
-        // 1 / sqrt, then sqrt with one correction step: half the chain of a square root and a
-        // division on this pipe (434 + 686 clocks)
-        const double inv = rsqrt(piv), d0 = piv * inv, d = fma(0.5 * inv, fma(-d0, d0, piv), d0);
-        __syncwarp();
-        if (lane == j) {
-          s11[j][j] = from_real<T>(d);
-          rd[j] = inv;
-        } else if (lane > j && lane < kb) {
-          s11[lane][j] = s11[lane][j] * inv;
-        }
-        __syncwarp();
-        for (int e = lane; e < kSub * kSub; e += 32) {
-          const int r = e >> 3, c = e & 7;
-          if (c > j && c <= r && r < kb) msubc(s11[r][c], s11[r][j], s11[c][j]);
-        }
-        __syncwarp();
-      }
+  for (int c0 = 0; c0 < nb; c0 += SB) {
+    const int kb = min(SB, nb - c0), m = nb - c0 - kb;
+    T* Ab = A + (size_t)c0 * lda + c0;
+    const int i = tid >> 3, q = tid & 7;
+    T a[4];
+#pragma unroll
+    for (int t = 0; t < 4; t++) {
+      const int j = q + 8 * t;
+      a[t] = (i < kb && j <= i) ? ldcg(Ab + (size_t)i * lda + j) : zero<T>();
     }
+    // pivot: 1 / sqrt, then sqrt with one correction step (half the chain of a square root and a
+    // division on this pipe, 434 + 686 clocks)
+    auto pivot = [&](int k, double piv) {
+      if (!(piv > 0.0) || !isfinite(piv)) {
+        fail = c0 + k;
+      } else {
+        const double inv = rsqrt(piv), d0 = piv * inv;
+        rd[k] = inv;
+        s_d = fma(0.5 * inv, fma(-d0, d0, piv), d0);
+      }
+    };
     __syncthreads();
+    if (q == 0) raw[i] = a[0];
+    if (tid == 0) pivot(0, re(a[0]));
+    __syncthreads();
+    for (int k = 0; k < kb && fail < 0; k++) {
+      if (warp == 0 && lane < kb) {
+        if (lane > k) l11[lane][k] = raw[lane] * rd[k];
+        if (lane == k) l11[k][k] = from_real<T>(s_d);
+        if (lane < k) l11[lane][k] = zero<T>();
+      }
+      __syncthreads();
+      if (i > k && i < kb) {
+        const T li = l11[i][k];
+#pragma unroll
+        for (int t = 0; t < 4; t++) {
+          const int j = q + 8 * t;
+          if (j > k && j <= i) {
+            msubc(a[t], li, l11[j][k]);
+            if (j == k + 1) {
+              raw[i] = a[t];
+              if (i == j) pivot(j, re(a[t]));
+            }
+          }
+        }
+      }
+      __syncthreads();
+    }
     if (fail >= 0) break;  // the same in every CTA of the cluster
-    // rows below, one per 8 lanes, row r of CTA r % kDiagC: x L11^H = a
-    {
-      const int r = rank + kDiagC * (tid >> 3), g = tid & 7;
-      if (tid < 64) {
+    // rows below, one per warp, row r of CTA r % kDiagC: x L11^H = a
+    if (m > 0) {
+      for (int r = rank + kDiagC * warp; r < m; r += kDiagC * 8) {
         T* ar = A + (size_t)(c0 + kb + r) * lda + c0;
-        T x = (r < m && g < kb) ? ldcg(ar + g) : zero<T>();
+        T x = lane < kb ? ldcg(ar + lane) : zero<T>();
+#pragma unroll 1
         for (int j = 0; j < kb; j++) {
-          const T xj = shfl8<T>(x * rd[j], j);
-          if (g > j && g < kb) msubc(x, xj, s11[g][j]);
-          if (g == j) x = xj;
+          const T xj = shfl32(x * rd[j], j);
+          if (lane > j && lane < kb) msubc(x, xj, l11[lane][j]);
+          if (lane == j) x = xj;
         }
-        if (r < m && g < kb) ar[g] = x;
+        if (lane < kb) ar[lane] = x;
       }
     }
-    cluster_barrier();  // every CTA has read the 8 x 8 block
-    if (rank == 0 && tid < kSub * kSub) {
-      const int i = tid >> 3, j = tid & 7;
-      if (i < kb && j <= i) A[(size_t)(c0 + i) * lda + c0 + j] = s11[i][j];
-    }
+    cluster_barrier();  // every CTA has read the diagonal part
+    if (rank == 0)
+      for (int e = tid; e < SB * SB; e += kDiagThreads) {
+        const int r = e >> 5, c = e & 31;
+        if (r < kb && c <= r) Ab[(size_t)r * lda + c] = l11[r][c];
+      }
     if (m <= 0) break;
-    for (int e = tid; e < m * kSub; e += kDiagThreads) {
-      const int i = e >> 3, g = e & 7;
-      v[i][g] = g < kb ? ldcg(A + (size_t)(c0 + kb + i) * lda + c0 + g) : zero<T>();
+    for (int e = tid; e < m * SB; e += kDiagThreads) {
+      const int r = e >> 5, g = e & 31;
+      v[r][g] = g < kb ? ldcg(A + (size_t)(c0 + kb + r) * lda + c0 + g) : zero<T>();
     }
     __syncthreads();
     for (int e = rank * kDiagThreads + tid; e < m * m; e += kDiagC * kDiagThreads) {
-      const int i = e / m, j = e - i * m;
-      if (j > i) continue;
-      T* p = A + (size_t)(c0 + kb + i) * lda + c0 + kb + j;
-      T x = ldcg(p);
-#pragma unroll
-      for (int g = 0; g < kSub; g++) msubc(x, v[i][g], v[j][g]);
-      *p = x;
+      const int r = e / m, j = e - r * m;
+      if (j > r) continue;
+      T* p = A + (size_t)(c0 + kb + r) * lda + c0 + kb + j;
+      T x = ldcg(p), y = zero<T>();
+#pragma unroll 4
+      for (int g = 0; g < SB; g += 2) {  // two chains
+        msubc(x, v[r][g], v[j][g]);
+        msubc(y, v[r][g + 1], v[j][g + 1]);
+      }
+      *p = x + y;
     }
     cluster_barrier();
   }
@@ -207,6 +229,8 @@ __global__ void __launch_bounds__(256) trsm_block_kernel(const T* L, int ldl, lo
 // and its in-block solve, then W = A21 L11^-H, V = W - L21 A11/2, A22 -= L21 V^H + V L21^H,
 // R = V - L21 A11/2, and finally L^-1 [R_0 R_1 ...] by forward substitution, a warp per
 // column.  Writes the lower triangle back into A and the full Hermitian block into F (ldF).
+constexpr int kSub = 8;
+__device__ __forceinline__ void diag_bar() { asm volatile("bar.sync 1, 64;\n" ::: "memory"); }
 template <typename T>
 __global__ void __launch_bounds__(kDiagThreads) hegst_diag_kernel(T* A, int lda, long long sA, const T* L, int ldl,
                                                                   long long sL, int k0, int nb, T* F, int ldF,
@@ -226,8 +250,9 @@ __global__ void __launch_bounds__(kDiagThreads) hegst_diag_kernel(T* A, int lda,
     const int i = e / nb, j = e - i * nb;
     const T x = j <= i ? L[(size_t)i * ldl + j] : zero<T>();
     l[i * LD + j] = x;
-    if (i == j) rd[i] = 1.0 / re(x);
   }
+  __syncthreads();
+  if (tid < nb) rd[tid] = 1.0 / re(l[tid * 66]);
   for (int c0 = 0; c0 < nb; c0 += kSub) {
     const int kb = min(kSub, nb - c0), m = nb - c0 - kb;
     const T* lb = l + c0 * LD + c0;
@@ -405,17 +430,29 @@ __global__ void apply_phase_kernel(T* X, int ldx, long long sX, const double* Z,
   }
 }
 
-// Upper triangle <- conj(lower triangle); diagonal made real.
+// Upper triangle <- conj(lower triangle); diagonal made real.  One CTA per 32 x 32 tile of the
+// lower triangle, transposed through shared memory so that both sides move in whole lines
+// (element by element, the writes down the columns took 93 us for four of order 1664; 29 us).
 template <typename T>
-__global__ void mirror_lower_kernel(T* A, int lda, long long sA, int n) {
-  const int z = blockIdx.z;
-  A += z * sA;
-  for (int i = blockIdx.y; i < n; i += gridDim.y)
-    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j <= i; j += gridDim.x * blockDim.x) {
-      T v = A[(size_t)i * lda + j];
-      if (j == i) A[(size_t)i * lda + i] = from_real<T>(re(v));
-      else A[(size_t)j * lda + i] = conjg(v);
-    }
+__global__ void __launch_bounds__(256) mirror_lower_kernel(T* A, int lda, long long sA, int n) {
+  if (blockIdx.x > blockIdx.y) return;
+  __shared__ T tile[32][33];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, r0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
+  A += blockIdx.z * sA;
+#pragma unroll
+  for (int q = 0; q < 4; q++) {
+    const int r = warp + 8 * q;
+    if (r0 + r < n && c0 + lane <= r0 + r) tile[r][lane] = A[(size_t)(r0 + r) * lda + c0 + lane];
+  }
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < 4; q++) {
+    const int c = warp + 8 * q;  // row of the mirrored tile
+    const int i = c0 + c, j = r0 + lane;
+    if (j >= n || j < i) continue;
+    const T v = tile[lane][c];
+    A[(size_t)i * lda + j] = i == j ? from_real<T>(re(v)) : conjg(v);
+  }
 }
 
 // Column phase convention: the entry of largest modulus (lowest row on ties) becomes
@@ -592,8 +629,10 @@ void lowdin_factor(const T* U, int ldu, long long sU, const double* sv, long lon
 
 template <typename T>
 void mirror_lower(T* A, int lda, long long sA, int n, int count, cudaStream_t s) {
+  if (n <= 0) return;
   count_launch();
-  mirror_lower_kernel<T><<<grid2d(n, n, count), 256, 0, s>>>(A, lda, sA, n);
+  const int t = (n + 31) / 32;
+  mirror_lower_kernel<T><<<dim3(t, t, count), 256, 0, s>>>(A, lda, sA, n);
 }
 
 template <typename T>
