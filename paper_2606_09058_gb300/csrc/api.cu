@@ -105,7 +105,6 @@ struct gks_ctx {
   size_t oz_bytes = 0;
   cudaGraphExec_t gexec = nullptr;     // graph of the last captured solve
   SolveKey gkey{};
-  bool shared = false;                 // a batch's context: other problems run beside this one
   std::vector<gks_ctx*> subs;          // per-problem contexts of gks_solve_batched
   std::vector<cudaStream_t> workers;   // fork/join streams of gks_solve_batched
   cudaGraphExec_t bexec = nullptr;     // graph of the last captured batch
@@ -968,7 +967,7 @@ bool hetrd_digit_run(gks_ctx* c, T* A, int M, int nk) {
   if (M < 3) return true;
   // items per launch: at least one CTA each, all resident
   int per = nk;
-  while (per > 1 && hetrd_panel_ctas<T>(M - 1, per, c->shared) < 1) per = (per + 1) / 2;
+  while (per > 1 && hetrd_panel_ctas<T>(M - 1, per) < 1) per = (per + 1) / 2;
   const int gs = panel_gs(nk);
   PanelArgs<T> pa{};
   pa.lda = M;
@@ -979,7 +978,6 @@ bool hetrd_digit_run(gks_ctx* c, T* A, int M, int nk) {
   pa.sv = M;
   pa.sP = panel_partials(M, gs);
   pa.gs = gs;
-  pa.shared = c->shared;
   pa.hd.sD = (long long)((ldd + 31) / 32 * 32) * ldd * npl;
   pa.hd.ldd = ldd;
   // the grid barriers' CTAs are all resident: a limit chosen for copies does not cut them short
@@ -1999,7 +1997,6 @@ gks_status gks_solve_batched(gks_ctx* ctx, int64_t count, const gks_problem* pro
   }
   for (auto* sc : ctx->subs) {
     sc->tuned = ctx->tuned;
-    sc->shared = P > 1;
   }
   auto body = [&]() -> gks_status {
     cudaEvent_t fork;

@@ -35,7 +35,7 @@ __device__ __forceinline__ zc shfl32(zc v, int src) { return zc{shfl32(v.x, src)
 // memory, L2 reads), with two cluster barriers per sub-block; the diagonal parts, a serial
 // chain of 67-clock operations, are done by every CTA for itself.
 // Measured, one block (complex / real): two-sided reduction 794 / 265 us on one CTA column by
-// column, 175 / 91 us here (190 / 90 with sub-blocks of 16); Cholesky 207 / 103 us on one CTA,
+// column, 163 / 80 us here (190 / 90 with sub-blocks of 16, 420 / 153 on one CTA); Cholesky 207 / 103 us on one CTA,
 // 110 / 76 us with sub-blocks of 8, 83 / 59 us here.
 constexpr int kDiagC = 8, kDiagThreads = 256;
 __device__ __forceinline__ void cluster_barrier() {
@@ -240,7 +240,7 @@ __global__ void __launch_bounds__(kDiagThreads) hegst_diag_kernel(T* A, int lda,
   __shared__ T s11[kSub][kSub + 1];
   __shared__ double rd[64];
   T* v = l + 64 * 65;  // [64][kSub + 1]
-  constexpr int LD = 65, LV = kSub + 1;
+  constexpr int LD = 65, LV = kSub + 1, C = kDiagC;
   const int z = blockIdx.y, rank = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   A += z * sA + (size_t)k0 * lda + k0;
   L += z * sL + (size_t)k0 * ldl + k0;
@@ -295,22 +295,28 @@ __global__ void __launch_bounds__(kDiagThreads) hegst_diag_kernel(T* A, int lda,
     }
     __syncthreads();
     // rows below, one per 8 lanes: W, V
-    const int r = rank + kDiagC * (tid >> 3), g = tid & 7;
-    T* ar = A + (size_t)(c0 + kb + r) * lda + c0;
-    T x = zero<T>(), h = zero<T>();
-    if (tid < 64) {
-      x = (r < m && g < kb) ? ldcg(ar + g) : zero<T>();
-      for (int j = 0; j < kb; j++) {
-        const T xj = shfl8<T>(x * rd[c0 + j], j);
-        if (g > j && g < kb) msubc(x, xj, lb[g * LD + j]);
-        if (g == j) x = xj;
-      }
-      if (r < m && g < kb) {
-        const T* lr = l + (c0 + kb + r) * LD + c0;
-        for (int j = 0; j < kb; j++) mac(h, lr[j], s11[j][g]);
-        h = 0.5 * h;
-        x = x - h;
-        ar[g] = x;
+    constexpr int NR = (56 + 32 * C - 1) / (32 * C);  // rows per 8 lanes
+    const int g = tid & 7;
+    T x[NR], h[NR];
+#pragma unroll
+    for (int q = 0; q < NR; q++) {
+      const int r = rank + C * ((tid >> 3) + 32 * q);
+      T* ar = A + (size_t)(c0 + kb + r) * lda + c0;
+      x[q] = (r < m && g < kb) ? ldcg(ar + g) : zero<T>();
+      h[q] = zero<T>();
+      if (__any_sync(0xffffffffu, r < m)) {
+        for (int j = 0; j < kb; j++) {
+          const T xj = shfl8<T>(x[q] * rd[c0 + j], j);
+          if (g > j && g < kb) msubc(x[q], xj, lb[g * LD + j]);
+          if (g == j) x[q] = xj;
+        }
+        if (r < m && g < kb) {
+          const T* lr = l + (c0 + kb + r) * LD + c0;
+          for (int j = 0; j < kb; j++) mac(h[q], lr[j], s11[j][g]);
+          h[q] = 0.5 * h[q];
+          x[q] = x[q] - h[q];
+          ar[g] = x[q];
+        }
       }
     }
     cluster_barrier();  // every CTA has read the 8 x 8 block
@@ -327,7 +333,7 @@ __global__ void __launch_bounds__(kDiagThreads) hegst_diag_kernel(T* A, int lda,
       v[i * LV + q] = q < kb ? ldcg(A + (size_t)(c0 + kb + i) * lda + c0 + q) : zero<T>();
     }
     __syncthreads();
-    for (int e = rank * kDiagThreads + tid; e < m * m; e += kDiagC * kDiagThreads) {
+    for (int e = rank * kDiagThreads + tid; e < m * m; e += C * kDiagThreads) {
       const int i = e / m, j = e - i * m;
       if (j > i) continue;
       T* p = A + (size_t)(c0 + kb + i) * lda + c0 + kb + j;
@@ -342,11 +348,15 @@ __global__ void __launch_bounds__(kDiagThreads) hegst_diag_kernel(T* A, int lda,
       *p = a;
     }
     cluster_barrier();
-    if (tid < 64 && r < m && g < kb) ar[g] = x - h;
+#pragma unroll
+    for (int q = 0; q < NR; q++) {
+      const int r = rank + C * ((tid >> 3) + 32 * q);
+      if (r < m && g < kb) A[(size_t)(c0 + kb + r) * lda + c0 + g] = x[q] - h[q];
+    }
   }
   cluster_barrier();  // every R is in place
   // column c: rows from its sub-block's end, x_i = (g_i - sum L_ik x_k) / l_ii
-  for (int c = rank + kDiagC * warp; c < nb; c += kDiagC * (kDiagThreads / 32)) {
+  for (int c = rank + C * warp; c < nb; c += C * (kDiagThreads / 32)) {
     const int s0 = min(nb, (c / kSub + 1) * kSub);
     T x0 = zero<T>(), x1 = zero<T>();
     if (lane >= s0 && lane < nb) x0 = ldcg(A + (size_t)lane * lda + c);
@@ -549,15 +559,15 @@ static dim3 grid2d(int rows, int cols, int count) {
 
 // Launch of a diagonal-block kernel on one cluster per item.
 template <typename... P, typename... Q>
-static void diag_launch(void (*k)(P...), int count, size_t sm, cudaStream_t s, Q... args) {
+static void diag_launch(void (*k)(P...), int ctas, int count, size_t sm, cudaStream_t s, Q... args) {
   cudaLaunchConfig_t cfg{};
   cudaLaunchAttribute at{};
-  cfg.gridDim = dim3(kDiagC, count);
+  cfg.gridDim = dim3(ctas, count);
   cfg.blockDim = dim3(kDiagThreads);
   cfg.dynamicSmemBytes = sm;
   cfg.stream = s;
   at.id = cudaLaunchAttributeClusterDimension;
-  at.val.clusterDim.x = kDiagC;
+  at.val.clusterDim.x = ctas;
   at.val.clusterDim.y = at.val.clusterDim.z = 1;
   cfg.attrs = &at;
   cfg.numAttrs = 1;
@@ -567,7 +577,7 @@ static void diag_launch(void (*k)(P...), int count, size_t sm, cudaStream_t s, Q
 
 template <typename T>
 void potf2(T* A, int lda, long long sA, int k0, int nb, DevStatus* st, int count, cudaStream_t s) {
-  diag_launch(potf2_kernel<T>, count, 0, s, A, lda, sA, k0, nb, st);
+  diag_launch(potf2_kernel<T>, kDiagC, count, 0, s, A, lda, sA, k0, nb, st);
 }
 
 template <typename T, int MODE>
@@ -601,7 +611,7 @@ void hegst_diag(T* A, int lda, long long sA, const T* L, int ldl, long long sL, 
                 long long sF, int count, cudaStream_t s) {
   const size_t sm = sizeof(T) * (64 * 65 + 64 * (kSub + 1));
   cudaFuncSetAttribute(hegst_diag_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  diag_launch(hegst_diag_kernel<T>, count, sm, s, A, lda, sA, L, ldl, sL, k0, nb, F, ldF, sF);
+  diag_launch(hegst_diag_kernel<T>, kDiagC, count, sm, s, A, lda, sA, L, ldl, sL, k0, nb, F, ldF, sF);
 }
 
 template <typename T>

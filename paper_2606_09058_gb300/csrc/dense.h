@@ -96,7 +96,6 @@ struct PanelArgs {
   unsigned* bar;
   unsigned base, basev;
   int early;
-  bool shared;  // other problems' reductions run beside this one
   HemvDigits hd;
   DevStatus* st;
   long long wait;
@@ -104,7 +103,7 @@ struct PanelArgs {
 // CTAs per item of the grid form for a panel of order jh on `items` items (0: not even one
 // per item fits).
 template <typename T>
-int hetrd_panel_ctas(int jh, int items, bool shared);
+int hetrd_panel_ctas(int jh, int items);
 // base and basev advance by the launch's arrivals.  False if the launch was refused (then
 // nothing ran).
 template <typename T>

@@ -1158,10 +1158,12 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
     }
     // where the partial products of this lane's first row of the next part lie (the integer
     // divisions before the barrier)
-    const int grp = tid >> 3, gl = tid & 7;
-    const int prow = grp < 40 ? c0 + grp : j - 1, pl = grp < 40 ? gl : lane, pn = grp < 40 ? 8 : 32;
+    // (16 lanes per row where one pass of 20 rows does, else 8 and passes of 40)
+    const int lr = ce - c0 <= 20 ? 4 : 3, LR = 1 << lr, RP = 320 >> lr;
+    const int grp = tid >> lr, gl = tid & (LR - 1);
+    const int prow = warp < 10 ? c0 + grp : j - 1, pl = warp < 10 ? gl : lane, pn = warp < 10 ? LR : 32;
     int pb0 = 0, pb1 = -1, pg0 = 0, pg1 = 0;
-    if (grp < 40 ? prow < ce : warp == 11) {
+    if (warp < 10 ? prow < ce : warp == 11) {
       pb0 = pr.owner((prow >> 5) * pr.C) + pl;
       pb1 = pr.owner(((prow >> 5) + 1) * pr.C - 1);
       if (pb0 <= pb1) {
@@ -1184,19 +1186,19 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
       }
       return v;
     };
-    // groups of 8 lanes of warps 0-9, one row each (40 rows at a time); kq and row j-1's p on
-    // the other two warps; the first rows' loads go out before y arrives
+    // groups of LR lanes of warps 0-9, one row each; kq and row j-1's p on the other two warps;
+    // the first rows' loads go out before y arrives
     T* an = arow2 + ((j - 1) & 1) * a.sv;
     const int ke = a.early ? 0 : k;  // steps of the corrections still to do
     T pv0 = zero<T>(), u0[4], q0[4];
     double dsum = 0.0;
-    if (grp < 40) {
+    if (warp < 10) {
       if (c0 + grp < ce) {
         const T* Uc = U + (size_t)(c0 + grp) * ldu;
         const T* Qc = Q + (size_t)(c0 + grp) * ldu;
 #pragma unroll
         for (int q = 0; q < 4; q++) {
-          const int sq = max(min(gl + 8 * q, ke - 1), 0);
+          const int sq = max(min(gl + LR * q, ke - 1), 0);
           u0[q] = ke > 0 ? Uc[sq] : zero<T>();
           q0[q] = ke > 0 ? Qc[sq] : zero<T>();
         }
@@ -1228,15 +1230,15 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
     double n2 = 0.0;
     int ex = NOEXP;
     bool synced = false;
-    for (int base = c0; base < ce || !synced; base += 40) {
+    for (int base = c0; base < ce || !synced; base += RP) {
       const int c = base + grp;
-      const bool ok = c < ce && grp < 40;
+      const bool ok = c < ce && warp < 10;
       T pv = pv0, corr = zero<T>(), rs = zero<T>(), uc = zero<T>(), aold = zero<T>();
       int dc = 0;
       if (ok) {
         const T* Uc = U + (size_t)c * ldu;
         const T* Qc = Q + (size_t)c * ldu;
-        if (synced) pv = p_from(c, pr.owner((c >> 5) * pr.C) + gl, pr.owner(((c >> 5) + 1) * pr.C - 1), 8);
+        if (synced) pv = p_from(c, pr.owner((c >> 5) * pr.C) + gl, pr.owner(((c >> 5) + 1) * pr.C - 1), LR);
         if (gl == 0) {
           uc = ldcg(Uc + k);
           if (a.early) corr = ldcg(Qc + k);
@@ -1245,25 +1247,31 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
             dc = deq(rmax[c]);
           }
         }
-        for (int s0 = gl; s0 < ke; s0 += 32) {  // four steps' loads in flight
+        for (int s0 = gl; s0 < ke; s0 += 4 * LR) {  // four steps' loads in flight
           if (synced || s0 > gl) {
 #pragma unroll
             for (int q = 0; q < 4; q++) {
-              const int sq = min(s0 + 8 * q, ke - 1);
+              const int sq = min(s0 + LR * q, ke - 1);
               u0[q] = Uc[sq];
               q0[q] = Qc[sq];
             }
           }
 #pragma unroll
           for (int q = 0; q < 4; q++) {
-            const int sq = s0 + 8 * q;
+            const int sq = s0 + LR * q;
             if (sq < ke) correct(corr, rs, u0[q], q0[q], sq);
           }
         }
       }
-      if (grp < 40) {
-        pv = group8_sum(pv - corr);
-        if (ke > 0 && rowupd) rs = group8_sum(rs);
+      if (warp < 10) {
+        pv = pv - corr;
+        const bool upd = ke > 0 && rowupd;
+        if (LR == 16) {
+          pv += shfl_xor(pv, 8);
+          if (upd) rs += shfl_xor(rs, 8);
+        }
+        pv = group8_sum(pv);
+        if (upd) rs = group8_sum(rs);
       }
       if (!synced) {  // kq and row j-1's share
         __syncthreads();
@@ -1300,13 +1308,14 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
 }
 
 // CTAs per item: as many as leave each at most kPanelTiles digit tiles and kPanelRows<T> rows
-// (the FP64 corrections of its rows cost an SM 1.2 us per 4 rows and 32 earlier steps, complex),
-// at most one per SM over all items.
-constexpr int kPanelTiles = 12;
-// With other problems' reductions on other streams (a batch): half the SMs at most.
-constexpr int kPanelShare = 76;
+// (the split of its FP64 corrections), up to the SMs.  Twice as many (12 tiles, 8 / 4 rows) is
+// 2 % faster for one problem (order 1152 real: 20.0 against 20.6 ms the whole call) but leaves
+// no SMs to other streams' reductions: eight uneven systems of order 208 to 1144 on eight
+// streams 57 ms against 43; half as many 36 ms, and one problem 4 % slower.  The count depends
+// on the problem alone, so a solve in a batch gives the bits of the solve by itself.
+constexpr int kPanelTiles = 24;
 template <typename T>
-constexpr int kPanelRows = sizeof(T) == 16 ? 4 : 8;
+constexpr int kPanelRows = sizeof(T) == 16 ? 8 : 16;
 template <typename T>
 static int panel_capacity() {
   static const int cap = [] {
@@ -1350,26 +1359,23 @@ static int panel_cluster() {
 }
 
 template <typename T>
-int hetrd_panel_ctas(int jh, int items, bool shared) {
-  const int cap = shared ? std::min(panel_capacity<T>(), kPanelShare) : panel_capacity<T>();
-  const int top = std::min(cap / items, kPanelCtas);
+int hetrd_panel_ctas(int jh, int items) {
+  const int top = std::min(panel_capacity<T>() / items, kPanelCtas);
   const long long tiles = (long long)((jh + 31) / 32) * ((jh + 15) / 16);
   return (int)std::min<long long>(
       top, std::max<long long>((tiles + kPanelTiles - 1) / kPanelTiles, (jh + kPanelRows<T> - 1) / kPanelRows<T>));
 }
 
 // The cluster form: one cluster of up to 16 CTAs per item, barriers through shared-memory
-// mbarriers, no co-residency of the whole grid needed.  For a problem of its own it pays at
-// the smallest orders only (16 SMs do the FP64 corrections: order 640 real 20 us per step
-// against 12.7 us on 80 CTAs), beside other streams' reductions up to 1000 digit tiles (eight
-// uneven systems of order 208 to 1144: 61 ms with whole-GPU grids, 52 ms on half the SMs, 37
-// ms with clusters below 1000 tiles), and where the grid form cannot give every item a CTA.
+// mbarriers, no co-residency of the whole grid needed.  It pays at the smallest orders only
+// (16 SMs do the FP64 corrections: order 640 real 20 us per step against 12.7 us on 80 CTAs),
+// and where the grid form cannot give every item a CTA.
 template <typename T>
-static int panel_cluster_ctas(int jh, int items, bool shared) {
-  const long long kClusterTiles = shared ? 1000 : 64;
+static int panel_cluster_ctas(int jh, int items) {
+  constexpr long long kClusterTiles = 64;
   const int c = panel_cluster<T>();
   const long long tiles = (long long)((jh + 31) / 32) * ((jh + 15) / 16);
-  if (c == 0 || (tiles > kClusterTiles && hetrd_panel_ctas<T>(jh, items, shared) >= 1)) return 0;
+  if (c == 0 || (tiles > kClusterTiles && hetrd_panel_ctas<T>(jh, items) >= 1)) return 0;
   return c;
 }
 
@@ -1377,8 +1383,8 @@ template <typename T>
 constexpr int kEarlyTiles = sizeof(T) == 16 ? 60 : 150;
 template <typename T>
 bool hetrd_panel(PanelArgs<T> a, int items, unsigned* base, unsigned* basev, cudaStream_t s) {
-  const int cl = std::min(panel_cluster_ctas<T>(a.jh, items, a.shared), a.gs >= 16 ? 16 : a.gs >= 8 ? 8 : 0);
-  const int G = cl > 0 ? cl : std::min(a.gs, hetrd_panel_ctas<T>(a.jh, items, a.shared));
+  const int cl = std::min(panel_cluster_ctas<T>(a.jh, items), a.gs >= 16 ? 16 : a.gs >= 8 ? 8 : 0);
+  const int G = cl > 0 ? cl : std::min(a.gs, hetrd_panel_ctas<T>(a.jh, items));
   int maxseg = (a.jh + 31) / 32 / G + 2;
   const int steps = a.jh - a.jl + 1;
   // U y1 + Q y2 behind the product from kEarlyTiles tiles per CTA up
@@ -1598,7 +1604,7 @@ void narrow_lower(const T* A, int lda, long long sA, TL* B, int ldb, long long s
   template void gather_reflectors<T, T>(const T*, int, long long, const double*, long long, int, int, T*,    \
                                         int, long long, double*, long long, int, cudaStream_t);               \
   template void hetrd_digits<T>(const T*, int, long long, int, const HemvDigits&, int, cudaStream_t);           \
-  template int hetrd_panel_ctas<T>(int, int, bool);                                                              \
+  template int hetrd_panel_ctas<T>(int, int);                                                              \
   template bool hetrd_panel<T>(PanelArgs<T>, int, unsigned*, unsigned*, cudaStream_t);
 INST(double)
 INST(zc)
