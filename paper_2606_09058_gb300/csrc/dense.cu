@@ -4,6 +4,9 @@
 // phase, spinor overlap).
 #include "dense.h"
 
+#include <algorithm>
+#include <cmath>
+
 namespace gks {
 
 // acc -= a * b, acc -= a * conj(b): two fused operations per component.
@@ -17,16 +20,11 @@ __device__ __forceinline__ void msub(zc& acc, zc a, zc b) {
 __device__ __forceinline__ void msubc(double& acc, double a, double b) { acc = fma(-a, b, acc); }
 __device__ __forceinline__ void msubc(zc& acc, zc a, zc b) { msub(acc, a, conjg(b)); }
 
-template <typename T>
-__device__ __forceinline__ T shfl8(T v, int src);
-template <>
-__device__ __forceinline__ double shfl8<double>(double v, int src) { return __shfl_sync(0xffffffffu, v, src, 8); }
-template <>
-__device__ __forceinline__ zc shfl8<zc>(zc v, int src) {
-  return zc{__shfl_sync(0xffffffffu, v.x, src, 8), __shfl_sync(0xffffffffu, v.y, src, 8)};
-}
-__device__ __forceinline__ double shfl32(double v, int src) { return __shfl_sync(0xffffffffu, v, src); }
-__device__ __forceinline__ zc shfl32(zc v, int src) { return zc{shfl32(v.x, src), shfl32(v.y, src)}; }
+// the value of lane src of each group of G lanes
+template <int G>
+__device__ __forceinline__ double shfl_g(double v, int src) { return __shfl_sync(0xffffffffu, v, src, G); }
+template <int G>
+__device__ __forceinline__ zc shfl_g(zc v, int src) { return zc{shfl_g<G>(v.x, src), shfl_g<G>(v.y, src)}; }
 
 // Diagonal blocks (64 x 64) on a cluster of kDiagC CTAs, in sub-blocks (32 columns of the
 // Cholesky factorization, 8 of the two-sided reduction).  One SM does 1.7 FP64 multiply-adds
@@ -114,7 +112,7 @@ __global__ void __launch_bounds__(kDiagThreads) potf2_kernel(T* A, int lda, long
         T x = lane < kb ? ldcg(ar + lane) : zero<T>();
 #pragma unroll 1
         for (int j = 0; j < kb; j++) {
-          const T xj = shfl32(x * rd[j], j);
+          const T xj = shfl_g<32>(x * rd[j], j);
           if (lane > j && lane < kb) msubc(x, xj, l11[lane][j]);
           if (lane == j) x = xj;
         }
@@ -163,13 +161,11 @@ __global__ void __launch_bounds__(kDiagThreads) potf2_kernel(T* A, int lda, long
 // entries, so nothing but the columns of L is read.  The steps are a rolled loop on rotating
 // registers (unrolled they are 30 to 100 KB of code that each launch runs through once).
 // The FP64 pipe bounds it: one warp instruction per 64 clocks and SM partition whatever its
-// active lanes, 19 clocks over the four.  With many right-hand sides G = 8 wastes least (5.5
-// instructions per step for 4 right-hand sides); with few, G = 32 has the shorter chain (2.5
-// per step) on four times the warps.
+// active lanes, 19 clocks over the four: trsm_pick.
 // Measured against 832 real right-hand sides: 184 us with a thread per right-hand side and
-// 64 of them per CTA, 20 us here; 4992 complex: 530, 137 us.
+// 64 of them per CTA, 20 us here.
 template <typename T, int MODE, int G>
-__global__ void __launch_bounds__(256) trsm_block_kernel(const T* L, int ldl, long long sL, T* B, int ldb,
+__global__ void __launch_bounds__(512) trsm_block_kernel(const T* L, int ldl, long long sL, T* B, int ldb,
                                                          long long sB, int nb, int nrhs) {
   constexpr int E = 64 / G;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -206,7 +202,7 @@ __global__ void __launch_bounds__(256) trsm_block_kernel(const T* L, int ldl, lo
 #pragma unroll 1
     for (int jj = 0; jj < G; jj++, col += 64) {
       const T y = x[0] * rd[G * J + jj];
-      const T xj = G == 8 ? shfl8<T>(y, jj) : shfl32(y, jj);
+      const T xj = shfl_g<G>(y, jj);
       if (g > jj) msub(x[0], xj, col[0]);
       if (g == jj) x[0] = xj;
 #pragma unroll
@@ -306,7 +302,7 @@ __global__ void __launch_bounds__(kDiagThreads) hegst_diag_kernel(T* A, int lda,
       h[q] = zero<T>();
       if (__any_sync(0xffffffffu, r < m)) {
         for (int j = 0; j < kb; j++) {
-          const T xj = shfl8<T>(x[q] * rd[c0 + j], j);
+          const T xj = shfl_g<8>(x[q] * rd[c0 + j], j);
           if (g > j && g < kb) msubc(x[q], xj, lb[g * LD + j]);
           if (g == j) x[q] = xj;
         }
@@ -363,7 +359,7 @@ __global__ void __launch_bounds__(kDiagThreads) hegst_diag_kernel(T* A, int lda,
     if (lane + 32 >= s0 && lane + 32 < nb) x1 = ldcg(A + (size_t)(lane + 32) * lda + c);
 #pragma unroll 1
     for (int i = s0; i < nb; i++) {
-      const T xi = shfl32(i < 32 ? x0 : x1, i & 31) * rd[i];
+      const T xi = shfl_g<32>(i < 32 ? x0 : x1, i & 31) * rd[i];
       if (i < 31 && lane > i && lane < nb) msub(x0, l[lane * LD + i], xi);
       if (lane + 32 > i && lane + 32 < nb) msub(x1, l[(lane + 32) * LD + i], xi);
       if (lane == (i & 31)) {
@@ -413,7 +409,7 @@ __global__ void __launch_bounds__(128) larft_kernel(const T* G, int ldG, long lo
   if (lane == (i & 31)) (i < 32 ? a0 : a1) = from_real<T>(ts[i]);
 #pragma unroll 1
   for (int c = i; c > 0; c--) {
-    const T tc = shfl32(c < 32 ? a0 : a1, c & 31);
+    const T tc = shfl_g<32>(c < 32 ? a0 : a1, c & 31);
     if (lane < c) mac(a0, gs[c * 65 + lane], tc);
     if (lane + 32 < c) mac(a1, gs[c * 65 + lane + 32], tc);
     if (lane == ((c - 1) & 31)) {
@@ -580,30 +576,55 @@ void potf2(T* A, int lda, long long sA, int k0, int nb, DevStatus* st, int count
   diag_launch(potf2_kernel<T>, kDiagC, count, 0, s, A, lda, sA, k0, nb, st);
 }
 
-template <typename T, int MODE>
+template <typename T, int MODE, int G>
 static void trsm_launch(const T* L, int ldl, long long sL, T* B, int ldb, long long sB, int nb, int nrhs, int count,
-                        cudaStream_t s) {
-  const int sm = (int)(64 * 64 * sizeof(T) + 64 * sizeof(double));
+                        int w, cudaStream_t s) {
+  const int sm = (int)(64 * 64 * sizeof(T) + 64 * sizeof(double)), per = 32 * w / G;
+  cudaFuncSetAttribute(trsm_block_kernel<T, MODE, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
   count_launch();
-  if ((long long)nrhs * count <= 8 * 152) {  // a warp per right-hand side, 4 per CTA
-    cudaFuncSetAttribute(trsm_block_kernel<T, MODE, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-    trsm_block_kernel<T, MODE, 32><<<dim3((nrhs + 3) / 4, count), 128, sm, s>>>(L, ldl, sL, B, ldb, sB, nb, nrhs);
-    return;
+  trsm_block_kernel<T, MODE, G><<<dim3((nrhs + per - 1) / per, count), 32 * w, sm, s>>>(L, ldl, sL, B, ldb, sB, nb,
+                                                                                        nrhs);
+}
+
+// Lanes per right-hand side and warps per CTA (4 to 16): those with the least FP64 pipe time
+// of the fullest SM, which is the instructions of a step (four right-hand sides: 20 / 24 / 32
+// for 8 / 16 / 32 lanes complex, 5.5 / 7 / 10 real) times 19 clocks for each of its warps or 64
+// for each on its fullest partition.  A last wave of a few CTAs costs as much as a full one
+// (4992 right-hand sides in CTAs of 32 are 156 on 152 SMs).
+// Measured, all launches of a call (32 lanes up to 1216 right-hand sides, 8 above, 4 or 8
+// warps, against this rule): order 4992 complex 32.2 / 29.1 ms, eight of order 832 complex
+// 5.5 / 5.0, a spinor problem of order 2496 12.2 / 11.2; order 832 real unchanged.
+template <typename T, int MODE>
+static void trsm_pick(const T* L, int ldl, long long sL, T* B, int ldb, long long sB, int nb, int nrhs, int count,
+                      cudaStream_t s) {
+  int G = 8, w = 4;
+  double best = 1e300;
+  for (int g = 8; g <= 32; g *= 2) {
+    const int e = 64 / g - 1;
+    const double instr = sizeof(T) == 16 ? 6.0 + 2.0 * e : 2.0 + 0.5 * e;
+    for (int v = 4; v <= 16; v++) {
+      const long long per = 32 * v / g, ctas = (nrhs + per - 1) / per * count;
+      const double warps = (double)((ctas + 151) / 152) * v;
+      const double t = instr * std::max(19.0 * warps, 64.0 * std::ceil(warps / 4.0));
+      if (t < best) {
+        best = t;
+        G = g;
+        w = v;
+      }
+    }
   }
-  // warps per CTA: 4 right-hand sides each, four warps (one per SM partition) or more
-  const int w = (long long)nrhs * count >= 2 * 32 * 152 ? 8 : 4;
-  cudaFuncSetAttribute(trsm_block_kernel<T, MODE, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-  trsm_block_kernel<T, MODE, 8><<<dim3((nrhs + 4 * w - 1) / (4 * w), count), 32 * w, sm, s>>>(L, ldl, sL, B, ldb, sB,
-                                                                                             nb, nrhs);
+  if (G == 8) trsm_launch<T, MODE, 8>(L, ldl, sL, B, ldb, sB, nb, nrhs, count, w, s);
+  else if (G == 16) trsm_launch<T, MODE, 16>(L, ldl, sL, B, ldb, sB, nb, nrhs, count, w, s);
+  else trsm_launch<T, MODE, 32>(L, ldl, sL, B, ldb, sB, nb, nrhs, count, w, s);
 }
 
 template <typename T>
 void trsm_block(int mode, const T* L, int ldl, long long sL, T* B, int ldb, long long sB, int nb, int nrhs,
                 int count, cudaStream_t s) {
   if (nrhs <= 0 || nb <= 0 || count <= 0) return;
-  if (mode == TRSM_RIGHT_CONJ) trsm_launch<T, TRSM_RIGHT_CONJ>(L, ldl, sL, B, ldb, sB, nb, nrhs, count, s);
-  else if (mode == TRSM_LEFT) trsm_launch<T, TRSM_LEFT>(L, ldl, sL, B, ldb, sB, nb, nrhs, count, s);
-  else trsm_launch<T, TRSM_LEFT_CONJ>(L, ldl, sL, B, ldb, sB, nb, nrhs, count, s);
+  if (mode == TRSM_RIGHT_CONJ) trsm_pick<T, TRSM_RIGHT_CONJ>(L, ldl, sL, B, ldb, sB, nb, nrhs, count, s);
+  else if (mode == TRSM_LEFT) trsm_pick<T, TRSM_LEFT>(L, ldl, sL, B, ldb, sB, nb, nrhs, count, s);
+  else trsm_pick<T, TRSM_LEFT_CONJ>(L, ldl, sL, B, ldb, sB, nb, nrhs, count, s);
 }
 
 template <typename T>
