@@ -103,6 +103,11 @@ struct gks_ctx {
   std::map<std::tuple<int, int, int>, int> tuned;  // (order bucket, element size, spin) -> width
   void* oz = nullptr;                  // digit workspace of the split-product GEMM
   size_t oz_bytes = 0;
+  // stages that run beside the main stream: their stream, fork and join events and split workspace
+  cudaStream_t side = nullptr;
+  cudaEvent_t fork = nullptr, join = nullptr;
+  void* side_oz = nullptr;
+  size_t side_oz_bytes = 0;
   cudaGraphExec_t gexec = nullptr;     // graph of the last captured solve
   SolveKey gkey{};
   std::vector<gks_ctx*> subs;          // per-problem contexts of gks_solve_batched
@@ -209,6 +214,17 @@ void release_oz(gks_ctx* c) {
   if (c->oz) cudaFree(c->oz);
   c->oz = nullptr;
   c->oz_bytes = 0;
+}
+
+void release_side(gks_ctx* c) {
+  if (c->side_oz) cudaFree(c->side_oz);
+  if (c->side) cudaStreamDestroy(c->side);
+  if (c->fork) cudaEventDestroy(c->fork);
+  if (c->join) cudaEventDestroy(c->join);
+  c->side_oz = nullptr;
+  c->side_oz_bytes = 0;
+  c->side = nullptr;
+  c->fork = c->join = nullptr;
 }
 
 void release_extra(gks_ctx* c) {
@@ -522,6 +538,40 @@ struct StageRec {
     nvtxRangePop();
   }
 };
+
+// Work of `body` on the context's side stream from where the main stream stands, its split
+// products on a workspace of their own (the same dispatch, so the same bits as on the main
+// stream); side_join makes the main stream wait for it.  The side stream has the higher
+// priority: it carries chains of small kernels beside large ones.  Without a stream (creation
+// failed) `body` runs on the main stream.  Both are captured when the main stream is.
+bool side_ready(gks_ctx* c) {
+  if (c->side) return true;
+  int lo = 0, hi = 0;
+  cudaDeviceGetStreamPriorityRange(&lo, &hi);
+  if (cudaEventCreateWithFlags(&c->fork, cudaEventDisableTiming) == cudaSuccess &&
+      cudaEventCreateWithFlags(&c->join, cudaEventDisableTiming) == cudaSuccess &&
+      cudaStreamCreateWithPriority(&c->side, cudaStreamNonBlocking, hi) == cudaSuccess)
+    return true;
+  cudaGetLastError();
+  release_side(c);
+  return false;
+}
+template <typename F>
+void on_side(gks_ctx* c, F body) {
+  auto swap = [&]() {
+    std::swap(c->stream, c->side);
+    std::swap(c->oz, c->side_oz);
+    std::swap(c->oz_bytes, c->side_oz_bytes);
+    c->prof.stream = c->stream;
+  };
+  cudaEventRecord(c->fork, c->stream);
+  cudaStreamWaitEvent(c->side, c->fork, 0);
+  swap();
+  body();
+  swap();
+  cudaEventRecord(c->join, c->side);
+}
+void side_join(gks_ctx* c) { cudaStreamWaitEvent(c->stream, c->join, 0); }
 
 double cmul(int es) { return es == 16 ? 8.0 : 2.0; }
 
@@ -875,7 +925,11 @@ void hegst_level(gks_ctx* c, T* A, int lda, long long sA, const T* L, int ldl, l
 // The same reduction with outer panels of nbb columns: the diagonal nbb block by
 // hegst_level, then the panel steps with K = nbb products (A21 L11^-H by 64-wide block
 // substitution, the Hermitian A11' as a full copy for the two half-updates, the rank-2nbb
-// trailing update), and the deferred substitution L^-1 [R_0 R_1 ...] blocked the same way.
+// trailing update), and the substitution L^-1 [R_0 R_1 ...] of row block K0 as soon as the
+// columns left of it are final.  hegst_level is a chain of some 60 small kernels on few SMs
+// that touches the diagonal block alone, so it runs beside the substitutions, which do not
+// (whole call, one after the other / beside: order 4992 complex 400 / 387 ms, four of order
+// 1625 complex 102 / 98.7, order 1079 real, two channels, 30.2 / 29.0, order 832 20.6 / 20.0).
 template <typename T>
 void hegst_run(gks_ctx* c, T* A, int lda, long long sA, const T* L, int ldl, long long sL, int n, int nk) {
   cudaStream_t s = c->stream;
@@ -886,18 +940,19 @@ void hegst_run(gks_ctx* c, T* A, int lda, long long sA, const T* L, int ldl, lon
     return;
   }
   T* FB = at<T>(c, c->oFB);
+  const bool beside = side_ready(c);
   for (int K0 = 0; K0 < n; K0 += nbb) {
-    const int KB = std::min(nbb, n - K0);
+    const int KB = std::min(nbb, n - K0), rows = n - K0 - KB;
     T* A11 = A + (size_t)K0 * lda + K0;
     const T* L11 = L + (size_t)K0 * ldl + K0;
-    hegst_level<T>(c, A11, lda, sA, L11, ldl, sL, KB, nk);
-    const int rows = n - K0 - KB;
-    if (rows <= 0) continue;
     const T* L21 = L + (size_t)(K0 + KB) * ldl + K0;
     T* A21 = A + (size_t)(K0 + KB) * lda + K0;
     T* A22 = A21 + KB;
+    auto level = [&]() { hegst_level<T>(c, A11, lda, sA, L11, ldl, sL, KB, nk); };
+    if (beside) on_side(c, level);
+    else level();
     // A21 <- A21 L11^-H: column blocks left to right, X_j = (A_j - X_<j L11[j,<j]^H) L11[j,j]^-H
-    for (int j0 = 0; j0 < KB; j0 += NB) {
+    for (int j0 = 0; rows > 0 && j0 < KB; j0 += NB) {
       const int jb = std::min(NB, KB - j0);
       if (j0 > 0)
         gmx<T>(c, nk, OP_N, OP_C, rows, jb, j0, -1.0, A21, lda, sA, L11 + (size_t)j0 * ldl, ldl, sL, 1.0, A21 + j0,
@@ -905,6 +960,24 @@ void hegst_run(gks_ctx* c, T* A, int lda, long long sA, const T* L, int ldl, lon
       Rec r(c, PC_TRSM, cmul(es) * 0.5 * jb * jb * rows * nk, (2.0 * rows * jb + 0.5 * jb * jb) * es * nk);
       trsm_block<T>(TRSM_RIGHT_CONJ, L11 + (size_t)j0 * ldl + j0, ldl, sL, A21 + j0, lda, sA, jb, rows, nk, s);
     }
+    // rows K0 .. K0 + KB of L^-1 [R_0 R_1 ...], and their share of the rows below
+    for (int r0 = K0; K0 > 0 && r0 < K0 + KB; r0 += NB) {
+      const int rb = std::min(NB, K0 + KB - r0);
+      T* Ai = A + (size_t)r0 * lda;
+      {
+        Rec r(c, PC_TRSM, cmul(es) * 0.5 * rb * rb * K0 * nk, (2.0 * K0 * rb + 0.5 * rb * rb) * es * nk);
+        trsm_block<T>(TRSM_LEFT, L + (size_t)r0 * ldl + r0, ldl, sL, Ai, lda, sA, rb, K0, nk, s);
+      }
+      const int below = K0 + KB - r0 - rb;
+      if (below > 0)
+        gmx<T>(c, nk, OP_N, OP_N, below, K0, rb, -1.0, L + (size_t)(r0 + rb) * ldl + r0, ldl, sL, Ai, lda, sA, 1.0,
+               A + (size_t)(r0 + rb) * lda, lda, sA);
+    }
+    if (K0 > 0 && rows > 0)
+      gmx<T>(c, nk, OP_N, OP_N, rows, K0, KB, -1.0, L21, ldl, sL, A + (size_t)K0 * lda, lda, sA, 1.0,
+             A + (size_t)(K0 + KB) * lda, lda, sA);
+    if (beside) side_join(c);
+    if (rows <= 0) continue;
     {
       Rec r(c, PC_MISC);
       copy2d<T>(FB, nbb, c->sFB, A11, lda, sA, KB, KB, nk, s);
@@ -914,26 +987,6 @@ void hegst_run(gks_ctx* c, T* A, int lda, long long sA, const T* L, int ldl, lon
     gmx<T>(c, nk, OP_N, OP_C, rows, rows, KB, -1.0, L21, ldl, sL, A21, lda, sA, 1.0, A22, lda, sA, 1);
     gmx<T>(c, nk, OP_N, OP_C, rows, rows, KB, -1.0, A21, lda, sA, L21, ldl, sL, 1.0, A22, lda, sA, 1);
     gmx<T>(c, nk, OP_N, OP_N, rows, KB, KB, -0.5, L21, ldl, sL, FB, nbb, c->sFB, 1.0, A21, lda, sA);
-  }
-  // deferred substitution over the outer-block-strictly-lower part
-  for (int R0 = nbb; R0 < n; R0 += nbb) {
-    const int RB = std::min(nbb, n - R0);
-    for (int r0 = R0; r0 < R0 + RB; r0 += NB) {
-      const int rb = std::min(NB, R0 + RB - r0);
-      T* Ai = A + (size_t)r0 * lda;
-      {
-        Rec r(c, PC_TRSM, cmul(es) * 0.5 * rb * rb * R0 * nk, (2.0 * R0 * rb + 0.5 * rb * rb) * es * nk);
-        trsm_block<T>(TRSM_LEFT, L + (size_t)r0 * ldl + r0, ldl, sL, Ai, lda, sA, rb, R0, nk, s);
-      }
-      const int below = R0 + RB - r0 - rb;
-      if (below > 0)
-        gmx<T>(c, nk, OP_N, OP_N, below, R0, rb, -1.0, L + (size_t)(r0 + rb) * ldl + r0, ldl, sL, Ai, lda, sA, 1.0,
-               A + (size_t)(r0 + rb) * lda, lda, sA);
-    }
-    const int below = n - R0 - RB;
-    if (below > 0)
-      gmx<T>(c, nk, OP_N, OP_N, below, R0, RB, -1.0, L + (size_t)(R0 + RB) * ldl + R0, ldl, sL,
-             A + (size_t)R0 * lda, lda, sA, 1.0, A + (size_t)(R0 + RB) * lda, lda, sA);
   }
 }
 
@@ -1400,7 +1453,7 @@ gks_status solve_t(gks_ctx* c, const SolveKey& key) {
   cudaStream_t s = c->stream;
   // the scratch of the largest split product (the density matrix) at once: growing it product
   // by product would wait for the stream each time
-  if (split_worth(c, items, M, M, nev, es, 0))
+  if (!(key.flags & GKS_EIGEN_ONLY) && split_worth(c, items, M, M, nev, es, 0))
     oz_reserve(c, ozaki_workspace_bytes(M, M, nev, es == 16, sform(c)), items);
   double* eps = static_cast<double*>(const_cast<void*>(key.eps));
   T* C = static_cast<T*>(const_cast<void*>(key.C));
@@ -1901,12 +1954,14 @@ gks_status gks_destroy(gks_ctx* ctx) {
     release_ws(sc);
     release_aws(sc);
     release_oz(sc);
+    release_side(sc);
     delete sc;
   }
   for (auto w : ctx->workers) cudaStreamDestroy(w);
   release_ws(ctx);
   release_aws(ctx);
   release_oz(ctx);
+  release_side(ctx);
   release_extra(ctx);
   delete ctx;
   return GKS_OK;
