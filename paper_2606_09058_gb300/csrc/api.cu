@@ -103,11 +103,13 @@ struct gks_ctx {
   std::map<std::tuple<int, int, int>, int> tuned;  // (order bucket, element size, spin) -> width
   void* oz = nullptr;                  // digit workspace of the split-product GEMM
   size_t oz_bytes = 0;
-  // stages that run beside the main stream: their stream, fork and join events and split workspace
-  cudaStream_t side = nullptr;
-  cudaEvent_t fork = nullptr, join = nullptr;
-  void* side_oz = nullptr;
-  size_t side_oz_bytes = 0;
+  // stages that run beside the main stream: their streams and split workspaces, and events
+  struct Lane {
+    cudaStream_t stream = nullptr;
+    void* oz = nullptr;
+    size_t oz_bytes = 0;
+  } lane[2];
+  std::vector<cudaEvent_t> events;
   cudaGraphExec_t gexec = nullptr;     // graph of the last captured solve
   SolveKey gkey{};
   std::vector<gks_ctx*> subs;          // per-problem contexts of gks_solve_batched
@@ -216,15 +218,14 @@ void release_oz(gks_ctx* c) {
   c->oz_bytes = 0;
 }
 
-void release_side(gks_ctx* c) {
-  if (c->side_oz) cudaFree(c->side_oz);
-  if (c->side) cudaStreamDestroy(c->side);
-  if (c->fork) cudaEventDestroy(c->fork);
-  if (c->join) cudaEventDestroy(c->join);
-  c->side_oz = nullptr;
-  c->side_oz_bytes = 0;
-  c->side = nullptr;
-  c->fork = c->join = nullptr;
+void release_lanes(gks_ctx* c) {
+  for (auto& l : c->lane) {
+    if (l.oz) cudaFree(l.oz);
+    if (l.stream) cudaStreamDestroy(l.stream);
+    l = {};
+  }
+  for (auto e : c->events) cudaEventDestroy(e);
+  c->events.clear();
 }
 
 void release_extra(gks_ctx* c) {
@@ -539,39 +540,45 @@ struct StageRec {
   }
 };
 
-// Work of `body` on the context's side stream from where the main stream stands, its split
-// products on a workspace of their own (the same dispatch, so the same bits as on the main
-// stream); side_join makes the main stream wait for it.  The side stream has the higher
-// priority: it carries chains of small kernels beside large ones.  Without a stream (creation
-// failed) `body` runs on the main stream.  Both are captured when the main stream is.
-bool side_ready(gks_ctx* c) {
-  if (c->side) return true;
+// Lanes: work beside the main stream, split products on a workspace of their own (the same
+// dispatch, so the same bits as on the main stream).  The lanes have the higher priority: they
+// carry chains of small kernels beside large ones.  lane_fork lets lane q start where the main
+// stream stands, lane_run enqueues `body` on it, main_wait makes the main stream wait for an
+// event.  All of it is captured when the main stream is, and every lane is joined before the
+// stage that forked it returns.  False if streams or events cannot be created: the caller then
+// runs everything on the main stream.
+enum { EV_FORK = 0, EV_LEVEL = 2, EV_PANEL = 3 };  // forks of lanes 0 and 1, join of lane 0, panels
+bool lanes_ready(gks_ctx* c, int panels) {
   int lo = 0, hi = 0;
   cudaDeviceGetStreamPriorityRange(&lo, &hi);
-  if (cudaEventCreateWithFlags(&c->fork, cudaEventDisableTiming) == cudaSuccess &&
-      cudaEventCreateWithFlags(&c->join, cudaEventDisableTiming) == cudaSuccess &&
-      cudaStreamCreateWithPriority(&c->side, cudaStreamNonBlocking, hi) == cudaSuccess)
-    return true;
-  cudaGetLastError();
-  release_side(c);
-  return false;
+  bool ok = true;
+  for (auto& l : c->lane)
+    if (ok && !l.stream) ok = cudaStreamCreateWithPriority(&l.stream, cudaStreamNonBlocking, hi) == cudaSuccess;
+  while (ok && (int)c->events.size() < EV_PANEL + panels) {
+    cudaEvent_t e;
+    ok = cudaEventCreateWithFlags(&e, cudaEventDisableTiming) == cudaSuccess;
+    if (ok) c->events.push_back(e);
+  }
+  if (!ok) cudaGetLastError();
+  return ok;
+}
+void lane_fork(gks_ctx* c, int q) {
+  cudaEventRecord(c->events[EV_FORK + q], c->stream);
+  cudaStreamWaitEvent(c->lane[q].stream, c->events[EV_FORK + q], 0);
 }
 template <typename F>
-void on_side(gks_ctx* c, F body) {
+void lane_run(gks_ctx* c, int q, F body) {
   auto swap = [&]() {
-    std::swap(c->stream, c->side);
-    std::swap(c->oz, c->side_oz);
-    std::swap(c->oz_bytes, c->side_oz_bytes);
+    std::swap(c->stream, c->lane[q].stream);
+    std::swap(c->oz, c->lane[q].oz);
+    std::swap(c->oz_bytes, c->lane[q].oz_bytes);
     c->prof.stream = c->stream;
   };
-  cudaEventRecord(c->fork, c->stream);
-  cudaStreamWaitEvent(c->side, c->fork, 0);
   swap();
   body();
   swap();
-  cudaEventRecord(c->join, c->side);
 }
-void side_join(gks_ctx* c) { cudaStreamWaitEvent(c->stream, c->join, 0); }
+void main_wait(gks_ctx* c, int e) { cudaStreamWaitEvent(c->stream, c->events[e], 0); }
 
 double cmul(int es) { return es == 16 ? 8.0 : 2.0; }
 
@@ -763,9 +770,10 @@ void rho_run(gks_ctx* c, const T* C, int ldc, long long sC, T* rho, long long sR
 // leading dimension ld, item stride sL), two levels.  Outer panels of nbb columns: inside a
 // panel, 64-wide steps (diagonal block in shared memory, L21 = A21 L11^-H by substitution,
 // rank-64 update of the rest of the panel only); after the panel, one rank-nbb update of
-// the trailing matrix (the product that dominates, with K = nbb).
-template <typename T>
-void potrf_run(gks_ctx* c, T* L, int n, int ld, long long sL, int nk) {
+// the trailing matrix (the product that dominates, with K = nbb).  after(p, K0, KB) is called
+// when panel p's columns K0 .. K0 + KB are final.
+template <typename T, typename F>
+void potrf_run(gks_ctx* c, T* L, int n, int ld, long long sL, int nk, F after) {
   cudaStream_t s = c->stream;
   const int es = sizeof(T);
   const int nbb = c->nbb;
@@ -788,12 +796,18 @@ void potrf_run(gks_ctx* c, T* L, int n, int ld, long long sL, int nk) {
       const int w = K0 + KB - (k0 + kb);  // panel columns right of this step
       if (w > 0) gmx<T>(c, nk, OP_N, OP_C, rows, w, kb, -1.0, L21, ld, sL, L21, ld, sL, 1.0, L21 + kb, ld, sL, 1);
     }
+    after(K0 / nbb, K0, KB);
     const int rows2 = n - K0 - KB;
     if (rows2 > 0) {
       T* P = L + (size_t)(K0 + KB) * ld + K0;
       gmx<T>(c, nk, OP_N, OP_C, rows2, rows2, KB, -1.0, P, ld, sL, P, ld, sL, 1.0, P + KB, ld, sL, 1);
     }
   }
+}
+
+template <typename T>
+void potrf_run(gks_ctx* c, T* L, int n, int ld, long long sL, int nk) {
+  potrf_run<T>(c, L, n, ld, sL, nk, [](int, int, int) {});
 }
 
 // X <- L^-1 X (conj = false) or L^-H X (conj = true) for the n x ncols block X (leading
@@ -930,17 +944,20 @@ void hegst_level(gks_ctx* c, T* A, int lda, long long sA, const T* L, int ldl, l
 // that touches the diagonal block alone, so it runs beside the substitutions, which do not
 // (whole call, one after the other / beside: order 4992 complex 400 / 387 ms, four of order
 // 1625 complex 102 / 98.7, order 1079 real, two channels, 30.2 / 29.0, order 832 20.6 / 20.0).
+// chol: L's panel p is final with event EV_PANEL + p (a factorization on lane 1).
 template <typename T>
-void hegst_run(gks_ctx* c, T* A, int lda, long long sA, const T* L, int ldl, long long sL, int n, int nk) {
+void hegst_run(gks_ctx* c, T* A, int lda, long long sA, const T* L, int ldl, long long sL, int n, int nk,
+               bool chol = false) {
   cudaStream_t s = c->stream;
   const int es = sizeof(T);
   const int nbb = c->nbb;
   if (n <= nbb || nbb <= NB) {
+    if (chol) main_wait(c, EV_PANEL + (n - 1) / nbb);
     hegst_level<T>(c, A, lda, sA, L, ldl, sL, n, nk);
     return;
   }
   T* FB = at<T>(c, c->oFB);
-  const bool beside = side_ready(c);
+  const bool beside = lanes_ready(c, 0);
   for (int K0 = 0; K0 < n; K0 += nbb) {
     const int KB = std::min(nbb, n - K0), rows = n - K0 - KB;
     T* A11 = A + (size_t)K0 * lda + K0;
@@ -948,9 +965,17 @@ void hegst_run(gks_ctx* c, T* A, int lda, long long sA, const T* L, int ldl, lon
     const T* L21 = L + (size_t)(K0 + KB) * ldl + K0;
     T* A21 = A + (size_t)(K0 + KB) * lda + K0;
     T* A22 = A21 + KB;
-    auto level = [&]() { hegst_level<T>(c, A11, lda, sA, L11, ldl, sL, KB, nk); };
-    if (beside) on_side(c, level);
-    else level();
+    auto level = [&]() {
+      hegst_level<T>(c, A11, lda, sA, L11, ldl, sL, KB, nk);
+      if (beside) cudaEventRecord(c->events[EV_LEVEL], c->stream);
+    };
+    if (chol) main_wait(c, EV_PANEL + K0 / nbb);
+    if (beside) {
+      lane_fork(c, 0);
+      lane_run(c, 0, level);
+    } else {
+      level();
+    }
     // A21 <- A21 L11^-H: column blocks left to right, X_j = (A_j - X_<j L11[j,<j]^H) L11[j,j]^-H
     for (int j0 = 0; rows > 0 && j0 < KB; j0 += NB) {
       const int jb = std::min(NB, KB - j0);
@@ -976,7 +1001,7 @@ void hegst_run(gks_ctx* c, T* A, int lda, long long sA, const T* L, int ldl, lon
     if (K0 > 0 && rows > 0)
       gmx<T>(c, nk, OP_N, OP_N, rows, K0, KB, -1.0, L21, ldl, sL, A + (size_t)K0 * lda, lda, sA, 1.0,
              A + (size_t)(K0 + KB) * lda, lda, sA);
-    if (beside) side_join(c);
+    if (beside) main_wait(c, EV_LEVEL);
     if (rows <= 0) continue;
     {
       Rec r(c, PC_MISC);
@@ -1474,6 +1499,7 @@ gks_status solve_t(gks_ctx* c, const SolveKey& key) {
     if (!reuse) copy2d<T>(L, n, sLk, S, n, (long long)n * n, n, n, nk, s);
   }
   const bool lowdin = c->reduction == GKS_REDUCE_LOWDIN;
+  bool chol = false;
   auto refused = [c] {
     return fail(c, GKS_ECUDA, "tridiagonalization: cooperative launch refused (not enough resident CTAs)");
   };
@@ -1499,11 +1525,26 @@ gks_status solve_t(gks_ctx* c, const SolveKey& key) {
     copy2d<T>(A, M, c->sMM, H, M, (long long)M * M, M, M, items, s);  // H again (A held S)
   } else if (!reuse) {
     c->l_valid = false;
-    StageRec sr(c, PS_POTRF);
-    potrf_run<T>(c, L, n, n, sLk, nk);
-    if (sp) {
-      Rec r(c, PC_MISC);
-      copy2d<T>(L + c->sMM, n, sLk, L, n, sLk, n, n, nk, s);
+    // on lane 1: the reduction takes a panel's columns as soon as they are final, so that the
+    // factorization's chains of small kernels run beside the reduction's products
+    // (whole call, one after the other / beside: order 4992 complex 387 / 376 ms, four of order
+    // 1625 complex 98.7 / 95.1, order 832 real 20.0 / 19.1)
+    chol = lanes_ready(c, (n + c->nbb - 1) / c->nbb);
+    auto factor = [&]() {
+      StageRec sr(c, PS_POTRF);
+      potrf_run<T>(c, L, n, n, sLk, nk, [&](int p, int K0, int KB) {
+        if (sp) {
+          Rec r(c, PC_MISC);
+          copy2d<T>(L + c->sMM + K0, n, sLk, L + K0, n, sLk, n, KB, nk, c->stream);
+        }
+        if (chol) cudaEventRecord(c->events[EV_PANEL + p], c->stream);
+      });
+    };
+    if (chol) {
+      lane_fork(c, 1);
+      lane_run(c, 1, factor);
+    } else {
+      factor();
     }
     c->lkey = key;
     c->l_valid = true;
@@ -1523,12 +1564,12 @@ gks_status solve_t(gks_ctx* c, const SolveKey& key) {
       // H'^{ss'} = L^-1 H^{ss'} L^-H per spin block (paper Sec. 3.2 Part 3-3): the two
       // Hermitian diagonal blocks two-sided, the lower off-diagonal block by a left and a
       // right triangular solve
-      hegst_run<T>(c, A, M, c->sMM, L, n, c->sMM, n, nk);
+      hegst_run<T>(c, A, M, c->sMM, L, n, c->sMM, n, nk, chol);
       hegst_run<T>(c, A + (size_t)n * M + n, M, c->sMM, L, n, c->sMM, n, nk);
       trsm_left_run<T>(c, L, n, c->sMM, A + (size_t)n * M, M, c->sMM, n, n, nk, false);
       trsm_right_conj_run<T>(c, L, n, c->sMM, A + (size_t)n * M, M, c->sMM, n, n, nk);
     } else {
-      hegst_run<T>(c, A, M, c->sMM, L, n, c->sMM, M, items);
+      hegst_run<T>(c, A, M, c->sMM, L, n, c->sMM, M, items, chol);
     }
   }
   // (a3-a4) Householder tridiagonalization with a real-making phase
@@ -1954,14 +1995,14 @@ gks_status gks_destroy(gks_ctx* ctx) {
     release_ws(sc);
     release_aws(sc);
     release_oz(sc);
-    release_side(sc);
+    release_lanes(sc);
     delete sc;
   }
   for (auto w : ctx->workers) cudaStreamDestroy(w);
   release_ws(ctx);
   release_aws(ctx);
   release_oz(ctx);
-  release_side(ctx);
+  release_lanes(ctx);
   release_extra(ctx);
   delete ctx;
   return GKS_OK;
