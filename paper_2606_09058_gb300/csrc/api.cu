@@ -158,7 +158,7 @@ struct gks_ctx {
       oweights, oeb, odc, oticket, oAf, oRY, oRT, oRR, onrm, orstat, operm, oflag, oBd, oV2, otau2, oprog, oerr, oqr, oD, oarow, oppart, opy, opP, opdot, opnrm, opmex, opbar, ormax,
       otau1, oT1, oP1, oP2, oVT, oXb, oGb, oYb, oZb, oXp, oVw, otw, oGw, oTw, oYw, oY2w;
   int ldt2 = 0, nblkmax = 0;
-  long long sMM, sF, sFB, sU, spart, sy, sV, sG, sT, sY, sVec;
+  long long oUQ, sUQ, sMM, sF, sFB, sU, spart, sy, sV, sG, sT, sY, sVec;
 };
 
 namespace {
@@ -316,6 +316,8 @@ gks_status ensure_ws(gks_ctx* c, int m, int n, int nk, int es, int nc) {
   c->oFB = a.take<char>(elems(c->sFB));
   c->oU = a.take<char>(elems(c->sU));
   c->oQ = a.take<char>(elems(c->sU));
+  c->sUQ = 3LL * m * std::min(kPanelMax, nbb);
+  c->oUQ = a.take<char>(elems(c->sUQ));
   c->opart = a.take<char>(elems(c->spart));
   c->oy = a.take<char>(elems(c->sy));
   c->ouw = a.take<double>((size_t)3 * m * nk);
@@ -1015,20 +1017,32 @@ void hegst_run(gks_ctx* c, T* A, int lda, long long sA, const T* L, int ldl, lon
   }
 }
 
-// Deferred update of a panel with kp steps: A[0:n, 0:n] -= U Q^H + Q U^H (lower triangle).
+// Deferred update of a panel with kp steps: A[0:n, 0:n] -= U Q^H + Q U^H (lower triangle), one
+// split product of twice the inner length (panel_pack), or two products on the FP64 kernel
+// (which gains nothing from the packing) and in single precision.
 template <typename T>
 void panel_deferred(gks_ctx* c, T* A, int M, int n, int kp, int nk) {
   T* U = at<T>(c, c->oU);
   T* Q = at<T>(c, c->oQ);
   const int ldu = c->nbb;
+  if constexpr (std::is_same<T, double>::value || std::is_same<T, zc>::value)
+    if (n > 0 && split_worth(c, nk, n, n, 2 * kp, sizeof(T), 1)) {
+      T* W = at<T>(c, c->oUQ);
+      {
+        Rec r(c, PC_HETRD_VEC, 0.0, 5.0 * sizeof(T) * n * (double)kp * nk);
+        panel_pack<T>(U, Q, ldu, c->sU, n, kp, W, c->sUQ, nk, c->stream);
+      }
+      gmx<T>(c, nk, OP_N, OP_C, n, n, 2 * kp, -1.0, W, 3 * kp, c->sUQ, W + kp, 3 * kp, c->sUQ, 1.0, A, M, c->sMM, 1);
+      return;
+    }
   gmx<T>(c, nk, OP_N, OP_C, n, n, kp, -1.0, U, ldu, c->sU, Q, ldu, c->sU, 1.0, A, M, c->sMM, 1);
   gmx<T>(c, nk, OP_N, OP_C, n, n, kp, -1.0, Q, ldu, c->sU, U, ldu, c->sU, 1.0, A, M, c->sMM, 1);
 }
 
 // Steps per panel.  The per-step FP64 corrections grow with the panel length, the digits and
-// the deferred update come once per panel.  Reductions in ms at 64 / 96 / 128 steps: complex
-// 1625 (four items) 55.3 / 60.3 / 64.4, 2496 63.2 / 65.3 / 68.3, 4992 242.8 / 237.2 / 238.9; real
-// 832 10.8 / 11.1 / 11.7, 2808 49.9 / 49.6 / 50.2.
+// the deferred update come once per panel.  Reductions in ms at 48 / 64 / 96 / 128 steps: complex
+// 1625 (four items) 52.4 / 52.3 / 57.0 / 61.6, 2496 62.5 / 61.0 / 62.6 / 64.7, 4992 239.5 / 230.6 /
+// 228.8 / 231.4; real 832 11.2 / 11.0 / 11.5 / 12.0, 2808 50.2 / 48.7 / 48.9 / 49.3.
 int panel_width(const gks_ctx* c, int M) {
   return std::min(M < 3072 ? 64 : M < 6144 ? 96 : kPanelMax, c->nbb);
 }

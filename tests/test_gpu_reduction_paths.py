@@ -64,6 +64,19 @@ def test_panel_edges(ctx, cplx, m, nk):
     _check_eigenpairs(H, S, sol.eps.cpu().numpy(), sol.C.cpu().numpy())
 
 
+@pytest.mark.parametrize("cplx,m", [(True, 66), (True, 300), (False, 640)])
+@pytest.mark.parametrize("shift", [-61, 60])
+def test_deferred_update_scales(ctx, cplx, m, shift):
+    """The deferred update as one product with balanced columns: H and 2^shift H give the same
+    eigenvalues up to the scale, within 8 m u ||H|| each."""
+    H, S = _pencils(m, 1, cplx)
+    a, b = (ctx.solve(torch.as_tensor(H * f).cuda(), torch.as_tensor(S).cuda(), 0.1 * f, 0.8 * m).eps.cpu().numpy()[0]
+            for f in (1.0, 2.0 ** shift))
+    assert np.abs(a - b / 2.0 ** shift).max() <= 16 * m * U * 10.0 * np.linalg.norm(H[0], 2)
+    _check_eigenpairs(H, S, a[None], ctx.solve(torch.as_tensor(H).cuda(), torch.as_tensor(S).cuda(), 0.1,
+                                               0.8 * m).C.cpu().numpy())
+
+
 @pytest.mark.parametrize("cplx", [False, True])
 @pytest.mark.parametrize("m,count", [(65, 1), (70, 151), (129, 7), (192, 40), (200, 9), (321, 30)])
 def test_triangular_solves_by_lanes_and_warps(ctx, cplx, m, count):
