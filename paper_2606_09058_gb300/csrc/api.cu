@@ -113,6 +113,7 @@ struct gks_ctx {
   cudaGraphExec_t gexec = nullptr;     // graph of the last captured solve
   SolveKey gkey{};
   std::vector<gks_ctx*> subs;          // per-problem contexts of gks_solve_batched
+  bool batched = false;                // a problem's context of gks_solve_batched
   std::vector<cudaStream_t> workers;   // fork/join streams of gks_solve_batched
   cudaGraphExec_t bexec = nullptr;     // graph of the last captured batch
   std::vector<SolveKey> bkey;
@@ -347,7 +348,7 @@ gks_status ensure_ws(gks_ctx* c, int m, int n, int nk, int es, int nc) {
   c->op = a.take<char>(elems(m));
   c->oph = a.take<char>(elems(m));
   c->otau = a.take<double>((size_t)m * nk);
-  c->otb = a.take<double>((size_t)nbb * nk);
+  c->otb = a.take<double>((size_t)2 * nbb * nk);
   c->od = a.take<double>((size_t)m * nk);
   c->oe = a.take<double>((size_t)m * nk);
   c->oZ = a.take<double>(MM * nk);
@@ -549,7 +550,9 @@ struct StageRec {
 // event.  All of it is captured when the main stream is, and every lane is joined before the
 // stage that forked it returns.  False if streams or events cannot be created: the caller then
 // runs everything on the main stream.
-enum { EV_FORK = 0, EV_LEVEL = 2, EV_OFF = 3, EV_PANEL = 4 };  // forks of lanes 0 and 1, their joins, panels
+// forks of lanes 0 and 1, ends of the reduction's work on them, WY blocks ready (two buffers),
+// buffers free again, panels of the factor
+enum { EV_FORK = 0, EV_LEVEL = 2, EV_OFF = 3, EV_WY = 4, EV_FREE = 6, EV_PANEL = 8 };
 bool lanes_ready(gks_ctx* c, int panels) {
   int lo = 0, hi = 0;
   cudaDeviceGetStreamPriorityRange(&lo, &hi);
@@ -1346,47 +1349,95 @@ void q1_apply_run(gks_ctx* c, const T* A, T* X, int ldx, long long sX, int M, in
   }
 }
 
-// X <- Q X with Q = P_{M-1} ... P_2 (reflectors stored by the reduction), compact WY in
-// blocks of nbb reflectors: B = I - V T V^H.  X is M x ncols (ldx, sX).  T (upper
-// triangular) is assembled from the 64-wide diagonal blocks (larft on G = V^H V) by the merge
+// V and T of block blk (from 0) of the reflectors stored by the reduction, compact WY in blocks
+// of nbb: B = I - V T V^H.  T (upper triangular) is assembled from the 64-wide diagonal blocks
+// (larft on G = V^H V) by the merge
 //   T[:s, s:s+k] = -T[:s, :s] G[:s, s:s+k] T[s:s+k, s:s+k].
+// Two buffers in turn (the reduction's U and Q and the two-sided reduction's FB are free here).
+template <typename T>
+struct WyBlock {
+  T *V, *Tm;
+  double* tb;
+};
+template <typename T>
+WyBlock<T> wy_block(gks_ctx* c, int blk, int nk) {
+  return {at<T>(c, blk & 1 ? c->oU : c->oV), at<T>(c, blk & 1 ? c->oFB : c->oT),
+          at<double>(c, c->otb) + (size_t)(blk & 1) * c->nbb * nk};
+}
 template <typename T, typename TA = T>
-void backtransform_run(gks_ctx* c, const TA* A, T* X, int ldx, long long sX, int M, int ncols, int nk) {
+void wy_prepare(gks_ctx* c, const TA* A, int M, int nk, int blk) {
   cudaStream_t s = c->stream;
   const int nbb = c->nbb;
-  T* V = at<T>(c, c->oV);
+  const WyBlock<T> w = wy_block<T>(c, blk, nk);
   T* G = at<T>(c, c->oG);
-  T* Tm = at<T>(c, c->oT);
-  T* Y = at<T>(c, c->oY);
-  T* Y2 = at<T>(c, c->oY2);
-  double* tau = at<double>(c, c->otau);
-  double* tb = at<double>(c, c->otb);
-  if (M < 3) return;
-  cudaMemsetAsync(Tm, 0, sizeof(T) * (size_t)c->sT * nk, s);
-  for (int j0 = 2; j0 <= M - 1; j0 += nbb) {
-    const int j1 = std::min(j0 + nbb - 1, M - 1), nbk = j1 - j0 + 1;
+  T* P = at<T>(c, c->oQ);
+  const int j0 = 2 + blk * nbb, j1 = std::min(j0 + nbb - 1, M - 1), nbk = j1 - j0 + 1;
+  if (blk < 2) cudaMemsetAsync(w.Tm, 0, sizeof(T) * (size_t)c->sT * nk, s);
+  {
+    Rec r(c, PC_BACKTR_AUX);
+    gather_reflectors<TA, T>(A, M, c->sMM, at<double>(c, c->otau), M, j0, j1, w.V, nbb, c->sV, w.tb, nbb, nk, s);
+  }
+  gmx<T>(c, nk, OP_C, OP_N, nbk, nbk, j1, 1.0, w.V, nbb, c->sV, w.V, nbb, c->sV, 0.0, G, nbb, c->sG);
+  for (int s0 = 0; s0 < nbk; s0 += NB) {
+    const int ks = std::min(NB, nbk - s0);
+    T* Tss = w.Tm + (size_t)s0 * nbb + s0;
     {
       Rec r(c, PC_BACKTR_AUX);
-      gather_reflectors<TA, T>(A, M, c->sMM, tau, M, j0, j1, V, nbb, c->sV, tb, nbb, nk, s);
+      larft<T>(G + (size_t)s0 * nbb + s0, nbb, c->sG, w.tb + s0, nbb, ks, Tss, nbb, c->sT, nk, s);
     }
-    gmx<T>(c, nk, OP_C, OP_N, nbk, nbk, j1, 1.0, V, nbb, c->sV, V, nbb, c->sV, 0.0, G, nbb, c->sG);
-    for (int s0 = 0; s0 < nbk; s0 += NB) {
-      const int ks = std::min(NB, nbk - s0);
-      {
-        Rec r(c, PC_BACKTR_AUX);
-        larft<T>(G + (size_t)s0 * nbb + s0, nbb, c->sG, tb + s0, nbb, ks, Tm + (size_t)s0 * nbb + s0, nbb, c->sT,
-                 nk, s);
-      }
-      if (s0 > 0) {
-        // P = G[:s0, s0:s0+ks] T_ss (P in Y2, ld NB), then T[:s0, s0:s0+ks] = -T[:s0, :s0] P
-        gmx<T>(c, nk, OP_N, OP_N, s0, ks, ks, 1.0, G + s0, nbb, c->sG, Tm + (size_t)s0 * nbb + s0, nbb, c->sT, 0.0,
-               Y2, NB, c->sY);
-        gmx<T>(c, nk, OP_N, OP_N, s0, ks, s0, -1.0, Tm, nbb, c->sT, Y2, NB, c->sY, 0.0, Tm + s0, nbb, c->sT);
-      }
+    if (s0 > 0) {
+      // P = G[:s0, s0:s0+ks] T_ss (ld NB), then T[:s0, s0:s0+ks] = -T[:s0, :s0] P
+      gmx<T>(c, nk, OP_N, OP_N, s0, ks, ks, 1.0, G + s0, nbb, c->sG, Tss, nbb, c->sT, 0.0, P, NB, c->sU);
+      gmx<T>(c, nk, OP_N, OP_N, s0, ks, s0, -1.0, w.Tm, nbb, c->sT, P, NB, c->sU, 0.0, w.Tm + s0, nbb, c->sT);
     }
+  }
+}
+// Blocks first and second on lane 0, from where the main stream stands.
+int wy_blocks(const gks_ctx* c, int M) { return M < 3 ? 0 : (M - 2 + c->nbb - 1) / c->nbb; }
+template <typename T, typename TA = T>
+void wy_ahead(gks_ctx* c, const TA* A, int M, int nk, int blk) {
+  lane_run(c, 0, [&]() {
+    wy_prepare<T, TA>(c, A, M, nk, blk);
+    cudaEventRecord(c->events[EV_WY + (blk & 1)], c->stream);
+  });
+}
+template <typename T, typename TA = T>
+bool wy_start(gks_ctx* c, const TA* A, int M, int nk) {
+  if (wy_blocks(c, M) == 0 || !lanes_ready(c, 0)) return false;
+  lane_fork(c, 0);
+  for (int blk = 0; blk < std::min(2, wy_blocks(c, M)); blk++) wy_ahead<T, TA>(c, A, M, nk, blk);
+  return true;
+}
+
+// X <- Q X with Q = P_{M-1} ... P_2, block by block.  X is M x ncols (ldx, sX).  The blocks' T
+// factors are chains of small kernels: they are made on lane 0, two blocks ahead.  Not in a
+// batch, where other problems fill the GPU and the streams share eight hardware queues (eight
+// uneven systems 36.7 ms without, 45 with), and not before the divide and conquer is done (its
+// leaves, chains of FP64 operations in single warps, then take 1.7 ms instead of 0.2).
+// Measured, whole call, without / with: order 4992 complex 365 / 358 ms, spinor order 2496
+// 101.5 / 98.0, order 2808 real 87.5 / 85.3, order 832 17.9 / 17.7.
+template <typename T, typename TA = T>
+void backtransform_run(gks_ctx* c, const TA* A, T* X, int ldx, long long sX, int M, int ncols, int nk) {
+  const int nbb = c->nbb;
+  T* Y = at<T>(c, c->oY);
+  T* Y2 = at<T>(c, c->oY2);
+  const int blocks = wy_blocks(c, M);
+  if (blocks == 0) return;
+  const bool beside = !c->batched && wy_start<T, TA>(c, A, M, nk);
+  for (int blk = 0; blk < blocks; blk++) {
+    const int j0 = 2 + blk * nbb, j1 = std::min(j0 + nbb - 1, M - 1), nbk = j1 - j0 + 1;
+    const WyBlock<T> w = wy_block<T>(c, blk, nk);
+    const T *V = w.V, *Tm = w.Tm;
+    if (beside) main_wait(c, EV_WY + (blk & 1));
+    else wy_prepare<T, TA>(c, A, M, nk, blk);
     gmx<T>(c, nk, OP_C, OP_N, nbk, ncols, j1, 1.0, V, nbb, c->sV, X, ldx, sX, 0.0, Y, ncols, c->sY);
     gmx<T>(c, nk, OP_N, OP_N, nbk, ncols, nbk, 1.0, Tm, nbb, c->sT, Y, ncols, c->sY, 0.0, Y2, ncols, c->sY);
     gmx<T>(c, nk, OP_N, OP_N, j1, ncols, nbk, -1.0, V, nbb, c->sV, Y2, ncols, c->sY, 1.0, X, ldx, sX);
+    if (beside && blk + 2 < blocks) {
+      cudaEventRecord(c->events[EV_FREE + (blk & 1)], c->stream);
+      cudaStreamWaitEvent(c->lane[0].stream, c->events[EV_FREE + (blk & 1)], 0);
+      wy_ahead<T, TA>(c, A, M, nk, blk + 2);
+    }
   }
 }
 
@@ -1546,6 +1597,9 @@ gks_status solve_t(gks_ctx* c, const SolveKey& key) {
     chol = lanes_ready(c, (n + c->nbb - 1) / c->nbb);
     auto factor = [&]() {
       StageRec sr(c, PS_POTRF);
+      const int rest = n - c->nbb;  // the first trailing update's scratch at once
+      if (rest > 0 && split_worth(c, nk, rest, rest, c->nbb, es, 1))
+        oz_reserve(c, ozaki_workspace_bytes(rest, rest, c->nbb, es == 16, sform(c)), nk);
       potrf_run<T>(c, L, n, n, sLk, nk, [&](int p, int K0, int KB) {
         if (sp) {
           Rec r(c, PC_MISC);
@@ -2098,6 +2152,7 @@ gks_status gks_solve_batched(gks_ctx* ctx, int64_t count, const gks_problem* pro
   while ((int64_t)ctx->subs.size() < count) {
     gks_ctx* sc = new gks_ctx();
     sc->device = ctx->device;
+    sc->batched = true;
     sc->f_cut = ctx->f_cut;
     sc->gemm_mode = ctx->gemm_mode;
     sc->slices = ctx->slices;
