@@ -10,7 +10,9 @@
  *    and row-major.  Complex data is interleaved (re, im) double pairs.
  *  - Hermitian inputs are read from their LOWER triangle only (row >= column).
  *  - M is the matrix order: M = n (collinear, spin-polarized) or 2n (noncollinear).
- *  - All work is enqueued on the stream given at context creation.  gks_solve returns
+ *  - All work is enqueued on the stream given at context creation, and on streams of the
+ *    context's own that fork from it and are joined to it within the call (both are captured
+ *    when that stream is).  gks_solve returns
  *    host-side validation status; device-side failures (S not positive definite, no
  *    convergence, invalid occupation parameters) are returned by gks_sync.
  *  - Errors never cross the ABI as exceptions and never trap on the device.  The text
@@ -51,7 +53,8 @@ typedef enum { GKS_COLLINEAR = 0, GKS_NONCOLLINEAR = 1, GKS_SPIN_POLARIZED = 2 }
 
 /* Arithmetic of the eigensolve.  GKS_FP64: every stage FP64-accurate (products as exact
  * split-bf16 tensor-core products with FP64 accumulation).  GKS_MIXED_SPLITBF16: H' is
- * rounded to single precision and tridiagonalized on the FP32 pipe, the divide and
+ * tridiagonalized in single precision on the FP32 pipe (up to 2.4e8 bytes of H' in the digit
+ * form of gks_hemv on a copy, which is faster there and more accurate), the divide and
  * conquer stays FP64, the back-transform products take 5 digits (about FP32 accuracy),
  * then opts.refine_sweeps Ogita-Aishima sweeps refine every eigenpair of H' with
  * FP64-accurate products (Ogita & Aishima 2018); the Cholesky of S, the reduction to H',
@@ -71,7 +74,7 @@ typedef enum { GKS_REDUCE_CHOLESKY = 0, GKS_REDUCE_LOWDIN = 1 } gks_reduction;
 
 /* Reduction of H' to real tridiagonal form.  GKS_TRIDIAG_ONE_STAGE: Householder steps whose
  * rank-2 updates are deferred over panels and applied as tensor-core products (the
- * matrix-vector half runs on the FP64 pipe).  GKS_TRIDIAG_TWO_STAGE (paper Sec. 6: the
+ * matrix-vector half: gks_hemv).  GKS_TRIDIAG_TWO_STAGE (paper Sec. 6: the
  * one-stage reduction is matrix-vector bound): dense -> band of width opts.band by panel QR
  * with two-sided updates as tensor-core products, band -> tridiagonal by a persistent
  * bulge-chasing kernel (bounded waits), and the back-transform applies the chase's
@@ -94,13 +97,13 @@ typedef enum { GKS_SPLIT_RESIDUES = 0, GKS_SPLIT_DIGITS = 1 } gks_split;
 
 /* The Hermitian matrix-vector step of the one-stage reduction (opts.hemv), about half of
  * the reduction's work and bound by the arithmetic unit that runs it (paper Sec. 6).
- * GKS_HEMV_DIGITS: the stale block of each panel as 8 signed 7-bit digits of Re and Im of
- * every entry (scaled by a power of two of the block's largest entry, 56 bits below it),
- * the vector the same, products of digit pairs up to the 56-bit level as exact 8-bit
- * integer dot products with 32-bit sums, weighted and summed in FP64: the error is that of
- * the 56-bit truncation, relative to the largest entries (normwise).  GKS_HEMV_FP64: FP64
- * multiply-adds (three real products per complex product).  Mixed precision keeps its
- * single-precision step. */
+ * GKS_HEMV_DIGITS: the stale block of each panel, equilibrated symmetrically by powers of
+ * two, as 7 balanced base-256 digits of Re and Im of every entry (54 bits, rounded), the
+ * vector the same, products of digit pairs up to the 2^-56 level as exact 8-bit integer dot
+ * products with 32-bit sums, weighted and summed in FP64: the error is that of the 54-bit
+ * rounding, relative to the equilibrated entries; all steps of a panel run in one
+ * persistent launch.  GKS_HEMV_FP64: FP64 multiply-adds (three real products per complex
+ * product), two launches per step. */
 typedef enum { GKS_HEMV_DIGITS = 0, GKS_HEMV_FP64 = 1 } gks_hemv;
 
 /* gks_solve flags. */
@@ -155,7 +158,8 @@ typedef struct {
                           More occupied states (f >= f_cut) than n_ev is a device-side
                           GKS_EINVAL. */
   long long wait_limit;/* bound of every device-side wait, in SM clock cycles (0 = 2^32,
-                          about two seconds); past it the waiting kernel stops, frees its
+                          about two seconds; the grid barriers of the one-stage reduction
+                          wait at least 2^28); past it the waiting kernel stops, frees its
                           resources and gks_sync returns GKS_ETIMEOUT */
   const char* autotune_cache; /* file of tuned widths: read at gks_create if it exists, rewritten
                           by gks_tune and gks_tune_set; NULL = none.  The string is copied. */

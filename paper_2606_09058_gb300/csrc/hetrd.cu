@@ -12,10 +12,13 @@
 //
 // On GB300 the Hermitian matrix-vector product that dominates each step is bound by the
 // FP64 pipe, not by HBM: a complex element read once feeds two complex multiply-adds
-// (16 flops per 16 bytes), above the DFMA pipe's balance point of ~0.15 flop/byte.  The
-// rank-2 updates are therefore deferred over panels of steps and applied as GEMMs (the
-// panel form below), which the product dispatcher can send to the tensor cores.
+// (16 flops per 16 bytes), above the DFMA pipe's balance point of ~0.15 flop/byte.  It runs
+// as exact 8-bit integer dot products on digits of the panel's stale block (the persistent
+// panel kernel below; two launches per step in FP64 or single precision are the other form),
+// and the rank-2 updates are deferred over panels of steps and applied as products, which
+// the product dispatcher can send to the tensor cores.
 #include <algorithm>
+#include <atomic>
 #include <type_traits>
 
 #include "dense.h"
@@ -1316,11 +1319,22 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
 constexpr int kPanelTiles = 24;
 template <typename T>
 constexpr int kPanelRows = sizeof(T) == 16 ? 8 : 16;
+// Per device, found once: the value of `find` for the current device (kernel attributes are
+// per device too).
+template <typename F>
+static int per_device(std::atomic<int> (&known)[64], F find) {
+  int dev = 0;
+  cudaGetDevice(&dev);
+  if (dev >= 64) return find(dev);
+  int v = known[dev].load();  // value + 1
+  if (v == 0) known[dev].store(v = find(dev) + 1);
+  return v - 1;
+}
 template <typename T>
 static int panel_capacity() {
-  static const int cap = [] {
-    int dev = 0, sms = 0, per = 0;
-    cudaGetDevice(&dev);
+  static std::atomic<int> known[64];
+  return per_device(known, [](int dev) {
+    int sms = 0, per = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     cudaFuncSetAttribute(hetrd_panel_kernel<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          PanelSmem<T>::TOTAL);
@@ -1328,13 +1342,13 @@ static int panel_capacity() {
                                                   PanelSmem<T>::TOTAL);
     cudaGetLastError();
     return sms * (per > 0 ? 1 : 0);
-  }();
-  return cap;
+  });
 }
 // Largest cluster of panel CTAs that can be resident (16, 8 or 0), attributes set.
 template <typename T>
 static int panel_cluster() {
-  static const int best = [] {
+  static std::atomic<int> known[64];
+  return per_device(known, [](int) {
     auto k = hetrd_panel_kernel<T, true>;
     cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, PanelSmem<T>::TOTAL);
     cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
@@ -1354,8 +1368,7 @@ static int panel_cluster() {
       cudaGetLastError();
     }
     return 0;
-  }();
-  return best;
+  });
 }
 
 template <typename T>

@@ -1,5 +1,7 @@
-// FP64-accurate GEMM from exact bf16 tensor-core products (split-integer products in the
-// manner of Ozaki, Ogita, Oishi and Rump's error-free splitting).
+// FP64-accurate GEMM from exact bf16 tensor-core products, in two forms: residues modulo 16
+// coprime moduli and the Chinese remainder theorem (the default; Ozaki, Uchino and Imamura),
+// described at the moduli below, and digit pairs (Ozaki, Ogita, Oishi and Rump's error-free
+// splitting):
 //
 // Each row i of op(A) is scaled by 2^-e_i (e_i = 1 + floor(log2 max_k |a_ik|), so every
 // entry is below 1 in magnitude) and cut into S digits of 6 bits, truncating toward zero:
@@ -17,8 +19,8 @@
 // column 2j+1 = (Im b, Re b); then (A' B')[i][2j] = Re c_ij and [i][2j+1] = Im c_ij.
 //
 // On GB300 the bf16 tensor cores (tcgen05) run the 45 digit products of S = 9 at an
-// FP64-equivalent rate of 13-18 TFLOP/s on large products, against 1.2 TFLOP/s for the
-// FP64 pipe.
+// FP64-equivalent rate of 18 TFLOP/s and the 16 residue products at 73 TFLOP/s on a complex
+// product of order 4096, against 1.06 TFLOP/s for the FP64 pipe.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cudaTypedefs.h>
