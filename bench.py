@@ -704,9 +704,9 @@ def main():
     # launch processes, so the live per-launch algorithmic bytes times that ratio is reported.
     # DRAM bytes / algorithmic bytes of one launch from an ncu capture (profiles/) of the
     # kernel as it stands: the FP64 matrix-vector step (16-row blocks on the 64-atom k-batch)
-    # and its digit form (one k-point of the 512-atom batch, the tiled copy-ring version:
-    # DRAM bytes = the digit block)
-    TRAFFIC_RATIO = {("hetrd_hemv", "fp64"): 1.04, ("hetrd_hemv", "digits"): 1.019}
+    # and the digit form's panel kernel (first panel of one k-point of the 512-atom batch: the
+    # digit blocks and the panel's rows)
+    TRAFFIC_RATIO = {("hetrd_hemv", "fp64"): 1.04, ("hetrd_hemv", "digits"): 1.056}
     kern = [p for p in prof if not p["name"].startswith("stage:")]
     dom = max(kern, key=lambda p: p["ms"]) if kern else None
     roof = None

@@ -29,6 +29,7 @@
 #include <cmath>
 #include <cstdlib>
 #include <mutex>
+#include <type_traits>
 
 #include "dense.h"
 #include "tcgen05.cuh"
@@ -70,10 +71,11 @@ __device__ __forceinline__ float crt_fold(float x, float m, float inv) {
 // into o[0..S); sh = 6S - e (digits) or p - e (residues).  Integer and FP32 operations only
 // (the FP64 pipe takes 1.7 operations per SM clock): u = trunc(|x| 2^sh) is the significand
 // shifted by the exponent difference.
+// cs = 1 or -1 is a further sign (the conjugation's).
 // Digits (RES false): the S base-64 digits of u, most significant first, with x's sign.
 // Residues (RES true): u < 2^62 in 21-bit limbs, reduced modulo each of the first S moduli by
-// Horner's rule in exact FP32 steps (|r| 2^7 + limb < 2^22), then x's sign: symmetric
-// residues |r| <= 128.  11 FP32 operations per modulus in place of five 32-bit integer
+// Horner's rule in exact FP32 steps (|r| 2^7 + |limb| < 2^22), the limbs with x's sign:
+// symmetric residues |r| <= 128.  11 FP32 operations per modulus in place of five 32-bit integer
 // remainders by a constant.
 // With wt (operand B) the residues are those of y_l times the integer, y_l = (M / m_l)^-1 mod
 // m_l in symmetric form: the product's residues then carry the weights of the
@@ -82,16 +84,16 @@ struct CrtWeights {
   float y[CRT_MAXMOD];
 };
 template <bool RES>
-__device__ __forceinline__ void split_vals(double x, int sh, int S, float (&o)[16], const CrtWeights* wt) {
+__device__ __forceinline__ void split_vals(double x, int sh, int S, float cs, float (&o)[16], const CrtWeights* wt) {
   const unsigned long long bits = (unsigned long long)__double_as_longlong(x);
   const int xe = (int)((bits >> 52) & 0x7ff);
   const unsigned long long m = xe == 0x7ff ? 0ull : (bits & 0xfffffffffffffull) | (xe ? (1ull << 52) : 0ull);
   const int s = (xe ? xe : 1) - 1075 + sh;
   const unsigned long long u = s >= 0 ? (s < 64 ? m << s : 0ull) : (s > -64 ? m >> -s : 0ull);
-  const float sg = (bits >> 63) ? -1.0f : 1.0f;
+  const float sg = (bits >> 63) ? -cs : cs;
   if constexpr (RES) {
-    const float a0 = (float)(uint32_t)(u & 0x1fffffull), a1 = (float)(uint32_t)((u >> 21) & 0x1fffffull),
-                a2 = (float)(uint32_t)(u >> 42);
+    const float a0 = sg * (float)(uint32_t)(u & 0x1fffffull), a1 = sg * (float)(uint32_t)((u >> 21) & 0x1fffffull),
+                a2 = sg * (float)(uint32_t)(u >> 42);
 #pragma unroll
     for (int l = 0; l < CRT_MAXMOD; l++) {
       constexpr uint32_t lim = 1u << 21;
@@ -99,7 +101,7 @@ __device__ __forceinline__ void split_vals(double x, int sh, int S, float (&o)[1
       const float mf = (float)mi, inv = 1.0f / mf, w = 2u * wi > mi ? (float)wi - mf : (float)wi;
       const float r2 = crt_fold(a2, mf, inv);
       const float r1 = crt_fold(__fmaf_rn(r2, w, a1), mf, inv);
-      o[l] = sg * crt_fold(__fmaf_rn(r1, w, a0), mf, inv);
+      o[l] = crt_fold(__fmaf_rn(r1, w, a0), mf, inv);
       if (wt) o[l] = crt_fold(o[l] * wt->y[l], mf, inv);
     }
   } else {
@@ -134,12 +136,24 @@ struct SplitOp {
   __nv_bfloat16* D;             // planes [S][rows][Kp], item stride sD, plane stride sstride
   long long sstride, sD;
   __device__ bool contig() const { return (role == 0) == (op == OP_N); }  // k contiguous in memory
+  // element k of vector v, up to signs (KS: scaled by kz)
+  template <bool KS>
   __device__ T at(const T* Xz, const double* kz, int v, int k) const {
     T x = contig() ? Xz[(size_t)v * ld + k] : Xz[(size_t)k * ld + v];
-    if (op == OP_C) x = conjg(x);
-    return kz ? x * kz[k] : x;
+    if constexpr (KS) x = x * kz[k];
+    return x;
   }
+  // the sign of the imaginary part that the conjugation asks for: 1 or -1
+  __device__ float conj_sign() const { return op == OP_C ? -1.0f : 1.0f; }
 };
+// f<true>() with a scaled operand, f<false>() without: the FP64 multiplications (and the
+// conjugation's, moved to the split values' signs) do not reach the unscaled path, whose
+// reading they bound: scale pass of a complex 4096^2 pair 227 us with them, 92 us without.
+template <typename F>
+__device__ __forceinline__ void scaled_or_not(const double* kz, F f) {
+  if (kz) f(std::true_type{});
+  else f(std::false_type{});
+}
 template <typename T>
 struct SplitPair {
   SplitOp<T> o[2];
@@ -166,8 +180,8 @@ __device__ __forceinline__ void emit_pair(const SplitOp<T>& q, __nv_bfloat16* D,
   const CrtWeights* wt = q.role ? &y : nullptr;
   float o0[16], o1[16];
   if constexpr (sizeof(T) == 16) {
-    split_vals<RES>(x0.x, sh, S, o0, wt);
-    split_vals<RES>(x0.y, sh, S, o1, wt);
+    split_vals<RES>(x0.x, sh, S, 1.0f, o0, wt);
+    split_vals<RES>(x0.y, sh, S, q.conj_sign(), o1, wt);
     const size_t k = 2 * ((size_t)k0 + lane);
     if (q.role == 0) {
       store_pair(o0, o1, 1.0f, D + (size_t)v * Kp + k, q.sstride, S);
@@ -176,8 +190,8 @@ __device__ __forceinline__ void emit_pair(const SplitOp<T>& q, __nv_bfloat16* D,
       store_pair(o1, o0, 1.0f, D + (size_t)(2 * v + 1) * Kp + k, q.sstride, S);
     }
   } else {
-    split_vals<RES>(x0, sh, S, o0, wt);
-    split_vals<RES>(x1, sh, S, o1, wt);
+    split_vals<RES>(x0, sh, S, 1.0f, o0, wt);
+    split_vals<RES>(x1, sh, S, 1.0f, o1, wt);
     store_pair(o0, o1, 1.0f, D + (size_t)v * Kp + k0 + 2 * lane, q.sstride, S);
   }
 }
@@ -208,13 +222,15 @@ __global__ void __launch_bounds__(256) oz_scale_kernel(const SplitPair<T> sp, in
       const int v = v0 + vv;
       if (v >= q.nvec) break;
       uint32_t m = 0;
-      for (int k = k0 + lane; k < k1; k += 128) {  // four loads in flight per lane
-        T x[4];
+      scaled_or_not(kz, [&](auto ks) {
+        for (int k = k0 + lane; k < k1; k += 128) {  // four loads in flight per lane
+          T x[4];
 #pragma unroll
-        for (int t = 0; t < 4; t++) x[t] = k + 32 * t < k1 ? q.at(X, kz, v, k + 32 * t) : zero<T>();
+          for (int t = 0; t < 4; t++) x[t] = k + 32 * t < k1 ? q.template at<decltype(ks)::value>(X, kz, v, k + 32 * t) : zero<T>();
 #pragma unroll
-        for (int t = 0; t < 4; t++) m = max(m, mag_key(x[t]));
-      }
+          for (int t = 0; t < 4; t++) m = max(m, mag_key(x[t]));
+        }
+      });
       m = __reduce_max_sync(0xffffffffu, m);
       if (lane == 0) put(v, m);
     }
@@ -222,13 +238,15 @@ __global__ void __launch_bounds__(256) oz_scale_kernel(const SplitPair<T> sp, in
     uint32_t m = 0;
     const int v = v0 + lane;
     if (v < q.nvec)
-      for (int k = k0 + warp; k < k1; k += 64) {  // eight loads in flight per lane
-        T x[8];
+      scaled_or_not(kz, [&](auto ks) {
+        for (int k = k0 + warp; k < k1; k += 64) {  // eight loads in flight per lane
+          T x[8];
 #pragma unroll
-        for (int t = 0; t < 8; t++) x[t] = k + 8 * t < k1 ? q.at(X, kz, v, k + 8 * t) : zero<T>();
+          for (int t = 0; t < 8; t++) x[t] = k + 8 * t < k1 ? q.template at<decltype(ks)::value>(X, kz, v, k + 8 * t) : zero<T>();
 #pragma unroll
-        for (int t = 0; t < 8; t++) m = max(m, mag_key(x[t]));
-      }
+          for (int t = 0; t < 8; t++) m = max(m, mag_key(x[t]));
+        }
+      });
     pm[warp][lane] = m;
     __syncthreads();
     if (warp == 0 && v < q.nvec) {
@@ -264,23 +282,25 @@ __global__ void __launch_bounds__(256) oz_split_kernel(const SplitPair<T> sp, in
   const double* kz = q.ksc ? q.ksc + z * q.sks : nullptr;
   const int* ex = q.ex + z * q.sE;
   __nv_bfloat16* D = q.D + z * q.sD;
-  if (q.contig()) {  // lanes along k
+  scaled_or_not(kz, [&](auto ks) {
+    if (q.contig()) {  // lanes along k
 #pragma unroll
-    for (int w = 0; w < 4; w++) {
-      const int vv = warp + 8 * w, v = v0 + vv;
+      for (int w = 0; w < 4; w++) {
+        const int vv = warp + 8 * w, v = v0 + vv;
 #pragma unroll
-      for (int t = 0; t < TK; t += 32) {
-        const int k = k0 + t + lane;
-        tile[t + lane][vv] = (v < q.nvec && k < K) ? q.at(X, kz, v, k) : zero<T>();
+        for (int t = 0; t < TK; t += 32) {
+          const int k = k0 + t + lane;
+          tile[t + lane][vv] = (v < q.nvec && k < K) ? q.template at<decltype(ks)::value>(X, kz, v, k) : zero<T>();
+        }
+      }
+    } else {  // lanes along the vectors
+#pragma unroll
+      for (int w = 0; w < TK / 8; w++) {
+        const int kk = warp + 8 * w, k = k0 + kk, v = v0 + lane;
+        tile[kk][lane] = (k < K && v < q.nvec) ? q.template at<decltype(ks)::value>(X, kz, v, k) : zero<T>();
       }
     }
-  } else {  // lanes along the vectors
-#pragma unroll
-    for (int w = 0; w < TK / 8; w++) {
-      const int kk = warp + 8 * w, k = k0 + kk, v = v0 + lane;
-      tile[kk][lane] = (k < K && v < q.nvec) ? q.at(X, kz, v, k) : zero<T>();
-    }
-  }
+  });
   __syncthreads();
 #pragma unroll 1
   for (int vv = warp; vv < 32; vv += 8) {
@@ -311,16 +331,19 @@ __global__ void __launch_bounds__(256) oz_fused_kernel(const SplitPair<T> sp, in
   if (kdev) K = min(K, max(0, kdev[z]));
   const T* X = q.X + item_off(z, q.sX, q.sX2, nb2);
   const double* kz = q.ksc ? q.ksc + z * q.sks : nullptr;
-  if (q.contig()) {
-    const int v = v0 + warp;
+  scaled_or_not(kz, [&](auto ks) {
+    if (q.contig()) {
+      const int v = v0 + warp;
 #pragma unroll 4
-    for (int k = lane; k < kpl; k += 32) rows[warp * ldk + k] = (v < q.nvec && k < K) ? q.at(X, kz, v, k) : zero<T>();
-  } else {
-    const int v = v0 + (tid & 7);
+      for (int k = lane; k < kpl; k += 32)
+        rows[warp * ldk + k] = (v < q.nvec && k < K) ? q.template at<decltype(ks)::value>(X, kz, v, k) : zero<T>();
+    } else {
+      const int v = v0 + (tid & 7);
 #pragma unroll 4
-    for (int k = tid >> 3; k < kpl; k += 32)
-      rows[(tid & 7) * ldk + k] = (v < q.nvec && k < K) ? q.at(X, kz, v, k) : zero<T>();
-  }
+      for (int k = tid >> 3; k < kpl; k += 32)
+        rows[(tid & 7) * ldk + k] = (v < q.nvec && k < K) ? q.template at<decltype(ks)::value>(X, kz, v, k) : zero<T>();
+    }
+  });
   __syncthreads();
   const int v = v0 + warp;
   if (v >= q.nvp) return;
