@@ -929,34 +929,43 @@ struct CrtRecon {
   int n;
 };
 
-// 128-bit magnitude (hi, lo) times 2^e to the nearest double (ties to even), from its bits
-// (through ldexp only where the result leaves the normal range).
-__device__ __forceinline__ double u128_scaled(unsigned long long hi, unsigned long long lo, bool neg, int e) {
-  if (hi == 0ull && lo == 0ull) return 0.0;
-  const int lz = hi ? __clzll((long long)hi) : 64 + __clzll((long long)lo);
-  unsigned long long h, l;
-  if (lz == 0) {
-    h = hi;
-    l = lo;
-  } else if (lz < 64) {
-    h = (hi << lz) | (lo >> (64 - lz));
-    l = lo << lz;
+// 128-bit magnitude (w3 the top word) times 2^e to the nearest double (ties to even), from its
+// bits: h the 64 bits from the leading one, l what is left of them, the 53-bit mantissa's
+// leading one and a rounding carry added into the exponent (through ldexp only where the
+// result leaves the normal range).  Most values fill the top word.
+__device__ __forceinline__ double u128_scaled(uint32_t w3, uint32_t w2, uint32_t w1, uint32_t w0, bool neg, int e) {
+  uint32_t h1, h0, l = 0;
+  int lz;
+  if (w3) {
+    lz = __clz((int)w3);
+    h1 = __funnelshift_l(w2, w3, lz);
+    h0 = __funnelshift_l(w1, w2, lz);
+    l = __funnelshift_l(w0, w1, lz) | (w0 << lz);
+  } else if (w2) {
+    lz = __clz((int)w2);
+    h1 = __funnelshift_l(w1, w2, lz);
+    h0 = __funnelshift_l(w0, w1, lz);
+    l = w0 << lz;
+    lz += 32;
+  } else if (w1) {
+    lz = __clz((int)w1);
+    h1 = __funnelshift_l(w0, w1, lz);
+    h0 = w0 << lz;
+    lz += 64;
   } else {
-    h = lo << (lz - 64);
-    l = 0ull;
+    if (!w0) return 0.0;
+    lz = __clz((int)w0);
+    h1 = w0 << lz;
+    h0 = 0;
+    lz += 96;
   }
-  unsigned long long mant = h >> 11;  // 53 significant bits
-  const unsigned long long rest = h & 0x7ffull;
-  if (rest > 0x400ull || (rest == 0x400ull && (l != 0ull || (mant & 1ull)))) mant++;
-  int ex = 127 - lz;  // position of the leading bit
-  if (mant >> 53) {
-    mant >>= 1;
-    ex++;
-  }
-  const unsigned long long sgn = neg ? 1ull << 63 : 0ull, frac = mant & ((1ull << 52) - 1);
-  const int be = ex + e + 1023;
-  if (be > 0 && be < 2047) return __longlong_as_double((long long)(sgn | ((unsigned long long)be << 52) | frac));
-  return ldexp(__longlong_as_double((long long)(sgn | ((unsigned long long)(ex + 1023) << 52) | frac)), e);
+  const uint32_t rest = ((h0 & 0x7ffu) << 1) | (l != 0u), odd = (h0 >> 11) & 1u;
+  const unsigned long long mant = (((unsigned long long)(h1 >> 11) << 32) | __funnelshift_r(h0, h1, 11)) +
+                                  (rest + odd > 0x800u ? 1ull : 0ull);
+  const int be = 127 - lz + 1022;  // the exponent field below the leading one of mant
+  const unsigned long long sgn = neg ? 1ull << 63 : 0ull;
+  if ((unsigned)(be + e) < 2046u) return __longlong_as_double((long long)(sgn | (((unsigned long long)(be + e) << 52) + mant)));
+  return ldexp(__longlong_as_double((long long)(sgn | (((unsigned long long)be << 52) + mant))), e);
 }
 
 // The signed integer X of the bytes of element el, as a double times 2^e.  S is
@@ -997,7 +1006,7 @@ __device__ __forceinline__ double crt_value(const uint32_t (&w)[CRT_MAXMOD][2], 
     lo = 0ull - lo;
     hi = ~hi + (lo == 0ull ? 1ull : 0ull);
   }
-  return u128_scaled(hi, lo, neg, e);
+  return u128_scaled((uint32_t)(hi >> 32), (uint32_t)hi, (uint32_t)(lo >> 32), (uint32_t)lo, neg, e);
 }
 
 // C = alpha 2^{e_i + f_j - 2p} X + beta C for the logical outputs (lower: j <= i only).
