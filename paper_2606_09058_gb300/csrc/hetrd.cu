@@ -436,6 +436,8 @@ __global__ void __launch_bounds__(256) hetrd_dmax_kernel(const T* A, int lda, lo
 // hetrd_digits_kernel: 32 x 32 tiles of the full Hermitian [0:n16, 0:n16] (zero outside
 // [0:n, 0:n]); tiles above the diagonal come from the transposed lower tile through shared
 // memory, conjugated.  64 threads: thread t packs row t / 2, columns 16 (t % 2) .. + 15.
+// Bound by integer operations once the tile's loads are in flight together (order 4992 complex:
+// 349 us with one load at a time, 246 us with eight).
 template <typename T>
 __global__ void __launch_bounds__(64) hetrd_digits_kernel(const T* A, int lda, long long sA, int n, HemvDigits hd) {
   constexpr int NPL = sizeof(T) == 16 ? 2 * kDig : kDig;
@@ -448,7 +450,8 @@ __global__ void __launch_bounds__(64) hetrd_digits_kernel(const T* A, int lda, l
   const bool upper = C0 > R0;
   // source tile: (R0, C0) itself, or (C0, R0) for tiles above the diagonal
   const int sr0 = upper ? C0 : R0, sc0 = upper ? R0 : C0;
-  for (int e = tid; e < 32 * 32; e += 64) {
+#pragma unroll 8
+  for (int e = tid; e < 32 * 32; e += 64) {  // eight loads in flight
     const int yy = e >> 5, xx = e & 31;
     const int r = sr0 + yy, c = sc0 + xx;
     tile[yy][xx] = (r < n && c < n && c <= r) ? A[(size_t)r * lda + c] : zero<T>();
@@ -1582,14 +1585,14 @@ void widen_copy(const T* src, TV* dst, long long n, cudaStream_t s) {
 // W = [U 2^h | Q 2^-h | U 2^h] (n rows of 3 kp), h per column the power of two that brings
 // the column's largest entries of U and Q together: the deferred update U Q^H + Q U^H is then
 // one product W[:, 0:2kp] W[:, kp:3kp]^H whose rows are scaled as the two products' rows were.
-// CTAs of 64 bytes of a row; the second reading comes from L2.  HBM-bound (5 entries moved per
+// CTAs of 32 bytes of a row; the second reading comes from L2.  HBM-bound (5 entries moved per
 // entry of U); the update's reconstruction and C traffic halve: reduction of order 4992 complex
 // 235.7 -> 229.5 ms, four of 1625 54.6 -> 52.5, order 2808 real 50.3 -> 48.8.
-constexpr int kPackThreads = 512;
+constexpr int kPackThreads = 1024;
 template <typename T>
 __global__ void __launch_bounds__(kPackThreads) panel_pack_kernel(const T* U, const T* Q, int ldu, long long sU, int n,
                                                                   int kp, T* W, long long sW) {
-  constexpr int C = 64 / sizeof(T);
+  constexpr int C = 32 / sizeof(T);
   __shared__ int top[2][C];
   const int z = blockIdx.y, c = threadIdx.x % C, k = blockIdx.x * C + c, r0 = threadIdx.x / C;
   U += z * sU;
@@ -1600,7 +1603,7 @@ __global__ void __launch_bounds__(kPackThreads) panel_pack_kernel(const T* U, co
   auto mag = [](T v) { return max(__double2hiint(fabs(re(v))), __double2hiint(fabs(im(v)))); };
   if (k < kp) {
     int mu = 0, mq = 0;
-#pragma unroll 4
+#pragma unroll 8
     for (int r = r0; r < n; r += kPackThreads / C) {
       mu = max(mu, mag(U[(size_t)r * ldu + k]));
       mq = max(mq, mag(Q[(size_t)r * ldu + k]));
@@ -1626,7 +1629,7 @@ __global__ void __launch_bounds__(kPackThreads) panel_pack_kernel(const T* U, co
 template <typename T>
 void panel_pack(const T* U, const T* Q, int ldu, long long sU, int n, int kp, T* W, long long sW, int count,
                 cudaStream_t s) {
-  constexpr int C = 64 / sizeof(T);
+  constexpr int C = 32 / sizeof(T);
   count_launch();
   panel_pack_kernel<T><<<dim3((kp + C - 1) / C, count), kPackThreads, 0, s>>>(U, Q, ldu, sU, n, kp, W, sW);
 }
