@@ -51,27 +51,22 @@ __device__ __forceinline__ int deq(unsigned long long bits) { return (bscale(bit
 constexpr int kDig = 7;
 constexpr int kMaxLevel = 7;  // digit pairs s + t <= kMaxLevel
 
-// The digits of x below 2^e into d[0..kDig), most significant first.  Integer operations on
+// The digits of x below 2^e as the bytes of one word.  Integer operations on
 // the bits of x only (the FP64 pipe is slow on this GPU): |x| = m 2^{x_e - 1075} with the
 // 53-bit significand m, so trunc(|x| 2^{55 - e}) = m shifted by x_e - 1020 - e, and
-// rounding halves it with a carry.  Balanced digits from the least significant up keep the
-// leading one within [-65, 65].
-__device__ __forceinline__ void digits8(double x, int e, int (&d)[kDig]) {
+// rounding halves it with a carry.  The balanced digits d_s, least significant d_{kDig-1} in
+// byte 0, are the bytes of v + sum 128 256^i less 128 each (a flipped top bit); the leading
+// one, in byte 6, stays within [-65, 65] and needs neither.
+__device__ __forceinline__ unsigned long long digit_bytes(double x, int e) {
+  constexpr unsigned long long bias = 0x0000808080808080ull;
+  static_assert(kDig == 7, "six balanced bytes below the leading one");
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
   const int xe = (int)((b >> 52) & 0x7ff);
   const unsigned long long m = (b & 0xfffffffffffffull) | (xe ? (1ull << 52) : 0ull);
   const int sh = (xe ? xe : 1) - 1020 - e;
   const unsigned long long q2 = sh >= 0 ? (m << sh) : (sh > -64 ? (m >> -sh) : 0ull);
-  const long long q = (long long)((q2 + 1) >> 1);
-  long long v = (b >> 63) ? -q : q;
-#pragma unroll
-  for (int s = kDig - 1; s >= 1; s--) {
-    int t = (int)(v & 255);
-    t = t >= 128 ? t - 256 : t;
-    d[s] = t;
-    v = (v - t) >> 8;
-  }
-  d[0] = (int)v;
+  const unsigned long long q = (q2 + 1) >> 1;
+  return (((b >> 63) ? 0ull - q : q) + bias) ^ bias;
 }
 
 // |Re|, |Im| maximum of a value as the bits of a non-negative double (bits of non-negative
@@ -91,25 +86,36 @@ __device__ __forceinline__ unsigned long long maxbits(T a) {
 template <typename T, int NPL>
 __device__ __forceinline__ void store_digit_block(const T (&vals)[16], const int (&e)[16], signed char* dst) {
   uint4 o[NPL];
-#pragma unroll
-  for (int q = 0; q < NPL; q++) o[q] = make_uint4(0u, 0u, 0u, 0u);
-  auto put = [&](int plane, int el, int dv) {
-    const uint32_t bb = (uint32_t)(dv & 0xff) << (8 * (el & 3));
-    if ((el >> 2) == 0) o[plane].x |= bb;
-    else if ((el >> 2) == 1) o[plane].y |= bb;
-    else if ((el >> 2) == 2) o[plane].z |= bb;
-    else o[plane].w |= bb;
+  auto put = [&](int plane, int w, uint32_t v) {
+    if (w == 0) o[plane].x = v;
+    else if (w == 1) o[plane].y = v;
+    else if (w == 2) o[plane].z = v;
+    else o[plane].w = v;
+  };
+  // digits first .. first - 3 of four elements, whose bytes are 0 .. 3 of x0 .. x3: a 4 x 4
+  // byte transpose, one word per plane
+  auto put4 = [&](int base, int first, int w, uint32_t x0, uint32_t x1, uint32_t x2, uint32_t x3) {
+    const uint32_t a = __byte_perm(x0, x1, 0x5140), b = __byte_perm(x2, x3, 0x5140);
+    const uint32_t c = __byte_perm(x0, x1, 0x7362), d = __byte_perm(x2, x3, 0x7362);
+    put(base + first, w, __byte_perm(a, b, 0x5410));
+    put(base + first - 1, w, __byte_perm(a, b, 0x7632));
+    put(base + first - 2, w, __byte_perm(c, d, 0x5410));
+    if (first > 2) put(base + first - 3, w, __byte_perm(c, d, 0x7632));
+  };
+  auto put7 = [&](int base, int w, const unsigned long long (&d)[4]) {
+    put4(base, 6, w, (uint32_t)d[0], (uint32_t)d[1], (uint32_t)d[2], (uint32_t)d[3]);
+    put4(base, 2, w, (uint32_t)(d[0] >> 32), (uint32_t)(d[1] >> 32), (uint32_t)(d[2] >> 32), (uint32_t)(d[3] >> 32));
   };
 #pragma unroll
-  for (int el = 0; el < 16; el++) {
-    int d[kDig];
-    digits8((double)re(vals[el]), e[el], d);
+  for (int w = 0; w < 4; w++) {
+    unsigned long long d[4];
 #pragma unroll
-    for (int sp = 0; sp < kDig; sp++) put(sp, el, d[sp]);
+    for (int q = 0; q < 4; q++) d[q] = digit_bytes((double)re(vals[4 * w + q]), e[4 * w + q]);
+    put7(0, w, d);
     if constexpr (NPL == 2 * kDig) {
-      digits8((double)im(vals[el]), e[el], d);
 #pragma unroll
-      for (int sp = 0; sp < kDig; sp++) put(kDig + sp, el, d[sp]);
+      for (int q = 0; q < 4; q++) d[q] = digit_bytes((double)im(vals[4 * w + q]), e[4 * w + q]);
+      put7(kDig, w, d);
     }
   }
   uint4* out = reinterpret_cast<uint4*>(dst);
@@ -436,8 +442,9 @@ __global__ void __launch_bounds__(256) hetrd_dmax_kernel(const T* A, int lda, lo
 // hetrd_digits_kernel: 32 x 32 tiles of the full Hermitian [0:n16, 0:n16] (zero outside
 // [0:n, 0:n]); tiles above the diagonal come from the transposed lower tile through shared
 // memory, conjugated.  64 threads: thread t packs row t / 2, columns 16 (t % 2) .. + 15.
-// Bound by integer operations once the tile's loads are in flight together (order 4992 complex:
-// 349 us with one load at a time, 246 us with eight).
+// Bound by integer operations and HBM once the tile's loads are in flight together (order 4992
+// complex: 349 us with one load at a time, 246 us with eight, 144 us with the digits as the bytes of one
+// biased word and byte transposes).
 template <typename T>
 __global__ void __launch_bounds__(64) hetrd_digits_kernel(const T* A, int lda, long long sA, int n, HemvDigits hd) {
   constexpr int NPL = sizeof(T) == 16 ? 2 * kDig : kDig;
@@ -972,13 +979,12 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
             }
           }
           vfetch(t + 8);
-          int d[kDig];
-          digits8(xv, xe, d);
+          const unsigned long long d = digit_bytes(xv, xe);
           unsigned char* ub = ubuf + (warp * 2 + (i & 1)) * (NPL * 16);
           if (CPX || lane < 16) {
 #pragma unroll
             for (int q = 0; q < kDig; q++)
-              ub[((lane >> 4) * kDig + q) * 16 + (lane & 15)] = (unsigned char)(d[q] & 0xff);
+              ub[((lane >> 4) * kDig + q) * 16 + (lane & 15)] = (unsigned char)(d >> (8 * (kDig - 1 - q)));
           }
           __syncwarp();  // the digits are written, and every lane is done with the stage refilled next
           issue(C, t + 8 * (STG - 1), t1, i + STG - 1);
