@@ -681,6 +681,13 @@ constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >
 static_assert(SMEM <= 227 * 1024, "shared memory of the residue kernel");
 }  // namespace crtc
 
+// Whether one fold of a chunk sum (|x| <= 2^24) fits the stored byte.  The quotient may miss by
+// one next to a half (1 / m is rounded: an error up to 0.004 at |x / m| = 65793), which leaves
+// |r| = (m + 1) / 2: 127 at most from modulus 253 down, but 128 for 255, where the byte stands
+// for -128, congruent modulo 256 only.  Modulus 256 divides exactly.  A second fold (|x| < 2^14)
+// has the exact quotient.
+__host__ __device__ constexpr bool crt_one_fold(int l) { return crt_mod(l) == 256u || crt_mod(l) <= 253u; }
+
 // Four symmetric residues as bytes r + 128 (r = 128, modulus 256 only, wraps to -128): adding
 // 1.5 * 2^23 leaves r in the low bits of the float, so no conversion instruction is needed.
 __device__ __forceinline__ uint32_t crt_bytes(float r0, float r1, float r2, float r3) {
@@ -834,7 +841,7 @@ __global__ void __launch_bounds__(tcg::THREADS, 1)
       auto put = [&](int word, uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3) {
         out[lane * 8 + (word ^ (lane & 7))] = make_uint4(w0, w1, w2, w3);
       };
-      if (nchunk == 1) {  // K' <= 1024: every accumulator folds straight to its bytes
+      if (nchunk == 1 && crt_one_fold(l)) {  // K' <= 1024: the accumulator folds straight to its bytes
         const int b = u & 1;
         const uint32_t uph = (uint32_t)((u >> 1) & 1);
         u++;
