@@ -205,9 +205,13 @@ void release_aws(gks_ctx* c) {
   c->am = -1;
 }
 
-void release_graph(gks_ctx* c) {
+void release_solve_graph(gks_ctx* c) {
   if (c->gexec) cudaGraphExecDestroy(c->gexec);
   c->gexec = nullptr;
+}
+
+void release_graph(gks_ctx* c) {
+  release_solve_graph(c);
   if (c->bexec) cudaGraphExecDestroy(c->bexec);
   c->bexec = nullptr;
   c->bkey.clear();
@@ -600,7 +604,9 @@ int oz_reserve(gks_ctx* c, size_t item, int count) {
   // grown in doublings: each growth waits for the stream
   const size_t need = item * per, want = std::max(need, std::min(2 * c->oz_bytes, kOzCap));
   if (need > c->oz_bytes) {
+    // a captured solve holds the buffer's address (c->oz may be a lane's): it is captured anew
     cudaStreamSynchronize(c->stream);
+    release_solve_graph(c);
     release_oz(c);
     if (cudaMalloc(&c->oz, want) == cudaSuccess) {
       c->oz_bytes = want;
