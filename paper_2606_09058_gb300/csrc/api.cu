@@ -110,8 +110,10 @@ struct gks_ctx {
     size_t oz_bytes = 0;
   } lane[2];
   std::vector<cudaEvent_t> events;
-  cudaGraphExec_t gexec = nullptr;     // graph of the last captured solve
-  SolveKey gkey{};
+  cudaGraphExec_t gexec = nullptr;     // graph of the solve with key gkey
+  bool capturing = false;              // inside capture(): nothing may be allocated or freed
+  bool short_scratch = false;          // a product of the capture found its scratch too small
+  SolveKey gkey{};                     // graph mode: the last solve that ran on this workspace
   std::vector<gks_ctx*> subs;          // per-problem contexts of gks_solve_batched
   bool batched = false;                // a problem's context of gks_solve_batched
   std::vector<cudaStream_t> workers;   // fork/join streams of gks_solve_batched
@@ -247,6 +249,7 @@ void release_extra(gks_ctx* c) {
 
 void release_ws(gks_ctx* c) {
   release_graph(c);
+  c->gkey = SolveKey{};
   c->l_valid = false;
   if (c->ws) cudaFree(c->ws);
   if (c->st) cudaFree(c->st);
@@ -289,15 +292,25 @@ int mixed_form(const gks_ctx* c, int m, int nk, int es) {
   return (double)m * m * nk * es <= kMixedDigitBytes ? 2 : 1;
 }
 
+// What the context's options make of a shape, and whether its workspace is of that kind.
+struct WsForm {
+  int width, mixed, two, dig;
+};
+WsForm ws_form(const gks_ctx* c, int m, int nk, int es, int nc) {
+  const int mixed = mixed_form(c, m, nk, es);
+  return {pick_width(c, m, es, shape_spin(nc)), mixed, c->tridiag == GKS_TRIDIAG_TWO_STAGE ? c->band : 0,
+          (c->hemv == 0 && !mixed) || mixed == 2 ? 1 : 0};
+}
+bool ws_matches(const gks_ctx* c, int m, int n, int nk, int es, int nc) {
+  const WsForm f = ws_form(c, m, nk, es, nc);
+  return c->ws && c->m == m && c->n == n && c->nk == nk && c->es == es && c->nc == nc && c->nbb == f.width &&
+         c->wsmixed == f.mixed && c->wstwo == f.two && c->wsdig == f.dig;
+}
+
 // Workspace for nk items of order m (element size es, n = basis per spin, nc = spin mode).
 gks_status ensure_ws(gks_ctx* c, int m, int n, int nk, int es, int nc) {
-  const int want = pick_width(c, m, es, shape_spin(nc));
-  const int mixed = mixed_form(c, m, nk, es);
-  const int two = c->tridiag == GKS_TRIDIAG_TWO_STAGE ? c->band : 0;
-  const int dig = (c->hemv == 0 && !mixed) || mixed == 2 ? 1 : 0;
-  if (c->ws && c->m == m && c->n == n && c->nk == nk && c->es == es && c->nc == nc && c->nbb == want &&
-      c->wsmixed == mixed && c->wstwo == two && c->wsdig == dig)
-    return GKS_OK;
+  if (ws_matches(c, m, n, nk, es, nc)) return GKS_OK;
+  const auto [want, mixed, two, dig] = ws_form(c, m, nk, es, nc);
   release_ws(c);
   c->nbb = want;
   const size_t MM = (size_t)m * m;
@@ -603,6 +616,10 @@ int oz_reserve(gks_ctx* c, size_t item, int count) {
   const int nch = (count + maxper - 1) / maxper, per = (count + nch - 1) / nch;
   // grown in doublings: each growth waits for the stream
   const size_t need = item * per, want = std::max(need, std::min(2 * c->oz_bytes, kOzCap));
+  if (need > c->oz_bytes && c->capturing) {
+    c->short_scratch = true;  // the graph is dropped and the call runs eagerly
+    return 0;
+  }
   if (need > c->oz_bytes) {
     // a captured solve holds the buffer's address (c->oz may be a lane's): it is captured anew
     cudaStreamSynchronize(c->stream);
@@ -1926,7 +1943,9 @@ gks_status enqueue_solve(gks_ctx* ctx, const SolveKey& k) {
 
 bool same_key(const SolveKey& a, const SolveKey& b) { return std::memcmp(&a, &b, sizeof(SolveKey)) == 0; }
 
-// Capture whatever `body` enqueues on c->stream into a graph and instantiate it.
+// Capture whatever `body` enqueues on c->stream into a graph and instantiate it.  *out stays
+// null where the scratch that the eager run left does not do (an allocation failed then): the
+// caller runs eagerly.
 template <typename F>
 gks_status capture(gks_ctx* c, cudaGraphExec_t* out, F body) {
   const bool prof_on = c->prof.on;
@@ -1936,10 +1955,22 @@ gks_status capture(gks_ctx* c, cudaGraphExec_t* out, F body) {
     c->prof.on = prof_on;
     return cuda_check(c, "graph capture begin");
   }
+  auto mark = [c](bool on) {
+    c->capturing = on;
+    for (auto* sc : c->subs) sc->capturing = on;
+  };
+  mark(true);
   gks_status rc = body();
+  mark(false);
   cudaError_t e = cudaStreamEndCapture(c->stream, &g);
   c->prof.on = prof_on;
-  if (rc) {
+  bool dropped = c->short_scratch;
+  c->short_scratch = false;
+  for (auto* sc : c->subs) {
+    dropped = dropped || sc->short_scratch;
+    sc->short_scratch = false;
+  }
+  if (rc || dropped) {
     if (g) cudaGraphDestroy(g);
     return rc;
   }
@@ -2115,23 +2146,26 @@ gks_status gks_solve(gks_ctx* ctx, const void* H, const void* S, int64_t n, int6
   const int M = spin_mode == GKS_NONCOLLINEAR ? (int)(2 * n) : (int)n;
   const int items = spin_mode == GKS_SPIN_POLARIZED ? (int)(2 * nk) : (int)nk;
   const int es = dtype == GKS_R64 ? 8 : 16;
-  // capture only when the workspace (order, batch, type and width) and the saved copies
-  // are already in place, so that nothing is allocated or freed while the stream is being
-  // captured
+  // capture only when the solve before ran the same path (shape, flags, and the H and C it
+  // used) and its workspace and saved copies are still in place, so that nothing is allocated
+  // or freed while the stream is being captured
   const bool saved_ok = !(flags & GKS_SAVE_FOR_BACKWARD) ||
                         (ctx->sv_valid && ctx->svkey.n == k.n && ctx->svkey.nk == k.nk &&
                          ctx->svkey.dtype == k.dtype && ctx->svkey.spin == k.spin);
-  const bool ready = ctx->ws && ctx->m == M && ctx->nk == items && ctx->es == es &&
-                     ctx->nbb == pick_width(ctx, M, es, shape_spin(spin_mode)) && ctx->gkey.H == k.H && ctx->gkey.C == k.C &&
-                     saved_ok;
+  const SolveKey& g = ctx->gkey;
+  const bool ready = ws_matches(ctx, M, (int)n, items, es, spin_mode) && g.H == k.H && g.C == k.C && g.n == k.n &&
+                     g.nk == k.nk && g.dtype == k.dtype && g.spin == k.spin && g.flags == k.flags && saved_ok;
+  release_solve_graph(ctx);
+  auto eager = [&]() {
+    const gks_status r = enqueue_solve(ctx, k);
+    ctx->gkey = r ? SolveKey{} : k;
+    return r;
+  };
+  if (!ready) return eager();
   ctx->gkey = k;
-  if (ctx->gexec) {
-    cudaGraphExecDestroy(ctx->gexec);
-    ctx->gexec = nullptr;
-  }
-  if (!ready) return enqueue_solve(ctx, k);
   rc = capture(ctx, &ctx->gexec, [&]() { return enqueue_solve(ctx, k); });
   if (rc) return rc;
+  if (!ctx->gexec) return eager();
   cudaGraphLaunch(ctx->gexec, ctx->stream);
   return cuda_check(ctx, "graph launch");
 }
@@ -2224,6 +2258,10 @@ gks_status gks_solve_batched(gks_ctx* ctx, int64_t count, const gks_problem* pro
   }
   gks_status rc = capture(ctx, &ctx->bexec, body);
   if (rc) return rc;
+  if (!ctx->bexec) {
+    rc = body();
+    return rc ? rc : cuda_check(ctx, "gks_solve_batched launch");
+  }
   cudaGraphLaunch(ctx->bexec, ctx->stream);
   return cuda_check(ctx, "batch graph launch");
 }

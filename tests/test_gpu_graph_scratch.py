@@ -82,3 +82,36 @@ def test_captured_eigenpairs_between_larger_calls(lib, n, cplx):
         c.occupy()
         c.solve(True)
     c.stream.synchronize()
+
+
+@pytest.mark.parametrize("cplx", [False, True])
+@pytest.mark.parametrize("n", [416, 832])
+def test_full_solve_after_captured_eigenpairs(lib, n, cplx):
+    """Another path on the same buffers runs eagerly before it is captured, also after other
+    entry points have replaced the workspace."""
+    c = _Case(lib, n, cplx)
+    with torch.cuda.stream(c.stream):
+        for _ in range(3):
+            c.solve(True)
+        for _ in range(3):
+            c.solve(False)
+        for _ in range(3):
+            c.solve(False, reuse_s=True)
+        c.solve(True)
+        c.graph.potrf(c.S.clone())
+        c.graph.potrf(torch.eye(40, dtype=c.S.dtype, device="cuda")[None].contiguous())
+        c.graph.potrf(c.S.clone())
+        for _ in range(3):
+            c.solve(True)
+    c.stream.synchronize()
+
+
+def test_workspace_of_another_form_between_solves(lib):
+    c = _Case(lib, 160, False)
+    with torch.cuda.stream(c.stream):
+        for _ in range(3):
+            c.solve(False)
+        c.graph.he2hb(c.H.clone(), 16)
+        for _ in range(3):
+            c.solve(False)
+    c.stream.synchronize()
