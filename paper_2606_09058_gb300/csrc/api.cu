@@ -2812,6 +2812,10 @@ gks_status gks_stedc(gks_ctx* ctx, const double* d, const double* e, int64_t m, 
   DeviceGuard dg(ctx->device);
   gks_status rc = ensure_ws(ctx, (int)m, (int)m, (int)count, 8, 0);
   if (rc) return rc;
+  // the merges' product lists are bound to the caller's Z from here on: a captured solve reads
+  // the same lists, so it is dropped
+  release_solve_graph(ctx);
+  ctx->gkey = SolveKey{};
   cudaStream_t s = ctx->stream;
   cudaMemsetAsync(ctx->st, 0, sizeof(DevStatus) * count, s);
   double* dw = at<double>(ctx, ctx->od);

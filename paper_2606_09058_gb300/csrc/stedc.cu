@@ -777,7 +777,10 @@ size_t dc_split_item_bytes(const DcPlan* p, int min_half, int S) {
 void dc_solve(DcPlan* p, double* d, double* e, long long sde, double* lam, double* Z, long long sZ, void* work,
               DevStatus* st, cudaStream_t s, Prof* prof, const DcSplit* sp) {
   const int m = p->m, cnt = p->count;
-  if (p->zbound != Z || p->wbound != work || p->sZbound != sZ) build_gemm_lists(p, Z, sZ, work);
+  if (p->zbound != Z || p->wbound != work || p->sZbound != sZ) {
+    if (p->zbound) cudaStreamSynchronize(s);  // work in flight may still read the lists
+    build_gemm_lists(p, Z, sZ, work);
+  }
   const size_t item = dc_item_bytes(m);
   DcWs w0 = dc_ws(work, m);
   // lam ping-pong: leaves write lamA (item stride = item bytes / 8 doubles)

@@ -115,3 +115,25 @@ def test_workspace_of_another_form_between_solves(lib):
         for _ in range(3):
             c.solve(False)
     c.stream.synchronize()
+
+
+@pytest.mark.parametrize("n", [70, 260])
+def test_tridiagonal_entry_between_solves(lib, n):
+    """gks_stedc shares the merges' product lists with the solve."""
+    c = _Case(lib, n, False)
+    d, e = (torch.rand(1, n, dtype=torch.float64, device="cuda") for _ in range(2))
+    with torch.cuda.stream(c.stream):
+        lam, Z = c.eager.stedc(d, e)
+        for _ in range(3):
+            c.solve(False)
+        lam2, Z2 = c.graph.stedc(d, e)
+        keep = Z2.clone()
+        assert torch.equal(lam2, lam) and torch.equal(Z2, Z)
+        for _ in range(3):
+            c.solve(False)
+        assert torch.equal(Z2, keep)
+        c.graph.solve_into(c.H, c.S, KT, c.ne, sync=False, **c.out)  # in flight
+        lam2, Z2 = c.graph.stedc(d, e)
+        assert torch.equal(lam2, lam) and torch.equal(Z2, Z)
+        assert all(torch.equal(c.out[k], c.ref_out[k]) for k in c.out)
+    c.stream.synchronize()
