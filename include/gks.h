@@ -103,7 +103,8 @@ typedef enum { GKS_SPLIT_RESIDUES = 0, GKS_SPLIT_DIGITS = 1 } gks_split;
  * products with 32-bit sums, weighted and summed in FP64: the error is that of the 54-bit
  * rounding, relative to the equilibrated entries; all steps of a panel run in one
  * persistent launch.  GKS_HEMV_FP64: FP64 multiply-adds (three real products per complex
- * product), two launches per step. */
+ * product), two launches per step.  Mixed precision: its digit form (up to 2.4e8 bytes of H')
+ * with GKS_HEMV_DIGITS only; with GKS_HEMV_FP64 single precision at every order. */
 typedef enum { GKS_HEMV_DIGITS = 0, GKS_HEMV_FP64 = 1 } gks_hemv;
 
 /* gks_solve flags. */

@@ -285,11 +285,12 @@ int shape_spin(int spin) { return spin == GKS_NONCOLLINEAR ? 1 : 0; }
 // persistent digit form on an FP64 copy of H' (2), which is more accurate and, its steps being
 // shorter, faster until its traffic (14 bytes per complex entry against 4) outweighs them.
 // Measured per step (single precision / digits): real order 1404 35 / 15 us, 6000 55 / 32 us;
-// complex 1404 41 / 22 us, 4000 59 / 39 us, eight items of 1404 47 / 50 us.
+// complex 1404 41 / 22 us, 4000 59 / 39 us, eight items of 1404 47 / 50 us.  opts.hemv =
+// GKS_HEMV_FP64 asks for no digits: the single-precision steps at every order.
 constexpr double kMixedDigitBytes = 2.4e8;
 int mixed_form(const gks_ctx* c, int m, int nk, int es) {
   if (c->precision == GKS_FP64) return 0;
-  return (double)m * m * nk * es <= kMixedDigitBytes ? 2 : 1;
+  return c->hemv == GKS_HEMV_DIGITS && (double)m * m * nk * es <= kMixedDigitBytes ? 2 : 1;
 }
 
 // What the context's options make of a shape, and whether its workspace is of that kind.
