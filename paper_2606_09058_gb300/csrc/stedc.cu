@@ -120,8 +120,11 @@ __global__ void __launch_bounds__(32) dc_leaf_kernel(const double* d, const doub
   bool ok = true;
   for (int l = 0; l < n && ok; l++) {
     for (int sweep = 0;; sweep++) {
-      // the first negligible off-diagonal from l on
-      const bool neg = lane >= l && lane < n - 1 && fabs(ee[lane]) <= DC_U * (fabs(dd[lane]) + fabs(dd[lane + 1]));
+      // the first negligible off-diagonal from l on (below 1e-150 of the block its square, which
+      // the shift and the rotations take, underflows: beside equal zero diagonal entries the
+      // shift would be 0 / 0)
+      const bool neg = lane >= l && lane < n - 1 &&
+                       fabs(ee[lane]) <= fmax(DC_U * (fabs(dd[lane]) + fabs(dd[lane + 1])), 1e-150);
       const unsigned mask = __ballot_sync(0xffffffffu, neg);
       const int q = mask ? __ffs(mask) - 1 : n - 1;
       __syncwarp();
