@@ -220,6 +220,16 @@ __device__ __forceinline__ double2 secular_scale(double spread, double rho2) {
   return make_double2(__hiloint2double((2045 - ex) << 20, 0), __hiloint2double((ex + 1) << 20, 0));
 }
 
+// Powers of two (x, y = 1 / x) for a merge whose entries lie outside 2^-340 .. 2^340 (a block that
+// is tiny beside the rest of T): in its own units the squares of the secular sums and of the
+// vectors neither overflow nor vanish.  1 otherwise, and then no bit changes.
+__device__ __forceinline__ double2 node_scale(double top) {
+  const int ex = (__double2hiint(top) >> 20) & 0x7ff;
+  if (top == 0.0 || (ex > 683 && ex < 1363)) return make_double2(1.0, 1.0);
+  const int k = max(-1000, min(1000, 1023 - ex));
+  return make_double2(__hiloint2double((1023 + k) << 20, 0), __hiloint2double((1023 - k) << 20, 0));
+}
+
 __device__ __forceinline__ DcWs item_ws(const DcArgs& a, int z) { return dc_ws(a.ws + z * a.sitem, a.m); }
 
 // Exclusive sum of v over the CTA (1024 threads), total in *all.
@@ -251,7 +261,8 @@ __device__ int block_scan(int v, int* scratch, int* all) {
 // compaction, the test between neighbouring survivors runs for all pairs at once on the
 // unrotated values (which are the current ones unless the pair before rotated), and one
 // thread walks the runs that start at a pair that fails it.  (Walking every pole from global
-// memory took 6.3 ms for the last merge of order 4992.)
+// memory took 6.3 ms for the last merge of order 4992.)  Poles are kept in the node's units
+// (node_scale, left in ds[0], ds[1] for the merge's other kernels) up to dc_colmap_kernel.
 __global__ void __launch_bounds__(1024) dc_merge_prep_kernel(DcArgs a, const DcNode* nodes) {
   __shared__ double red[32];
   __shared__ int scan[32], s_nrot, s_bad;
@@ -262,7 +273,7 @@ __global__ void __launch_bounds__(1024) dc_merge_prep_kernel(DcArgs a, const DcN
   const double* lam = a.lam + z * a.slam;
   const double* Zc = a.Zc + z * a.sZ;
   const double beta = a.e[z * a.sde + s - 1];
-  const double rho2 = 2.0 * fabs(beta);
+  double rho2 = 2.0 * fabs(beta);
   const double sg = beta < 0.0 ? -1.0 : 1.0;
   const double isq2 = 0.70710678118654752440;
   double *ds = w.ds + off, *zs = w.zs + off, *dK = w.dK + off, *zK = w.zK + off, *dD = w.dD + off;
@@ -299,6 +310,13 @@ __global__ void __launch_bounds__(1024) dc_merge_prep_kernel(DcArgs a, const DcN
   if (tid == 0) s_nrot = s_bad = 0;
   __syncthreads();
   for (int k = 0; k < 32; k++) dmax = fmax(dmax, red[k]);
+  const double2 unit = node_scale(fmax(dmax, rho2));
+  if (unit.x != 1.0) {
+    for (int i = tid; i < n; i += nt) ds[i] *= unit.x;
+    dmax *= unit.x;
+    rho2 *= unit.x;
+    __syncthreads();
+  }
   const double tol = 8.0 * DC_U * fmax(dmax, rho2);
   // survivors (in dK, zK, idxK) and negligible z_i (in dD, idxD), each in ascending order
   const int per = (n + nt - 1) / nt, p0 = min(n, tid * per), p1 = min(n, p0 + per);
@@ -408,6 +426,8 @@ __global__ void __launch_bounds__(1024) dc_merge_prep_kernel(DcArgs a, const DcN
     }
   }
   if (tid == 0) {
+    ds[0] = unit.x;
+    ds[1] = unit.y;
     w.cnt[3 * off + 0] = K;
     w.cnt[3 * off + 1] = nD;
     w.cnt[3 * off + 2] = s_nrot;
@@ -494,7 +514,7 @@ __global__ void dc_secular_kernel(DcArgs a, const DcNode* nodes, DevStatus* st) 
   const int lane = threadIdx.x & 31;
   const int j = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (j >= K) return;
-  const double rho2 = 2.0 * fabs(a.e[z * a.sde + s - 1]);
+  const double rho2 = 2.0 * fabs(a.e[z * a.sde + s - 1]) * w.ds[off];
   const double* dK = w.dK + off;
   const double* zK = w.zK + off;
   const float2* xf = reinterpret_cast<const float2*>(w.xf + off);
@@ -592,7 +612,7 @@ __global__ void dc_zhat_kernel(DcArgs a, const DcNode* nodes) {
   const int K = w.cnt[3 * off];
   const int lane = threadIdx.x & 31, i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (i >= K) return;
-  const double rho2 = 2.0 * fabs(a.e[z * a.sde + s - 1]);
+  const double rho2 = 2.0 * fabs(a.e[z * a.sde + s - 1]) * w.ds[off];
   const double* dK = w.dK + off;
   const double di = dK[i];
   // a warp per entry, the factors over the lanes (each near 1 but for the nearest: no overflow)
@@ -616,17 +636,18 @@ __global__ void dc_colmap_kernel(DcArgs a, const DcNode* nodes) {
   const int K = w.cnt[3 * off], nD = w.cnt[3 * off + 1];
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   double* lamNew = a.lamNew + z * a.slam;
+  const double unit = w.ds[off + 1];
   if (t < K) {
     double v = w.lamK[off + t];
     int pos = t + lower_bound_d(w.dD + off, nD, v);
     w.colsrc[off + pos] = t;
-    lamNew[off + pos] = v;
+    lamNew[off + pos] = v * unit;
   } else if (t < K + nD) {
     int i = t - K;
     double v = w.dD[off + i];
     int pos = i + upper_bound_d(w.lamK + off, K, v);
     w.colsrc[off + pos] = -1 - i;
-    lamNew[off + pos] = v;
+    lamNew[off + pos] = v * unit;
   }
 }
 

@@ -17,10 +17,10 @@ def ctx():
     return gks.Context(0)
 
 
-@pytest.mark.parametrize("c", [5e-324, 1e-300, 1e-170, 1.4e-162, 1e-155, 1e-150, 1e-140])
-@pytest.mark.parametrize("scale", [1.0, 1e100, 1e-100])
-@pytest.mark.parametrize("m", [3, 7, 16])
-def test_tiny_couplings(ctx, m, scale, c):
+C = [5e-324, 1e-300, 1e-170, 1.4e-162, 1e-155, 1e-150, 1e-140]
+
+
+def _check(ctx, m, scale, c):
     d, e = np.zeros(m), np.full(m, c)
     d[-1] = 1.0
     e[m - 1:] = 0.0
@@ -32,3 +32,18 @@ def test_tiny_couplings(ctx, m, scale, c):
     assert np.abs(lam / scale - ref).max() <= 8 * m * u
     assert np.abs(Z.T @ Z - np.eye(m)).max() <= 16 * m * u
     assert np.abs(T @ Z - Z * (lam / scale)).max() <= 16 * m * u
+
+
+@pytest.mark.parametrize("c", C)
+@pytest.mark.parametrize("scale", [1.0, 1e100, 1e-100])
+@pytest.mark.parametrize("m", [3, 7, 16])
+def test_tiny_couplings(ctx, m, scale, c):
+    _check(ctx, m, scale, c)
+
+
+@pytest.mark.parametrize("c", C)
+@pytest.mark.parametrize("scale", [1.0, 1e100, 1e-100])
+@pytest.mark.parametrize("m", [17, 40, 70, 300])
+def test_tiny_blocks_beside_a_large_one(ctx, m, scale, c):
+    """Merges whose whole spectrum lies far below the rest of T."""
+    _check(ctx, m, scale, c)
