@@ -698,7 +698,12 @@ __device__ __forceinline__ bool grid_wait(unsigned* cnt, unsigned target, unsign
 }
 
 // The same over the CTAs of a cluster: an mbarrier of G arrivals in every CTA.  Lanes below G
-// arrive on the barrier of CTA `lane`; a thread waits for its own CTA's phase.
+// arrive on the barrier of CTA `lane`; a thread waits for its own CTA's phase.  Consecutive
+// phases alternate between two mbarriers: an arrival names no sender and arrivals at different
+// CTAs are not ordered, so that on one mbarrier a CTA that has seen phase n could arrive for n + 1
+// at a CTA where another's arrival for n is still on its way, and complete n there in its place.
+// With two, an arrival for n + 2 on the mbarrier of n follows everyone's for n + 1, which
+// follow their completions of n.
 __device__ __forceinline__ void cluster_arrive(uint64_t* bar, int cta) {
   asm volatile(
       "{\n .reg .b32 ra;\n mapa.shared::cluster.u32 ra, %0, %1;\n"
@@ -750,7 +755,7 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
   T* qjs = ujs + (kPanelMax + 1);
   __shared__ T s_inv, s_upiv, s_sub, s_pj, s_us[64];
   __shared__ double s_tau, s_kq, s_red[12];
-  __shared__ __align__(8) uint64_t s_bar[2];  // cluster form: all threads', the vector warps'
+  __shared__ __align__(8) uint64_t s_bar[4];  // cluster form: two for all threads, two for the vector warps
   __shared__ int s_fu, s_ok, s_abort, s_rede[12];
 
   const int z = blockIdx.y, b = blockIdx.x, G = gridDim.x;
@@ -811,8 +816,9 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
     arrived += CL ? 1u : (unsigned)G;
     if (CL) {
       if (warp == 0) {
-        if (lane < G) cluster_arrive(&s_bar[0], lane);
-        if (lane == 0 && !cluster_wait(&s_bar[0], (arrived - 1) & 1u, a.wait)) s_abort = 1;
+        uint64_t* sb = &s_bar[(arrived - 1) & 1u];
+        if (lane < G) cluster_arrive(sb, lane);
+        if (lane == 0 && !cluster_wait(sb, ((arrived - 1) >> 1) & 1u, a.wait)) s_abort = 1;
       }
     } else if (tid == 0) {
       red_release(bar);
@@ -855,7 +861,7 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
   if (tid == 0) s_abort = 0;
   if (CL) {
     if (tid == 0) {
-      for (int q = 0; q < 2; q++)
+      for (int q = 0; q < 4; q++)
         asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"((unsigned)__cvta_generic_to_shared(&s_bar[q])),
                      "r"(G));
       asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
@@ -1106,8 +1112,9 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
         bar_named<2, 128>();
         arrivedv += CL ? 1u : (unsigned)G;
         if (CL) {
-          if (warp == 8 && lane < G) cluster_arrive(&s_bar[1], lane);
-          if (vt == 0 && !cluster_wait(&s_bar[1], (arrivedv - 1) & 1u, a.wait)) s_abort = 1;
+          uint64_t* sb = &s_bar[2 + ((arrivedv - 1) & 1u)];
+          if (warp == 8 && lane < G) cluster_arrive(sb, lane);
+          if (vt == 0 && !cluster_wait(sb, ((arrivedv - 1) >> 1) & 1u, a.wait)) s_abort = 1;
         } else if (vt == 0) {
           red_release(bar + 1);
           if (!grid_wait(bar + 1, arrivedv, bar + 2, a.wait)) s_abort = 1;
