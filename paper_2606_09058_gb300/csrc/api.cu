@@ -1084,9 +1084,6 @@ bool hetrd_digit_run(gks_ctx* c, T* A, int M, int nk) {
   const int es = sizeof(T), pw = panel_width(c, M);
   const int ldd = (M + 15) / 16 * 16, npl = es == 16 ? 14 : 7;
   if (M < 3) return true;
-  // items per launch: at least one CTA each, all resident
-  int per = nk;
-  while (per > 1 && hetrd_panel_ctas<T>(M - 1, per) < 1) per = (per + 1) / 2;
   const int gs = panel_gs(nk);
   PanelArgs<T> pa{};
   pa.lda = M;
@@ -1105,7 +1102,8 @@ bool hetrd_digit_run(gks_ctx* c, T* A, int M, int nk) {
   HemvDigits hd = pa.hd;
   hd.D = at<signed char>(c, c->oD);
   hd.rmax = at<unsigned long long>(c, c->ormax);
-  std::vector<unsigned> base((nk + per - 1) / per, 0u), basev(base);
+  const int chunk = hetrd_panel_items<T>(M - 1, nk);
+  std::vector<unsigned> base((nk + chunk - 1) / chunk, 0u), basev(base);
   for (int jh = M - 1; jh >= 2; jh -= pw) {
     const int jl = std::max(2, jh - pw + 1), steps = jh - jl + 1;  // steps jh .. jl in this panel
     {
@@ -1120,6 +1118,7 @@ bool hetrd_digit_run(gks_ctx* c, T* A, int M, int nk) {
     }
     {
       Rec r(c, PC_HETRD_HEMV, fl, by);
+      const int per = hetrd_panel_items<T>(jh, nk);  // chunk, or every item once the cluster form runs
       for (int z0 = 0, q = 0; z0 < nk; z0 += per, q++) {
         const int cnt = std::min(per, nk - z0);
         pa.A = A + z0 * c->sMM;

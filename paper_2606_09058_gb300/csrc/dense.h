@@ -104,10 +104,10 @@ struct PanelArgs {
   DevStatus* st;
   long long wait;
 };
-// CTAs per item of the grid form for a panel of order jh on `items` items (0: not even one
-// per item fits).
+// Items per launch, of `items`, for panels of order jh and below: all in the cluster form, else
+// as many as the grid form can give a resident CTA each.
 template <typename T>
-int hetrd_panel_ctas(int jh, int items);
+int hetrd_panel_items(int jh, int items);
 // base and basev advance by the launch's arrivals.  False if the launch was refused (then
 // nothing ran).
 template <typename T>

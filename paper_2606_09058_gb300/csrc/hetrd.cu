@@ -1360,35 +1360,33 @@ static int panel_capacity() {
     return sms * (per > 0 ? 1 : 0);
   });
 }
-// Largest cluster of panel CTAs that can be resident (16, 8 or 0), attributes set.
-template <typename T>
-static int panel_cluster() {
+// Clusters of c panel CTAs (c = 16, 8, 4, 2, 1) that are resident at once, attributes set.
+template <typename T, int c>
+static int panel_clusters() {
   static std::atomic<int> known[64];
   return per_device(known, [](int) {
     auto k = hetrd_panel_kernel<T, true>;
     cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, PanelSmem<T>::TOTAL);
     cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    for (int c = 16; c >= 8; c /= 2) {
-      cudaLaunchConfig_t cfg{};
-      cudaLaunchAttribute at{};
-      at.id = cudaLaunchAttributeClusterDimension;
-      at.val.clusterDim.x = c;
-      at.val.clusterDim.y = at.val.clusterDim.z = 1;
-      cfg.gridDim = dim3(c);
-      cfg.blockDim = dim3(kPanelThreads);
-      cfg.dynamicSmemBytes = PanelSmem<T>::TOTAL;
-      cfg.attrs = &at;
-      cfg.numAttrs = 1;
-      int n = 0;
-      if (cudaOccupancyMaxActiveClusters(&n, k, &cfg) == cudaSuccess && n > 0) return c;
-      cudaGetLastError();
-    }
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = c;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.gridDim = dim3(c);
+    cfg.blockDim = dim3(kPanelThreads);
+    cfg.dynamicSmemBytes = PanelSmem<T>::TOTAL;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, k, &cfg) == cudaSuccess && n > 0) return n;
+    cudaGetLastError();
     return 0;
   });
 }
 
 template <typename T>
-int hetrd_panel_ctas(int jh, int items) {
+static int hetrd_panel_ctas(int jh, int items) {
   const int top = std::min(panel_capacity<T>() / items, kPanelCtas);
   const long long tiles = (long long)((jh + 31) / 32) * ((jh + 15) / 16);
   return (int)std::min<long long>(
@@ -1397,22 +1395,36 @@ int hetrd_panel_ctas(int jh, int items) {
 
 // The cluster form: one cluster of up to 16 CTAs per item, barriers through shared-memory
 // mbarriers, no co-residency of the whole grid needed.  It pays at the smallest orders only
-// (16 SMs do the FP64 corrections: order 640 real 20 us per step against 12.7 us on 80 CTAs),
-// and where the grid form cannot give every item a CTA.
+// (16 SMs do the FP64 corrections: order 640 real 20 us per step against 12.7 us on 80 CTAs).
+// The largest cluster of which the GPU holds one per item: a step of these orders is latency,
+// and waves of clusters repeat it.  All panels of a call, clusters of 16 in waves / this rule:
+// order 104 complex, 8 items 2.77 / 1.58 ms, 64 items 13.9 / 2.9, 512 items 105 / 14; order 40
+// real, 1000 items 48.8 / 3.2 (two launches per step in FP64: 3.8).
+constexpr long long kClusterTiles = 64;
+static bool panel_in_cluster(int jh) {
+  return (long long)((jh + 31) / 32) * ((jh + 15) / 16) <= kClusterTiles;
+}
 template <typename T>
-static int panel_cluster_ctas(int jh, int items) {
-  constexpr long long kClusterTiles = 64;
-  const int c = panel_cluster<T>();
-  const long long tiles = (long long)((jh + 31) / 32) * ((jh + 15) / 16);
-  if (c == 0 || (tiles > kClusterTiles && hetrd_panel_ctas<T>(jh, items) >= 1)) return 0;
-  return c;
+static int panel_cluster_ctas(int items) {
+  if (panel_clusters<T, 16>() >= items) return 16;
+  if (panel_clusters<T, 8>() >= items) return 8;
+  if (panel_clusters<T, 4>() >= items) return 4;
+  if (panel_clusters<T, 2>() >= items) return 2;
+  return panel_clusters<T, 1>() > 0 ? 1 : 0;
+}
+
+template <typename T>
+int hetrd_panel_items(int jh, int items) {
+  if (panel_in_cluster(jh) && panel_cluster_ctas<T>(items) > 0) return items;
+  while (items > 1 && panel_capacity<T>() < items) items = (items + 1) / 2;
+  return items;
 }
 
 template <typename T>
 constexpr int kEarlyTiles = sizeof(T) == 16 ? 60 : 150;
 template <typename T>
 bool hetrd_panel(PanelArgs<T> a, int items, unsigned* base, unsigned* basev, cudaStream_t s) {
-  const int cl = std::min(panel_cluster_ctas<T>(a.jh, items), a.gs >= 16 ? 16 : a.gs >= 8 ? 8 : 0);
+  const int cl = panel_in_cluster(a.jh) ? panel_cluster_ctas<T>(items) : 0;
   const int G = cl > 0 ? cl : std::min(a.gs, hetrd_panel_ctas<T>(a.jh, items));
   int maxseg = (a.jh + 31) / 32 / G + 2;
   const int steps = a.jh - a.jl + 1;
@@ -1686,7 +1698,7 @@ void narrow_lower(const T* A, int lda, long long sA, TL* B, int ldb, long long s
                                         int, long long, double*, long long, int, cudaStream_t);               \
   template void hetrd_digits<T>(const T*, int, long long, int, const HemvDigits&, int, cudaStream_t);           \
   template void panel_pack<T>(const T*, const T*, int, long long, int, int, T*, long long, int, cudaStream_t);    \
-  template int hetrd_panel_ctas<T>(int, int);                                                              \
+  template int hetrd_panel_items<T>(int, int);                                                             \
   template bool hetrd_panel<T>(PanelArgs<T>, int, unsigned*, unsigned*, cudaStream_t);
 INST(double)
 INST(zc)
