@@ -647,12 +647,28 @@ int oz_reserve(gks_ctx* c, size_t item, int count) {
 // take 0.073 us (complex 0.294) per inner index on their SM, whatever shares the other SMs.
 // Measured (FP64 kernel / split product): real 832 x 256 x 64 35 / 39 us, 832 x 832 x 64 95 / 52
 // us, 2500 x 64 x 64 29 / 42 us; complex 256 x 256 x 64 42 / 38 us, 192 x 64 x 192 64 / 38 us.
-constexpr double kSplitUs = 32.0;
+// A large batch of products far below a tile moves little but padding: beyond what L2 holds, the
+// planes and residues at their padded sizes (rows to 128, embedded columns to 256, K to 64; 16 of
+// each), written and read, add their time at about 4 TB/s, against the rounds of the tiles that
+// the FP64 kernel takes there (density matrices of all items, FP64 kernel / split product: 1000
+// of order 40 real 0.36 / 0.70 ms, complex 1.00 / 0.85; 300 of order 64 real 0.12 / 0.24, complex
+// 0.42 / 0.30; 300 of order 104 real 0.71 / 0.37).
+constexpr double kSplitUs = 32.0, kSplitCached = 1e8, kSplitBytesPerUs = 4e6;
 bool split_worth(gks_ctx* c, int count, int M, int N, int K, int es, int lower) {
   if (c->gemm_mode == 2) return true;
   if (c->gemm_mode != 0 || M < 32 || (es == 16 ? 2 * N : N) < 32 || K < 32) return false;
   const long long tiles = (long long)((M + 15) / 16) * ((N + 15) / 16) * count / (lower ? 2 : 1);
-  return (double)((tiles + 151) / 152) * K * (es == 16 ? 0.294 : 0.073) >= kSplitUs;
+  const double round = K * (es == 16 ? 0.294 : 0.073);
+  if ((double)((tiles + 151) / 152) * round < kSplitUs) return false;
+  auto up = [](int v, int to) { return (double)((v + to - 1) / to * to); };
+  const int e = es == 16 ? 2 : 1;
+  const double Mp = up(M, 128), Np = up(e * N, 256), Kp = up(e * K, 64);
+  const double bytes = 2.0 * 16.0 * count * ((Mp + Np) * Kp * 2.0 + Mp * Np);
+  if (bytes <= kSplitCached) return true;
+  const int t = gemm_tile(M, N, count, es);  // of the FP64 kernel
+  const long long tm = (M + t - 1) / t, tn = (N + t - 1) / t, w = t / 16;
+  const long long padded = (lower && M == N ? tm * (tm + 1) / 2 : tm * tn) * w * w * count;
+  return (double)((padded + 151) / 152) * round >= kSplitUs + (bytes - kSplitCached) / kSplitBytesPerUs;
 }
 
 // Smallest half of a merge whose products (half x 2 half x half, `items` of them per launch) are

@@ -119,28 +119,29 @@ __global__ void __launch_bounds__(256) gemm_kernel(GemmBatch gb) {
   }
 }
 
-template <typename T, int TM>
-static bool gemm_try(const GemmBatch& b, int maxM, int maxN, cudaStream_t s, long long want) {
-  constexpr int BM = 16 * TM;
-  dim3 grid((maxN + BM - 1) / BM, (maxM + BM - 1) / BM, b.count);
-  if ((long long)grid.x * grid.y * grid.z < want) return false;
-  count_launch();
-  gemm_kernel<T, TM><<<grid, 256, 0, s>>>(b);
-  return true;
-}
-
 // The largest tile that still gives four CTAs per SM (608), else the smallest.  A
 // 832 x 64 x 64 real product: 13 CTAs of 64 x 64 took 150 us, 208 of 16 x 16 take 12 us.
+int gemm_tile(int maxM, int maxN, int count, int es) {
+  for (int t = es == 16 ? 32 : 64; t > 16; t /= 2)
+    if ((long long)((maxM + t - 1) / t) * ((maxN + t - 1) / t) * count >= 4 * 152) return t;
+  return 16;
+}
+
+template <typename T, int TM>
+static void gemm_launch(const GemmBatch& b, int maxM, int maxN, cudaStream_t s) {
+  constexpr int BM = 16 * TM;
+  count_launch();
+  gemm_kernel<T, TM><<<dim3((maxN + BM - 1) / BM, (maxM + BM - 1) / BM, b.count), 256, 0, s>>>(b);
+}
+
 template <typename T>
 void gemm(const GemmBatch& b, int maxM, int maxN, cudaStream_t s) {
   if (maxM <= 0 || maxN <= 0 || b.count <= 0) return;
-  constexpr long long want = 4 * 152;
-  if constexpr (sizeof(T) == 16) {
-    if (!gemm_try<T, 2>(b, maxM, maxN, s, want)) gemm_try<T, 1>(b, maxM, maxN, s, 0);
-  } else {
-    if (gemm_try<T, 4>(b, maxM, maxN, s, want) || gemm_try<T, 2>(b, maxM, maxN, s, want)) return;
-    gemm_try<T, 1>(b, maxM, maxN, s, 0);
-  }
+  const int t = gemm_tile(maxM, maxN, b.count, sizeof(T));
+  if constexpr (sizeof(T) != 16)
+    if (t == 64) return gemm_launch<T, 4>(b, maxM, maxN, s);
+  if (t == 32) gemm_launch<T, 2>(b, maxM, maxN, s);
+  else gemm_launch<T, 1>(b, maxM, maxN, s);
 }
 
 template <typename T>

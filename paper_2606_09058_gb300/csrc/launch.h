@@ -36,6 +36,8 @@ struct GemmBatch {
 };
 
 template <typename T> void gemm(const GemmBatch& b, int maxM, int maxN, cudaStream_t s);
+// Side of the output tile that gemm takes for `count` products of elements of es bytes.
+int gemm_tile(int maxM, int maxN, int count, int es);
 
 // Number of kernel launches issued by this library (process-wide).
 void count_launch(int n = 1);
