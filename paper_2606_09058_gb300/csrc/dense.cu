@@ -26,7 +26,7 @@ __device__ __forceinline__ double shfl_g(double v, int src) { return __shfl_sync
 template <int G>
 __device__ __forceinline__ zc shfl_g(zc v, int src) { return zc{shfl_g<G>(v.x, src), shfl_g<G>(v.y, src)}; }
 
-// Diagonal blocks (64 x 64) on a cluster of kDiagC CTAs, in sub-blocks (32 columns of the
+// Diagonal blocks (64 x 64) on a cluster of C CTAs, in sub-blocks (32 columns of the
 // Cholesky factorization, 8 of the two-sided reduction).  One SM does 1.7 FP64 multiply-adds
 // per clock: the 64^3 operations of a complex two-sided reduction alone keep it busy for 0.3
 // ms, so the panel rows and the trailing updates are spread over the cluster (data in global
@@ -35,7 +35,7 @@ __device__ __forceinline__ zc shfl_g(zc v, int src) { return zc{shfl_g<G>(v.x, s
 // Measured, one block (complex / real): two-sided reduction 794 / 265 us on one CTA column by
 // column, 163 / 80 us here (190 / 90 with sub-blocks of 16, 420 / 153 on one CTA); Cholesky 207 / 103 us on one CTA,
 // 110 / 76 us with sub-blocks of 8, 83 / 59 us here.
-constexpr int kDiagC = 8, kDiagThreads = 256;
+constexpr int kDiagThreads = 256;
 __device__ __forceinline__ void cluster_barrier() {
   asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
 }
@@ -46,7 +46,7 @@ __device__ __forceinline__ void cluster_barrier() {
 // A 32-column sub-block's own part: thread (i, q) holds row i, columns q + 8 t in registers; a
 // step scales the pivot column (one warp), then every element takes its rank-one update, the
 // next pivot's owner going on to its reciprocal square root while the others still update.
-template <typename T>
+template <typename T, int C>
 __global__ void __launch_bounds__(kDiagThreads) potf2_kernel(T* A, int lda, long long sA, int k0, int nb,
                                                              DevStatus* st) {
   constexpr int SB = 32;
@@ -105,9 +105,9 @@ __global__ void __launch_bounds__(kDiagThreads) potf2_kernel(T* A, int lda, long
       __syncthreads();
     }
     if (fail >= 0) break;  // the same in every CTA of the cluster
-    // rows below, one per warp, row r of CTA r % kDiagC: x L11^H = a
+    // rows below, one per warp, row r of CTA r % C: x L11^H = a
     if (m > 0) {
-      for (int r = rank + kDiagC * warp; r < m; r += kDiagC * 8) {
+      for (int r = rank + C * warp; r < m; r += C * 8) {
         T* ar = A + (size_t)(c0 + kb + r) * lda + c0;
         T x = lane < kb ? ldcg(ar + lane) : zero<T>();
 #pragma unroll 1
@@ -131,7 +131,7 @@ __global__ void __launch_bounds__(kDiagThreads) potf2_kernel(T* A, int lda, long
       v[r][g] = g < kb ? ldcg(A + (size_t)(c0 + kb + r) * lda + c0 + g) : zero<T>();
     }
     __syncthreads();
-    for (int e = rank * kDiagThreads + tid; e < m * m; e += kDiagC * kDiagThreads) {
+    for (int e = rank * kDiagThreads + tid; e < m * m; e += C * kDiagThreads) {
       const int r = e / m, j = e - r * m;
       if (j > r) continue;
       T* p = A + (size_t)(c0 + kb + r) * lda + c0 + kb + j;
@@ -227,7 +227,7 @@ __global__ void __launch_bounds__(512) trsm_block_kernel(const T* L, int ldl, lo
 // column.  Writes the lower triangle back into A and the full Hermitian block into F (ldF).
 constexpr int kSub = 8;
 __device__ __forceinline__ void diag_bar() { asm volatile("bar.sync 1, 64;\n" ::: "memory"); }
-template <typename T>
+template <typename T, int C>
 __global__ void __launch_bounds__(kDiagThreads) hegst_diag_kernel(T* A, int lda, long long sA, const T* L, int ldl,
                                                                   long long sL, int k0, int nb, T* F, int ldF,
                                                                   long long sF) {
@@ -236,7 +236,7 @@ __global__ void __launch_bounds__(kDiagThreads) hegst_diag_kernel(T* A, int lda,
   __shared__ T s11[kSub][kSub + 1];
   __shared__ double rd[64];
   T* v = l + 64 * 65;  // [64][kSub + 1]
-  constexpr int LD = 65, LV = kSub + 1, C = kDiagC;
+  constexpr int LD = 65, LV = kSub + 1;
   const int z = blockIdx.y, rank = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   A += z * sA + (size_t)k0 * lda + k0;
   L += z * sL + (size_t)k0 * ldl + k0;
@@ -553,6 +553,14 @@ static dim3 grid2d(int rows, int cols, int count) {
   return dim3(gx, gy, count);
 }
 
+// CTAs per diagonal block: the largest cluster with all items side by side (clusters of 8 and 4
+// do not fill every processing cluster's SMs).  A second wave costs more than a wider cluster
+// gains.  Two-sided reduction of 64 x 64 blocks, complex, in us on 8 / 4 / 2 / 1 CTAs: 8 items
+// 163 / 194 / 266 / 421, 19 items 208 / 194 / 266 / 421, 76 items 585 / 448 / 266 / 423, 1000
+// items 5779 / 3760 / 2837 / 2552; Cholesky 85 / 89 / 110 / 154, 112 / 90 / 111 / 153, 218 / 165 /
+// 112 / 155, 2129 / 1306 / 956 / 784.  Real blocks cross at the same counts.
+static int diag_ctas(int count) { return count <= 8 ? 8 : count <= 32 ? 4 : count <= 76 ? 2 : 1; }
+
 // Launch of a diagonal-block kernel on one cluster per item.
 template <typename... P, typename... Q>
 static void diag_launch(void (*k)(P...), int ctas, int count, size_t sm, cudaStream_t s, Q... args) {
@@ -573,7 +581,12 @@ static void diag_launch(void (*k)(P...), int ctas, int count, size_t sm, cudaStr
 
 template <typename T>
 void potf2(T* A, int lda, long long sA, int k0, int nb, DevStatus* st, int count, cudaStream_t s) {
-  diag_launch(potf2_kernel<T>, kDiagC, count, 0, s, A, lda, sA, k0, nb, st);
+  auto run = [&](auto k, int c) { diag_launch(k, c, count, 0, s, A, lda, sA, k0, nb, st); };
+  const int c = diag_ctas(count);
+  if (c == 8) run(potf2_kernel<T, 8>, c);
+  else if (c == 4) run(potf2_kernel<T, 4>, c);
+  else if (c == 2) run(potf2_kernel<T, 2>, c);
+  else run(potf2_kernel<T, 1>, c);
 }
 
 template <typename T, int MODE, int G>
@@ -631,8 +644,15 @@ template <typename T>
 void hegst_diag(T* A, int lda, long long sA, const T* L, int ldl, long long sL, int k0, int nb, T* F, int ldF,
                 long long sF, int count, cudaStream_t s) {
   const size_t sm = sizeof(T) * (64 * 65 + 64 * (kSub + 1));
-  cudaFuncSetAttribute(hegst_diag_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  diag_launch(hegst_diag_kernel<T>, kDiagC, count, sm, s, A, lda, sA, L, ldl, sL, k0, nb, F, ldF, sF);
+  auto run = [&](auto k, int c) {
+    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    diag_launch(k, c, count, sm, s, A, lda, sA, L, ldl, sL, k0, nb, F, ldF, sF);
+  };
+  const int c = diag_ctas(count);
+  if (c == 8) run(hegst_diag_kernel<T, 8>, c);
+  else if (c == 4) run(hegst_diag_kernel<T, 4>, c);
+  else if (c == 2) run(hegst_diag_kernel<T, 2>, c);
+  else run(hegst_diag_kernel<T, 1>, c);
 }
 
 template <typename T>
