@@ -5,6 +5,7 @@
 // little memory bandwidth: a 64 x 64 register-tiled CTA at K-step 16 asks for under one
 // byte of shared memory per DFMA.  The kernel therefore favours many independent CTAs
 // (grouped problems of different shapes in one launch) over deep software pipelining.
+#include <algorithm>
 #include <atomic>
 #include <cstdio>
 
@@ -35,7 +36,7 @@ __global__ void __launch_bounds__(256) gemm_kernel(GemmBatch gb) {
   __shared__ T As[BK][BM];
   __shared__ T Bs[BK][BN];
 
-  const int z = blockIdx.z;
+  const int z = gb.z0 + blockIdx.z;
   GemmDesc d;
   if (gb.list) {
     d = gb.list[z];
@@ -138,10 +139,19 @@ template <typename T>
 void gemm(const GemmBatch& b, int maxM, int maxN, cudaStream_t s) {
   if (maxM <= 0 || maxN <= 0 || b.count <= 0) return;
   const int t = gemm_tile(maxM, maxN, b.count, sizeof(T));
-  if constexpr (sizeof(T) != 16)
-    if (t == 64) return gemm_launch<T, 4>(b, maxM, maxN, s);
-  if (t == 32) gemm_launch<T, 2>(b, maxM, maxN, s);
-  else gemm_launch<T, 1>(b, maxM, maxN, s);
+  // a grid holds 65535 products (the first merges of many small tridiagonals are more)
+  for (int z0 = 0; z0 < b.count; z0 += 65535) {
+    GemmBatch part = b;
+    part.z0 = z0;
+    part.count = std::min(b.count - z0, 65535);
+    if constexpr (sizeof(T) != 16)
+      if (t == 64) {
+        gemm_launch<T, 4>(part, maxM, maxN, s);
+        continue;
+      }
+    if (t == 32) gemm_launch<T, 2>(part, maxM, maxN, s);
+    else gemm_launch<T, 1>(part, maxM, maxN, s);
+  }
 }
 
 template <typename T>

@@ -33,6 +33,7 @@ struct GemmBatch {
   double alpha, beta;
   int nb2;                // > 0: two-level batch, item z at (z / nb2) sX + (z % nb2) sX2
   long long sA2, sB2, sC2;
+  int z0;                 // first product of a launch (set by gemm)
 };
 
 template <typename T> void gemm(const GemmBatch& b, int maxM, int maxN, cudaStream_t s);

@@ -45,3 +45,14 @@ def _check(H, S, sol, m):
 def test_items(ctx, m, nk, cplx):
     H, S = _pencils(m, nk, cplx)
     _check(H, S, ctx.solve(H, S, 0.05, 0.6 * m), m)
+
+
+def test_more_merges_than_a_grid_holds(ctx):
+    """20000 tridiagonals of order 34: 80000 products in the first merges."""
+    m, nk = 34, 20000
+    g = torch.Generator(device="cuda").manual_seed(3)
+    d, e = (torch.randn(nk, m, dtype=torch.float64, device="cuda", generator=g) for _ in range(2))
+    lam, Z = ctx.stedc(d, e)
+    T = torch.diag_embed(d) + torch.diag_embed(e[:, :-1], 1) + torch.diag_embed(e[:, :-1], -1)
+    assert (T @ Z - Z * lam[:, None, :]).abs().max() <= 32 * m * U * T.abs().sum(-1).max()
+    assert (Z.mT @ Z - torch.eye(m, dtype=torch.float64, device="cuda")).abs().max() <= 32 * m * U
