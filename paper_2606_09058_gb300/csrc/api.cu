@@ -101,15 +101,19 @@ struct gks_ctx {
   int nbb_default = 256;               // opts.block, used for shapes the tuner has not seen
   bool nbb_fixed = false;              // opts.block given: no size-dependent default
   std::map<std::tuple<int, int, int>, int> tuned;  // (order bucket, element size, spin) -> width
-  void* oz = nullptr;                  // digit workspace of the split-product GEMM
-  size_t oz_bytes = 0;
-  // stages that run beside the main stream: their streams and split workspaces, and events
+  // digit workspace of the split-product GEMM, and the stages that run beside the main stream:
+  // their streams and split workspaces, and events
   struct Lane {
     cudaStream_t stream = nullptr;
     void* oz = nullptr;
     size_t oz_bytes = 0;
-  } lane[2];
-  std::vector<cudaEvent_t> events;
+  };
+  struct Scratch {
+    void* oz = nullptr;
+    size_t oz_bytes = 0;
+    Lane lane[2];
+    std::vector<cudaEvent_t> events;
+  } sx;
   cudaGraphExec_t gexec = nullptr;     // graph of the solve with key gkey
   bool capturing = false;              // inside capture(): nothing may be allocated or freed
   bool short_scratch = false;          // a product of the capture found its scratch too small
@@ -117,6 +121,8 @@ struct gks_ctx {
   std::vector<gks_ctx*> subs;          // per-problem contexts of gks_solve_batched
   bool batched = false;                // a problem's context of gks_solve_batched
   std::vector<cudaStream_t> workers;   // fork/join streams of gks_solve_batched
+  std::vector<Scratch> wsx;            // and the scratch of a large batch's problems (share_scratch)
+  bool bshare = false;                 // the last batch shared it
   cudaGraphExec_t bexec = nullptr;     // graph of the last captured batch
   std::vector<SolveKey> bkey;
   cudaStream_t stream = nullptr;
@@ -220,19 +226,19 @@ void release_graph(gks_ctx* c) {
 }
 
 void release_oz(gks_ctx* c) {
-  if (c->oz) cudaFree(c->oz);
-  c->oz = nullptr;
-  c->oz_bytes = 0;
+  if (c->sx.oz) cudaFree(c->sx.oz);
+  c->sx.oz = nullptr;
+  c->sx.oz_bytes = 0;
 }
 
-void release_lanes(gks_ctx* c) {
-  for (auto& l : c->lane) {
+void release_scratch(gks_ctx::Scratch& x) {
+  if (x.oz) cudaFree(x.oz);
+  for (auto& l : x.lane) {
     if (l.oz) cudaFree(l.oz);
     if (l.stream) cudaStreamDestroy(l.stream);
-    l = {};
   }
-  for (auto e : c->events) cudaEventDestroy(e);
-  c->events.clear();
+  for (auto e : x.events) cudaEventDestroy(e);
+  x = {};
 }
 
 void release_extra(gks_ctx* c) {
@@ -575,33 +581,33 @@ bool lanes_ready(gks_ctx* c, int panels) {
   int lo = 0, hi = 0;
   cudaDeviceGetStreamPriorityRange(&lo, &hi);
   bool ok = true;
-  for (auto& l : c->lane)
+  for (auto& l : c->sx.lane)
     if (ok && !l.stream) ok = cudaStreamCreateWithPriority(&l.stream, cudaStreamNonBlocking, hi) == cudaSuccess;
-  while (ok && (int)c->events.size() < EV_PANEL + panels) {
+  while (ok && (int)c->sx.events.size() < EV_PANEL + panels) {
     cudaEvent_t e;
     ok = cudaEventCreateWithFlags(&e, cudaEventDisableTiming) == cudaSuccess;
-    if (ok) c->events.push_back(e);
+    if (ok) c->sx.events.push_back(e);
   }
   if (!ok) cudaGetLastError();
   return ok;
 }
 void lane_fork(gks_ctx* c, int q) {
-  cudaEventRecord(c->events[EV_FORK + q], c->stream);
-  cudaStreamWaitEvent(c->lane[q].stream, c->events[EV_FORK + q], 0);
+  cudaEventRecord(c->sx.events[EV_FORK + q], c->stream);
+  cudaStreamWaitEvent(c->sx.lane[q].stream, c->sx.events[EV_FORK + q], 0);
 }
 template <typename F>
 void lane_run(gks_ctx* c, int q, F body) {
   auto swap = [&]() {
-    std::swap(c->stream, c->lane[q].stream);
-    std::swap(c->oz, c->lane[q].oz);
-    std::swap(c->oz_bytes, c->lane[q].oz_bytes);
+    std::swap(c->stream, c->sx.lane[q].stream);
+    std::swap(c->sx.oz, c->sx.lane[q].oz);
+    std::swap(c->sx.oz_bytes, c->sx.lane[q].oz_bytes);
     c->prof.stream = c->stream;
   };
   swap();
   body();
   swap();
 }
-void main_wait(gks_ctx* c, int e) { cudaStreamWaitEvent(c->stream, c->events[e], 0); }
+void main_wait(gks_ctx* c, int e) { cudaStreamWaitEvent(c->stream, c->sx.events[e], 0); }
 
 double cmul(int es) { return es == 16 ? 8.0 : 2.0; }
 
@@ -616,27 +622,27 @@ int oz_reserve(gks_ctx* c, size_t item, int count) {
   const int maxper = (int)std::max<size_t>(1, std::min<size_t>((size_t)count, kOzCap / item));
   const int nch = (count + maxper - 1) / maxper, per = (count + nch - 1) / nch;
   // grown in doublings: each growth waits for the stream
-  const size_t need = item * per, want = std::max(need, std::min(2 * c->oz_bytes, kOzCap));
-  if (need > c->oz_bytes && c->capturing) {
+  const size_t need = item * per, want = std::max(need, std::min(2 * c->sx.oz_bytes, kOzCap));
+  if (need > c->sx.oz_bytes && c->capturing) {
     c->short_scratch = true;  // the graph is dropped and the call runs eagerly
     return 0;
   }
-  if (need > c->oz_bytes) {
-    // a captured solve holds the buffer's address (c->oz may be a lane's): it is captured anew
+  if (need > c->sx.oz_bytes) {
+    // a captured solve holds the buffer's address (sx.oz may be a lane's): it is captured anew
     cudaStreamSynchronize(c->stream);
     release_solve_graph(c);
     release_oz(c);
-    if (cudaMalloc(&c->oz, want) == cudaSuccess) {
-      c->oz_bytes = want;
+    if (cudaMalloc(&c->sx.oz, want) == cudaSuccess) {
+      c->sx.oz_bytes = want;
     } else {
       cudaGetLastError();
-      c->oz = nullptr;
-      if (want == need || cudaMalloc(&c->oz, need) != cudaSuccess) {
+      c->sx.oz = nullptr;
+      if (want == need || cudaMalloc(&c->sx.oz, need) != cudaSuccess) {
         cudaGetLastError();
-        c->oz = nullptr;
+        c->sx.oz = nullptr;
         return 0;
       }
-      c->oz_bytes = need;
+      c->sx.oz_bytes = need;
     }
   }
   return per;
@@ -705,7 +711,7 @@ void gmx(gks_ctx* c, int count, int opA, int opB, int M, int N, int K, double al
     const long long skip = (c->debug & GKS_DEBUG_SKIP_COPY) ? 3 : -1;
     c->debug &= ~GKS_DEBUG_SKIP_COPY;
     if (!ozaki_gemm<T>(opA, opB, M, N, K, alpha, A + z0 * sA, lda, sA, B + z0 * sB, ldb, sB, beta, C + z0 * sC, ldc,
-                       sC, cnt, lower, sform(c), c->oz, c->st ? c->st : c->gst, c->stream, nullptr, 0, nullptr,
+                       sC, cnt, lower, sform(c), c->sx.oz, c->st ? c->st : c->gst, c->stream, nullptr, 0, nullptr,
                        c->wait_cycles, skip))
       gmp<T>(c, cnt, opA, opB, M, N, K, alpha, A + z0 * sA, lda, sA, B + z0 * sB, ldb, sB, beta, C + z0 * sC, ldc, sC,
              lower);
@@ -753,7 +759,7 @@ void gmx2(gks_ctx* c, int count, int nb2, int opA, int opB, int M, int N, int K,
   auto split = [&](const T* Ap, const T* Bp, T* Cp, int cnt, int nb, long long a1, long long a2, long long b1,
                    long long b2, long long c1, long long c2) {
     Rec r(c, PC_OZAKI, gemm_flops(es, M, N, K, 0, cnt), gemm_bytes(es, M, N, K, 0, cnt, beta != 0.0));
-    if (!ozaki_gemm<T>(opA, opB, M, N, K, alpha, Ap, lda, a1, Bp, ldb, b1, beta, Cp, ldc, c1, cnt, 0, sform(c), c->oz,
+    if (!ozaki_gemm<T>(opA, opB, M, N, K, alpha, Ap, lda, a1, Bp, ldb, b1, beta, Cp, ldc, c1, cnt, 0, sform(c), c->sx.oz,
                        c->st ? c->st : c->gst, c->stream, nullptr, 0, nullptr, c->wait_cycles, -1, a2, b2, c2, nb))
       fp64(Ap, Bp, Cp, cnt, nb, a1, a2, b1, b2, c1, c2);
   };
@@ -790,7 +796,7 @@ void rho_run(gks_ctx* c, const T* C, int ldc, long long sC, T* rho, long long sR
   for (; per > 0 && z0 < nk; z0 += per) {
     const int cnt = std::min(per, nk - z0);
     if (!ozaki_gemm<T>(OP_N, OP_C, M, M, K, 1.0, C + z0 * sC, ldc, sC, C + z0 * sC, ldc, sC, 0.0, rho + z0 * sR, M,
-                       sR, cnt, 1, sform(c), c->oz, c->st ? c->st : c->gst, c->stream, ks + z0 * sks, sks,
+                       sR, cnt, 1, sform(c), c->sx.oz, c->st ? c->st : c->gst, c->stream, ks + z0 * sks, sks,
                        nrho + z0, c->wait_cycles))
       break;  // tensor maps unavailable: the FP64 kernel takes the remaining items
   }
@@ -1012,7 +1018,7 @@ void hegst_run(gks_ctx* c, T* A, int lda, long long sA, const T* L, int ldl, lon
     T* A22 = A21 + KB;
     auto level = [&]() {
       hegst_level<T>(c, A11, lda, sA, L11, ldl, sL, KB, nk);
-      if (beside) cudaEventRecord(c->events[EV_LEVEL], c->stream);
+      if (beside) cudaEventRecord(c->sx.events[EV_LEVEL], c->stream);
     };
     if (chol) main_wait(c, EV_PANEL + K0 / nbb);
     if (beside) {
@@ -1437,7 +1443,7 @@ template <typename T, typename TA = T>
 void wy_ahead(gks_ctx* c, const TA* A, int M, int nk, int blk) {
   lane_run(c, 0, [&]() {
     wy_prepare<T, TA>(c, A, M, nk, blk);
-    cudaEventRecord(c->events[EV_WY + (blk & 1)], c->stream);
+    cudaEventRecord(c->sx.events[EV_WY + (blk & 1)], c->stream);
   });
 }
 template <typename T, typename TA = T>
@@ -1473,8 +1479,8 @@ void backtransform_run(gks_ctx* c, const TA* A, T* X, int ldx, long long sX, int
     gmx<T>(c, nk, OP_N, OP_N, nbk, ncols, nbk, 1.0, Tm, nbb, c->sT, Y, ncols, c->sY, 0.0, Y2, ncols, c->sY);
     gmx<T>(c, nk, OP_N, OP_N, j1, ncols, nbk, -1.0, V, nbb, c->sV, Y2, ncols, c->sY, 1.0, X, ldx, sX);
     if (beside && blk + 2 < blocks) {
-      cudaEventRecord(c->events[EV_FREE + (blk & 1)], c->stream);
-      cudaStreamWaitEvent(c->lane[0].stream, c->events[EV_FREE + (blk & 1)], 0);
+      cudaEventRecord(c->sx.events[EV_FREE + (blk & 1)], c->stream);
+      cudaStreamWaitEvent(c->sx.lane[0].stream, c->sx.events[EV_FREE + (blk & 1)], 0);
       wy_ahead<T, TA>(c, A, M, nk, blk + 2);
     }
   }
@@ -1500,7 +1506,7 @@ bool standard_eig(gks_ctx* c, T* A, T* X, long long sX, double* w, int M, int it
     const size_t item = dc_split_item_bytes(c->dc, sp.min_half, sform(c));
     if (item > 0) {
       sp.per = oz_reserve(c, item, items);
-      sp.work = c->oz;
+      sp.work = c->sx.oz;
     }
   }
   dc_solve(c->dc, d, e, M, w, Z, c->sMM, c->ws + c->odc, c->st, s, &c->prof, &sp);
@@ -1644,7 +1650,7 @@ gks_status solve_t(gks_ctx* c, const SolveKey& key) {
           Rec r(c, PC_MISC);
           copy2d<T>(L + c->sMM + K0, n, sLk, L + K0, n, sLk, n, KB, nk, c->stream);
         }
-        if (chol) cudaEventRecord(c->events[EV_PANEL + p], c->stream);
+        if (chol) cudaEventRecord(c->sx.events[EV_PANEL + p], c->stream);
       });
     };
     if (chol) {
@@ -1677,7 +1683,7 @@ gks_status solve_t(gks_ctx* c, const SolveKey& key) {
       auto off = [&]() {
         trsm_left_run<T>(c, L, n, c->sMM, A + (size_t)n * M, M, c->sMM, n, n, nk, false);
         trsm_right_conj_run<T>(c, L, n, c->sMM, A + (size_t)n * M, M, c->sMM, n, n, nk);
-        if (beside) cudaEventRecord(c->events[EV_OFF], c->stream);
+        if (beside) cudaEventRecord(c->sx.events[EV_OFF], c->stream);
       };
       if (beside && !chol) lane_fork(c, 1);
       if (beside) lane_run(c, 1, off);
@@ -1742,7 +1748,7 @@ gks_status solve_t(gks_ctx* c, const SolveKey& key) {
       const size_t item = dc_split_item_bytes(c->dc, sp_.min_half, sform(c));
       if (item > 0) {
         sp_.per = oz_reserve(c, item, items);
-        sp_.work = c->oz;
+        sp_.work = c->sx.oz;
       }
     }
     dc_solve(c->dc, d, e, M, eps, Z, c->sMM, c->ws + c->odc, c->st, s, &c->prof, &sp_);
@@ -1957,6 +1963,52 @@ gks_status enqueue_solve(gks_ctx* ctx, const SolveKey& k) {
   return solve_t<zc>(ctx, k);
 }
 
+// Split scratch of one problem of a batch: the main stream's (the density matrix's product), and
+// a lane's (the factorization's first trailing update).
+void scratch_estimate(gks_ctx* c, const SolveKey& k, size_t* main, size_t* lane) {
+  const bool nc = k.spin == GKS_NONCOLLINEAR;
+  const int n = (int)k.n, M = nc ? 2 * n : n, es = k.dtype == GKS_R64 ? 8 : 16;
+  const int items = (int)k.nk * (k.spin == GKS_SPIN_POLARIZED ? 2 : 1), nev = ncols_of(c, M);
+  const int w = pick_width(c, M, es, shape_spin(k.spin)), rest = n - w;
+  auto need = [&](int m, int cols, int K, int count, int lower) -> size_t {
+    if (m <= 0 || !split_worth(c, count, m, cols, K, es, lower)) return 0;
+    const size_t item = ozaki_workspace_bytes(m, cols, K, es == 16, sform(c));
+    return std::max(item, std::min(item * count, kOzCap));
+  };
+  *main = need(M, M, nev, items, 0);
+  *lane = need(rest, rest, w, (int)k.nk, 1);
+}
+
+// Whether a batch's problems share scratch by worker stream (a worker's problems run one after
+// another): where scratch of their own would take more than the 12 GB that one launch may.  Own
+// scratch costs less time (48 systems of order 208 to 1144: 132 against 134 ms, first pass 182
+// against 472 when the shared one grows), so smaller batches keep it.  The shared scratch is
+// sized for the largest problem at once: growing it waits for the worker.
+void share_scratch(gks_ctx* ctx, const std::vector<SolveKey>& keys, int P) {
+  size_t all = 0;
+  std::vector<size_t> main(P, 0), lane(P, 0);
+  for (size_t b = 0; b < keys.size(); b++) {
+    size_t m = 0, l = 0;
+    scratch_estimate(ctx->subs[b], keys[b], &m, &l);
+    const gks_ctx::Scratch& x = ctx->subs[b]->sx;
+    all += std::max(m + 2 * l, x.oz_bytes + x.lane[0].oz_bytes + x.lane[1].oz_bytes);
+    main[b % P] = std::max(main[b % P], m);
+    lane[b % P] = std::max(lane[b % P], l);
+  }
+  ctx->bshare = all > kOzCap;
+  if (!ctx->bshare) return;
+  for (auto* sc : ctx->subs) release_scratch(sc->sx);
+  for (int w = 0; w < P; w++) {
+    gks_ctx* sc = ctx->subs[w];
+    sc->stream = ctx->workers[w];
+    std::swap(sc->sx, ctx->wsx[w]);
+    if (main[w]) oz_reserve(sc, main[w], 1);
+    if (lane[w] && lanes_ready(sc, 0))
+      for (int q = 0; q < 2; q++) lane_run(sc, q, [&]() { oz_reserve(sc, lane[w], 1); });
+    std::swap(sc->sx, ctx->wsx[w]);
+  }
+}
+
 bool same_key(const SolveKey& a, const SolveKey& b) { return std::memcmp(&a, &b, sizeof(SolveKey)) == 0; }
 
 // Capture whatever `body` enqueues on c->stream into a graph and instantiate it.  *out stays
@@ -2125,15 +2177,14 @@ gks_status gks_destroy(gks_ctx* ctx) {
   for (auto sc : ctx->subs) {
     release_ws(sc);
     release_aws(sc);
-    release_oz(sc);
-    release_lanes(sc);
+    release_scratch(sc->sx);
     delete sc;
   }
+  for (auto& x : ctx->wsx) release_scratch(x);
   for (auto w : ctx->workers) cudaStreamDestroy(w);
   release_ws(ctx);
   release_aws(ctx);
-  release_oz(ctx);
-  release_lanes(ctx);
+  release_scratch(ctx->sx);
   release_extra(ctx);
   delete ctx;
   return GKS_OK;
@@ -2204,6 +2255,7 @@ gks_status gks_solve_batched(gks_ctx* ctx, int64_t count, const gks_problem* pro
     cudaStream_t w;
     if (cudaStreamCreateWithFlags(&w, cudaStreamNonBlocking) != cudaSuccess) return cuda_check(ctx, "stream create");
     ctx->workers.push_back(w);
+    ctx->wsx.emplace_back();
   }
   while ((int64_t)ctx->subs.size() < count) {
     gks_ctx* sc = new gks_ctx();
@@ -2239,7 +2291,9 @@ gks_status gks_solve_batched(gks_ctx* ctx, int64_t count, const gks_problem* pro
       gks_ctx* sc = ctx->subs[b];
       sc->stream = ctx->workers[b % P];
       sc->prof.stream = sc->stream;
+      if (ctx->bshare) std::swap(sc->sx, ctx->wsx[b % P]);
       rc = enqueue_solve(sc, keys[b]);
+      if (ctx->bshare) std::swap(sc->sx, ctx->wsx[b % P]);
       if (rc) ctx->err = "problem " + std::to_string(b) + ": " + sc->err;
     }
     for (int w = 0; w < P; w++) {
@@ -2253,6 +2307,7 @@ gks_status gks_solve_batched(gks_ctx* ctx, int64_t count, const gks_problem* pro
     return rc;
   };
   if (!ctx->graph) {
+    share_scratch(ctx, keys, P);
     gks_status rc = body();
     return rc ? rc : cuda_check(ctx, "gks_solve_batched launch");
   }
@@ -2269,6 +2324,7 @@ gks_status gks_solve_batched(gks_ctx* ctx, int64_t count, const gks_problem* pro
                      !std::equal(keys.begin(), keys.end(), ctx->bkey.begin(), same_key);
   ctx->bkey = keys;
   if (first) {  // eager run: allocates every problem's workspace and merge lists
+    share_scratch(ctx, keys, P);
     gks_status rc = body();
     return rc ? rc : cuda_check(ctx, "gks_solve_batched launch");
   }
