@@ -127,7 +127,11 @@ enum {
 enum {
   /* The next split product on this context leaves out one operand copy in every CTA, so
    * that its bounded waits expire and gks_sync reports GKS_ETIMEOUT; no fault, no trap. */
-  GKS_DEBUG_SKIP_COPY = 1
+  GKS_DEBUG_SKIP_COPY = 1,
+  /* The first panel of the next one-stage reduction (digit form) waits at one of its barriers
+   * for an arrival more than its CTAs make, so that the bounded waits expire and gks_sync
+   * reports GKS_ETIMEOUT. */
+  GKS_DEBUG_LATE_ARRIVAL = 2
 };
 
 typedef struct {

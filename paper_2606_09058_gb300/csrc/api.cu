@@ -1120,6 +1120,8 @@ bool hetrd_digit_run(gks_ctx* c, T* A, int M, int nk) {
   pa.hd.ldd = ldd;
   // the grid barriers' CTAs are all resident: a limit chosen for copies does not cut them short
   pa.wait = std::max(c->wait_cycles, 1ll << 28);
+  pa.late = (c->debug & GKS_DEBUG_LATE_ARRIVAL) ? 1 : 0;
+  c->debug &= ~GKS_DEBUG_LATE_ARRIVAL;
   cudaMemsetAsync(at<unsigned>(c, c->opbar), 0, sizeof(unsigned) * 4 * nk, s);
   HemvDigits hd = pa.hd;
   hd.D = at<signed char>(c, c->oD);
@@ -1165,6 +1167,7 @@ bool hetrd_digit_run(gks_ctx* c, T* A, int M, int nk) {
           return false;
         }
       }
+      pa.late = 0;
     }
     panel_deferred<T>(c, A, M, jl, steps, nk);
   }
@@ -2141,7 +2144,7 @@ gks_status gks_create(gks_ctx** ctx, const gks_opts* opts) {
         (c->tridiag != GKS_TRIDIAG_ONE_STAGE && c->tridiag != GKS_TRIDIAG_TWO_STAGE) || c->band < 2 ||
         c->band > 32 || (c->split != GKS_SPLIT_RESIDUES && c->split != GKS_SPLIT_DIGITS) ||
         (c->hemv != GKS_HEMV_DIGITS && c->hemv != GKS_HEMV_FP64) ||
-        (opts->debug & ~GKS_DEBUG_SKIP_COPY)) {
+        (opts->debug & ~(GKS_DEBUG_SKIP_COPY | GKS_DEBUG_LATE_ARRIVAL))) {
       delete c;
       return GKS_EINVAL;
     }

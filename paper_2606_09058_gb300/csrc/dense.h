@@ -103,6 +103,7 @@ struct PanelArgs {
   HemvDigits hd;
   DevStatus* st;
   long long wait;
+  int late;  // test hook: arrivals that the vector warps' barrier waits for beyond those made
 };
 // Items per launch, of `items`, for panels of order jh and below: all in the cluster form, else
 // as many as the grid form can give a resident CTA each.

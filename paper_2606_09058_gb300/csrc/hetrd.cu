@@ -863,7 +863,7 @@ __global__ void __launch_bounds__(kPanelThreads, 1) hetrd_panel_kernel(const Pan
     if (tid == 0) {
       for (int q = 0; q < 4; q++)
         asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"((unsigned)__cvta_generic_to_shared(&s_bar[q])),
-                     "r"(G));
+                     "r"(q < 2 ? G : G + a.late));
       asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
     cluster_sync_all();
@@ -1431,7 +1431,7 @@ bool hetrd_panel(PanelArgs<T> a, int items, unsigned* base, unsigned* basev, cud
   // U y1 + Q y2 behind the product from kEarlyTiles tiles per CTA up
   a.early = (long long)((a.jh + 31) / 32) * ((a.jh + 15) / 16) >= (long long)kEarlyTiles<T> * G;
   a.base = *base;
-  a.basev = *basev;
+  a.basev = *basev + a.late;
   cudaLaunchConfig_t cfg{};
   cudaLaunchAttribute at{};
   cfg.gridDim = dim3(G, items);

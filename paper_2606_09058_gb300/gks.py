@@ -19,6 +19,7 @@ GKS_COLLINEAR, GKS_NONCOLLINEAR, GKS_SPIN_POLARIZED = 0, 1, 2
 GKS_FP64, GKS_MIXED_TF32, GKS_MIXED_SPLITBF16 = 0, 1, 2
 GKS_REUSE_S_FACTOR, GKS_SAVE_FOR_BACKWARD, GKS_EIGEN_ONLY = 1, 2, 4
 GKS_DEBUG_SKIP_COPY = 1
+GKS_DEBUG_LATE_ARRIVAL = 2
 GKS_SPLIT_RESIDUES, GKS_SPLIT_DIGITS = 0, 1
 GKS_HEMV_DIGITS, GKS_HEMV_FP64 = 0, 1
 _SPIN = {"collinear": GKS_COLLINEAR, "noncollinear": GKS_NONCOLLINEAR, "spin_polarized": GKS_SPIN_POLARIZED}
