@@ -1643,11 +1643,17 @@ gks_status solve_t(gks_ctx* c, const SolveKey& key) {
     // (whole call, one after the other / beside: order 4992 complex 387 / 376 ms, four of order
     // 1625 complex 98.7 / 95.1, order 832 real 20.0 / 19.1)
     chol = lanes_ready(c, (n + c->nbb - 1) / c->nbb);
+    const int rest = n - c->nbb;  // the first trailing update's scratch at once
+    const size_t first = rest > 0 && split_worth(c, nk, rest, rest, c->nbb, es, 1)
+                             ? ozaki_workspace_bytes(rest, rest, c->nbb, es == 16, sform(c)) : 0;
+    if (chol) {
+      lane_fork(c, 1);
+      // no memory for a second workspace: on the main stream, with its own
+      if (first) lane_run(c, 1, [&]() { chol = oz_reserve(c, first, nk) > 0; });
+    }
     auto factor = [&]() {
       StageRec sr(c, PS_POTRF);
-      const int rest = n - c->nbb;  // the first trailing update's scratch at once
-      if (rest > 0 && split_worth(c, nk, rest, rest, c->nbb, es, 1))
-        oz_reserve(c, ozaki_workspace_bytes(rest, rest, c->nbb, es == 16, sform(c)), nk);
+      if (!chol && first) oz_reserve(c, first, nk);
       potrf_run<T>(c, L, n, n, sLk, nk, [&](int p, int K0, int KB) {
         if (sp) {
           Rec r(c, PC_MISC);
@@ -1656,12 +1662,8 @@ gks_status solve_t(gks_ctx* c, const SolveKey& key) {
         if (chol) cudaEventRecord(c->sx.events[EV_PANEL + p], c->stream);
       });
     };
-    if (chol) {
-      lane_fork(c, 1);
-      lane_run(c, 1, factor);
-    } else {
-      factor();
-    }
+    if (chol) lane_run(c, 1, factor);
+    else factor();
     c->lkey = key;
     c->l_valid = true;
   }
@@ -2043,6 +2045,7 @@ gks_status capture(gks_ctx* c, cudaGraphExec_t* out, F body) {
   }
   if (rc || dropped) {
     if (g) cudaGraphDestroy(g);
+    if (dropped) cudaGetLastError();  // a lane that was forked for nothing
     return rc;
   }
   if (e != cudaSuccess || !g) return fail(c, GKS_ECUDA, std::string("graph capture: ") + cudaGetErrorString(e));
