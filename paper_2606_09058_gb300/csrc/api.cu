@@ -1098,8 +1098,7 @@ int panel_width(const gks_ctx* c, int M) {
 
 // One-stage Householder tridiagonalization with the digit form of the matrix-vector step:
 // per panel the digits of the stale block, one persistent launch for its steps, and the
-// deferred update as two lower-triangle products with K = the panel's step count.  False if
-// a cooperative launch was refused.
+// deferred update (panel_deferred).  False if a launch was refused.
 template <typename T>
 bool hetrd_digit_run(gks_ctx* c, T* A, int M, int nk) {
   cudaStream_t s = c->stream;
@@ -2284,9 +2283,7 @@ gks_status gks_solve_batched(gks_ctx* ctx, int64_t count, const gks_problem* pro
     sc->band = ctx->band;
     ctx->subs.push_back(sc);
   }
-  for (auto* sc : ctx->subs) {
-    sc->tuned = ctx->tuned;
-  }
+  for (auto* sc : ctx->subs) sc->tuned = ctx->tuned;
   auto body = [&]() -> gks_status {
     cudaEvent_t fork;
     cudaEventCreateWithFlags(&fork, cudaEventDisableTiming);

@@ -61,11 +61,11 @@ struct HemvDigits {
   int ldd;                   // columns per row, multiple of 16
   unsigned long long* rmax;  // [item][ldd] row maxima of the stale block (bits of doubles)
 };
-// Digits of the stale block [0:n, 0:n] (FP64 forms only).
 // W = [U | Q | U] scaled by columns, the operands of the deferred update as one product.
 template <typename T>
 void panel_pack(const T* U, const T* Q, int ldu, long long sU, int n, int kp, T* W, long long sW, int count,
                 cudaStream_t s);
+// Digits of the stale block [0:n, 0:n] (FP64 forms only).
 template <typename T>
 void hetrd_digits(const T* A, int lda, long long sA, int n, const HemvDigits& hd, int count, cudaStream_t s);
 // One panel of the digit form: steps jh .. jl.  Per item (strides in elements): arow 2 x sv,

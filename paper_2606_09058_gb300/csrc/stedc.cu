@@ -99,7 +99,7 @@ __global__ void dc_tear_kernel(double* d, const double* e, long long sde, const 
 // 220 us here.
 __global__ void __launch_bounds__(32) dc_leaf_kernel(const double* d, const double* e, long long sde, double* lam,
                                                      long long slam, double* Z, long long sZ, int m,
-                                                     const int* leaves, int nleaves, DevStatus* st) {
+                                                     const int* leaves, DevStatus* st) {
   __shared__ double dd[DC_LEAF], ee[DC_LEAF], zr[DC_LEAF][33];
   const int z = blockIdx.y, leaf = blockIdx.x, lane = threadIdx.x;
   const int off = leaves[2 * leaf], n = leaves[2 * leaf + 1];
@@ -817,8 +817,7 @@ void dc_solve(DcPlan* p, double* d, double* e, long long sde, double* lam, doubl
   dc_tear_kernel<<<cnt, 256, 0, s>>>(d, e, sde, p->d_splits, (int)p->splits.size());
   const int nleaves = (int)p->leaves.size() / 2;
   count_launch();
-  dc_leaf_kernel<<<dim3(nleaves, cnt), 32, 0, s>>>(d, e, sde, lamBuf[0], slam, zbuf0, sZ0, m, p->d_leaves, nleaves,
-                                                   st);
+  dc_leaf_kernel<<<dim3(nleaves, cnt), 32, 0, s>>>(d, e, sde, lamBuf[0], slam, zbuf0, sZ0, m, p->d_leaves, st);
   prof->end(tok, PC_DC_LEAF, 0.0, 0.0);
   for (int t = 0; t < p->depth; t++) {
     DcLevel& L = p->levels[t];
