@@ -141,7 +141,9 @@ typedef struct {
   double f_cut;        /* occupations below f_cut are left out of rho (default 1e-16) */
   int profile;         /* 1: record CUDA events around every launch group (see gks_profile) */
   int graph;           /* 1: capture each solve (and each batch) into a CUDA graph and replay it
-                          while the arguments are unchanged; needs a non-default stream */
+                          while the arguments are unchanged; needs a non-default stream.  A graph
+                          that the caller captures holds the context's workspace: it is valid
+                          until a call of another shape or entry point replaces that */
   int gemm;            /* FP64 products: 0 = large ones as exact split-bf16 tensor-core products
                           with FP64 accumulation, small ones on the FP64 pipe (default);
                           1 = FP64 pipe only; 2 = split products for every product */
