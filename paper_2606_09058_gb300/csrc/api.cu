@@ -648,6 +648,14 @@ int oz_reserve(gks_ctx* c, size_t item, int count) {
   return per;
 }
 
+// Planes and residues of one split product in the residue form (bytes).
+double split_bytes(int M, int N, int K, int es) {
+  auto up = [](int v, int to) { return (double)((v + to - 1) / to * to); };
+  const int e = es == 16 ? 2 : 1;
+  const double Mp = up(M, 128), Np = up(e * N, 256), Kp = up(e * K, 64);
+  return 16.0 * ((Mp + Np) * Kp * 2.0 + Mp * Np);
+}
+
 // Split products where the FP64 kernel would take longer than their fixed cost (three or four
 // launches, about 30 us) and every dimension is at least 32.  The FP64 kernel's 16 x 16 tiles
 // take 0.073 us (complex 0.294) per inner index on their SM, whatever shares the other SMs.
@@ -666,10 +674,7 @@ bool split_worth(gks_ctx* c, int count, int M, int N, int K, int es, int lower) 
   const long long tiles = (long long)((M + 15) / 16) * ((N + 15) / 16) * count / (lower ? 2 : 1);
   const double round = K * (es == 16 ? 0.294 : 0.073);
   if ((double)((tiles + 151) / 152) * round < kSplitUs) return false;
-  auto up = [](int v, int to) { return (double)((v + to - 1) / to * to); };
-  const int e = es == 16 ? 2 : 1;
-  const double Mp = up(M, 128), Np = up(e * N, 256), Kp = up(e * K, 64);
-  const double bytes = 2.0 * 16.0 * count * ((Mp + Np) * Kp * 2.0 + Mp * Np);
+  const double bytes = 2.0 * count * split_bytes(M, N, K, es);  // written and read
   if (bytes <= kSplitCached) return true;
   const int t = gemm_tile(M, N, count, es);  // of the FP64 kernel
   const long long tm = (M + t - 1) / t, tn = (N + t - 1) / t, w = t / 16;
@@ -1976,7 +1981,7 @@ void scratch_estimate(gks_ctx* c, const SolveKey& k, size_t* main, size_t* lane)
   const int w = pick_width(c, M, es, shape_spin(k.spin)), rest = n - w;
   auto need = [&](int m, int cols, int K, int count, int lower) -> size_t {
     if (m <= 0 || !split_worth(c, count, m, cols, K, es, lower)) return 0;
-    const size_t item = ozaki_workspace_bytes(m, cols, K, es == 16, sform(c));
+    const size_t item = (size_t)(1.01 * split_bytes(m, cols, K, es)) + 4096;  // and the scale codes
     return std::max(item, std::min(item * count, kOzCap));
   };
   *main = need(M, M, nev, items, 0);

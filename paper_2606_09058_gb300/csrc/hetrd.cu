@@ -1427,6 +1427,7 @@ template <typename T>
 bool hetrd_panel(PanelArgs<T> a, int items, unsigned* base, unsigned* basev, cudaStream_t s) {
   const int cl = panel_in_cluster(a.jh) ? panel_cluster_ctas<T>(items) : 0;
   const int G = cl > 0 ? cl : std::min(a.gs, hetrd_panel_ctas<T>(a.jh, items));
+  if (G < 1) return false;
   int maxseg = (a.jh + 31) / 32 / G + 2;
   const int steps = a.jh - a.jl + 1;
   // U y1 + Q y2 behind the product from kEarlyTiles tiles per CTA up
